@@ -1,0 +1,271 @@
+// fx.cuh -- 3x3 complex matrix products of FP64-class accuracy on the integer
+// pipe, for fields of SU(3) links.
+//
+// GB300 retires 2.2 FP64 multiply-adds per clock and SM and 32 integer ones
+// of 32 x 32 + 64 bits, which are exact, so a product of link matrices is
+// computed in fixed point.  A number |v| <= 1 is held as
+//   v = h 2^-30 + l 2^-60,   h, l signed 32-bit, |l| <= 2^29,
+// that is, to 2^-60 (FP64 rounds numbers near 1 to 2^-53), and
+//   a b = (h_a h_b) 2^-60 + (h_a l_b + l_a h_b) 2^-90 + O(2^-62):
+// three multiply-adds into two 64-bit sums.  Of the cross sum m only the high
+// word is kept (2^-58, rounded), which needs no 64-bit shift.  A complex
+// product takes three real ones (Gauss): with P1 = sum ar br, P2 = sum ai bi,
+// P3 = sum (ar + ai)(br + bi), the real part is P1 - P2 and the imaginary
+// part P3 - P1 - P2, all exact in the h sums.  Error of an entry: about 2^-58,
+// thirty times below that of the FP64 chain of six multiply-adds.
+// One product costs a warp 1.3 k clocks of an SM quarter (81 x 3 wide
+// multiply-adds at 4 clocks each, the rest on the ALU pipe beside them;
+// measured; 1.5 k with four real products per complex one), against 6.3 k in
+// FP64.
+//
+// Range.  Every factor is unitary to 2^-12 or a product of such (checked for
+// the input links, see k_fx_links), so rows and columns have norm <= 1.01;
+// by Cauchy-Schwarz an entry's h sums stay below 2^61.1, and its cross sums,
+// with |ar + ai| and |br + bi| of row norm sqrt 2, below 2 sqrt(2) sqrt(3)
+// 2^60 < 2^62.4.
+#pragma once
+#include "su3.cuh"
+
+namespace stag {
+namespace fx {
+
+using su3::Dims;
+
+// One matrix: entry e = 3 row + column, [2 e] real, [2 e + 1] imaginary part.
+struct FM {
+  int h[18], l[18];
+};
+
+// Inline PTX: from C the compiler forms some of these as a 64-bit product and
+// an addition (1.3 times the time of a matrix product).
+__device__ __forceinline__ void wmad(long long& acc, int a, int b) {
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
+}
+__device__ __forceinline__ long long wmul(int a, int b) {
+  long long r;
+  asm("mul.wide.s32 %0, %1, %2;" : "=l"(r) : "r"(a), "r"(b));
+  return r;
+}
+
+// int64 in units of 2^-60 -> (h, l): h = round(s / 2^30), l = s - h 2^30
+__device__ __forceinline__ void split1(long long s, int& h, int& l) {
+  h = (int)((s + (1LL << 29)) >> 30);
+  l = ((int)((unsigned)s << 2)) >> 2;
+}
+__device__ __forceinline__ long long join1(int h, int l) { return ((long long)h << 30) + l; }
+
+// One entry of a b, in units of 2^-60.
+__device__ __forceinline__ void entry(const FM& a, const FM& b, int i, int j, long long& re, long long& im) {
+  constexpr long long half = 0x80000000LL;  // rounds the high word of a cross sum
+  long long p1, p2, p3, m1 = half, m2 = half, m3 = half;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int e = 2 * (3 * i + k), f = 2 * (3 * k + j);
+    const int sh = a.h[e] + a.h[e + 1], sl = a.l[e] + a.l[e + 1];
+    const int th = b.h[f] + b.h[f + 1], tl = b.l[f] + b.l[f + 1];
+    if (k == 0) {
+      p1 = wmul(a.h[e], b.h[f]);
+      p2 = wmul(a.h[e + 1], b.h[f + 1]);
+      p3 = wmul(sh, th);
+    } else {
+      wmad(p1, a.h[e], b.h[f]);
+      wmad(p2, a.h[e + 1], b.h[f + 1]);
+      wmad(p3, sh, th);
+    }
+    wmad(m1, a.h[e], b.l[f]);
+    wmad(m1, a.l[e], b.h[f]);
+    wmad(m2, a.h[e + 1], b.l[f + 1]);
+    wmad(m2, a.l[e + 1], b.h[f + 1]);
+    wmad(m3, sh, tl);
+    wmad(m3, sl, th);
+  }
+  // high words, units of 2^-58; the differences are below 2^31 whatever the terms (unsigned: modulo 2^32)
+  const unsigned c1 = (unsigned)(m1 >> 32), c2 = (unsigned)(m2 >> 32), c3 = (unsigned)(m3 >> 32);
+  re = p1 - p2 + (long long)(int)(c1 - c2) * 4;
+  im = p3 - p1 - p2 + (long long)(int)(c3 - c1 - c2) * 4;
+}
+
+// a b
+__device__ __forceinline__ FM mul(const FM& a, const FM& b) {
+  FM c;
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      long long re, im;
+      entry(a, b, i, j, re, im);
+      const int e = 2 * (3 * i + j);
+      split1(re, c.h[e], c.l[e]);
+      split1(im, c.h[e + 1], c.l[e + 1]);
+    }
+  return c;
+}
+
+// s (units of 2^-60) += a b; up to seven products of unitary matrices fit
+__device__ __forceinline__ void mac(long long (&s)[18], const FM& a, const FM& b) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      long long re, im;
+      entry(a, b, i, j, re, im);
+      const int e = 2 * (3 * i + j);
+      s[e] += re;
+      s[e + 1] += im;
+    }
+}
+
+__device__ __forceinline__ void clear(long long (&s)[18]) {
+#pragma unroll
+  for (int i = 0; i < 18; ++i) s[i] = 0;
+}
+
+// ------------------------------------------------------------ conversions (no FP64 instruction)
+// v 2^60 (|v| < 2, truncated towards zero)
+__device__ __forceinline__ long long fixed60(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const int r = 1023 - (int)((b >> 52) & 0x7ff);
+  const unsigned long long m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 8;  // 1.f at 2^60
+  const long long q = (long long)(m >> (r > 63 ? 63 : r));
+  return (long long)b < 0 ? -q : q;
+}
+// s 2^k, rounded to nearest; the result must be a normal number (or s = 0)
+__device__ __forceinline__ double double_of(long long s, int k) {
+  const unsigned long long a0 = (unsigned long long)(s < 0 ? -s : s);
+  const int z = __clzll((long long)a0);
+  const unsigned long long a = a0 << (z & 63);
+  const unsigned long long m = (a >> 11) + ((a >> 10) & 1);  // 53 bits, leading bit at 52
+  unsigned long long b = ((unsigned long long)(unsigned)(1023 + 62 - z + k) << 52) + m;
+  b = a0 == 0 ? 0 : b;
+  return __longlong_as_double((long long)(b | ((unsigned long long)s & 0x8000000000000000ull)));
+}
+// A coefficient |c| <= 1 in the same form, and c s for |s| <= 2^60.
+struct Coef {
+  int h, l;
+};
+__device__ __forceinline__ long long scaled(Coef c, long long s) {
+  int h, l;
+  split1(s, h, l);
+  long long p = wmul(c.h, h), m = 0x80000000LL;
+  wmad(m, c.h, l);
+  wmad(m, c.l, h);
+  return p + ((long long)(int)(m >> 32) << 2);
+}
+// Host: c = coefficient 2^k with a common k for a set of coefficients.
+inline Coef make_coef(double c) {  // |c| <= 1
+  Coef r;
+  const double s = c * 0x1p30;
+  const long long h = (long long)(s < 0 ? s - 0.5 : s + 0.5);
+  r.h = (int)h;
+  r.l = (int)((s - (double)h) * 0x1p30);
+  return r;
+}
+
+// ------------------------------------------------------------ field layout
+// Tiles of 32 consecutive sites; in a tile, one row of 32 int4 {re.h, re.l,
+// im.h, im.l} per entry: [site / 32][slot][entry][site % 32].  A warp's loads
+// over consecutive sites are whole 512-byte rows, and the nine entries of a
+// matrix lie at constant offsets from one address.
+constexpr int TS = 32;
+inline size_t field_bytes(long long V, int slots) { return (size_t)((V + TS - 1) / TS) * TS * slots * 9 * sizeof(int4); }
+__device__ __forceinline__ size_t row0(int slots, int site, int slot) {
+  return (size_t)((site >> 5) * slots + slot) * 288 + (site & 31);
+}
+template <int SLOTS> __device__ __forceinline__ FM ld(const int4* __restrict__ f, int slot, int site) {
+  FM m;
+  const int4* p = f + row0(SLOTS, site, slot);
+#pragma unroll
+  for (int e = 0; e < 9; ++e) {
+    const int4 q = __ldg(p + e * 32);
+    m.h[2 * e] = q.x;
+    m.l[2 * e] = q.y;
+    m.h[2 * e + 1] = q.z;
+    m.l[2 * e + 1] = q.w;
+  }
+  return m;
+}
+template <int SLOTS> __device__ __forceinline__ void st(int4* __restrict__ f, int slot, int site, const FM& m) {
+  int4* p = f + row0(SLOTS, site, slot);
+#pragma unroll
+  for (int e = 0; e < 9; ++e) p[e * 32] = make_int4(m.h[2 * e], m.l[2 * e], m.h[2 * e + 1], m.l[2 * e + 1]);
+}
+// m, or its adjoint (adj: 0 or -1): one code path for factors that are daggered
+// in some terms of a loop keeps the loop inside the instruction cache.
+__device__ __forceinline__ void adjoint_if(FM& m, int adj) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    m.h[8 * i + 1] = (m.h[8 * i + 1] ^ adj) - adj;
+    m.l[8 * i + 1] = (m.l[8 * i + 1] ^ adj) - adj;
+#pragma unroll
+    for (int j = i + 1; j < 3; ++j) {
+      const int e = 2 * (3 * i + j), f = 2 * (3 * j + i);
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const int eh = m.h[e + c], el = m.l[e + c], fh = m.h[f + c], fl = m.l[f + c], sg = c ? adj : 0;
+        m.h[e + c] = ((adj ? fh : eh) ^ sg) - sg;
+        m.l[e + c] = ((adj ? fl : el) ^ sg) - sg;
+        m.h[f + c] = ((adj ? eh : fh) ^ sg) - sg;
+        m.l[f + c] = ((adj ? el : fl) ^ sg) - sg;
+      }
+    }
+  }
+}
+
+// A site's index and coordinates in 32 bits (the entry points take at most 2^31
+// sites): 64-bit index products would run on the wide multiply-add pipe.
+struct Site {
+  int lex;
+  su3::C4 c;
+};
+__device__ __forceinline__ Site site_of(const Dims& d, int x) {
+  Site p;
+  p.lex = x;
+  const int r = x / d.L0, q = r / d.L1;
+  p.c.x = x - r * d.L0;
+  p.c.y = r - q * d.L1;
+  p.c.t = q / d.L2;
+  p.c.z = q - p.c.t * d.L2;
+  return p;
+}
+// The index of p moved by k = +-1 along mu (periodic).
+__device__ __forceinline__ int next_lex(const Dims& d, const Site& p, int mu, int k) {
+  const int L = su3::extent(d, mu), v = p.c.get(mu);
+  const int st = mu == 0 ? 1 : mu == 1 ? d.L0 : mu == 2 ? d.L0 * d.L1 : d.L0 * d.L1 * d.L2;
+  const int w = v + k;
+  return p.lex + st * ((w >= L ? w - L : w < 0 ? w + L : w) - v);
+}
+__device__ __forceinline__ Site next(const Dims& d, const Site& p, int mu, int k) {
+  Site q = p;
+  q.lex = next_lex(d, p, mu, k);
+  const int L = su3::extent(d, mu);
+  int w = p.c.get(mu) + k;
+  w = w >= L ? w - L : w < 0 ? w + L : w;
+  q.c.x = mu == 0 ? w : q.c.x;
+  q.c.y = mu == 1 ? w : q.c.y;
+  q.c.z = mu == 2 ? w : q.c.z;
+  q.c.t = mu == 3 ? w : q.c.t;
+  return q;
+}
+
+// ------------------------------------------------------------ canonical fields
+// A block of 128 threads takes one tile of 32 sites; warp w the direction
+// mu = w of each.  The canonical field [V][4][3][3] of those sites is one
+// contiguous 18 KB piece, moved through shared memory with whole-warp
+// contiguous accesses; there a site takes 592 B (37 16-byte words, odd: the
+// eight threads of a 128-bit access phase fall in different bank groups).
+constexpr int SITE_W = 37;
+
+// Bits of *status, set by k_fx_links: some link is not unitary to 2^-12 (or
+// not finite); some link is at least 2^-5 away from the unit matrix.
+enum : int { FX_NOT_UNITARY = 1, FX_AWAY = 2 };
+// The integer kernels run on FX_AWAY alone.  Links all close to the unit
+// matrix stay on the FP64 kernels: their small entries, and a force made of
+// them, would be known to 2^-58 absolute where FP64 keeps 2^-53 relative.
+__device__ __forceinline__ bool usable(const int* status) { return __ldcg(status) == FX_AWAY; }
+
+// Fixed-point copy of the thin links [V][4][3][3] into slots slot0 + mu of a
+// field with `slots` slots, and *status (fx.cu).
+int launch_fx_links(long long V, const double2* U, int4* out, int slots, int slot0, int* status, cudaStream_t st);
+
+}  // namespace fx
+}  // namespace stag

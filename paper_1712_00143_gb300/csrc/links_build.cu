@@ -9,20 +9,27 @@
 //                                               + U_nu(x-nu)^dag U_mu(x-nu) U_nu(x-nu+mu) ]
 //   L_mu(x) = c3 U_mu(x) U_mu(x+mu) U_mu(x+2mu)
 // One thread per (site, direction): 12 staple products and 2 Naik products
-// of 3x3 complex matrices (about 1500 FP64 FMA), inputs from L2 (each thin
-// link is read by up to 19 threads), outputs written once in the canonical
-// layout.  Bound by the FP64 pipe on GB300 (about 1.2 TFLOP/s).
-#include "su3.cuh"
+// of 3x3 complex matrices (about 1500 real multiply-adds), inputs from L2
+// (each thin link is read by up to 19 threads).  Links that are SU(3) matrices
+// go through the fixed-point products of fx.cuh on the integer pipe; any
+// other input, and links all close to 1, through the FP64 kernel.
+#include <cmath>
+
+#include "fx.cuh"
 
 namespace stag {
 namespace lb {
 using namespace su3;
 
+// FP64 form: bound by the FP64 pipe (10.8 ms at 32^4, 1.2 TFLOP/s).  With a
+// status word it runs only when the integer kernel may not, in a grid of a
+// few blocks per SM whose blocks return at once otherwise.
 __global__ void __launch_bounds__(128) k_build_links(Dims d, long long V, const double2* __restrict__ U,
                                                      double2* __restrict__ F, double2* __restrict__ Lk, double c1,
-                                                     double cst, double c3) {
-  const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (idx >= 4 * V) return;
+                                                     double cst, double c3, const int* status) {
+  if (status && fx::usable(status)) return;
+  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < 4 * V;
+       idx += (long long)gridDim.x * blockDim.x) {
   const int mu = (int)(idx / V);
   const long long x = idx - (long long)mu * V;
   C4 c;
@@ -71,6 +78,63 @@ __global__ void __launch_bounds__(128) k_build_links(Dims d, long long V, const 
   double2* l = Lk + (x * 4 + mu) * 9;
 #pragma unroll
   for (int i = 0; i < 9; ++i) l[i] = make_double2(c3 * l3.e[i].x, c3 * l3.e[i].y);
+  }
+}
+
+// The fat links (12 products) or the Naik links (2 products) on the integer
+// pipe; two launches keep each loop's code small.  A block takes a tile of 32
+// sites, its warp w the direction mu = w: link loads are whole 512-byte rows,
+// the four directions of a site share their staples' links in L1, and the
+// outputs leave through shared memory as one contiguous piece.  The
+// coefficients, scaled by 2^-k to at most 1, are applied in fixed point too:
+// FP64 instructions at the end would cost a tenth of the whole kernel.  Bound
+// by the integer pipe (65 % busy with two blocks per SM; three or four blocks
+// measured the same).  24^4: conversion 0.06, fat 0.84, Naik 0.17 ms; the call
+// at 32^4 3.42 ms against 10.84 ms with the FP64 kernel.
+template <bool FAT>
+__global__ void __launch_bounds__(128, FAT ? 2 : 3) k_build_links_fx(Dims d, long long V, const int4* __restrict__ U,
+                                                        const int* __restrict__ status, double2* __restrict__ out,
+                                                        fx::Coef c1, fx::Coef cst, int k) {
+  if (!fx::usable(status)) return;
+  __shared__ double2 sm[fx::TS * fx::SITE_W];
+  const long long x0 = (long long)blockIdx.x * fx::TS;
+  const int ns = (int)(V - x0 < fx::TS ? V - x0 : fx::TS);
+  const int mu = threadIdx.x >> 5, s = threadIdx.x & 31;
+  if (s < ns) {
+    const fx::Site p = fx::site_of(d, (int)x0 + s), pm = fx::next(d, p, mu, 1);
+    double2* o = sm + s * fx::SITE_W + mu * 9;
+    long long acc[18];
+    fx::clear(acc);
+    if constexpr (FAT) {
+      // t = 0..5: direction nu, upper (U_nu(x) U_mu(x+nu) U_nu(x+mu)^dag) and
+      // lower (U_nu(x-nu)^dag U_mu(x-nu) U_nu(x-nu+mu)) staple
+#pragma unroll 1
+      for (int t = 0; t < 6; ++t) {
+        const int o3 = t >> 1, nu = o3 < mu ? o3 : o3 + 1, low = t & 1;
+        const int xm = fx::next_lex(d, p, nu, -1), xp = fx::next_lex(d, p, nu, 1);
+        fx::FM a = fx::ld<4>(U, nu, low ? xm : p.lex);
+        fx::adjoint_if(a, -low);
+        a = fx::mul(a, fx::ld<4>(U, mu, low ? xm : xp));
+        fx::FM c = fx::ld<4>(U, nu, low ? fx::next_lex(d, pm, nu, -1) : pm.lex);
+        fx::adjoint_if(c, low - 1);
+        fx::mac(acc, a, c);
+      }
+      const fx::FM u = fx::ld<4>(U, mu, p.lex);
+#pragma unroll
+      for (int e = 0; e < 18; ++e)  // the staple sum, of norm up to 6, enters as an eighth
+        acc[e] = fx::scaled(c1, fx::join1(u.h[e], u.l[e])) + fx::scaled(cst, (acc[e] + 4) >> 3);
+    } else {
+      // U_mu(x) U_mu(x+mu) U_mu(x+2mu)
+      fx::FM a = fx::mul(fx::ld<4>(U, mu, p.lex), fx::ld<4>(U, mu, pm.lex));
+      fx::mac(acc, a, fx::ld<4>(U, mu, fx::next_lex(d, pm, mu, 1)));
+#pragma unroll
+      for (int e = 0; e < 18; ++e) acc[e] = fx::scaled(c1, acc[e]);
+    }
+#pragma unroll
+    for (int e = 0; e < 9; ++e) o[e] = make_double2(fx::double_of(acc[2 * e], k), fx::double_of(acc[2 * e + 1], k));
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < ns * 36; i += 128) out[x0 * 36 + i] = sm[(i / 36) * fx::SITE_W + i % 36];
 }
 
 }  // namespace lb
@@ -96,9 +160,51 @@ extern "C" int stag_build_links(const int dims[4], const void* thin, void* fat, 
   };
   if (overlap(thin, fat) || overlap(thin, lng) || overlap(fat, lng)) return STAG_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
-  ProfScope ps("links", st);
-  const long long n = 4 * V;
-  lb::k_build_links<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(d, V, (const double2*)thin, (double2*)fat,
-                                                                  (double2*)lng, c1, c_staple, c3);
-  return last_launch_status();
+  const double2* U = (const double2*)thin;
+  auto fp64 = [&](const int* status) {
+    ProfScope ps("links", st);
+    const long long want = (4 * V + 127) / 128;
+    const unsigned grid = (unsigned)(status && want > 152 * 8 ? 152 * 8 : want);
+    lb::k_build_links<<<grid, 128, 0, st>>>(d, V, U, (double2*)fat, (double2*)lng, c1, c_staple, c3, status);
+    return last_launch_status();
+  };
+  // Coefficients as fixed point with a power of two taken out; beyond 2^+-900
+  // (or not finite) the FP64 kernel, whose range is wider.
+  const double big = std::fmax(std::fabs(c1), 8.0 * std::fabs(c_staple)), big3 = std::fabs(c3);
+  int k = 0, k3 = 0;
+  if (!(big > 0x1p-900 && big < 0x1p900 && big3 > 0x1p-900 && big3 < 0x1p900) || c1 != c1 || c_staple != c_staple)
+    return fp64(nullptr);
+  std::frexp(big, &k);
+  std::frexp(big3, &k3);
+  // the fixed-point copy of the links (576 B per site) in stream-ordered
+  // scratch; without room for it the FP64 kernel does the work
+  char* scratch = nullptr;
+  if (cudaMallocAsync((void**)&scratch, 256 + fx::field_bytes(V, 4), st) != cudaSuccess) {
+    cudaGetLastError();
+    return fp64(nullptr);
+  }
+  int* status = (int*)scratch;
+  int4* Uf = (int4*)(scratch + 256);
+  const unsigned tiles = (unsigned)((V + fx::TS - 1) / fx::TS);
+  const fx::Coef none{0, 0};
+  int s;
+  {
+    ProfScope ps("links", st);
+    s = fx::launch_fx_links(V, U, Uf, 4, 0, status, st);
+  }
+  if (!s) {
+    ProfScope ps("links", st);
+    lb::k_build_links_fx<true><<<tiles, 128, 0, st>>>(d, V, Uf, status, (double2*)fat, fx::make_coef(std::ldexp(c1, -k)),
+                                                      fx::make_coef(std::ldexp(c_staple, 3 - k)), k - 60);
+    s = last_launch_status();
+  }
+  if (!s) {
+    ProfScope ps("links", st);
+    lb::k_build_links_fx<false><<<tiles, 128, 0, st>>>(d, V, Uf, status, (double2*)lng,
+                                                       fx::make_coef(std::ldexp(c3, -k3)), none, k3 - 60);
+    s = last_launch_status();
+  }
+  if (!s) s = fp64(status);
+  const int f = cuda_status(cudaFreeAsync(scratch, st));
+  return s ? s : f;
 }
