@@ -18,9 +18,12 @@
 // (nu, rho distinct and != mu, s, r = +-1), and the force is
 //   F_mu(x) = (beta/3) TA[U_mu(x) Sigma_mu(x)],  TA(M) = (M - M^dag)/2 - Tr(M - M^dag)/6,
 // so that moving the link as exp(eps X) U changes S by -eps Re Tr(X F).
-// FP64 throughout; bound by the FP64 pipe on GB300.  The staples are built
-// from a stored table of three-link staples (below).
-#include "su3.cuh"
+// The staples are built from a stored table of three-link staples (below): on
+// the integer pipe (fx.cuh) when the links are SU(3) matrices, otherwise, and
+// when they are all close to 1, by the FP64 kernels.
+#include <cmath>
+
+#include "fx.cuh"
 
 namespace stag {
 namespace gf {
@@ -84,10 +87,13 @@ __device__ __forceinline__ M3 hop_at(const double2* __restrict__ U, const Dims& 
   return hop_link(U, d, p, dir, sgn);
 }
 
+// FP64 form; it and k_gauge_force_reuse run only when the integer kernels may
+// not (*status), in grids of a few blocks per SM that return at once otherwise.
 __global__ void __launch_bounds__(128) k_gf_staples(Dims d, long long V, const double2* __restrict__ U,
-                                                    double2* __restrict__ T) {
-  const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (idx >= 24 * V) return;
+                                                    double2* __restrict__ T, const int* status) {
+  if (fx::usable(status)) return;
+  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < 24 * V;
+       idx += (long long)gridDim.x * blockDim.x) {
   const int k = (int)(idx / V);  // mu * 6 + (other direction index) * 2 + sign
   const long long x = idx - (long long)k * V;
   const int mu = k / 6, o = (k % 6) >> 1, s = (k & 1) ? -1 : 1;
@@ -110,6 +116,7 @@ __global__ void __launch_bounds__(128) k_gf_staples(Dims d, long long V, const d
   double2* out = T + tslot(x, mu, nu, s);
 #pragma unroll
   for (int i = 0; i < 9; ++i) out[i] = m.e[i];
+  }
 }
 
 // acc += c m
@@ -123,9 +130,11 @@ __device__ __forceinline__ void axpy3(M3& acc, double c, const M3& m) {
 
 __global__ void __launch_bounds__(128) k_gauge_force_reuse(Dims d, long long V, const double2* __restrict__ U,
                                                            const double2* __restrict__ T, double2* __restrict__ F,
-                                                           double beta, double cpl, double crt, double cpg) {
-  const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (idx >= 4 * V) return;
+                                                           double beta, double cpl, double crt, double cpg,
+                                                           const int* status) {
+  if (fx::usable(status)) return;
+  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < 4 * V;
+       idx += (long long)gridDim.x * blockDim.x) {
   const int mu = (int)(idx / V);
   const long long x = idx - (long long)mu * V;
   Pos p0;
@@ -194,6 +203,197 @@ __global__ void __launch_bounds__(128) k_gauge_force_reuse(Dims d, long long V, 
 #pragma unroll
     for (int j = 0; j < 3; ++j)
       f[3 * i + j] = make_double2(k * a.e[3 * i + j].x, k * (a.e[3 * i + j].y - (i == j ? tr3 : 0.0)));
+  }
+}
+
+// ------------------------------------------------------------ fixed point
+// One field of 28 matrices per site: T(y; mu nu s) in slots 0..23, U_mu in 24..27.
+constexpr int SLOTS = 28, U0 = 24;
+__device__ __forceinline__ int fslot(int mu, int nu, int s) {
+  return mu * 6 + (nu < mu ? nu : nu - 1) * 2 + (s < 0 ? 1 : 0);
+}
+
+// The staple table, from the links in slots 24..27 of the same field: a block
+// takes 32 sites, its warp w the six staples of mu = w.  T is stored as the
+// adjoint of the path walked the other way, A B C with A or C daggered.
+__global__ void __launch_bounds__(128, 3) k_gf_staples_fx(Dims d, long long V, int4* __restrict__ T,
+                                                          const int* __restrict__ status) {
+  if (!fx::usable(status)) return;
+  const int x = blockIdx.x * fx::TS + (threadIdx.x & 31);
+  const int mu = threadIdx.x >> 5;
+  if (x >= V) return;
+  const fx::Site p = fx::site_of(d, x), pm = fx::next(d, p, mu, 1);
+#pragma unroll 1
+  for (int t = 0; t < 6; ++t) {
+    const int o = t >> 1, nu = o < mu ? o : o + 1, low = t & 1;
+    const int xm = fx::next_lex(d, p, nu, -1), xp = fx::next_lex(d, p, nu, 1);
+    fx::FM a = fx::ld<SLOTS>(T, U0 + nu, low ? xm : x);
+    fx::adjoint_if(a, -low);
+    a = fx::mul(a, fx::ld<SLOTS>(T, U0 + mu, low ? xm : xp));
+    fx::FM c = fx::ld<SLOTS>(T, U0 + nu, low ? fx::next_lex(d, pm, nu, -1) : pm.lex);
+    fx::adjoint_if(c, low - 1);
+    a = fx::mul(a, c);
+    fx::adjoint_if(a, -1);
+    fx::st<SLOTS>(T, mu * 6 + t, x, a);
+  }
+}
+
+// The force.  The products are grouped so that a factor common to several
+// staples is multiplied once, 51 per link:
+//   group 0    U_mu(x+mu) [sum_{nu,s} T(x+mu; mu nu s) T(x; mu nu s)]             rectangles 1
+//   group 1    [sum_{nu,s} T(x; mu nu s) T(x-mu; mu nu s)] U_mu(x-mu)             rectangles 2
+//   2..7       h(x+mu, nu, s) [c_rt T(x+s nu; mu nu s) h(x+s nu, nu, -s)
+//                              + c_pg sum_{rho,r} T(x+s nu; mu rho r) Q]          rectangles 3, parallelograms
+// All groups run through the same two matrix products (sum += a b inside a
+// group, S += P Q at its end), and what is done per entry runs in loops over
+// shared memory: code beyond the instruction cache cost 1.4 issue slots per
+// instruction (twelve warps, each at another place).  The coefficients, scaled
+// by 2^-k so that |c_pl| 6 + |c_rt| 18 + |c_pg| 24 <= 1, keep S within range.
+// Sums that are touched once per group (S, and a group's rectangle 3) wait in
+// shared memory, a column per thread: in registers they cost the third block
+// of an SM (255 registers, 4.4 ms at 24^4).  Bound by the integer pipe, 67 % busy (ncu),
+// the rest the latency of the table's loads at three warps per scheduler.
+// 24^4: conversion 0.06, table 0.72, force 3.6 ms; the call 4.6 ms against
+// 21.3 ms with the FP64 kernels.
+struct ForceCoef {
+  fx::Coef pl8, rt8, rt, pg4;  // 8 c_pl, 8 c_rt, c_rt, 4 c_pg, each times 2^-k
+  double off, diag;            // beta/3 times 2^(k-60) / 2 and / 3
+};
+__global__ void __launch_bounds__(128, 3) k_gauge_force_fx(Dims d, long long V, const int4* __restrict__ T,
+                                                           const int* __restrict__ status, double2* __restrict__ F,
+                                                           ForceCoef cf) {
+  if (!fx::usable(status)) return;
+  extern __shared__ __align__(16) unsigned char gf_sm[];
+  long long(*S)[128] = (long long(*)[128])gf_sm;  // [18][128]
+  long long(*lone)[128] = S + 18;                  // a group's rectangle 3
+  long long(*hold)[128] = S + 36;                  // a group's sum, then its weighted sum
+  double2* out = (double2*)gf_sm;                  // the block's output, at the end
+  const long long x0 = (long long)blockIdx.x * fx::TS;
+  const int ns = (int)(V - x0 < fx::TS ? V - x0 : fx::TS);
+  const int mu = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
+  double dg[3];    // the force: imaginary parts of the diagonal,
+  double2 off[3];  // entries 01, 02, 12
+  if (lane < ns) {
+    const fx::Site p0 = fx::site_of(d, (int)x0 + lane);
+    const fx::Site pp = fx::next(d, p0, mu, 1);
+    const int x = p0.lex, xm = fx::next_lex(d, p0, mu, -1);  // x, x - mu; pp = x + mu
+    {  // plaquettes
+      long long acc[18];
+      fx::clear(acc);
+#pragma unroll 1
+      for (int t = 0; t < 6; ++t) {
+        const fx::FM b = fx::ld<SLOTS>(T, mu * 6 + t, x);
+#pragma unroll
+        for (int e = 0; e < 18; ++e) acc[e] += fx::join1(b.h[e], b.l[e]);
+      }
+#pragma unroll
+      for (int e = 0; e < 18; ++e) S[e][tid] = acc[e];
+#pragma unroll 2
+      for (int e = 0; e < 18; ++e) {
+        S[e][tid] = fx::scaled(cf.pl8, S[e][tid] >> 3);
+        lone[e][tid] = 0;
+      }
+    }
+#pragma unroll 1
+    for (int g = 0; g < 8; ++g) {
+      // group g >= 2: its (nu, s); ps = x + s nu; qs = x (s > 0) or x - nu
+      const int gt = g < 2 ? 0 : g - 2, go = gt >> 1, gnu = go < mu ? go : go + 1, gs = (gt & 1) ? -1 : 1;
+      const int ps = fx::next_lex(d, p0, gnu, gs), qs = gs > 0 ? x : ps;
+      long long acc[18];
+      fx::clear(acc);
+      const int items = g < 2 ? 6 : 5;
+#pragma unroll 1
+      for (int t = 0; t < items; ++t) {
+        int sa, sb, xa = ps, xb = qs, adj;
+        if (g < 2) {
+          sa = sb = mu * 6 + t;
+          xa = g == 0 ? pp.lex : x;
+          xb = g == 0 ? x : xm;
+          adj = 0;
+        } else if (t == 0) {
+          sa = mu * 6 + gt;
+          sb = U0 + gnu;
+          adj = gs > 0 ? -1 : 0;
+        } else {
+          // (rho, r): the two directions other than mu and nu, both signs
+          int rho = (t - 1) >> 1;
+          const int lo = gnu < mu ? gnu : mu, hi = gnu < mu ? mu : gnu, r = (t & 1) ? 1 : -1;
+          rho += rho >= lo ? 1 : 0;
+          rho += rho >= hi ? 1 : 0;
+          sa = fslot(mu, rho, r);
+          sb = fslot(gnu, rho, r);
+          adj = gs > 0 ? 0 : -1;
+        }
+        const fx::FM a = fx::ld<SLOTS>(T, sa, xa);
+        fx::FM b = fx::ld<SLOTS>(T, sb, xb);
+        fx::adjoint_if(b, adj);
+        fx::mac(acc, a, b);
+        if (g >= 2 && t == 0) {
+#pragma unroll
+          for (int e = 0; e < 18; ++e) {
+            lone[e][tid] = acc[e];
+            acc[e] = 0;
+          }
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < 18; ++e) hold[e][tid] = acc[e];
+      {
+        const fx::Coef ca = g < 2 ? cf.rt8 : cf.pg4, cb = cf.rt;
+        const int sh = g < 2 ? 3 : 2;
+#pragma unroll 2
+        for (int e = 0; e < 18; ++e) {
+          int h, l;  // lone is 0 for the first two groups
+          fx::split1(fx::scaled(ca, hold[e][tid] >> sh) + fx::scaled(cb, lone[e][tid]), h, l);
+          ((int2*)&hold[e][tid])[0] = make_int2(h, l);
+        }
+      }
+      // the other factor: U_mu(x+mu), U_mu(x-mu), else h(x+mu, nu, s)
+      const int xh = g == 1 ? xm : g == 0 || gs > 0 ? pp.lex : fx::next_lex(d, pp, gnu, -1);
+      fx::FM P = fx::ld<SLOTS>(T, U0 + (g < 2 ? mu : gnu), xh), Q;
+      fx::adjoint_if(P, g >= 2 && gs < 0 ? -1 : 0);
+#pragma unroll
+      for (int e = 0; e < 18; ++e) {
+        const int2 q = ((const int2*)&hold[e][tid])[0];
+        Q.h[e] = g == 1 ? P.h[e] : q.x;
+        Q.l[e] = g == 1 ? P.l[e] : q.y;
+        P.h[e] = g == 1 ? q.x : P.h[e];
+        P.l[e] = g == 1 ? q.y : P.l[e];
+      }
+      fx::clear(acc);
+      fx::mac(acc, P, Q);
+#pragma unroll
+      for (int e = 0; e < 18; ++e) S[e][tid] += acc[e];
+    }
+    // F = (beta/3) TA[U S]; the differences are exact
+    fx::FM s;
+#pragma unroll
+    for (int e = 0; e < 18; ++e) fx::split1(S[e][tid], s.h[e], s.l[e]);
+    long long w[18];
+    fx::clear(w);
+    fx::mac(w, fx::ld<SLOTS>(T, U0 + mu, x), s);
+    const long long tr = w[1] + w[9] + w[17];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      dg[i] = cf.diag * fx::double_of(3 * w[8 * i + 1] - tr, 0);
+      const int r = i == 2 ? 1 : 0, c = i == 0 ? 1 : 2;  // entries 01, 02, 12
+      const int e = 2 * (3 * r + c), f = 2 * (3 * c + r);
+      off[i] = make_double2(cf.off * fx::double_of(w[e] - w[f], 0), cf.off * fx::double_of(w[e + 1] + w[f + 1], 0));
+    }
+  }
+  __syncthreads();  // the sums' memory becomes the output's
+  if (lane < ns) {
+    double2* o = out + lane * fx::SITE_W + mu * 9;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const int r = i == 2 ? 1 : 0, c = i == 0 ? 1 : 2;
+      o[4 * i] = make_double2(0.0, dg[i]);
+      o[3 * r + c] = off[i];
+      o[3 * c + r] = make_double2(-off[i].x, off[i].y);
+    }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < ns * 36; i += 128) F[x0 * 36 + i] = out[(i / 36) * fx::SITE_W + i % 36];
 }
 
 }  // namespace gf
@@ -215,26 +415,68 @@ extern "C" int stag_gauge_force(const int dims[4], const void* thin, void* force
   if (p < q + bytes && q < p + bytes) return STAG_EINVAL;
   const su3::Dims d{dims[0], dims[1], dims[2], dims[3]};
   cudaStream_t st = (cudaStream_t)stream;
-  // the staple table (24 matrices per site, 3456 B) in stream-ordered scratch
-  double2* T = nullptr;
-  if (cudaMallocAsync((void**)&T, (size_t)V * 32 * 9 * sizeof(double2), st) != cudaSuccess) {
+  // stream-ordered scratch: the FP64 staple table (24 of 32 matrix slots per
+  // site, 4608 B) or the fixed-point field (28 matrices, 4032 B), whichever
+  // form runs
+  const size_t tbytes = (size_t)V * 32 * 9 * sizeof(double2), fbytes = fx::field_bytes(V, gf::SLOTS);
+  char* scratch = nullptr;
+  if (cudaMallocAsync((void**)&scratch, 256 + (tbytes > fbytes ? tbytes : fbytes), st) != cudaSuccess) {
     cudaGetLastError();
     return STAG_ENOMEM;
   }
+  int* status = (int*)scratch;
+  double2* T = (double2*)(scratch + 256);
+  int4* Tf = (int4*)(scratch + 256);
+  const double2* U = (const double2*)thin;
+  // coefficients with a power of two taken out (see k_gauge_force_fx); beyond
+  // 2^+-900, or not finite, the FP64 kernels, whose range is wider
+  const double big = std::fabs(c_pl) * 6 + std::fabs(c_rt) * 18 + std::fabs(c_pg) * 24;
+  const bool fixed = big > 0x1p-900 && big < 0x1p900 && std::fabs(beta) < 0x1p60;
   int s = STAG_OK;
-  {
+  if (fixed) {
+    int k = 0;
+    std::frexp(big, &k);
+    gf::ForceCoef cf;
+    cf.pl8 = fx::make_coef(std::ldexp(c_pl, 3 - k));
+    cf.rt8 = fx::make_coef(std::ldexp(c_rt, 3 - k));
+    cf.rt = fx::make_coef(std::ldexp(c_rt, -k));
+    cf.pg4 = fx::make_coef(std::ldexp(c_pg, 2 - k));
+    cf.off = std::ldexp(beta / 3.0, k - 61);
+    cf.diag = std::ldexp(beta / 9.0, k - 60);
+    const unsigned tiles = (unsigned)((V + fx::TS - 1) / fx::TS);
+    {
+      ProfScope ps("gauge_force", st);
+      s = fx::launch_fx_links(V, U, Tf, gf::SLOTS, gf::U0, status, st);
+    }
+    if (!s) {
+      ProfScope ps("gauge_force", st);
+      gf::k_gf_staples_fx<<<tiles, 128, 0, st>>>(d, V, Tf, status);
+      s = last_launch_status();
+    }
+    if (!s) {
+      ProfScope ps("gauge_force", st);
+      constexpr int smem = 3 * 18 * 128 * sizeof(long long);  // 54 KB, three blocks per SM
+      s = cuda_status(cudaFuncSetAttribute(gf::k_gauge_force_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+      if (!s) gf::k_gauge_force_fx<<<tiles, 128, smem, st>>>(d, V, Tf, status, (double2*)force, cf);
+      if (!s) s = last_launch_status();
+    }
+  } else {
+    s = cuda_status(cudaMemsetAsync(status, 0, sizeof(int), st));
+  }
+  const unsigned few = 152 * 8;
+  if (!s) {
     ProfScope ps("gauge_force", st);
-    const long long n = 24 * V;
-    gf::k_gf_staples<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(d, V, (const double2*)thin, T);
+    const long long n = (24 * V + 127) / 128;
+    gf::k_gf_staples<<<(unsigned)(fixed && n > few ? few : n), 128, 0, st>>>(d, V, U, T, status);
     s = last_launch_status();
   }
   if (!s) {
     ProfScope ps("gauge_force", st);
-    const long long n = 4 * V;
-    gf::k_gauge_force_reuse<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(d, V, (const double2*)thin, T,
-                                                                          (double2*)force, beta, c_pl, c_rt, c_pg);
+    const long long n = (4 * V + 127) / 128;
+    gf::k_gauge_force_reuse<<<(unsigned)(fixed && n > few ? few : n), 128, 0, st>>>(d, V, U, T, (double2*)force, beta, c_pl,
+                                                                                   c_rt, c_pg, status);
     s = last_launch_status();
   }
-  const int f = cuda_status(cudaFreeAsync(T, st));
+  const int f = cuda_status(cudaFreeAsync(scratch, st));
   return s ? s : f;
 }
