@@ -48,7 +48,7 @@ void Workspace::drop(const std::string& name) {
 
 int get_red_scratch(stag_lattice_s* lat, const char* name, RedScratch* out, int nv_max) {
   int st = 0;
-  int max_grid = (lat->g.Vh + 127) / 128;  // one block per 128 sites at most
+  int max_grid = (lat->g.Vh + 7) / 8;  // one block per 8 sites at most
   if (max_grid < 1024) max_grid = 1024;
   std::string n(name);
   double* p = (double*)lat->ws.get(n + ".partials", sizeof(double) * (size_t)nv_max * (size_t)max_grid, &st);
@@ -419,7 +419,8 @@ int stag_tuned_shape(stag_lattice_t lat, int prec, int kernel, int* block, int* 
     return STAG_OK;
   }
   if (block) *block = v < 2 ? 256 : 128;
-  if (min_blocks) *min_blocks = v == 1 ? 4 : v == 3 ? 8 : 1;
+  // (fixed-point FP64 links: 2 and 4 blocks, and few sites run in one shape of their own, dslash_impl.cuh)
+  if (min_blocks) *min_blocks = L.fixed ? (v == 1 ? 2 : v == 3 ? 4 : 1) : v == 1 ? 4 : v == 3 ? 8 : 1;
   if (us) *us = L.tuned_us[kernel];
   return STAG_OK;
 }
@@ -449,14 +450,29 @@ template Spinor<16> ws_spinor<16>(stag_lattice_s*, const std::string&, int*);
 template Spinor<15> ws_spinor<15>(stag_lattice_s*, const std::string&, int*);
 template Spinor<31> ws_spinor<31>(stag_lattice_s*, const std::string&, int*);
 
+// FP64 vectors are canonical in memory: the kernels can read and write the
+// caller's fields, unless the output overlaps the input.
+static bool disjoint(const void* a, const void* b, size_t n) {
+  const char *p = (const char*)a, *q = (const char*)b;
+  return p + n <= q || q + n <= p;
+}
+
 template <int P>
 static int dslash_p(stag_lattice_s* lat, double2* out, const double2* in, int out_parity, int nrhs, cudaStream_t st) {
   int s = 0;
+  const size_t n = (size_t)lat->g.Vh * 3;
+  if constexpr (P == 64) {
+    if (disjoint(out, in, n * nrhs * sizeof(double2))) {
+      for (int r = 0; r < nrhs && !s; ++r)
+        s = launch_dslash<64>(lat, Spinor<64>{out + r * n, lat->g.Vh}, Spinor<64>{const_cast<double2*>(in) + r * n, lat->g.Vh},
+                              out_parity, nullptr, st);
+      return s;
+    }
+  }
   Spinor<P> a = ws_spinor<P>(lat, "dslash.in", &s);
   if (s) return s;
   Spinor<P> b = ws_spinor<P>(lat, "dslash.out", &s);
   if (s) return s;
-  const size_t n = (size_t)lat->g.Vh * 3;
   for (int r = 0; r < nrhs; ++r) {
     if ((s = launch_from_canonical<P>(a, in + r * n, lat->g.Vh, st))) return s;
     if ((s = launch_dslash<P>(lat, b, a, out_parity, nullptr, st))) return s;
@@ -469,9 +485,18 @@ template <int P>
 static int apply_m_p(stag_lattice_s* lat, double2* out, const double2* in, double shift, cudaStream_t st) {
   constexpr int PA = Acc<P>::value;
   int s = 0;
-  Spinor<P> a = ws_spinor<P>(lat, "applym.in", &s);
-  if (s) return s;
   Spinor<P> t = ws_spinor<P>(lat, "applym.t", &s);
+  if (s) return s;
+  if constexpr (P == 64) {
+    if (disjoint(out, in, (size_t)lat->g.Vh * 3 * sizeof(double2))) {
+      const Spinor<64> x{const_cast<double2*>(in), lat->g.Vh};
+      if ((s = launch_dslash<64>(lat, t, x, 1, nullptr, st))) return s;
+      return launch_dslash_epi<64>(lat, Spinor<64>{out, lat->g.Vh}, t, 0, x, shift, Spinor<64>{nullptr, lat->g.Vh}, 0.0,
+                                   -1.0, 0, RedScratch{nullptr, nullptr, 0}, RedTarget{RED_STORE, nullptr, nullptr},
+                                   nullptr, st);
+    }
+  }
+  Spinor<P> a = ws_spinor<P>(lat, "applym.in", &s);
   if (s) return s;
   Spinor<PA> o = ws_spinor<PA>(lat, "applym.out", &s);
   if (s) return s;

@@ -15,6 +15,7 @@
 // neighbour vectors as one 128-bit record each, and neighbour indices are
 // computed from the site's coordinates (no index table).
 #pragma once
+#include "dslash_fx.cuh"
 #include "internal.h"
 
 namespace stag {
@@ -26,6 +27,7 @@ template <int P> struct DslashArgs {
   float fat_scale, long_scale;  // long_scale = c3/2 for two-row storage
   Spinor<P> in;
   int s_begin, s_end;  // output sites computed: [s_begin, s_end) (all: 0, Vh)
+  int kexp;            // fixed-point FP64 links: entries in units of 2^kexp
 };
 
 // The complex number k of a group of link chunks held in registers (k is a
@@ -122,6 +124,10 @@ template <int P, int NL>
 __device__ __forceinline__ void dslash_site(const DslashArgs<P>& a, int s, typename Prec<P>::A2 out[3]) {
   using A2 = typename Prec<P>::A2;
   using A = typename Prec<P>::A;
+  if constexpr (NL == kNLFixed) {
+    fxd::site(a, s, out);
+    return;
+  } else {
   constexpr int CPM = 18 + 2 * NL;  // complex entries per direction
   const int Vh = a.g.Vh;
   Coord c = cb_coords(a.g, s, a.out_parity);
@@ -175,6 +181,7 @@ __device__ __forceinline__ void dslash_site(const DslashArgs<P>& a, int s, typen
     out[i].x = fs * accF[i].x + ls * accL[i].x;
     out[i].y = fs * accF[i].y + ls * accL[i].y;
   }
+  }
 }
 
 // Launch shapes the autotuner chooses among: threads per block and the
@@ -183,6 +190,11 @@ __device__ __forceinline__ void dslash_site(const DslashArgs<P>& a, int s, typen
 constexpr int kNumShapes = 4;
 __host__ __device__ constexpr int shape_block(int v) { return v < 2 ? 256 : 128; }
 __host__ __device__ constexpr int shape_minb(int v) { return v == 1 ? 4 : v == 3 ? 8 : 1; }
+// The fixed-point form of the FP64 links needs about a hundred registers: 2
+// and 4 blocks.
+__host__ __device__ constexpr int shape_minb_nl(int v, int nl) {
+  return nl == kNLFixed ? (v == 1 ? 2 : v == 3 ? 4 : 1) : shape_minb(v);
+}
 
 template <int P, int NL, int B, int MINB>
 __global__ void __launch_bounds__(B, MINB) k_dslash(DslashArgs<P> a, Spinor<P> out, const int* flags) {
@@ -251,14 +263,45 @@ static DslashArgs<P> make_args(const stag_lattice_s* lat, Spinor<P> in, int out_
   a.in = in;
   a.s_begin = 0;
   a.s_end = lat->g.Vh;
+  a.kexp = L.kexp;
   return a;
+}
+
+// Fixed-point FP64 links, few sites: one hop per thread, eight sites per
+// block, one component of a site per thread in the epilogue (an FP64
+// instruction holds a warp for 58 clocks, whatever its lanes).  With one
+// thread per site a lattice of up to 2^15 sites per parity leaves most of the
+// chip's 608 warp schedulers with one warp or none.  One operator (two
+// halves), this form and the other: 8^4 12.3 and 28.7 us, 12 x 16^3 37.5 and
+// 49.2 us, 16^4 48.2 and 51.4 us.
+constexpr int kFewSites = 1 << 15;
+template <int RED>
+__global__ void __launch_bounds__(128)
+    k_dslash_few(DslashArgs<64> a, Spinor<64> out, Spinor<64> x, double ax, Spinor<64> y, double ay, double ad,
+                 int plain, RedBuf rb, RedTarget tgt, const int* flags) {
+  if (stopped(flags)) return;
+  const int s0 = a.s_begin + blockIdx.x * 8;
+  Acc1<double> red[1];
+  double d;
+  if (fxd::component16(a, s0, a.s_end, d)) {
+    const size_t at = (size_t)STAG_BOUND(s0 + (int)(threadIdx.x & 7), a.g.Vh, BOUND_VECTOR) * 6 + (threadIdx.x >> 3);
+    double o = d;
+    if (!plain) {
+      const double xv = __ldg((const double*)x.v + at);
+      o = ax * xv + ad * d;
+      if (ay != 0.0) o += ay * __ldg((const double*)y.v + at);
+      if (RED) red[0].add_prod(RED == 1 ? xv : o, o);
+    }
+    ((double*)out.v)[at] = o;
+  }
+  if (RED) grid_reduce_acc<1>(red, rb, tgt);
 }
 
 template <int P, int NL>
 static void dispatch_plain(int shape, const DslashArgs<P>& a, Spinor<P> out, const int* flags, cudaStream_t st) {
   const int Vh = a.s_end - a.s_begin;
 #define STAG_PL(V)                                                                                \
-  k_dslash<P, NL, shape_block(V), shape_minb(V)>                                                  \
+  k_dslash<P, NL, shape_block(V), shape_minb_nl(V, NL)>                                                  \
       <<<(Vh + shape_block(V) - 1) / shape_block(V), shape_block(V), 0, st>>>(a, out, flags)
   switch (shape) {
     case 1: STAG_PL(1); break;
@@ -275,7 +318,7 @@ static void dispatch_epi(int shape, const DslashArgs<P>& a, Spinor<Acc<P>::value
                          cudaStream_t st) {
   const int Vh = a.s_end - a.s_begin;
 #define STAG_EP(V)                                                                                \
-  k_dslash_epi<P, NL, RED, shape_block(V), shape_minb(V)>                                         \
+  k_dslash_epi<P, NL, RED, shape_block(V), shape_minb_nl(V, NL)>                                         \
       <<<(Vh + shape_block(V) - 1) / shape_block(V), shape_block(V), 0, st>>>(a, out, x, ax, y, ay, ad, rb, tgt, flags)
   switch (shape) {
     case 1: STAG_EP(1); break;
@@ -296,6 +339,18 @@ static int plain_with_shape(const stag_lattice_s* lat, int shape, Spinor<P> out,
     a.s_end = s1;
   }
   constexpr int NL2 = P == 64 ? 9 : 6;
+  if constexpr (P == 64) {
+    const int n = a.s_end - a.s_begin;
+    if (L.fixed && n <= kFewSites) {
+      k_dslash_few<0><<<(n + 7) / 8, 128, 0, st>>>(a, out, out, 0.0, out, 0.0, 0.0, 1, RedBuf{nullptr, nullptr},
+                                                         RedTarget{RED_STORE, nullptr, nullptr}, flags);
+      return last_launch_status();
+    }
+    if (L.fixed) {
+      dispatch_plain<P, kNLFixed>(shape, a, out, flags, st);
+      return last_launch_status();
+    }
+  }
   if (P == 64 || L.nl == 9)
     dispatch_plain<P, 9>(shape, a, out, flags, st);
   else
@@ -314,12 +369,33 @@ static int epi_with_shape(const stag_lattice_s* lat, int shape, Spinor<Acc<P>::v
     a.s_begin = s0;
     a.s_end = s1;
   }
-  const int G = (a.s_end - a.s_begin + shape_block(shape) - 1) / shape_block(shape);
-  if (red && G > rs.max_grid) return STAG_EINVAL;
+  const int n = a.s_end - a.s_begin;
   RedBuf rb{rs.partials, rs.counter};
+  if constexpr (P == 64) {
+    if (L.fixed && n <= kFewSites) {
+      const int G8 = (n + 7) / 8;
+      if (red && G8 > rs.max_grid) return STAG_EINVAL;
+#define STAG_E8(R) k_dslash_few<R><<<G8, 128, 0, st>>>(a, out, x, ax, y, ay, ad, 0, rb, tgt, flags)
+      if (red == 0) STAG_E8(0);
+      else if (red == 1) STAG_E8(1);
+      else STAG_E8(2);
+#undef STAG_E8
+      return last_launch_status();
+    }
+  }
+  const int G = (n + shape_block(shape) - 1) / shape_block(shape);
+  if (red && G > rs.max_grid) return STAG_EINVAL;
   constexpr int NL2 = P == 64 ? 9 : 6;
   const bool r12 = P != 64 && L.nl == 6;
 #define STAG_E(NL, R) dispatch_epi<P, NL, R>(shape, a, out, x, ax, y, ay, ad, rb, tgt, flags, st)
+  if constexpr (P == 64) {
+    if (L.fixed) {
+      if (red == 0) STAG_E(kNLFixed, 0);
+      else if (red == 1) STAG_E(kNLFixed, 1);
+      else STAG_E(kNLFixed, 2);
+      return last_launch_status();
+    }
+  }
   if (r12) {
     if (red == 0) STAG_E(NL2, 0);
     else if (red == 1) STAG_E(NL2, 1);

@@ -64,6 +64,7 @@ template <int P> struct DslashArgsM {
   const uint4* links;
   float fat_scale, long_scale;
   SpinorM<P> in;
+  int kexp;  // fixed-point FP64 links (dslash_fx.cuh)
 };
 
 // Loads the chunks holding the complex entries [k0, k0 + NE) of one hop and
@@ -143,6 +144,17 @@ template <int P, int NL, int N>
 __device__ __forceinline__ void dslash_site_m(const DslashArgsM<P>& a, int s, typename Prec<P>::A2 (&out)[N][3]) {
   using A2 = typename Prec<P>::A2;
   using A = typename Prec<P>::A;
+  if constexpr (NL == kNLFixed) {
+    static_assert(N == 1, "one right-hand side per thread");
+    DslashArgs<P> one;
+    one.g = a.g;
+    one.out_parity = a.out_parity;
+    one.links = a.links;
+    one.in = SpinorLoadM<P>::one(a.in, 0);
+    one.kexp = a.kexp;
+    fxd::site(one, s, out[0]);
+    return;
+  } else {
   constexpr int CPM = 18 + 2 * NL;
   const Geom& g = a.g;
   const int Vh = g.Vh;
@@ -184,6 +196,7 @@ __device__ __forceinline__ void dslash_site_m(const DslashArgsM<P>& a, int s, ty
       else
         hop_recon12_m<P, N>(out, b, off, a.in, cb_neighbour(g, s, c, mu, -3), !eta_bit(c, mu), ls);
     }
+  }
   }
 }
 

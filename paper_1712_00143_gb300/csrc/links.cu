@@ -13,8 +13,10 @@
 // two-row storage of the SU(3) part) form one list of complex numbers,
 // packed PER to a 16-byte chunk; chunk j of all sites is contiguous,
 // [chunk][site], so a warp's 128-bit loads of one chunk are coalesced.
+#include <cmath>
 #include <cstring>
 
+#include "fx.cuh"
 #include "internal.h"
 
 namespace stag {
@@ -160,6 +162,113 @@ static double max_abs(const double2* a, long long n_complex, unsigned long long*
   return v;
 }
 
+// ------------------------------------------------------------ fixed-point form of the FP64 copy
+// What decides whether (and in which unit) the FP64 copy can be held in fixed
+// point (dslash_fx.cuh): the largest entry, the smallest nonzero matrix (by
+// its largest entry), both as high words of the double, and the largest sum
+// over the sixteen hops of a row's norm.
+struct FxStats {
+  int max_hi, min_hi;
+  unsigned row;  // a float's bits
+};
+
+__device__ __forceinline__ float float_of_bits(double v) {  // |v| to float without the FP64 pipe; ends clamped
+  const int hi = __double2hiint(v) & 0x7fffffff;
+  const int e = hi >> 20;
+  if (e < 897) return 0.f;
+  if (e > 1150) return __int_as_float(0x7f800000);
+  return __int_as_float(((hi - (896 << 20)) << 3) | (int)((unsigned)__double2loint(v) >> 29));
+}
+
+// one thread per (parity, site); reads the copy once: bound by HBM
+__global__ void __launch_bounds__(128) k_fx_stats(const double2* __restrict__ L, int Vh, FxStats* st) {
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  int mx = 0, mn = 0x7fffffff;
+  float row = 0.f;
+  if (idx < 2 * Vh) {
+    const int p = idx / Vh, s = idx - p * Vh;
+    const double2* src = L + (size_t)p * 144 * Vh + s;
+    float sum[3] = {0.f, 0.f, 0.f};
+#pragma unroll 1
+    for (int t = 0; t < 16; ++t) {
+      int m = 0;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        float n2 = 0.f;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          const double2 w = __ldg(src + (size_t)(t * 9 + 3 * i + j) * Vh);
+          m = max(m, max(__double2hiint(w.x) & 0x7fffffff, __double2hiint(w.y) & 0x7fffffff));
+          const float a = float_of_bits(w.x), b = float_of_bits(w.y);
+          n2 += a * a + b * b;
+        }
+        sum[i] += sqrtf(n2);
+      }
+      mx = max(mx, m);
+      if (m > 0) mn = min(mn, m);
+    }
+    row = fmaxf(sum[0], fmaxf(sum[1], sum[2]));
+  }
+  mx = (int)__reduce_max_sync(0xffffffffu, (unsigned)mx);
+  mn = (int)__reduce_min_sync(0xffffffffu, (unsigned)mn);
+  const unsigned r = __reduce_max_sync(0xffffffffu, __float_as_uint(row));
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(&st->max_hi, mx);
+    atomicMin(&st->min_hi, mn);
+    atomicMax(&st->row, r);
+  }
+}
+
+// in place: two doubles -> {re.h, re.l, im.h, im.l} in units of 2^kexp, rounded to nearest
+__device__ __forceinline__ void fixed_entry(double v, int kexp, int& h, int& l) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const int r = 1023 + kexp - (int)((b >> 52) & 0x7ff);  // >= 1: |v| < 2^kexp
+  const unsigned long long m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 8;
+  const long long q = r > 62 ? 0 : (long long)((m + (1ull << (r - 1))) >> r);
+  fx::split1((long long)b < 0 ? -q : q, h, l);
+}
+__global__ void __launch_bounds__(256) k_fx_convert(double2* L, long long n, int kexp) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const double2 v = L[i];
+    int4 q;
+    fixed_entry(v.x, kexp, q.x, q.y);
+    fixed_entry(v.y, kexp, q.z, q.w);
+    ((int4*)L)[i] = q;
+  }
+}
+
+// The FP64 copy to fixed point, if every nonzero matrix lies within 2^-10 of
+// the largest entry (so that all keep FP64's relative accuracy) and the unit
+// is in the middle of the double range; else it stays in doubles.
+static int to_fixed(LinkCopy& L, const Geom& g, FxStats* scratch, cudaStream_t st) {
+  FxStats h{0, 0x7fffffff, 0u};
+  int status = cuda_status(cudaMemcpyAsync(scratch, &h, sizeof(h), cudaMemcpyHostToDevice, st));
+  if (status) return status;
+  {
+    ProfScope ps("links", st);
+    k_fx_stats<<<(2 * g.Vh + 127) / 128, 128, 0, st>>>((const double2*)L.data, g.Vh, scratch);
+  }
+  if ((status = last_launch_status())) return status;
+  if ((status = cuda_status(cudaMemcpyAsync(&h, scratch, sizeof(h), cudaMemcpyDeviceToHost, st)))) return status;
+  if ((status = cuda_status(cudaStreamSynchronize(st)))) return status;
+  float row;
+  memcpy(&row, &h.row, sizeof(row));
+  const int emax = h.max_hi >> 20, emin = h.min_hi >> 20;
+  if (emax < 1023 - 100 || emax > 1023 + 100 || emin < emax - 10) return STAG_OK;
+  int kexp = emax - 1022;  // |entry| < 2^kexp
+  for (double r = std::ldexp((double)row, -kexp); r > 9.0; r *= 0.5) ++kexp;
+  if (kexp > emax - 1022 + 4) return STAG_OK;
+  const long long n = (long long)2 * 144 * g.Vh;
+  {
+    ProfScope ps("links", st);
+    k_fx_convert<<<1216, 256, 0, st>>>((double2*)L.data, n, kexp);
+  }
+  if ((status = last_launch_status())) return status;
+  L.fixed = true;
+  L.kexp = kexp;
+  return STAG_OK;
+}
+
 int build_link_copy(stag_lattice_s* lat, int prec, int recon, const double2* fat, const double2* lng,
                     cudaStream_t st) {
   const Geom& g = lat->g;
@@ -216,6 +325,7 @@ int build_link_copy(stag_lattice_s* lat, int prec, int recon, const double2* fat
   if ((status = cuda_status(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st)))) return status;
   if ((status = cuda_status(cudaStreamSynchronize(st)))) return status;
   if (herr) return STAG_ENOTUNITARY;
+  if (prec == STAG_FP64 && (status = to_fixed(L, g, (FxStats*)(err + 8), st))) return status;
   L.present = true;
   return STAG_OK;
 }

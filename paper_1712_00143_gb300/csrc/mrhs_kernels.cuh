@@ -88,7 +88,7 @@ template <int P, int NL, int N, int RED, int SP, int MINB>
 __global__ void __launch_bounds__(MB, MINB)
     k_dslash_m_epi_v(DslashArgsM<P> a, SpinorM<Acc<P>::value> out, SpinorM<P> x, double ax,
                      SpinorM<Acc<P>::value> y, double ay, double ad, RedBuf rb, RedTarget tgt, const int* flags) {
-  static_assert(N % SP == 0 && (RED == 0 || RED == 3 || SP == 1), "variant");
+  static_assert(N % SP == 0 && (RED == 0 || RED == 3 || SP == 1 || NL == kNLFixed), "variant");
   using A2 = typename Prec<P>::A2;
   using A = typename Prec<P>::A;
   constexpr int PA = Acc<P>::value;
@@ -148,8 +148,15 @@ __global__ void __launch_bounds__(MB, MINB)
       }
     }
   }
-  if constexpr (RED != 0 && RED != 3) {
+  if constexpr (RED != 0 && RED != 3 && SP == 1) {
     grid_reduce_acc<N>(red, rb, tgt);
+  } else if constexpr (RED != 0 && RED != 3) {
+    // one system per thread: its sum among zeros
+    Acc1<A> all[N];
+#pragma unroll
+    for (int r = 0; r < N; ++r)
+      if (r == part) all[r] = red[0];
+    grid_reduce_acc<N>(all, rb, tgt);
   }
 }
 
@@ -163,6 +170,7 @@ template <int P> DslashArgsM<P> make_args_m(const stag_lattice_s* lat, SpinorM<P
   a.fat_scale = (float)(L.fat_scale * fx);
   a.long_scale = (float)((L.nl == 6 ? 0.5 * lat->c3 : (double)L.long_scale) * fx);
   a.in = in;
+  a.kexp = L.kexp;
   return a;
 }
 
@@ -232,6 +240,26 @@ void dispatch_epi(int v, const DslashArgsM<P>& a, SpinorM<Acc<P>::value> out, Sp
 #undef STAG_EPV
 }
 
+// Fixed-point FP64 links (dslash_fx.cuh): each thread takes one system of a
+// site, so that its sums and operands fit in registers; the N threads of a
+// site read the same links from L1.  Eight systems at 32^4: 1.41 ms per
+// half, bound by the integer pipe and the latency of the gathers.
+template <int N>
+void launch_plain_fixed(const DslashArgsM<64>& a, SpinorM<64> out, const int* flags, cudaStream_t st) {
+  constexpr int spb = MB / N;
+  k_dslash_mv<64, kNLFixed, N, N, 4><<<(a.g.Vh + spb - 1) / spb, MB, 0, st>>>(a, out, flags);
+}
+template <int N, int RED>
+int launch_epi_fixed(const DslashArgsM<64>& a, SpinorM<64> out, SpinorM<64> x, double ax, SpinorM<64> y, double ay,
+                     double ad, RedScratch rs, RedTarget tgt, const int* flags, cudaStream_t st) {
+  constexpr int spb = MB / N;
+  const int G = (a.g.Vh + spb - 1) / spb;
+  if (RED && G > rs.max_grid) return STAG_EINVAL;
+  k_dslash_m_epi_v<64, kNLFixed, N, RED, N, 4>
+      <<<G, MB, 0, st>>>(a, out, x, ax, y, ay, ad, RedBuf{rs.partials, rs.counter}, tgt, flags);
+  return last_launch_status();
+}
+
 template <int P, int N>
 int mdslash_v(const stag_lattice_s* lat, int v, SpinorM<P> out, SpinorM<P> in, int out_parity, const int* flags,
               cudaStream_t st) {
@@ -239,6 +267,12 @@ int mdslash_v(const stag_lattice_s* lat, int v, SpinorM<P> out, SpinorM<P> in, i
   if (!L.present) return STAG_EINVAL;
   DslashArgsM<P> a = make_args_m<P>(lat, in, out_parity);
   ProfScope ps(P == 64 ? "dslash_mrhs64" : "dslash_mrhs", st);
+  if constexpr (P == 64) {
+    if (L.fixed) {
+      launch_plain_fixed<N>(a, out, flags, st);
+      return last_launch_status();
+    }
+  }
   if (P != 64 && L.nl == 6)
     dispatch_plain<P, (P == 64 ? 9 : 6), N>(v, a, out, flags, st);
   else
@@ -255,6 +289,9 @@ int mdslash_epi_v(const stag_lattice_s* lat, int v, SpinorM<Acc<P>::value> out, 
   DslashArgsM<P> a = make_args_m<P>(lat, in, out_parity);
   if (RED && RED != 3 && (a.g.Vh + MB - 1) / MB > rs.max_grid) return STAG_EINVAL;
   ProfScope ps(P == 64 ? "dslash_mrhs64_epi" : "dslash_mrhs_epi", st);
+  if constexpr (P == 64 && RED != 3) {
+    if (L.fixed) return launch_epi_fixed<N, RED>(a, out, x, ax, y, ay, ad, rs, tgt, flags, st);
+  }
   RedBuf rb{rs.partials, rs.counter};
   if (P != 64 && L.nl == 6)
     dispatch_epi<P, (P == 64 ? 9 : 6), N, RED>(v, a, out, x, ax, y, ay, ad, rb, tgt, flags, st);

@@ -9,7 +9,7 @@
 // the entry point runs on it.
 #include <mutex>
 
-#include "dslash_impl.cuh"
+#include "internal.h"
 
 namespace stag {
 namespace {
@@ -64,21 +64,9 @@ extern "C" int stag_apply_m_noalloc(stag_lattice_t lat, void* out, const void* i
   Spinor<64> t{scratch, Vh};
   Spinor<64> o{out, Vh};
   Spinor<64> none{nullptr, Vh};
-  const int B = 256, G = (Vh + B - 1) / B;
   // t = D_oe in (odd sites): every entry of t is written before it is read
-  DslashArgs<64> a1 = make_args<64>(lat, x, 1);
-  {
-    ProfScope ps("dslash64", st);
-    k_dslash<64, 9, 256, 1><<<G, B, 0, st>>>(a1, t, nullptr);
-  }
-  if ((s = last_launch_status())) return s;
+  if ((s = launch_dslash<64>(lat, t, x, 1, nullptr, st))) return s;
   // out = (m^2 + shift) in - D_eo t (even sites)
-  DslashArgs<64> a2 = make_args<64>(lat, t, 0);
-  {
-    ProfScope ps("dslash64_epi", st);
-    k_dslash_epi<64, 9, 0, 256, 1><<<G, B, 0, st>>>(a2, o, x, mass * mass + shift, none, 0.0, -1.0,
-                                                    RedBuf{nullptr, nullptr}, RedTarget{RED_STORE, nullptr, nullptr},
-                                                    nullptr);
-  }
-  return last_launch_status();
+  return launch_dslash_epi<64>(lat, o, t, 0, x, mass * mass + shift, none, 0.0, -1.0, 0, RedScratch{nullptr, nullptr, 0},
+                               RedTarget{RED_STORE, nullptr, nullptr}, nullptr, st);
 }
