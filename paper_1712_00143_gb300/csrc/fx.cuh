@@ -255,9 +255,10 @@ __device__ __forceinline__ Site next(const Dims& d, const Site& p, int mu, int k
 // eight threads of a 128-bit access phase fall in different bank groups).
 constexpr int SITE_W = 37;
 
-// Bits of *status, set by k_fx_links: some link is not unitary to 2^-12 (or
-// not finite); some link is at least 2^-5 away from the unit matrix.
-enum : int { FX_NOT_UNITARY = 1, FX_AWAY = 2 };
+// Bits of *status.  Set by k_fx_links: some link is not unitary to 2^-12 (or
+// not finite); some link is at least 2^-5 away from the unit matrix.  Set by a
+// later kernel: some other input's exponent is out of range.
+enum : int { FX_NOT_UNITARY = 1, FX_AWAY = 2, FX_RANGE = 4 };
 // The integer kernels run on FX_AWAY alone.  Links all close to the unit
 // matrix stay on the FP64 kernels: their small entries, and a force made of
 // them, would be known to 2^-58 absolute where FP64 keeps 2^-53 relative.
