@@ -464,50 +464,33 @@ static int dslash_p(stag_lattice_s* lat, double2* out, const double2* in, int ou
   if constexpr (P == 64) {
     if (disjoint(out, in, n * nrhs * sizeof(double2))) {
       for (int r = 0; r < nrhs && !s; ++r)
-        s = launch_dslash<64>(lat, Spinor<64>{out + r * n, lat->g.Vh}, Spinor<64>{const_cast<double2*>(in) + r * n, lat->g.Vh},
-                              out_parity, nullptr, st);
+        s = launch_dslash_canonical<64>(lat, out + r * n, Spinor<64>{const_cast<double2*>(in) + r * n, lat->g.Vh},
+                                        out_parity, st);
       return s;
     }
   }
   Spinor<P> a = ws_spinor<P>(lat, "dslash.in", &s);
   if (s) return s;
-  Spinor<P> b = ws_spinor<P>(lat, "dslash.out", &s);
-  if (s) return s;
   for (int r = 0; r < nrhs; ++r) {
     if ((s = launch_from_canonical<P>(a, in + r * n, lat->g.Vh, st))) return s;
-    if ((s = launch_dslash<P>(lat, b, a, out_parity, nullptr, st))) return s;
-    if ((s = launch_to_canonical<P>(out + r * n, b, lat->g.Vh, st))) return s;
+    if ((s = launch_dslash_canonical<P>(lat, out + r * n, a, out_parity, st))) return s;
   }
   return STAG_OK;
 }
 
 template <int P>
 static int apply_m_p(stag_lattice_s* lat, double2* out, const double2* in, double shift, cudaStream_t st) {
-  constexpr int PA = Acc<P>::value;
   int s = 0;
   Spinor<P> t = ws_spinor<P>(lat, "applym.t", &s);
   if (s) return s;
-  if constexpr (P == 64) {
-    if (disjoint(out, in, (size_t)lat->g.Vh * 3 * sizeof(double2))) {
-      const Spinor<64> x{const_cast<double2*>(in), lat->g.Vh};
-      if ((s = launch_dslash<64>(lat, t, x, 1, nullptr, st))) return s;
-      return launch_dslash_epi<64>(lat, Spinor<64>{out, lat->g.Vh}, t, 0, x, shift, Spinor<64>{nullptr, lat->g.Vh}, 0.0,
-                                   -1.0, 0, RedScratch{nullptr, nullptr, 0}, RedTarget{RED_STORE, nullptr, nullptr},
-                                   nullptr, st);
-    }
+  Spinor<P> a{const_cast<double2*>(in), lat->g.Vh};
+  if (P != 64 || !disjoint(out, in, (size_t)lat->g.Vh * 3 * sizeof(double2))) {
+    a = ws_spinor<P>(lat, "applym.in", &s);
+    if (s) return s;
+    if ((s = launch_from_canonical<P>(a, in, lat->g.Vh, st))) return s;
   }
-  Spinor<P> a = ws_spinor<P>(lat, "applym.in", &s);
-  if (s) return s;
-  Spinor<PA> o = ws_spinor<PA>(lat, "applym.out", &s);
-  if (s) return s;
-  if ((s = launch_from_canonical<P>(a, in, lat->g.Vh, st))) return s;
   if ((s = launch_dslash<P>(lat, t, a, 1, nullptr, st))) return s;
-  RedScratch rs{nullptr, nullptr, 0};
-  Spinor<PA> none{nullptr, lat->g.Vh};
-  if ((s = launch_dslash_epi<P>(lat, o, t, 0, a, shift, none, 0.0, -1.0, 0, rs, RedTarget{RED_STORE, nullptr, nullptr},
-                                nullptr, st)))
-    return s;
-  return launch_to_canonical<PA>(out, o, lat->g.Vh, st);
+  return launch_dslash_epi_canonical<P>(lat, out, t, 0, a, shift, -1.0, st);
 }
 
 // Double-float: canonical FP64 in, split exactly, DF hops, DF out widened to FP64.

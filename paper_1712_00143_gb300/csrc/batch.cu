@@ -69,20 +69,28 @@ template <int P, int N>
 static int dslash_group(stag_lattice_s* lat, double2* out, const double2* in, int out_parity, cudaStream_t st) {
   int s = tune_mrhs<P, N>(lat, st);
   if (s) return s;
-  SpinorM<P> a = ws_spinorm<P>(lat, "mdslash.in", N, &s);
-  SpinorM<P> b = ws_spinorm<P>(lat, "mdslash.out", N, &s);
-  if (s) return s;
-  {
+  SpinorM<P> a{const_cast<double2*>(in), lat->g.Vh, N};
+  const size_t bytes = spinorm_bytes<64>(lat->g.Vh, N);
+  const char *pi = (const char*)in, *po = (const char*)out;
+  if (P != 64 || (pi < po + bytes && po < pi + bytes)) {  // (FP64 vectors are canonical in memory)
+    a = ws_spinorm<P>(lat, "mdslash.in", N, &s);
+    if (s) return s;
     ProfScope ps("convert", st);
     k_mfrom_canonical<P, N><<<grid_bw(lat->g.Vh), 256, 0, st>>>(a, in, N);
+    TRYB(last_launch_status());
   }
-  TRYB(last_launch_status());
-  TRYB((mdslash<P, N>(lat, b, a, out_parity, nullptr, st)));
-  {
-    ProfScope ps("convert", st);
-    k_mto_canonical<P, N><<<grid_bw(lat->g.Vh), 256, 0, st>>>(out, b, N);
-  }
-  return last_launch_status();
+  return mdslash_canonical<P, N>(lat, out, a, out_parity, st);
+}
+
+// The next group of `left` right-hand sides: 8 while there are as many, then
+// one or two launches.  (Six in one launch read the links once; 28x20x18x36,
+// fixed-point links with FP32 vectors: 75 us against 108 us as 4 + 2 with the
+// result converted in a pass of its own; three 43 against 76 us.)  16-bit vectors: 8, 4, 2, as their kernels with
+// more vectors per thread are slower per vector.
+template <int P> static int next_group(int left) {
+  if (left >= 8) return 8;
+  if (P == 16 || P == 15) return left >= 4 ? 4 : left >= 2 ? 2 : 1;
+  return left == 7 ? 4 : left == 5 ? 3 : left;
 }
 
 template <int P>
@@ -91,15 +99,23 @@ static int dslash_multi_p(stag_lattice_s* lat, double2* out, const double2* in, 
   const size_t n = (size_t)lat->g.Vh * 3;
   int r = 0;
   while (r < nrhs) {
-    const int left = nrhs - r;
-    int s;
-    if (left >= 8) s = dslash_group<P, 8>(lat, out + r * n, in + r * n, out_parity, st), r += 8;
-    else if (left >= 4) s = dslash_group<P, 4>(lat, out + r * n, in + r * n, out_parity, st), r += 4;
-    else if (left >= 2) s = dslash_group<P, 2>(lat, out + r * n, in + r * n, out_parity, st), r += 2;
-    else break;
+    const int N = next_group<P>(nrhs - r);
+    double2* o = out + r * n;
+    const double2* i = in + r * n;
+    int s = STAG_OK;
+    switch (N) {
+      case 8: s = dslash_group<P, 8>(lat, o, i, out_parity, st); break;
+      case 4: s = dslash_group<P, 4>(lat, o, i, out_parity, st); break;
+      case 2: s = dslash_group<P, 2>(lat, o, i, out_parity, st); break;
+      case 1: s = stag_dslash(lat, o, i, out_parity, P == 31 ? STAG_FX16L32 : prec_index<P>(), 1, st); break;
+      default:
+        if constexpr (P != 16 && P != 15) {
+          s = N == 6 ? dslash_group<P, 6>(lat, o, i, out_parity, st) : dslash_group<P, 3>(lat, o, i, out_parity, st);
+        }
+    }
     if (s) return s;
+    r += N;
   }
-  if (r < nrhs) return stag_dslash(lat, out + r * n, in + r * n, out_parity, P == 31 ? STAG_FX16L32 : prec_index<P>(), 1, st);
   return STAG_OK;
 }
 

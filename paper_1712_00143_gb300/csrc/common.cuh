@@ -364,7 +364,7 @@ template <int P> struct SpinorLoad16 {
       return (unsigned)(unsigned short)(short)a | ((unsigned)(unsigned short)(short)b << 16);
     }
   }
-  static __device__ __forceinline__ void st(const Spinor<P>& f, int s, const float2 o[3]) {
+  static __device__ __forceinline__ uint4 pack(const float2 o[3]) {
     float m = 0.f;
 #pragma unroll
     for (int c = 0; c < 3; ++c) m = fmaxf(m, fmaxf(fabsf(o[c].x), fabsf(o[c].y)));
@@ -375,11 +375,56 @@ template <int P> struct SpinorLoad16 {
     r.y = pack2(o[1].x * inv, o[1].y * inv);
     r.z = pack2(o[2].x * inv, o[2].y * inv);
     r.w = __float_as_uint(m / full);
-    ((uint4*)f.v)[STAG_BOUND(s, f.Vh, BOUND_VECTOR)] = r;
+    return r;
+  }
+  static __device__ __forceinline__ void st(const Spinor<P>& f, int s, const float2 o[3]) {
+    ((uint4*)f.v)[STAG_BOUND(s, f.Vh, BOUND_VECTOR)] = pack(o);
   }
 };
 template <> struct SpinorLoad<16> : SpinorLoad16<16> {};
 template <> struct SpinorLoad<15> : SpinorLoad16<15> {};
+
+// float -> double, exactly, on the integer pipe for normal numbers and zero
+// (a conversion holds a warp's FP64 pipe for tens of clocks; a store of eight
+// FP32 vectors as doubles at 32^4 spent 75 us in it against 46 us of traffic).
+__device__ __forceinline__ double widen_float(float f) {
+  const unsigned b = __float_as_uint(f), u = b & 0x7fffffffu;
+  if (u - 0x00800000u < 0x7f000000u)
+    return __hiloint2double((int)((b & 0x80000000u) | ((u >> 3) + 0x38000000u)), (int)(u << 29));
+  return (double)f;
+}
+// One site's vector as stored in format P (16-bit formats: rounded to it),
+// to the canonical field of doubles.  A warp whose lanes hold 32 consecutive
+// sites from a multiple of 32 on exchanges them through shared memory (stage:
+// 96 float2 per warp), so that its stores are whole 512-byte rows instead of
+// 16 bytes in every 48.
+template <int P>
+__device__ __forceinline__ void store_canonical(double2* out, int s, const typename Prec<P>::A2 o[3], float2* stage) {
+  if constexpr (P == 64) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) out[3 * (size_t)s + c] = o[c];
+  } else {
+    float2 q[3] = {o[0], o[1], o[2]};
+    if constexpr (P == 16 || P == 15) SpinorLoad16<P>::unpack(SpinorLoad16<P>::pack(o), q);
+    if (__activemask() == 0xffffffffu) {
+      const int lane = threadIdx.x & 31;
+      float2* w = stage + (threadIdx.x >> 5) * 96;
+      __syncwarp();
+#pragma unroll
+      for (int c = 0; c < 3; ++c) w[3 * lane + c] = q[c];
+      __syncwarp();
+      double2* p = out + 3 * (size_t)(s - lane) + lane;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const float2 v = w[32 * c + lane];
+        p[32 * c] = make_double2(widen_float(v.x), widen_float(v.y));
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) out[3 * (size_t)s + c] = make_double2(widen_float(q[c].x), widen_float(q[c].y));
+    }
+  }
+}
 
 // ------------------------------------------------------------------ solver state
 enum StateFlags : int {

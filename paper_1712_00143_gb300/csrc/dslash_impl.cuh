@@ -197,21 +197,27 @@ __host__ __device__ constexpr int shape_minb_nl(int v, int nl) {
 }
 
 template <int P, int NL, int B, int MINB>
-__global__ void __launch_bounds__(B, MINB) k_dslash(DslashArgs<P> a, Spinor<P> out, const int* flags) {
+__global__ void __launch_bounds__(B, MINB)
+    k_dslash(DslashArgs<P> a, Spinor<P> out, double2* can, const int* flags) {
   if (stopped(flags)) return;
   int s = a.s_begin + blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= a.s_end) return;
   typename Prec<P>::A2 d[3];
   dslash_site<P, NL>(a, s, d);
-  SpinorLoad<P>::st(out, s, d);
+  if (P != 64 && can) {
+    __shared__ float2 stage[P == 64 ? 1 : 3 * B];
+    store_canonical<P>(can, STAG_BOUND(s, a.g.Vh, BOUND_VECTOR), d, stage);
+  } else {
+    SpinorLoad<P>::st(out, s, d);
+  }
 }
 
 // out = ax x + ay y + ad (D in), with an FP64 reduction of Re<x,out> (RED=1)
 // or ||out||^2 (RED=2) finalised by the last block.
 template <int P, int NL, int RED, int B, int MINB>
 __global__ void __launch_bounds__(B, MINB)
-    k_dslash_epi(DslashArgs<P> a, Spinor<Acc<P>::value> out, Spinor<P> x, double ax, Spinor<Acc<P>::value> y,
-                 double ay, double ad, RedBuf rb, RedTarget tgt, const int* flags) {
+    k_dslash_epi(DslashArgs<P> a, Spinor<Acc<P>::value> out, double2* can, Spinor<P> x, double ax,
+                 Spinor<Acc<P>::value> y, double ay, double ad, RedBuf rb, RedTarget tgt, const int* flags) {
   using A2 = typename Prec<P>::A2;
   using A = typename Prec<P>::A;
   if (stopped(flags)) return;
@@ -238,7 +244,12 @@ __global__ void __launch_bounds__(B, MINB)
         o[i].y += cy * yv[i].y;
       }
     }
-    SpinorLoad<Acc<P>::value>::st(out, s, o);
+    if (P != 64 && RED == 0 && can) {
+      __shared__ float2 stage[P == 64 || RED ? 1 : 3 * B];
+      store_canonical<Acc<P>::value>(can, STAG_BOUND(s, a.g.Vh, BOUND_VECTOR), o, stage);
+    } else {
+      SpinorLoad<Acc<P>::value>::st(out, s, o);
+    }
     if (RED) {
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
@@ -298,11 +309,12 @@ __global__ void __launch_bounds__(128)
 }
 
 template <int P, int NL>
-static void dispatch_plain(int shape, const DslashArgs<P>& a, Spinor<P> out, const int* flags, cudaStream_t st) {
+static void dispatch_plain(int shape, const DslashArgs<P>& a, Spinor<P> out, double2* can, const int* flags,
+                           cudaStream_t st) {
   const int Vh = a.s_end - a.s_begin;
 #define STAG_PL(V)                                                                                \
   k_dslash<P, NL, shape_block(V), shape_minb_nl(V, NL)>                                                  \
-      <<<(Vh + shape_block(V) - 1) / shape_block(V), shape_block(V), 0, st>>>(a, out, flags)
+      <<<(Vh + shape_block(V) - 1) / shape_block(V), shape_block(V), 0, st>>>(a, out, can, flags)
   switch (shape) {
     case 1: STAG_PL(1); break;
     case 2: STAG_PL(2); break;
@@ -313,13 +325,13 @@ static void dispatch_plain(int shape, const DslashArgs<P>& a, Spinor<P> out, con
 }
 
 template <int P, int NL, int RED>
-static void dispatch_epi(int shape, const DslashArgs<P>& a, Spinor<Acc<P>::value> out, Spinor<P> x, double ax,
+static void dispatch_epi(int shape, const DslashArgs<P>& a, Spinor<Acc<P>::value> out, double2* can, Spinor<P> x, double ax,
                          Spinor<Acc<P>::value> y, double ay, double ad, RedBuf rb, RedTarget tgt, const int* flags,
                          cudaStream_t st) {
   const int Vh = a.s_end - a.s_begin;
 #define STAG_EP(V)                                                                                \
   k_dslash_epi<P, NL, RED, shape_block(V), shape_minb_nl(V, NL)>                                         \
-      <<<(Vh + shape_block(V) - 1) / shape_block(V), shape_block(V), 0, st>>>(a, out, x, ax, y, ay, ad, rb, tgt, flags)
+      <<<(Vh + shape_block(V) - 1) / shape_block(V), shape_block(V), 0, st>>>(a, out, can, x, ax, y, ay, ad, rb, tgt, flags)
   switch (shape) {
     case 1: STAG_EP(1); break;
     case 2: STAG_EP(2); break;
@@ -331,7 +343,7 @@ static void dispatch_epi(int shape, const DslashArgs<P>& a, Spinor<Acc<P>::value
 
 template <int P>
 static int plain_with_shape(const stag_lattice_s* lat, int shape, Spinor<P> out, Spinor<P> in, int out_parity,
-                            const int* flags, cudaStream_t st, int s0 = 0, int s1 = -1) {
+                            const int* flags, cudaStream_t st, int s0 = 0, int s1 = -1, double2* can = nullptr) {
   const LinkCopy& L = lat->links[prec_index<P>()];
   DslashArgs<P> a = make_args<P>(lat, in, out_parity);
   if (s1 >= 0) {
@@ -347,14 +359,14 @@ static int plain_with_shape(const stag_lattice_s* lat, int shape, Spinor<P> out,
       return last_launch_status();
     }
     if (L.fixed) {
-      dispatch_plain<P, kNLFixed>(shape, a, out, flags, st);
+      dispatch_plain<P, kNLFixed>(shape, a, out, can, flags, st);
       return last_launch_status();
     }
   }
   if (P == 64 || L.nl == 9)
-    dispatch_plain<P, 9>(shape, a, out, flags, st);
+    dispatch_plain<P, 9>(shape, a, out, can, flags, st);
   else
-    dispatch_plain<P, NL2>(shape, a, out, flags, st);
+    dispatch_plain<P, NL2>(shape, a, out, can, flags, st);
   return last_launch_status();
 }
 
@@ -362,7 +374,7 @@ template <int P>
 static int epi_with_shape(const stag_lattice_s* lat, int shape, Spinor<Acc<P>::value> out, Spinor<P> in,
                           int out_parity, Spinor<P> x, double ax, Spinor<Acc<P>::value> y, double ay, double ad,
                           int red, RedScratch rs, RedTarget tgt, const int* flags, cudaStream_t st, int s0 = 0,
-                          int s1 = -1) {
+                          int s1 = -1, double2* can = nullptr) {
   const LinkCopy& L = lat->links[prec_index<P>()];
   DslashArgs<P> a = make_args<P>(lat, in, out_parity);
   if (s1 >= 0) {
@@ -387,7 +399,7 @@ static int epi_with_shape(const stag_lattice_s* lat, int shape, Spinor<Acc<P>::v
   if (red && G > rs.max_grid) return STAG_EINVAL;
   constexpr int NL2 = P == 64 ? 9 : 6;
   const bool r12 = P != 64 && L.nl == 6;
-#define STAG_E(NL, R) dispatch_epi<P, NL, R>(shape, a, out, x, ax, y, ay, ad, rb, tgt, flags, st)
+#define STAG_E(NL, R) dispatch_epi<P, NL, R>(shape, a, out, can, x, ax, y, ay, ad, rb, tgt, flags, st)
   if constexpr (P == 64) {
     if (L.fixed) {
       if (red == 0) STAG_E(kNLFixed, 0);
@@ -426,6 +438,27 @@ int launch_dslash_epi(const stag_lattice_s* lat, Spinor<Acc<P>::value> out, Spin
   if (!L.present) return STAG_EINVAL;
   ProfScope ps(P == 64 ? "dslash64_epi" : "dslash_epi", st);
   return epi_with_shape<P>(lat, L.shape_epi, out, in, out_parity, x, ax, y, ay, ad, red, rs, tgt, flags, st);
+}
+
+// The same two with the result stored as canonical doubles (FP64 callers
+// pass the field itself), sparing a pass over it.
+template <int P>
+int launch_dslash_canonical(const stag_lattice_s* lat, double2* out, Spinor<P> in, int out_parity, cudaStream_t st) {
+  const LinkCopy& L = lat->links[prec_index<P>()];
+  if (!L.present) return STAG_EINVAL;
+  ProfScope ps(P == 64 ? "dslash64" : "dslash", st);
+  return plain_with_shape<P>(lat, L.shape_plain, Spinor<P>{out, in.Vh}, in, out_parity, nullptr, st, 0, -1, out);
+}
+template <int P>
+int launch_dslash_epi_canonical(const stag_lattice_s* lat, double2* out, Spinor<P> in, int out_parity, Spinor<P> x,
+                                double ax, double ad, cudaStream_t st) {
+  const LinkCopy& L = lat->links[prec_index<P>()];
+  if (!L.present) return STAG_EINVAL;
+  ProfScope ps(P == 64 ? "dslash64_epi" : "dslash_epi", st);
+  constexpr int PA = Acc<P>::value;
+  return epi_with_shape<P>(lat, L.shape_epi, Spinor<PA>{out, in.Vh}, in, out_parity, x, ax, Spinor<PA>{nullptr, in.Vh}, 0.0,
+                           ad, 0, RedScratch{nullptr, nullptr, 0}, RedTarget{RED_STORE, nullptr, nullptr}, nullptr, st, 0,
+                           -1, out);
 }
 
 // The same two kernels on the output sites [s0, s1) only (the interior of a
@@ -516,6 +549,9 @@ int tune_dslash(stag_lattice_s* lat, cudaStream_t st) {
                                     double, Spinor<Acc<P>::value>, double, double, int, RedScratch, RedTarget, \
                                     const int*, cudaStream_t);                                              \
   template int tune_dslash<P>(stag_lattice_s*, cudaStream_t);                                                  \
+  template int launch_dslash_canonical<P>(const stag_lattice_s*, double2*, Spinor<P>, int, cudaStream_t);         \
+  template int launch_dslash_epi_canonical<P>(const stag_lattice_s*, double2*, Spinor<P>, int, Spinor<P>, double, \
+                                              double, cudaStream_t);                                             \
   template int launch_dslash_range<P>(const stag_lattice_s*, Spinor<P>, Spinor<P>, int, int, int, const int*,    \
                                       cudaStream_t);                                                             \
   template int launch_dslash_epi_range<P>(const stag_lattice_s*, Spinor<Acc<P>::value>, Spinor<P>, int, Spinor<P>, \

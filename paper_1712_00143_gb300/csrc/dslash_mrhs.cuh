@@ -53,6 +53,9 @@ template <int P, int N, int RED>
 int mdslash_epi(const stag_lattice_s* lat, SpinorM<Acc<P>::value> out, SpinorM<P> in, int out_parity, SpinorM<P> x,
                 double ax, SpinorM<Acc<P>::value> y, double ay, double ad, RedScratch rs, RedTarget tgt,
                 const int* flags, cudaStream_t st);
+// the plain half with the result stored as N canonical fields of doubles
+template <int P, int N>
+int mdslash_canonical(const stag_lattice_s* lat, double2* out, SpinorM<P> in, int out_parity, cudaStream_t st);
 template <int P, int N> int tune_mrhs(stag_lattice_s* lat, cudaStream_t st);
 // <p_r, Ap_r> -> RED_MCG_ALPHA from the per-site values of mdslash_epi<P, N, 3>
 template <int P, int N>

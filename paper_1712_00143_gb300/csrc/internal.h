@@ -51,14 +51,14 @@ struct stag_lattice_s {
   double c3 = -1.0 / 24.0;
   int autotune = 1;  // time launch variants on this lattice (stag_link_opts.autotune)
   // launch variants of the N-right-hand-side kernels per (format, N = 2, 4,
-  // 8): the plain operator half and the epilogue form the batched CG runs
+  // 8, 3, 6): the plain operator half and the epilogue form the batched CG runs
   // (-1: not chosen yet), each with its time per launch (us)
   struct MrhsTune {
     int variant = -1;
     float us = 0.f;
     int variant_epi = -1;
     float us_epi = 0.f;
-  } mrhs[6][4];  // by the ABI precision (stag_prec), tuned per format
+  } mrhs[6][5];  // by the ABI precision (stag_prec), tuned per format
   stag::LinkCopy links[5];  // by stag_prec (STAG_DF64 = 4: FP64 split into hi + lo floats)
   stag::Workspace ws;
 };
@@ -147,6 +147,14 @@ template <int P>
 int launch_dslash_epi(const stag_lattice_s* lat, Spinor<Acc<P>::value> out, Spinor<P> in, int out_parity,
                       Spinor<P> x, double ax, Spinor<Acc<P>::value> y, double ay, double ad, int red,
                       RedScratch rs, RedTarget tgt, const int* flags, cudaStream_t st);
+
+// The plain operator half, and out = ax x + ad (D in), with the result stored
+// as a canonical field of doubles.
+template <int P>
+int launch_dslash_canonical(const stag_lattice_s* lat, double2* out, Spinor<P> in, int out_parity, cudaStream_t st);
+template <int P>
+int launch_dslash_epi_canonical(const stag_lattice_s* lat, double2* out, Spinor<P> in, int out_parity, Spinor<P> x,
+                                double ax, double ad, cudaStream_t st);
 
 // The plain and the fused-epilogue kernel on the output sites [s0, s1) only
 // (flags: a solver's stop word, or null).

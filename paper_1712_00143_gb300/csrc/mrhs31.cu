@@ -7,6 +7,8 @@ namespace stag {
 STAG_INSTANTIATE_MRHS_N(31, 2)
 STAG_INSTANTIATE_MRHS_N(31, 4)
 STAG_INSTANTIATE_MRHS_N(31, 8)
+STAG_INSTANTIATE_MRHS_PLAIN(31, 3)
+STAG_INSTANTIATE_MRHS_PLAIN(31, 6)
 STAG_INSTANTIATE_MRHS_RED3(31, 2)
 STAG_INSTANTIATE_MRHS_RED3(31, 4)
 STAG_INSTANTIATE_MRHS_RED3(31, 8)

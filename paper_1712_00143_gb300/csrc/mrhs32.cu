@@ -6,6 +6,8 @@ namespace stag {
 STAG_INSTANTIATE_MRHS_N(32, 2)
 STAG_INSTANTIATE_MRHS_N(32, 4)
 STAG_INSTANTIATE_MRHS_N(32, 8)
+STAG_INSTANTIATE_MRHS_PLAIN(32, 3)
+STAG_INSTANTIATE_MRHS_PLAIN(32, 6)
 STAG_INSTANTIATE_MRHS_RED3(32, 2)
 STAG_INSTANTIATE_MRHS_RED3(32, 4)
 STAG_INSTANTIATE_MRHS_RED3(32, 8)

@@ -39,9 +39,10 @@ constexpr int kNumMVariants = 6;
 
 // The variant used without tuning: FP32 with up to four right-hand sides
 // fits in 80 registers without spilling (six blocks, 24 warps, measured
-// faster than five); the other forms take no cap.
+// faster than five); six are split over two threads (one thread spills); the
+// other forms take no cap.
 __host__ __device__ constexpr int mrhs_default_variant(int p, int n) {
-  return ((p == 32 || p == 31) && n <= 4) ? 1 : 0;
+  return (p == 32 || p == 31) ? (n <= 4 ? 1 : n == 6 ? 2 : 0) : 0;
 }
 
 // Variants compiled for (format, Naik storage, N): the default always; the
@@ -56,21 +57,27 @@ __host__ __device__ constexpr bool mrhs_variant_built(int p, int nl, int n, int 
            ((p == 16 || p == 15) && n <= 4 && mvariant(v).minb != 6)));
 }
 
-template <int P, int NL, int N, int SP, int MINB>
+// CAN: the result goes to N canonical fields of doubles at out.v.
+template <int P, int NL, int N, int SP, int MINB, bool CAN>
 __global__ void __launch_bounds__(MB, MINB) k_dslash_mv(DslashArgsM<P> a, SpinorM<P> out, const int* flags) {
   static_assert(N % SP == 0, "right-hand sides split evenly");
   constexpr int NT = N / SP, SPB = MB / SP;
   if (stopped(flags)) return;
   const int part = threadIdx.x / SPB;
   const int s = blockIdx.x * SPB + (threadIdx.x - part * SPB);
-  if (s >= a.g.Vh) return;
-  const size_t off = spinor_bytes<P>(a.g.Vh) * (size_t)(part * NT);
-  a.in.v = (char*)a.in.v + off;
-  out.v = (char*)out.v + off;
+  if (s >= a.g.Vh || (MB % SP != 0 && part >= SP)) return;
+  a.in.v = (char*)a.in.v + spinor_bytes<P>(a.g.Vh) * (size_t)(part * NT);
+  out.v = (char*)out.v + spinor_bytes<CAN ? 64 : P>(a.g.Vh) * (size_t)(part * NT);
   typename Prec<P>::A2 d[NT][3];
   dslash_site_m<P, NL, NT>(a, s, d);
+  __shared__ float2 stage[CAN && P != 64 ? 3 * MB : 1];
 #pragma unroll
-  for (int r = 0; r < NT; ++r) SpinorLoadM<P>::st(out, s, r, d[r]);
+  for (int r = 0; r < NT; ++r) {
+    if constexpr (CAN)  // (blocks take a multiple of 32 sites in these formats)
+      store_canonical<P>((double2*)out.v + (size_t)r * 3 * a.g.Vh, STAG_BOUND(s, a.g.Vh, BOUND_VECTOR), d[r], stage);
+    else
+      SpinorLoadM<P>::st(out, s, r, d[r]);
+  }
 }
 
 // out_r = ax x_r + ay y_r + ad (D in)_r; RED = 1: Re<x_r, out_r>, RED = 2:
@@ -174,7 +181,10 @@ template <int P> DslashArgsM<P> make_args_m(const stag_lattice_s* lat, SpinorM<P
   return a;
 }
 
-__host__ __device__ constexpr int mrhs_nindex(int n) { return n == 2 ? 0 : n == 4 ? 1 : n == 8 ? 2 : 3; }
+__host__ __device__ constexpr int mrhs_nindex(int n) { return n == 2 ? 0 : n == 4 ? 1 : n == 8 ? 2 : n == 3 ? 3 : 4; }
+// Group sizes only stag_dslash forms (the batched solver's are 2, 4, 8): only
+// the plain half that stores canonical doubles is built.
+__host__ __device__ constexpr bool mrhs_plain_only(int n) { return n == 3 || n == 6; }
 
 // The variants a group of N right-hand sides of format P runs with on this
 // lattice: the plain operator half, and the epilogue form.
@@ -188,25 +198,31 @@ template <int P, int N> int mrhs_variant_epi(const stag_lattice_s* lat) {
 }
 
 template <int P, int NL, int N, int V>
-void launch_plain_v(int G, const DslashArgsM<P>& a, SpinorM<P> out, const int* flags, cudaStream_t st) {
+void launch_plain_v(int G, const DslashArgsM<P>& a, SpinorM<P> out, bool can, const int* flags, cudaStream_t st) {
   if constexpr (mrhs_variant_built(P, NL, N, V)) {
     constexpr MVariant mv = mvariant(V);
-    k_dslash_mv<P, NL, N, mv.sp, mv.minb><<<G, MB, 0, st>>>(a, out, flags);
+    if constexpr (!mrhs_plain_only(N)) {
+      if (!can) {
+        k_dslash_mv<P, NL, N, mv.sp, mv.minb, false><<<G, MB, 0, st>>>(a, out, flags);
+        return;
+      }
+    }
+    k_dslash_mv<P, NL, N, mv.sp, mv.minb, true><<<G, MB, 0, st>>>(a, out, flags);
   }
 }
 
 template <int P, int NL, int N>
-void dispatch_plain(int v, const DslashArgsM<P>& a, SpinorM<P> out, const int* flags, cudaStream_t st) {
+void dispatch_plain(int v, const DslashArgsM<P>& a, SpinorM<P> out, bool can, const int* flags, cudaStream_t st) {
   if (!mrhs_variant_built(P, NL, N, v)) v = mrhs_default_variant(P, N);
   const int spb = MB / mvariant(v).sp;
   const int G = (a.g.Vh + spb - 1) / spb;
   switch (v) {
-    case 0: launch_plain_v<P, NL, N, 0>(G, a, out, flags, st); break;
-    case 1: launch_plain_v<P, NL, N, 1>(G, a, out, flags, st); break;
-    case 2: launch_plain_v<P, NL, N, 2>(G, a, out, flags, st); break;
-    case 3: launch_plain_v<P, NL, N, 3>(G, a, out, flags, st); break;
-    case 4: launch_plain_v<P, NL, N, 4>(G, a, out, flags, st); break;
-    default: launch_plain_v<P, NL, N, 5>(G, a, out, flags, st);
+    case 0: launch_plain_v<P, NL, N, 0>(G, a, out, can, flags, st); break;
+    case 1: launch_plain_v<P, NL, N, 1>(G, a, out, can, flags, st); break;
+    case 2: launch_plain_v<P, NL, N, 2>(G, a, out, can, flags, st); break;
+    case 3: launch_plain_v<P, NL, N, 3>(G, a, out, can, flags, st); break;
+    case 4: launch_plain_v<P, NL, N, 4>(G, a, out, can, flags, st); break;
+    default: launch_plain_v<P, NL, N, 5>(G, a, out, can, flags, st);
   }
 }
 
@@ -247,7 +263,7 @@ void dispatch_epi(int v, const DslashArgsM<P>& a, SpinorM<Acc<P>::value> out, Sp
 template <int N>
 void launch_plain_fixed(const DslashArgsM<64>& a, SpinorM<64> out, const int* flags, cudaStream_t st) {
   constexpr int spb = MB / N;
-  k_dslash_mv<64, kNLFixed, N, N, 4><<<(a.g.Vh + spb - 1) / spb, MB, 0, st>>>(a, out, flags);
+  k_dslash_mv<64, kNLFixed, N, N, 4, false><<<(a.g.Vh + spb - 1) / spb, MB, 0, st>>>(a, out, flags);
 }
 template <int N, int RED>
 int launch_epi_fixed(const DslashArgsM<64>& a, SpinorM<64> out, SpinorM<64> x, double ax, SpinorM<64> y, double ay,
@@ -262,7 +278,7 @@ int launch_epi_fixed(const DslashArgsM<64>& a, SpinorM<64> out, SpinorM<64> x, d
 
 template <int P, int N>
 int mdslash_v(const stag_lattice_s* lat, int v, SpinorM<P> out, SpinorM<P> in, int out_parity, const int* flags,
-              cudaStream_t st) {
+              cudaStream_t st, bool can = false) {
   const LinkCopy& L = lat->links[prec_index<P>()];
   if (!L.present) return STAG_EINVAL;
   DslashArgsM<P> a = make_args_m<P>(lat, in, out_parity);
@@ -274,9 +290,9 @@ int mdslash_v(const stag_lattice_s* lat, int v, SpinorM<P> out, SpinorM<P> in, i
     }
   }
   if (P != 64 && L.nl == 6)
-    dispatch_plain<P, (P == 64 ? 9 : 6), N>(v, a, out, flags, st);
+    dispatch_plain<P, (P == 64 ? 9 : 6), N>(v, a, out, can, flags, st);
   else
-    dispatch_plain<P, 9, N>(v, a, out, flags, st);
+    dispatch_plain<P, 9, N>(v, a, out, can, flags, st);
   return last_launch_status();
 }
 
@@ -304,6 +320,11 @@ template <int P, int N>
 int mdslash(const stag_lattice_s* lat, SpinorM<P> out, SpinorM<P> in, int out_parity, const int* flags,
             cudaStream_t st) {
   return mdslash_v<P, N>(lat, mrhs_variant<P, N>(lat), out, in, out_parity, flags, st);
+}
+
+template <int P, int N>
+int mdslash_canonical(const stag_lattice_s* lat, double2* out, SpinorM<P> in, int out_parity, cudaStream_t st) {
+  return mdslash_v<P, N>(lat, mrhs_variant<P, N>(lat), SpinorM<P>{out, in.Vh, N}, in, out_parity, nullptr, st, true);
 }
 
 template <int P, int N, int RED>
@@ -334,6 +355,7 @@ template <int P, int N> int tune_mrhs(stag_lattice_s* lat, cudaStream_t st) {
     slot.variant = slot.variant_epi = def;
     return STAG_OK;
   }
+  if (mrhs_plain_only(N)) slot.variant_epi = def;
   const std::string key = tune_key("dslash_mrhs", abi_prec<P>(), L.nl, N, lat->dims);
   const std::string key_epi = tune_key("dslash_mrhs_epi", abi_prec<P>(), L.nl, N, lat->dims);
   auto cached = [&](const std::string& k, int* v, float* us) {
@@ -353,7 +375,7 @@ template <int P, int N> int tune_mrhs(stag_lattice_s* lat, cudaStream_t st) {
   const int Vh = lat->g.Vh;
   int s = 0;
   SpinorM<P> in{lat->ws.get("tunem.in", spinorm_bytes<P>(Vh, N), &s), Vh, N};
-  SpinorM<P> t{lat->ws.get("tunem.t", spinorm_bytes<P>(Vh, N), &s), Vh, N};
+  SpinorM<P> t{lat->ws.get("tunem.t", spinorm_bytes<mrhs_plain_only(N) ? 64 : P>(Vh, N), &s), Vh, N};
   SpinorM<PA> o{lat->ws.get("tunem.o", spinorm_bytes<PA>(Vh, N), &s), Vh, N};
   double* pw = (double*)lat->ws.get("tunem.pw", sizeof(float) * N * (size_t)Vh, &s);
   if (s) return s;
@@ -379,8 +401,8 @@ template <int P, int N> int tune_mrhs(stag_lattice_s* lat, cudaStream_t st) {
         if (it == 0) s = cuda_status(cudaEventRecord(e0, st));
         if (s) break;
         if (form == 0)
-          s = mdslash_v<P, N>(lat, v, t, in, 1, nullptr, st);
-        else
+          s = mdslash_v<P, N>(lat, v, t, in, 1, nullptr, st, mrhs_plain_only(N));
+        else if constexpr (!mrhs_plain_only(N))
           s = mdslash_epi_v<P, N, RED>(lat, v, o, t, 0, in, 0.01, none, 0.0, -1.0, rs,
                                        RedTarget{RED_STORE, nullptr, nullptr}, nullptr, st);
       }
@@ -453,7 +475,12 @@ int launch_mcg_alpha_pt(const stag_lattice_s* lat, const float* pt, McgState* g,
   return last_launch_status();
 }
 
+#define STAG_INSTANTIATE_MRHS_PLAIN(P, N)                                                                           \
+  template int mdslash_canonical<P, N>(const stag_lattice_s*, double2*, SpinorM<P>, int, cudaStream_t);             \
+  template int tune_mrhs<P, N>(stag_lattice_s*, cudaStream_t);
+
 #define STAG_INSTANTIATE_MRHS_N(P, N)                                                                               \
+  template int mdslash_canonical<P, N>(const stag_lattice_s*, double2*, SpinorM<P>, int, cudaStream_t);             \
   template int mdslash<P, N>(const stag_lattice_s*, SpinorM<P>, SpinorM<P>, int, const int*, cudaStream_t);         \
   template int mdslash_epi<P, N, 0>(const stag_lattice_s*, SpinorM<Acc<P>::value>, SpinorM<P>, int, SpinorM<P>,     \
                                     double, SpinorM<Acc<P>::value>, double, double, RedScratch, RedTarget,          \
