@@ -285,7 +285,7 @@ static DslashArgs<P> make_args(const stag_lattice_s* lat, Spinor<P> in, int out_
 // chip's 608 warp schedulers with one warp or none.  One operator (two
 // halves), this form and the other: 8^4 12.3 and 28.7 us, 12 x 16^3 37.5 and
 // 49.2 us, 16^4 48.2 and 51.4 us.
-constexpr int kFewSites = 1 << 15;
+// (kFewSites: internal.h)
 template <int RED>
 __global__ void __launch_bounds__(128)
     k_dslash_few(DslashArgs<64> a, Spinor<64> out, Spinor<64> x, double ax, Spinor<64> y, double ay, double ad,

@@ -192,6 +192,18 @@ int launch_ru_convert_dot(Spinor<Acc<P>::value> rh, Spinor<64> r, Spinor<P> p, C
 // p = rh + beta (p - ortho rh)
 template <int P> int launch_ru_p(Spinor<P> p, Spinor<Acc<P>::value> rh, CgState* state, cudaStream_t st);
 
+// The iterations up to the next stop flag as one cooperative kernel (cg_loop.cu)
+template <int P>
+int launch_cg_loop(stag_lattice_s* lat, Spinor<P> p, Spinor<P> p2, Spinor<P> t, Spinor<32> Ap, Spinor<32> xh,
+                   Spinor<32> rh, CgState* state, int pending, int most, RedScratch rs, unsigned* sync, cudaStream_t st);
+// Sites per parity up to which the fixed-point FP64 operator runs one hop per
+// thread (dslash_impl.cuh says why the line lies there).
+constexpr int kFewSites = 1 << 15;
+// Sites per parity up to which a mixed-precision solve takes it.  Queued
+// kernels against the loop, m = 0.1 to 1e-12: 8^4 6.37 and 2.93 ms, 12^4 7.7
+// and 4.6, 12^2 16^2 8.2 and 5.8, 16^4 8.8 and 8.3, 20^4 14.1 and 18.0 ms.
+constexpr int kLoopSites = 1 << 15;
+
 // Multi-shift: r -= alpha Ap; ||r||^2 -> RED_MS_BETA
 template <int P>
 int launch_ms_r_update(Spinor<Acc<P>::value> r, Spinor<Acc<P>::value> Ap, MsState* state, RedScratch rs,

@@ -81,7 +81,9 @@ static int cg_solve(stag_lattice_s* lat, double2* x_can, const double2* b_can, d
   double* dscal = (double*)lat->ws.get("cg.scalars", 64, &s);
   // reliable updates in double-float when the handle holds that link copy,
   // measured from an anchor (ya64, its residual radf): r = r_a - M (y - y_a)
-  const bool use_df = P != 64 && lat->links[STAG_DF64].present;
+  // (on few sites the FP64 operator is the faster one: dslash_impl.cuh)
+  const bool few = lat->links[STAG_FP64].fixed && Vh <= kFewSites;
+  const bool use_df = P != 64 && lat->links[STAG_DF64].present && !few;
   DfField radf{nullptr, Vh}, ydf{nullptr, Vh}, tdf{nullptr, Vh}, rdf{nullptr, Vh};
   Spinor<64> ya64{nullptr, Vh};
   if (use_df) {
@@ -98,10 +100,20 @@ static int cg_solve(stag_lattice_s* lat, double2* x_can, const double2* b_can, d
     TRY(launch_dslash_df(lat, tdf, ydf, 1, 1, nullptr, st));
     return launch_dslash_df_epi(lat, rdf, tdf, 1, 0, ydf, -shift, radf, 1.0, 1.0, nullptr, st);
   };
+  // small lattices: the iterations between two updates as one kernel
+  bool loop = P != 64 && Vh <= kLoopSites;
+  Spinor<P> p2{nullptr, Vh};
+  unsigned* sync = nullptr;
+  if (loop) {
+    if (P == 32 || P == 31) p2 = ws_spinor<P>(lat, "cg.p2", &s);
+    sync = (unsigned*)lat->ws.get("cg.sync", 64, &s);
+    if (s) return s;
+  }
   PinnedState pin(sizeof(CgState) + 64);
   if (!pin.h) return STAG_ENOMEM;
   CgState* hs = (CgState*)pin.h;
   double* hscal = (double*)((char*)pin.h + sizeof(CgState));
+  unsigned* hsync = (unsigned*)(hscal + 4);
 
   // ||b||^2 and the initial residual
   TRY(launch_from_canonical<64>(b64, b_can, Vh, st));
@@ -181,7 +193,20 @@ static int cg_solve(stag_lattice_s* lat, double2* x_can, const double2* b_can, d
         break;
       }
       const long long mark = prof_mark();
-      for (int i = 0; i < C; ++i) {
+      if constexpr (P != 64) {
+        if (loop) {
+          const int ls = launch_cg_loop<P>(lat, p, p2, t, Ap, xh, rh, dst, pending_p, 4096, rs, sync, st);
+          if (ls == STAG_OK) {
+            pending_p = true;
+            TRY(cuda_status(cudaMemcpyAsync(hsync, sync, 2 * sizeof(unsigned), cudaMemcpyDeviceToHost, st)));
+          } else if (ls == STAG_EINVAL) {
+            loop = false;
+          } else {
+            return ls;
+          }
+        }
+      }
+      for (int i = 0; i < C && !loop; ++i) {
         if (pending_p) TRY(launch_cg_xpay<P>(p, rh, dst, st));
         TRY(launch_dslash<P>(lat, t, p, 1, flags, st));
         TRY(launch_dslash_epi<P>(lat, Ap, t, 0, p, shift, none_spinor<PV>(Vh), 0.0, -1.0, 1, rs,
@@ -191,7 +216,8 @@ static int cg_solve(stag_lattice_s* lat, double2* x_can, const double2* b_can, d
       }
       TRY(cuda_status(cudaMemcpyAsync(hs, dst, sizeof(CgState), cudaMemcpyDeviceToHost, st)));
       TRY(cuda_status(cudaStreamSynchronize(st)));
-      if (hs->flags & F_STOP) prof_discard_since(mark);  // launches after the flag returned at once
+      if (loop && hsync[1]) return STAG_ETIMEOUT;
+      if ((hs->flags & F_STOP) && !loop) prof_discard_since(mark);  // launches after the flag returned at once
       prof_flush_completed();
       if (hs->flags & F_BREAKDOWN) {
         status = STAG_EBREAKDOWN;
