@@ -1,7 +1,7 @@
 // flags.h -- host-side handling of the library's device status words.
 //
-// Kernels that give up a bounded wait (the tensor-core layers' mbarrier
-// waits) record it in a device word instead of trapping, and the host turns
+// Kernels that give up a bounded wait (the grid barriers of the
+// CG loop) record it in a device word instead of trapping, and the host turns
 // the word into a status: read it; if it is set, clear it and report the
 // status that goes with it, so that the next check starts clean.  The
 // reading and clearing are passed in, so that the logic is the same with a

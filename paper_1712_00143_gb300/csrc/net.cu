@@ -7,8 +7,7 @@
 #include <cstring>
 #include <vector>
 
-#include "flags.h"
-#include "net_tc.cuh"
+#include "net_mma.cuh"
 
 struct stag_net_s {
   int nl = 0;
@@ -65,11 +64,20 @@ __global__ void k_adam(float* w, float* m, float* v, const float* __restrict__ g
   }
 }
 
+// FP64 scalars derived from a device norm are computed by one thread per
+// block: a square root and a division hold a warp's FP64 pipe for microseconds.
+template <class F> __device__ __forceinline__ double once_per_block(F f) {
+  __shared__ double v;
+  if (threadIdx.x == 0) v = f();
+  __syncthreads();
+  return v;
+}
+
 // One-channel input field: even sites r * scale, odd sites 0 (scale from a
 // device norm: sqrt(Vh / ||r||^2)).
 __global__ void k_net_embed(Spinor<32> r, const double* __restrict__ rr, float2* __restrict__ h0) {
   const int Vh = r.Vh;
-  const float sc = (float)sqrt((double)Vh / fmax(*rr, 1e-300));
+  const float sc = (float)once_per_block([&] { return sqrt((double)Vh / fmax(*rr, 1e-300)); });
   for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < Vh; s += gridDim.x * blockDim.x) {
     float2 v[3];
     SpinorLoad<32>::ld(r, s, v);
@@ -84,7 +92,7 @@ __global__ void k_net_embed(Spinor<32> r, const double* __restrict__ rr, float2*
 // z = prediction / scale on even sites (the network's output channel).
 __global__ void k_net_extract(const float2* __restrict__ hL, const double* __restrict__ rr, Spinor<32> z) {
   const int Vh = z.Vh;
-  const float inv = (float)sqrt(fmax(*rr, 0.0) / (double)Vh);
+  const float inv = (float)once_per_block([&] { return sqrt(fmax(*rr, 0.0) / (double)Vh); });
   for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < Vh; s += gridDim.x * blockDim.x) {
     float2 o[3];
 #pragma unroll
@@ -139,8 +147,9 @@ __global__ void k_net_pred_to_spinor(const float2* __restrict__ hL, Spinor<32> z
 __global__ void k_net_resid_loss(Spinor<32> mz, Spinor<32> r, const double* __restrict__ rr, Spinor<32> diff, RedBuf rb,
                                  RedTarget tgt) {
   const int Vh = r.Vh;
-  const double sc2 = (double)Vh / fmax(*rr, 1e-300);
-  const float sc = (float)sqrt(sc2);
+  const double sc2 = once_per_block([&] { return (double)Vh / fmax(*rr, 1e-300); });
+  __syncthreads();  // the block's word is used again
+  const float sc = (float)once_per_block([&] { return sqrt(sc2); });
   Acc1<float> acc;
   for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < Vh; s += gridDim.x * blockDim.x) {
     float2 a[3], b[3], o[3];
@@ -193,6 +202,7 @@ struct NetRun {
   float2* g1 = nullptr;
   float* part = nullptr;        // per-block partial sums for dW / db
   int part_blocks = 0;
+  bool training = false;
   double* scal = nullptr;       // rr, ee, loss
   RedScratch rs;
 };
@@ -202,6 +212,7 @@ static int net_run_init(stag_net_s* net, stag_lattice_s* lat, NetRun& R, bool tr
   R.net = net;
   R.lat = lat;
   R.Vh = lat->g.Vh;
+  R.training = training;
   R.ng.g = lat->g;
   const LinkCopy& L = lat->links[STAG_FP32];
   R.ng.links[0] = (const uint4*)L.data;
@@ -223,7 +234,7 @@ static int net_run_init(stag_net_s* net, stag_lattice_s* lat, NetRun& R, bool tr
   if (training) {
     R.g0 = (float2*)net->ws.get(pre + "g0", sites * cmax * 3 * sizeof(float2), &s);
     R.g1 = (float2*)net->ws.get(pre + "g1", sites * cmax * 3 * sizeof(float2), &s);
-    R.part_blocks = 2 * 152;
+    R.part_blocks = 3 * 152;
     R.part = (float*)net->ws.get(pre + "part", (size_t)R.part_blocks * NET_NDIR * cmax * cmax * sizeof(float), &s);
   }
   R.scal = (double*)net->ws.get(pre + "scal", 64, &s);
@@ -231,61 +242,10 @@ static int net_run_init(stag_net_s* net, stag_lattice_s* lat, NetRun& R, bool tr
   return get_red_scratch(lat, "net", &R.rs, 2);
 }
 
-template <int CIN, int COUT, bool GATE>
-static int launch_layer(const NetRun& R, int l, const float2* in, float2* pre, float2* out, const __nv_bfloat16* W,
-                        const float* b, int transpose, cudaStream_t st) {
-  const int n = 2 * R.Vh;
-  count_launch();
-  if constexpr (CIN == 16 && COUT == 16) {
-    // the channel mixing of a 16 -> 16 layer runs on the tensor cores
-    // one CTA per 64-site tile
-    static bool attr[2] = {false, false};
-    if (!attr[GATE]) {
-      cudaFuncSetAttribute(k_net_layer_tc<GATE>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::LAYER_SMEM);
-      attr[GATE] = true;
-    }
-    // the layer's bulk copies need 16-byte aligned input records
-    if (((uintptr_t)in & 15u) != 0) return STAG_EINVAL;
-    const int tiles = 2 * ((R.Vh + tc::TILE - 1) / tc::TILE);
-    k_net_layer_tc<GATE><<<tiles, 128, tc::LAYER_SMEM, st>>>(R.ng, in, pre, out, W, b, transpose);
-  } else if constexpr (COUT == 1 && CIN == 16 && !GATE) {
-    if (!transpose) {
-      // one output channel: site-local mix into the nine directions, then
-      // one transport per direction
-      k_net_mix_local<CIN><<<grid_for(n, 256), 256, 0, st>>>(n, in, W, R.U);
-      count_launch();
-      k_net_transport_sum<<<grid_for(n, 256), 256, 0, st>>>(R.ng, R.U, out);
-    } else {
-      k_net_layer<CIN, COUT, GATE><<<(n + 127) / 128, 128, 0, st>>>(R.ng, in, pre, out, W, b, transpose);
-    }
-  } else {
-    // 16 output channels: the block's outputs are staged in shared memory
-    const size_t smem = COUT == 16 ? (size_t)128 * 97 * sizeof(float) : 0;
-    static bool attr = false;
-    if (COUT == 16 && !attr) {
-      cudaFuncSetAttribute(k_net_layer<CIN, COUT, GATE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      attr = true;
-    }
-    k_net_layer<CIN, COUT, GATE><<<(n + 127) / 128, 128, smem, st>>>(R.ng, in, pre, out, W, b, transpose);
-  }
-  return STAG_OK;
-}
-
-// STAG_ETIMEOUT if a tensor-core layer gave up a bounded wait since the
-// last check (the flag is cleared here).  Synchronous.
-static int net_tc_status() {
-  auto read = [](int* v) {
-    const cudaError_t e = cudaMemcpyFromSymbol(v, tc::g_tc_error, sizeof(int));
-    if (e != cudaSuccess) cudaGetLastError();
-    return e == cudaSuccess ? 0 : 1;
-  };
-  auto clear = []() {
-    const int z = 0;
-    const cudaError_t e = cudaMemcpyToSymbol(tc::g_tc_error, &z, sizeof(int));
-    if (e != cudaSuccess) cudaGetLastError();
-    return e == cudaSuccess ? 0 : 1;
-  };
-  return take_flag(read, clear, STAG_ETIMEOUT);
+// Blocks of a kernel whose warps take 8 sites of one parity each, at most `most`.
+static int grid_groups(int Vh, int warps, int most) {
+  const int n = (2 * ((Vh + 7) / 8) + warps - 1) / warps;
+  return n < most ? n : most;
 }
 
 // Layer l forward (ch[l] -> ch[l+1]); supported widths 1 and 16.
@@ -296,14 +256,27 @@ static int layer_fwd(const NetRun& R, int l, cudaStream_t st) {
   const __nv_bfloat16* W = N->wb + N->woff[l];
   const float* b = gate ? N->w + N->boff[l] : nullptr;
   float2 *in = R.h[l], *out = R.h[l + 1], *pre = gate ? R.pre[l + 1] : R.h[l + 1];
+  // the gated value is kept for the backward pass only
+  if (!R.training && gate) pre = nullptr;
   ProfScope ps(ci == 16 && co == 16 ? "net_tc" : "net", st);
-  int ls;
-  if (ci == 1 && co == 16 && gate) ls = launch_layer<1, 16, true>(R, l, in, pre, out, W, b, 0, st);
-  else if (ci == 16 && co == 16 && gate) ls = launch_layer<16, 16, true>(R, l, in, pre, out, W, b, 0, st);
-  else if (ci == 16 && co == 1 && !gate) ls = launch_layer<16, 1, false>(R, l, in, pre, out, W, b, 0, st);
-  else if (ci == 1 && co == 1 && !gate) ls = launch_layer<1, 1, false>(R, l, in, pre, out, W, b, 0, st);
-  else return STAG_EINVAL;
-  if (ls) return ls;
+  const int n = 2 * R.Vh;
+  if (ci == 1 && co == 16 && gate) {
+    k_net_layer_1to16<true><<<grid_groups(R.Vh, 8, 1 << 20), 256, 0, st>>>(R.ng, in, pre, out, W, b);
+  } else if (ci == 16 && co == 16 && gate) {
+    if (((uintptr_t)in & 15u) != 0) return STAG_EINVAL;  // records are read as 16-byte words
+    k_net_layer_mma<<<grid_groups(R.Vh, nm::FW, 2 * 152), 32 * nm::FW, 0, st>>>(R.ng, in, pre, out, W, b);
+  } else if (ci == 16 && co == 1 && !gate) {
+    // one output channel: site-local mix into the directions, then one
+    // transport per direction, for the even sites the prediction is read on
+    k_net_mix_local16<<<(2 * ((R.Vh + 31) / 32) + 3) / 4, 128, 0, st>>>(R.Vh, in, W, R.U);
+    TRYN(last_launch_status());
+    count_launch();
+    k_net_transport_sum<<<grid_for(R.Vh, 256), 256, 0, st>>>(R.ng, R.U, out);
+  } else if (ci == 1 && co == 1 && !gate) {
+    k_net_layer_1to1<<<grid_for(n, 256), 256, 0, st>>>(R.ng, in, out, W);
+  } else {
+    return STAG_EINVAL;
+  }
   return last_launch_status();
 }
 
@@ -319,45 +292,46 @@ static int layer_bwd(const NetRun& R, int l, float2* g, float2* gin, bool want_i
     ProfScope ps("net_bwd", st);
     const int G = R.part_blocks;
     if (co == 16)
-      k_net_gate_bwd<16><<<G, 256, 0, st>>>(n2, R.pre[l + 1], g, N->w + N->boff[l], R.part);
+      k_net_gate_bwd16<<<G, 256, 0, st>>>(n2, R.pre[l + 1], g, N->w + N->boff[l], R.part);
     else
       return STAG_EINVAL;
     TRYN(last_launch_status());
-    k_net_sum_parts<<<1, 64, 0, st>>>(R.part, G, co, N->grad + N->boff[l]);
+    k_net_sum_parts<<<(co + 31) / 32, 256, 0, st>>>(R.part, G, co, N->grad + N->boff[l]);
     TRYN(last_launch_status());
   }
+  // dW, and the adjoint layer: co -> ci channels with W' (transposed, partner
+  // directions, sign).  16 -> 16: both from one pass over the transports.
+  const __nv_bfloat16* W = N->wb + N->woff[l];
+  const int nw = NET_NDIR * ci * co;
+  int G = 0;
   {
     ProfScope ps("net_bwd", st);
-    constexpr int TS = 16;
-    const int G = R.part_blocks;
-    const int nw = NET_NDIR * ci * co;
-#define STAG_DW(CI, CO)                                                                                  \
-  {                                                                                                      \
-    const size_t smem = (size_t)(TS * NET_NDIR * CI * 6 + TS * CO * 6) * sizeof(float);                   \
-    cudaFuncSetAttribute(k_net_dw<CI, CO, TS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);  \
-    k_net_dw<CI, CO, TS><<<G, 256, smem, st>>>(R.ng, R.h[l], g, R.part);                                  \
-  }
-    if (ci == 1 && co == 16) STAG_DW(1, 16)
-    else if (ci == 16 && co == 16) STAG_DW(16, 16)
-    else if (ci == 16 && co == 1) STAG_DW(16, 1)
-    else if (ci == 1 && co == 1) STAG_DW(1, 1)
-    else return STAG_EINVAL;
-#undef STAG_DW
+    if (ci == 16 && co == 16) {
+      if (!want_in) return STAG_EINVAL;  // (the first layer has one input channel)
+      G = grid_groups(R.Vh, nm::AW, R.part_blocks);
+      TRYN(cuda_status(cudaFuncSetAttribute(k_net_adjoint_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, nm::ADJ_SMEM)));
+      k_net_adjoint_mma<<<G, 32 * nm::AW, nm::ADJ_SMEM, st>>>(R.ng, g, R.h[l], gin, W, R.part);
+    } else if (ci == 1 && co == 16) {
+      G = grid_groups(R.Vh, 4, R.part_blocks);
+      k_net_dw_thin<<<G, 128, 0, st>>>(R.ng, R.h[l], g, 0, R.part);
+    } else if (ci == 16 && co == 1) {
+      G = grid_groups(R.Vh, 4, R.part_blocks);
+      k_net_dw_thin<<<G, 128, 0, st>>>(R.ng, g, R.h[l], 1, R.part);
+    } else if (ci == 1 && co == 1) {
+      G = 152;
+      k_net_dw_1to1<<<G, 256, 0, st>>>(R.ng, R.h[l], g, R.part);
+    } else {
+      return STAG_EINVAL;
+    }
     TRYN(last_launch_status());
-    k_net_sum_parts<<<grid_for(nw, 256), 256, 0, st>>>(R.part, G, nw, N->grad + N->woff[l]);
+    count_launch();
+    k_net_sum_parts<<<(nw + 31) / 32, 256, 0, st>>>(R.part, G, nw, N->grad + N->woff[l]);
     TRYN(last_launch_status());
   }
-  if (want_in) {
-    // adjoint layer: co -> ci channels with W' (transposed, partner directions, sign)
+  if (want_in && co == 1) {
     ProfScope ps("net_bwd", st);
-    const __nv_bfloat16* W = N->wb + N->woff[l];
-    int ls;
-    if (ci == 16 && co == 16) ls = launch_layer<16, 16, false>(R, l, g, gin, gin, W, nullptr, 1, st);
-    else if (ci == 16 && co == 1) ls = launch_layer<1, 16, false>(R, l, g, gin, gin, W, nullptr, 1, st);
-    else if (ci == 1 && co == 16) ls = launch_layer<16, 1, false>(R, l, g, gin, gin, W, nullptr, 1, st);
-    else if (ci == 1 && co == 1) ls = launch_layer<1, 1, false>(R, l, g, gin, gin, W, nullptr, 1, st);
-    else return STAG_EINVAL;
-    TRYN(ls);
+    if (ci != 16) return STAG_EINVAL;
+    k_net_layer_1to16<false><<<grid_groups(R.Vh, 8, 1 << 20), 256, 0, st>>>(R.ng, g, nullptr, gin, W, nullptr);
     TRYN(last_launch_status());
   }
   return STAG_OK;
@@ -585,8 +559,7 @@ int stag_net_loss_grad(stag_net_t n, stag_lattice_t lat, const void* r, const vo
   TRYN(net_loss_grad(R, rs, es, loss_kind, mass, R.scal + 2, st));
   TRYN(cuda_status(cudaMemcpyAsync(loss, R.scal + 2, sizeof(double), cudaMemcpyDeviceToHost, st)));
   TRYN(cuda_status(cudaMemcpyAsync(grad, n->grad, n->nparam * 4, cudaMemcpyDeviceToHost, st)));
-  TRYN(cuda_status(cudaStreamSynchronize(st)));
-  return net_tc_status();
+  return cuda_status(cudaStreamSynchronize(st));
 }
 
 int stag_tc_selftest(double* max_rel_err) {
@@ -662,8 +635,7 @@ int stag_net_train(stag_net_t n, const stag_train_pair* pairs, int npairs, const
   }
   if (losses)
     TRYN(cuda_status(cudaMemcpyAsync(losses, lossd, sizeof(double) * (size_t)npairs * tp->epochs, cudaMemcpyDeviceToHost, st)));
-  TRYN(cuda_status(cudaStreamSynchronize(st)));
-  return net_tc_status();
+  return cuda_status(cudaStreamSynchronize(st));
 }
 
 }  // extern "C"
@@ -927,7 +899,6 @@ static int fcg_solve(stag_lattice_s* lat, stag_net_s* net, double2* x_can, const
       TRYN(cuda_status(cudaMemcpyAsync(hs, dst, sizeof(FcgState), cudaMemcpyDeviceToHost, st)));
       TRYN(cuda_status(cudaStreamSynchronize(st)));
       prof_flush_completed();
-      TRYN(net_tc_status());
       if (hs->cg.flags & F_BREAKDOWN) {
         status = STAG_EBREAKDOWN;
         break;

@@ -2,7 +2,8 @@
 // preconditioner network (definition in include/stag.h, stag_net_create).
 //
 // Activations are full-lattice fields stored per parity: [2][Vh][C][3]
-// complex FP32, the C channels of a site contiguous.  A layer reads, for each
+// complex FP32, a site's channels contiguous (16 channels: in the word order
+// of net_mma.cuh).  A layer reads, for each
 // of its 9 directions d, the fat-link hop of the staggered operator (the
 // library's FP32 link copy: entries mu*CPM + 0..17 of the output parity's
 // chunk list hold the +mu and -mu hop matrices with eta and 1/2 folded in)
@@ -17,7 +18,9 @@
 namespace stag {
 
 constexpr int NET_NDIR = 9;
-constexpr int NET_MAXC = 16;
+template <int V> struct IntC {
+  static constexpr int value = V;
+};
 
 struct NetGeom {
   Geom g;
@@ -67,257 +70,228 @@ __device__ __forceinline__ void net_neighbour(const NetGeom& ng, int p, int s, i
   np = 1 - p;
 }
 
-// pre_c(x) = sum_d sum_c' W[d][c][c'] (T_d h_c')(x); GATE: out = pre * sigmoid(|pre|^2 - b_c).
-// Weights come in as bfloat16 [9][COUT][CIN]; wsign[d] multiplies direction d
-// (used for the adjoint pass: T_{1+2mu}^dag = -T_{2+2mu}).
-template <int CIN, int COUT, bool GATE>
-__global__ void __launch_bounds__(128) k_net_layer(NetGeom ng, const float2* __restrict__ hin, float2* __restrict__ pre,
-                                                  float2* __restrict__ hout, const __nv_bfloat16* __restrict__ W,
-                                                  const float* __restrict__ bias, int transpose) {
-  __shared__ float sw[NET_NDIR * COUT * CIN];
-  for (int i = threadIdx.x; i < NET_NDIR * COUT * CIN; i += blockDim.x) {
-    // transpose != 0: the adjoint layer -- W'[d][c][c'] = sign(d) * W[partner(d)][c'][c]
-    if (!transpose) {
-      sw[i] = __bfloat162float(W[i]);
-    } else {
-      const int d = i / (COUT * CIN), rem = i % (COUT * CIN), c = rem / CIN, cp = rem % CIN;
-      const int dd = d == 0 ? 0 : ((d & 1) ? d + 1 : d - 1);
-      const float sg = d == 0 ? 1.f : -1.f;
-      sw[i] = sg * __bfloat162float(W[(dd * CIN + cp) * COUT + c]);  // source layer is [9][CIN][COUT]
-    }
-  }
-  __syncthreads();
+// The single layer of a network without hidden channels: out(x) = sum_d W[d] (T_d h)(x).
+__global__ void __launch_bounds__(256) k_net_layer_1to1(NetGeom ng, const float2* __restrict__ hin, float2* __restrict__ hout,
+                                                       const __nv_bfloat16* __restrict__ W) {
   const int Vh = ng.g.Vh;
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  const bool valid = idx < 2 * Vh;
-  const int p = valid ? idx / Vh : 0, s = valid ? idx - p * Vh : 0;
-  float2 acc[COUT][3];
-#pragma unroll
-  for (int c = 0; c < COUT; ++c)
-#pragma unroll
-    for (int i = 0; i < 3; ++i) acc[c][i] = make_float2(0.f, 0.f);
+  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < 2 * Vh; idx += gridDim.x * blockDim.x) {
+    const int p = idx / Vh, s = idx - p * Vh;
+    float2 acc[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll 1
-  for (int d = 0; d < (valid ? NET_NDIR : 0); ++d) {
-    int np, ns;
-    net_neighbour(ng, p, s, d, np, ns);
-    float2 w[9];
-    if (d) load_hop_matrix(ng, p, s, d, w);
-    const float2* src = act_ptr(hin, CIN, Vh, np, ns);
-    if constexpr (COUT == 1 && CIN > 1) {
-      // one output channel: mix first, then transport once (T_d is linear
-      // and the weights are real, so sum_c' W T_d h_c' = T_d sum_c' W h_c')
-      float2 m[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-      const float* wr = sw + d * CIN;
-#pragma unroll 4
-      for (int cp = 0; cp < CIN; ++cp) {
-        const float k = wr[cp];
+    for (int d = 0; d < NET_NDIR; ++d) {
+      int np, ns;
+      net_neighbour(ng, p, s, d, np, ns);
+      const float k = __bfloat162float(W[d]);
+      const float2* src = hin + ((size_t)np * Vh + ns) * 3;
+      float2 v[3], t[3], w[9];
+      if (d) load_hop_matrix(ng, p, s, d, w);
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          const float2 v = __ldg(src + cp * 3 + i);
-          m[i].x = fmaf(k, v.x, m[i].x);
-          m[i].y = fmaf(k, v.y, m[i].y);
-        }
-      }
+      for (int i = 0; i < 3; ++i) v[i] = __ldg(src + i);
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
         if (d) {
-#pragma unroll
-          for (int j = 0; j < 3; ++j) cmac(acc[0][i], w[3 * i + j], m[j]);
-        } else {
-          acc[0][i].x += m[i].x;
-          acc[0][i].y += m[i].y;
-        }
-      }
-    } else {
-#pragma unroll 4
-    for (int cp = 0; cp < CIN; ++cp) {
-      float2 v[3], t[3];
-#pragma unroll
-      for (int i = 0; i < 3; ++i) v[i] = __ldg(src + cp * 3 + i);
-      if (d) {
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
           t[i] = make_float2(0.f, 0.f);
 #pragma unroll
           for (int j = 0; j < 3; ++j) cmac(t[i], w[3 * i + j], v[j]);
+        } else {
+          t[i] = v[i];
         }
-      } else {
-#pragma unroll
-        for (int i = 0; i < 3; ++i) t[i] = v[i];
-      }
-      const float* wr = sw + (d * COUT) * CIN + cp;
-#pragma unroll
-      for (int c = 0; c < COUT; ++c) {
-        const float k = wr[c * CIN];
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          acc[c][i].x = fmaf(k, t[i].x, acc[c][i].x);
-          acc[c][i].y = fmaf(k, t[i].y, acc[c][i].y);
-        }
+        acc[i].x = fmaf(k, t[i].x, acc[i].x);
+        acc[i].y = fmaf(k, t[i].y, acc[i].y);
       }
     }
-    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) hout[(size_t)idx * 3 + i] = acc[i];
   }
-  if constexpr (COUT == 16) {
-    // staged epilogue: the block's 128 sites x 16 channels go through shared
-    // memory so that consecutive threads store consecutive 24-byte channel
-    // vectors (a site's record is 384 bytes; per-site stores would be strided)
-    extern __shared__ float net_epi[];  // [blockDim][97]
-    float* e = net_epi + threadIdx.x * 97;
+}
+
+// Its weight gradient dW[d] = sum_x Re <g(x), (T_d h)(x)>: per-block sums, threads in order.
+__global__ void __launch_bounds__(256) k_net_dw_1to1(NetGeom ng, const float2* __restrict__ hin, const float2* __restrict__ g,
+                                                    float* __restrict__ part) {
+  __shared__ float sm[256];
+  const int Vh = ng.g.Vh;
+  for (int d = 0; d < NET_NDIR; ++d) {
+    float acc = 0.f;
+    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < 2 * Vh; idx += gridDim.x * blockDim.x) {
+      const int p = idx / Vh, s = idx - p * Vh;
+      int np, ns;
+      net_neighbour(ng, p, s, d, np, ns);
+      const float2* src = hin + ((size_t)np * Vh + ns) * 3;
+      float2 v[3], w[9];
+      if (d) load_hop_matrix(ng, p, s, d, w);
 #pragma unroll
-    for (int c = 0; c < 16; ++c)
+      for (int i = 0; i < 3; ++i) v[i] = __ldg(src + i);
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
-        e[c * 6 + 2 * i] = acc[c][i].x;
-        e[c * 6 + 2 * i + 1] = acc[c][i].y;
+        float2 t = v[i];
+        if (d) {
+          t = make_float2(0.f, 0.f);
+#pragma unroll
+          for (int j = 0; j < 3; ++j) cmac(t, w[3 * i + j], v[j]);
+        }
+        const float2 q = __ldg(g + (size_t)idx * 3 + i);
+        acc = fmaf(q.x, t.x, acc);
+        acc = fmaf(q.y, t.y, acc);
       }
+    }
+    sm[threadIdx.x] = acc;
     __syncthreads();
-    const int base = blockIdx.x * blockDim.x;
-    for (int q = threadIdx.x; q < (int)blockDim.x * 16; q += blockDim.x) {
-      const int sl = q >> 4, c = q & 15, site = base + sl;
-      if (site >= 2 * Vh) continue;
-      const float* ev = net_epi + sl * 97 + c * 6;
-      float2 v[3] = {make_float2(ev[0], ev[1]), make_float2(ev[2], ev[3]), make_float2(ev[4], ev[5])};
-      float2* ho = hout + ((size_t)site * 16 + c) * 3;
-      if (GATE) {
-        const float n2 = v[0].x * v[0].x + v[0].y * v[0].y + v[1].x * v[1].x + v[1].y * v[1].y + v[2].x * v[2].x +
-                         v[2].y * v[2].y;
-        const float sg = 1.f / (1.f + __expf(-(n2 - bias[c])));
-        float2* po = pre + ((size_t)site * 16 + c) * 3;
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          po[i] = v[i];
-          ho[i] = make_float2(v[i].x * sg, v[i].y * sg);
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < 3; ++i) ho[i] = v[i];
-      }
+    for (int o = 128; o > 0; o >>= 1) {
+      if ((int)threadIdx.x < o) sm[threadIdx.x] += sm[threadIdx.x + o];
+      __syncthreads();
     }
-    return;
-  }
-  if (!valid) return;
-  float2* po = act_ptr(pre, COUT, Vh, p, s);
-  float2* ho = act_ptr(hout, COUT, Vh, p, s);
-#pragma unroll
-  for (int c = 0; c < COUT; ++c) {
-    if (GATE) {
-      float n2 = 0.f;
-#pragma unroll
-      for (int i = 0; i < 3; ++i) n2 += acc[c][i].x * acc[c][i].x + acc[c][i].y * acc[c][i].y;
-      const float sg = 1.f / (1.f + __expf(-(n2 - bias[c])));
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        po[c * 3 + i] = acc[c][i];
-        ho[c * 3 + i] = make_float2(acc[c][i].x * sg, acc[c][i].y * sg);
-      }
-    } else {
-#pragma unroll
-      for (int i = 0; i < 3; ++i) ho[c * 3 + i] = acc[c][i];
-    }
+    if (threadIdx.x == 0) part[(size_t)blockIdx.x * NET_NDIR + d] = sm[0];
+    __syncthreads();
   }
 }
 
 // Gate backward: G_pre = s G_out + 2 s(1-s) Re<G_out, pre> pre  (in place on g)
 // and per-block partial sums of db_c = -sum s(1-s) Re<G_out, pre>.  One
-// thread per (site, channel): consecutive threads read and write consecutive
-// 24-byte channel vectors; a thread's channel stays fixed over the
-// grid-stride loop (the stride is a multiple of C).
-template <int C>
-__global__ void __launch_bounds__(256) k_net_gate_bwd(int n2vh, const float2* __restrict__ pre, float2* g,
-                                                     const float* __restrict__ bias, float* __restrict__ db_part) {
-  static_assert(C == 16, "one warp covers two sites of 16 channels");
-  __shared__ float sdb[8][C];
-  const int stride = gridDim.x * blockDim.x;
-  const int q0 = blockIdx.x * blockDim.x + threadIdx.x;
-  const int c = q0 & (C - 1);
-  const float bc = bias[c];
-  float db = 0.f;
-  for (int q = q0; q < n2vh * C; q += stride) {
-    const float2* pv = pre + (size_t)q * 3;
-    float2* gv = g + (size_t)q * 3;
-    float2 v[3], o[3];
-    float n2 = 0.f, pr = 0.f;
+// thread per (site, channel pair), three 16-byte words of each field (their
+// place in the record: net_mma.cuh); a thread's pair stays fixed over the
+// grid-stride loop.
+__global__ void __launch_bounds__(256) k_net_gate_bwd16(int n2vh, const float2* __restrict__ pre, float2* g,
+                                                       const float* __restrict__ bias, float* __restrict__ db_part) {
+  __shared__ float sdb[8][16];
+  const int stride = gridDim.x * blockDim.x, q0 = blockIdx.x * blockDim.x + threadIdx.x, pair = q0 & 7;
+  const float2 bc = make_float2(bias[2 * pair], bias[2 * pair + 1]);
+  float db[2] = {0.f, 0.f};
+  for (int q = q0; q < n2vh * 8; q += stride) {
+    const size_t at = (size_t)(q >> 3) * 24 + 12 * (pair >> 2) + (pair & 3);
+    const float4* pv = (const float4*)pre + at;
+    float4* gv = (float4*)g + at;
+    float2 v[2][3], o[2][3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      v[i] = pv[i];
-      o[i] = gv[i];
-      n2 += v[i].x * v[i].x + v[i].y * v[i].y;
-      pr += o[i].x * v[i].x + o[i].y * v[i].y;
+    for (int k = 0; k < 3; ++k) {
+      const float4 a = __ldg(pv + 4 * k), b = gv[4 * k];
+      v[(2 * k) / 3][(2 * k) % 3] = make_float2(a.x, a.y);
+      v[(2 * k + 1) / 3][(2 * k + 1) % 3] = make_float2(a.z, a.w);
+      o[(2 * k) / 3][(2 * k) % 3] = make_float2(b.x, b.y);
+      o[(2 * k + 1) / 3][(2 * k + 1) % 3] = make_float2(b.z, b.w);
     }
-    const float sg = 1.f / (1.f + __expf(-(n2 - bc)));
-    const float sp = sg * (1.f - sg);
-    db -= sp * pr;
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
-      gv[i] = make_float2(sg * o[i].x + 2.f * sp * pr * v[i].x, sg * o[i].y + 2.f * sp * pr * v[i].y);
+    for (int e = 0; e < 2; ++e) {
+      float n2 = 0.f, pr = 0.f;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        n2 += v[e][i].x * v[e][i].x + v[e][i].y * v[e][i].y;
+        pr += o[e][i].x * v[e][i].x + o[e][i].y * v[e][i].y;
+      }
+      const float sg = 1.f / (1.f + __expf(-(n2 - (e ? bc.y : bc.x))));
+      const float sp = sg * (1.f - sg);
+      db[e] -= sp * pr;
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+        o[e][i] = make_float2(sg * o[e][i].x + 2.f * sp * pr * v[e][i].x, sg * o[e][i].y + 2.f * sp * pr * v[e][i].y);
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const float2 a = o[(2 * k) / 3][(2 * k) % 3], b = o[(2 * k + 1) / 3][(2 * k + 1) % 3];
+      gv[4 * k] = make_float4(a.x, a.y, b.x, b.y);
+    }
   }
-  // lanes l and l + 16 hold the same channel; then warps in order
-  db += __shfl_xor_sync(0xffffffffu, db, 16);
+  // lanes l, l + 8, ... hold the same pair; then warps in order
+#pragma unroll
+  for (int e = 0; e < 2; ++e)
+#pragma unroll
+    for (int o = 8; o < 32; o <<= 1) db[e] += __shfl_xor_sync(0xffffffffu, db[e], o);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane < C) sdb[warp][lane] = db;
+  if (lane < 8) {
+    sdb[warp][2 * lane] = db[0];
+    sdb[warp][2 * lane + 1] = db[1];
+  }
   __syncthreads();
-  if (threadIdx.x < C) {
+  if (threadIdx.x < 16) {
     float v = 0.f;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += sdb[w][threadIdx.x];
-    db_part[(size_t)blockIdx.x * C + threadIdx.x] = v;
+    db_part[(size_t)blockIdx.x * 16 + threadIdx.x] = v;
   }
 }
 
-// Output layer with one channel, mix first: u_d(y) = sum_c' W[d][0][c'] h_c'(y)
-// for the nine directions at every site (site-local, read once), then
-// (see k_net_transport_sum) out(x) = sum_d (T_d u_d)(x).  U: [9][2 Vh][3].
-template <int CIN>
-__global__ void __launch_bounds__(256) k_net_mix_local(int n2vh, const float2* __restrict__ hin,
-                                                      const __nv_bfloat16* __restrict__ W, float2* __restrict__ U) {
-  __shared__ float sw[NET_NDIR * CIN];
-  for (int i = threadIdx.x; i < NET_NDIR * CIN; i += blockDim.x) sw[i] = __bfloat162float(W[i]);
+// Output layer with one channel, for even output sites x (the prediction is
+// read nowhere else).  Mix first: u_d(y) = sum_c' W[d][0][c'] h_c'(y),
+// site-local, for the directions that lead from y to an even site (y even:
+// d = 0, y odd: 1..8); then (k_net_transport_sum) out(x) = u_0(x) + sum_d
+// (T_d u_d)(x).  U: [9][Vh][3].
+// A warp takes 32 sites of one parity, whose records (one contiguous piece)
+// pass through shared memory with whole-warp accesses; there a record takes
+// 25 words (odd: no bank conflicts between sites).
+__global__ void __launch_bounds__(128) k_net_mix_local16(int Vh, const float2* __restrict__ hin,
+                                                        const __nv_bfloat16* __restrict__ W, float2* __restrict__ U) {
+  __shared__ float sw[NET_NDIR * 16];
+  __shared__ float4 rec[4][16 * 25];
+  for (int i = threadIdx.x; i < NET_NDIR * 16; i += blockDim.x) sw[i] = __bfloat162float(W[i]);
   __syncthreads();
-  for (int site = blockIdx.x * blockDim.x + threadIdx.x; site < n2vh; site += gridDim.x * blockDim.x) {
-    float2 u[NET_NDIR][3];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, per = (Vh + 31) / 32;
+  float4* r = rec[warp];
+  auto mix = [&](int p, int s0, auto first, auto count) {
+    constexpr int D0 = decltype(first)::value, ND = decltype(count)::value;
+    const int n = Vh - s0 < 32 ? Vh - s0 : 32;
+    const float4* src = (const float4*)hin + ((size_t)p * Vh + s0) * 24;
+    float2 u[ND][3];
 #pragma unroll
-    for (int d = 0; d < NET_NDIR; ++d)
+    for (int d = 0; d < ND; ++d)
 #pragma unroll
       for (int i = 0; i < 3; ++i) u[d][i] = make_float2(0.f, 0.f);
-    const float4* src = (const float4*)(hin + (size_t)site * CIN * 3);
+    // channels 0..7, then 8..15 (the halves of every record), 12 words per site each
+#pragma unroll 1
+    for (int q = 0; q < 2; ++q) {
+      __syncwarp();
 #pragma unroll
-    for (int k = 0; k < CIN * 3 / 2; ++k) {  // float4 k holds entries 2k, 2k + 1 (channel e / 3, colour e % 3)
-      const float4 f = __ldg(src + k);
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int e = 2 * k + h, cp = e / 3, i = e - 3 * cp;
-        const float vx = h ? f.z : f.x, vy = h ? f.w : f.y;
-#pragma unroll
-        for (int d = 0; d < NET_NDIR; ++d) {
-          const float w = sw[d * CIN + cp];
-          u[d][i].x = fmaf(w, vx, u[d][i].x);
-          u[d][i].y = fmaf(w, vy, u[d][i].y);
-        }
+      for (int k = 0; k < 12; ++k) {
+        const int w = k * 32 + lane, site = w / 12;
+        if (site < n) r[(site & 15) * 25 + (site >> 4) * 12 + w % 12] = __ldg(src + (size_t)site * 24 + 12 * q + w % 12);
       }
+      __syncwarp();
+      const float4* me = r + (lane & 15) * 25 + (lane >> 4) * 12;
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const float4 f = me[4 * k + t];
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int e = 2 * k + h, c = 2 * t + e / 3, i = e % 3;  // channel 8 q + c, colour i
+            const float vx = h ? f.z : f.x, vy = h ? f.w : f.y;
+#pragma unroll
+            for (int d = 0; d < ND; ++d) {
+              const float w = sw[(D0 + d) * 16 + 8 * q + c];
+              u[d][i].x = fmaf(w, vx, u[d][i].x);
+              u[d][i].y = fmaf(w, vy, u[d][i].y);
+            }
+          }
+        }
     }
+    if (lane < n) {
 #pragma unroll
-    for (int d = 0; d < NET_NDIR; ++d)
+      for (int d = 0; d < ND; ++d)
 #pragma unroll
-      for (int i = 0; i < 3; ++i) U[((size_t)d * n2vh + site) * 3 + i] = u[d][i];
+        for (int i = 0; i < 3; ++i) U[((size_t)(D0 + d) * Vh + s0 + lane) * 3 + i] = u[d][i];
+    }
+  };
+  for (int g = blockIdx.x * 4 + warp; g < 2 * per; g += gridDim.x * 4) {
+    if (g < per)
+      mix(0, g * 32, IntC<0>{}, IntC<1>{});
+    else
+      mix(1, (g - per) * 32, IntC<1>{}, IntC<NET_NDIR - 1>{});
   }
 }
 
-// out(x) = u_0(x) + sum_{d >= 1} hop_d(x) u_d(neighbour_d(x)).
+// out(x) = u_0(x) + sum_{d >= 1} hop_d(x) u_d(neighbour_d(x)), x even.
 __global__ void __launch_bounds__(256) k_net_transport_sum(NetGeom ng, const float2* __restrict__ U,
                                                           float2* __restrict__ hout) {
-  const int Vh = ng.g.Vh, n2 = 2 * Vh;
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n2; idx += gridDim.x * blockDim.x) {
-    const int p = idx / Vh, s = idx - p * Vh;
+  const int Vh = ng.g.Vh;
+  for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < Vh; s += gridDim.x * blockDim.x) {
     float2 acc[3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) acc[i] = __ldg(U + (size_t)idx * 3 + i);
-#pragma unroll 1
+    for (int i = 0; i < 3; ++i) acc[i] = __ldg(U + (size_t)s * 3 + i);
+#pragma unroll 2
     for (int d = 1; d < NET_NDIR; ++d) {
       int np, ns;
-      net_neighbour(ng, p, s, d, np, ns);
+      net_neighbour(ng, 0, s, d, np, ns);
       float2 w[9], v[3];
-      load_hop_matrix(ng, p, s, d, w);
-      const float2* src = U + ((size_t)d * n2 + (size_t)np * Vh + ns) * 3;
+      load_hop_matrix(ng, 0, s, d, w);
+      const float2* src = U + ((size_t)d * Vh + ns) * 3;
 #pragma unroll
       for (int j = 0; j < 3; ++j) v[j] = __ldg(src + j);
 #pragma unroll
@@ -326,108 +300,25 @@ __global__ void __launch_bounds__(256) k_net_transport_sum(NetGeom ng, const flo
         for (int j = 0; j < 3; ++j) cmac(acc[i], w[3 * i + j], v[j]);
     }
 #pragma unroll
-    for (int i = 0; i < 3; ++i) hout[(size_t)idx * 3 + i] = acc[i];
+    for (int i = 0; i < 3; ++i) hout[(size_t)s * 3 + i] = acc[i];
   }
 }
 
-// Weight gradient: dW[d][c][c'] = sum_x Re<G_pre_c(x), (T_d h_c')(x)>.
-// A block stages a tile of TS sites: the 9 transports of every input channel
-// and the output gradients, in shared memory; then thread (d, tile of 4x4
-// (c, c') pairs) accumulates over the tile's sites.  Per-block sums go to
-// part[block][9*COUT*CIN] (a fixed-order final sum follows).
-template <int CIN, int COUT, int TS>
-__global__ void __launch_bounds__(256) k_net_dw(NetGeom ng, const float2* __restrict__ hin,
-                                               const float2* __restrict__ g, float* __restrict__ part) {
-  constexpr int TC = (COUT + 3) / 4, TP = (CIN + 3) / 4;  // 4x4 tiles
-  constexpr int NT = NET_NDIR * TC * TP;                  // accumulating threads
-  extern __shared__ float smem[];
-  float* st = smem;                                  // [TS][9][CIN][6]
-  float* sg = smem + TS * NET_NDIR * CIN * 6;        // [TS][COUT][6]
-  const int Vh = ng.g.Vh;
-  const int n2 = 2 * Vh;
-  float acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
-  const int tid = threadIdx.x;
-  const int td = tid / (TC * TP), tr = tid % (TC * TP), tc = tr / TP, tp = tr % TP;
-  for (int base = blockIdx.x * TS; base < n2; base += gridDim.x * TS) {
-    __syncthreads();
-    // stage transports: item = (site in tile, d, channel)
-    for (int it = tid; it < TS * NET_NDIR * CIN; it += blockDim.x) {
-      const int ls = it / (NET_NDIR * CIN), rem = it % (NET_NDIR * CIN), d = rem / CIN, cp = rem % CIN;
-      const int site = base + ls;
-      float2 t[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-      if (site < n2) {
-        const int p = site / Vh, s = site - p * Vh;
-        int np, ns;
-        net_neighbour(ng, p, s, d, np, ns);
-        const float2* src = act_ptr(hin, CIN, Vh, np, ns) + cp * 3;
-        float2 v[3];
-#pragma unroll
-        for (int i = 0; i < 3; ++i) v[i] = __ldg(src + i);
-        if (d) {
-          float2 w[9];
-          load_hop_matrix(ng, p, s, d, w);
-#pragma unroll
-          for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) cmac(t[i], w[3 * i + j], v[j]);
-        } else {
-#pragma unroll
-          for (int i = 0; i < 3; ++i) t[i] = v[i];
-        }
-      }
-      float* dst = st + ((ls * NET_NDIR + d) * CIN + cp) * 6;
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        dst[2 * i] = t[i].x;
-        dst[2 * i + 1] = t[i].y;
-      }
-    }
-    for (int it = tid; it < TS * COUT * 6; it += blockDim.x) {
-      const int ls = it / (COUT * 6), rem = it % (COUT * 6);
-      const int site = base + ls;
-      sg[it] = site < n2 ? ((const float*)(g + (size_t)site * COUT * 3))[rem] : 0.f;
-    }
-    __syncthreads();
-    if (tid < NT) {
-      for (int ls = 0; ls < TS; ++ls) {
-        const float* tv = st + (ls * NET_NDIR + td) * CIN * 6;
-        const float* gv = sg + ls * COUT * 6;
-#pragma unroll
-        for (int i = 0; i < 6; ++i) {
-          float ga[4], tb[4];
-#pragma unroll
-          for (int a = 0; a < 4; ++a) ga[a] = (tc * 4 + a < COUT) ? gv[(tc * 4 + a) * 6 + i] : 0.f;
-#pragma unroll
-          for (int b = 0; b < 4; ++b) tb[b] = (tp * 4 + b < CIN) ? tv[(tp * 4 + b) * 6 + i] : 0.f;
-#pragma unroll
-          for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(ga[a], tb[b], acc[a][b]);
-        }
-      }
-    }
+// grad[i] += sum over blocks of part[block][i], in a fixed order: a block takes
+// 32 entries, eight threads each every eighth partial, then the eight in order.
+__global__ void __launch_bounds__(256) k_net_sum_parts(const float* __restrict__ part, int nblocks, int n, float* grad) {
+  __shared__ float sm[8][33];
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5, i = blockIdx.x * 32 + x;
+  float s = 0.f;
+  if (i < n) {
+#pragma unroll 4
+    for (int b = y; b < nblocks; b += 8) s += part[(size_t)b * n + i];
   }
-  if (tid < NT) {
-    float* out = part + (size_t)blockIdx.x * NET_NDIR * COUT * CIN;
+  sm[y][x] = s;
+  __syncthreads();
+  if (y == 0 && i < n) {
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const int c = tc * 4 + a, cp = tp * 4 + b;
-        if (c < COUT && cp < CIN) out[(td * COUT + c) * CIN + cp] = acc[a][b];
-      }
-  }
-}
-
-// grad[i] += sum over blocks of part[block][i] (fixed block order)
-__global__ void k_net_sum_parts(const float* __restrict__ part, int nblocks, int n, float* grad) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    float s = 0.f;
-    for (int b = 0; b < nblocks; ++b) s += part[(size_t)b * n + i];
+    for (int k = 1; k < 8; ++k) s += sm[k][x];
     grad[i] += s;
   }
 }

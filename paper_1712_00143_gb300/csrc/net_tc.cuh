@@ -1,20 +1,8 @@
-// net_tc.cuh -- the 16 -> 16 channel layers of the preconditioner network on
-// the fifth-generation tensor cores (tcgen05, accumulators in tensor memory).
-//
-// A layer computes pre_c(x) = sum_d sum_c' W[d][c][c'] (T_d h_c')(x).  For a
-// tile of 64 sites of one parity this is, per direction d, the product
-//     D[row][c] += sum_c' X_d[row][c'] W_d[c][c']
-// with row = (colour-and-re/im component j, site) -- 6 x 64 = 384 rows, real
-// weights act on real and imaginary parts alike -- K = 16 input channels and
-// N = 16 output channels: three 128 x 16 x 16 MMAs per direction, nine
-// directions accumulated in one tensor-memory accumulator of 3 x 16 columns.
-// The CUDA cores compute the transports X_d (3x3 complex link times colour
-// vector, FP32) and write them to shared memory as bfloat16 in two parts,
-// hi = bf16(x) and lo = bf16(x - hi), so hi + lo carries 16 significant bits
-// and the product with the bfloat16 weights is accurate to about 2^-17 (each
-// part is multiplied exactly and accumulated in FP32).  Directions are
-// double-buffered: the transports of d + 1 are written while the MMAs of d
-// run; an mbarrier signalled by tcgen05.commit guards buffer reuse.
+// net_tc.cuh -- tcgen05 helpers and the check of the fifth-generation tensor
+// cores on this GPU (stag_tc_selftest): 384 x 16 rows of bfloat16 operands,
+// nine accumulated K = 16 steps into tensor memory, against the CUDA cores.
+// The network's layers once ran in this form; they now take mma.sync straight
+// from registers (net_mma.cuh says why) with the same results.
 //
 // Shared-memory operand layout (no swizzle, K-major): 8-row x 16-byte core
 // matrices stored as 128 contiguous bytes; the two 16-byte K halves of a row
@@ -29,15 +17,11 @@
 namespace stag {
 namespace tc {
 
-constexpr int TILE = 64;                    // sites per CTA tile
-constexpr int ROWS = 6 * TILE;              // 384 MMA rows
+constexpr int ROWS = 384;                   // MMA rows
 constexpr int A_BYTES = ROWS * 16 * 2;      // one operand part of one direction: 12288 B
 constexpr int B_BYTES = 16 * 16 * 2;        // weights of one direction: 512 B
 constexpr int TMEM_COLS = 64;               // 3 x 16 accumulator columns, allocated as 64
-constexpr int E_STRIDE = 97;                // floats per site in the epilogue staging (96 + 1 pad)
 constexpr int SMEM_BYTES = 4 * A_BYTES + NET_NDIR * B_BYTES + 64;
-
-static_assert(TILE * E_STRIDE * 4 <= 4 * A_BYTES, "epilogue staging must fit in the operand buffers");
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -145,296 +129,9 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t&
   lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
-__device__ __forceinline__ void st_shared_v2(uint32_t addr, uint32_t a, uint32_t b) {
-  asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
-}
-
-__device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
-
-__device__ int g_tc_error;  // set (never cleared by kernels) when a bounded wait gave up
-
 constexpr long long WAIT_CYCLES = 4000000000LL;  // about two seconds at GB300 clocks
 
-// ---- layout of the layer kernel's shared memory (bytes from the 1024-aligned base)
-constexpr int REC = 16 * 3 * 8;                      // one site's 16 input channels: 384 B
-constexpr int REC_STRIDE = REC + 16;                 // staged records 400 B apart (bank groups)
-constexpr int S_BYTES = TILE * REC_STRIDE;           // one staged direction: 25600 B
-constexpr int L_A = 0;                               // A operand, hi and lo parts
-constexpr int L_S = L_A + 2 * A_BYTES;               // staged neighbour records, two directions
-constexpr int L_B = L_S + 2 * S_BYTES;               // B operand of the current direction
-constexpr int L_BAR = L_B + B_BYTES;                 // mbarriers, tensor-memory slot, status
-constexpr int LAYER_SMEM = L_BAR + 64;               // 76352 B: three CTAs per SM
-
-static_assert(TILE * E_STRIDE * 4 <= 2 * S_BYTES, "epilogue staging must fit in the record buffers");
-static_assert(L_S % 16 == 0 && L_B % 16 == 0 && L_BAR % 8 == 0 && REC_STRIDE % 16 == 0, "alignment");
-
-// Offset of chunk q (16 B) of staged record r.  Records sit 400 B apart, so
-// eight consecutive records read at one chunk index fall in eight different
-// 16-byte bank groups (25 r + q mod 8).
-__device__ __forceinline__ uint32_t rec_off(int r, int q) { return (uint32_t)(r * REC_STRIDE + q * 16); }
-
-// mbarrier arrival that also announces `bytes` of bulk-copy data for the phase.
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-// Bulk copy global -> shared of `bytes` (a multiple of 16, both addresses
-// 16-byte aligned), completion counted on *bar.
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-               "l"(src), "r"(bytes), "r"(smem_u32(bar))
-               : "memory");
-}
-
-__device__ __forceinline__ float4 ld_shared_v4(uint32_t addr) {
-  float4 v;
-  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
-  return v;
-}
-
 }  // namespace tc
-
-// 16 -> 16 layer on the tensor cores.  transpose != 0: the adjoint layer
-// (weights W'[d][c][c'] = sign(d) W[partner(d)][c'][c]).  GATE: hout =
-// pre * sigmoid(|pre|^2 - b_c) and pre stored; else hout = pre.
-//
-// Per direction d the CTA (64 sites of one parity, 128 threads) needs the
-// 384-byte input records of the 64 neighbour sites.  They are copied into
-// shared memory one direction ahead, one bulk copy per record issued by the
-// record's own site thread of channel half 0 (the copy engine moves the
-// bytes; completion is counted on a per-buffer mbarrier: 64 arrivals, each
-// announcing its 384 bytes; splitting each record between the site's two
-// threads balanced the warps but doubled the neighbour-index work and was
-// slower), so that the gather of d + 1 is in flight while the CUDA cores
-// transport direction d and the tensor cores mix it; the link matrix of
-// d + 1 is prefetched into registers the same way.  The A and B operands
-// are single-buffered: the MMAs of d - 1 (a few hundred cycles) are
-// complete long before the transports of d are, and the smaller footprint
-// lets three CTAs share an SM.  Every wait is bounded; a wait for copies is
-// kept even after an MMA wait gave up, so that no copy is in flight when
-// the CTA leaves.  Input activations must be 16-byte aligned (every
-// workspace buffer is).
-template <bool GATE>
-__global__ void __launch_bounds__(128, 3)
-    k_net_layer_tc(NetGeom ng, const float2* __restrict__ hin, float2* __restrict__ pre, float2* __restrict__ hout,
-                   const __nv_bfloat16* __restrict__ W, const float* __restrict__ bias, int transpose) {
-  using namespace tc;
-  extern __shared__ __align__(1024) unsigned char tc_smem[];
-  uint64_t* bar = (uint64_t*)(tc_smem + L_BAR);  // MMA completion
-  uint64_t* bar_s = bar + 1;                      // [2] record buffers
-  uint32_t* tmem_slot = (uint32_t*)(bar + 3);
-  int* s_ok = (int*)(tmem_slot + 1);
-
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int Vh = ng.g.Vh;
-  const int tiles_per_parity = (Vh + TILE - 1) / TILE;
-  const int p = blockIdx.x / tiles_per_parity;
-  const int s0 = (blockIdx.x - p * tiles_per_parity) * TILE;
-
-  // staging role: site s_local, channel half `half` (8 input channels)
-  const int s_local = tid & 63, half = tid >> 6;
-  const int s = s0 + s_local;
-  const bool valid = s < Vh;
-  const Coord crd = valid ? cb_coords(ng.g, s, p) : Coord{0, 0, 0, 0};
-  if (tid == 0) {
-    mbar_init(bar, 1);
-    mbar_init(&bar_s[0], TILE);
-    mbar_init(&bar_s[1], TILE);
-    *s_ok = 1;
-    fence_barrier_init();
-  }
-  if (warp == 0) tmem_alloc(tmem_slot, TMEM_COLS);
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
-  constexpr uint32_t IDESC = idesc_bf16(128, 16);
-  const uint32_t base = smem_u32(tc_smem);
-  const uint32_t hi_base = base + L_A, lo_base = base + L_A + A_BYTES;
-
-  // the record of this site's neighbour in direction d -> slot s_local of
-  // record buffer b (threads of half 0; a site past the end only arrives)
-  auto stage = [&](int d, int b) {
-    if (half) return;
-    if (valid) {
-      const int ns = d == 0 ? s : cb_neighbour(ng.g, s, crd, (d - 1) >> 1, (d & 1) ? 1 : -1);
-      mbar_arrive_expect_tx(&bar_s[b], (uint32_t)REC);
-      bulk_g2s(base + L_S + (uint32_t)b * S_BYTES + rec_off(s_local, 0), act_ptr(hin, 16, Vh, d ? 1 - p : p, ns),
-               (uint32_t)REC, &bar_s[b]);
-    } else {
-      mbar_arrive(&bar_s[b]);
-    }
-  };
-
-  // this thread's two weights of direction d (B operand entries tid and
-  // tid + 128: output channel c, input channel c'), read one direction ahead
-  auto load_weights = [&](int d, __nv_bfloat16 (&wb)[2]) {
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int i = tid + 128 * k, c = i >> 4, cp = i & 15;
-      if (!transpose) {
-        wb[k] = W[d * 256 + i];
-      } else {
-        const int dd = d == 0 ? 0 : ((d & 1) ? d + 1 : d - 1);
-        const float wv = __bfloat162float(W[(dd * 16 + cp) * 16 + c]);
-        wb[k] = __float2bfloat16_rn(d == 0 ? wv : -wv);  // exact: a sign change
-      }
-    }
-  };
-
-  stage(0, 0);
-  float2 w[9], wn[9];
-#pragma unroll
-  for (int e = 0; e < 9; ++e) w[e] = wn[e] = make_float2(0.f, 0.f);
-  __nv_bfloat16 wcur[2], wnext[2] = {__float2bfloat16_rn(0.f), __float2bfloat16_rn(0.f)};
-  load_weights(0, wcur);
-
-#pragma unroll 1
-  for (int d = 0; d < NET_NDIR; ++d) {
-    const int buf = d & 1;
-    if (d + 1 < NET_NDIR) {
-      // the record buffer of d + 1 was last read by the transports of d - 1,
-      // which every thread finished before the barrier ahead of that MMA,
-      // and its barrier's previous phase was waited for in iteration d - 1
-      stage(d + 1, buf ^ 1);
-      if (valid) load_hop_matrix(ng, p, s, d + 1, wn);
-      load_weights(d + 1, wnext);
-    }
-    if (tid == 0) {
-      // the records of d (phase d / 2 of their buffer's barrier): waited
-      // for whatever happened before, so that no copy outlives the CTA
-      if (!mbar_wait(&bar_s[buf], (uint32_t)((d >> 1) & 1), WAIT_CYCLES)) *s_ok = 0;
-      // the MMAs of d - 1 read the operand buffers: wait for them
-      if (d >= 1 && *s_ok && !mbar_wait(bar, (uint32_t)((d - 1) & 1), WAIT_CYCLES)) *s_ok = 0;
-    }
-    __syncthreads();
-
-    // weights of direction d -> B operand (N = output channel c, K = input channel c')
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int i = tid + 128 * k;
-      *(__nv_bfloat16*)(tc_smem + L_B + op_offset(i >> 4, i & 15)) = wcur[k];
-    }
-
-    const uint32_t rb = base + L_S + (uint32_t)buf * S_BYTES;
-    // packed bf16 words of this thread's 8 channels for the six rows: [row][word]
-    // (words 0, 1 from channel group g = 0, words 2, 3 from g = 1), hi and lo
-    uint32_t hw[6][4], lw[6][4];
-#pragma unroll
-    for (int g = 0; g < 2; ++g) {
-      float2 v[4][3], t[4][3];
-#pragma unroll
-      for (int q = 0; q < 6; ++q) {
-        const float4 u = ld_shared_v4(rb + rec_off(s_local, half * 12 + g * 6 + q));
-        v[(2 * q) / 3][(2 * q) % 3] = make_float2(u.x, u.y);
-        v[(2 * q + 1) / 3][(2 * q + 1) % 3] = make_float2(u.z, u.w);
-      }
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        if (d) {
-#pragma unroll
-          for (int i = 0; i < 3; ++i) {
-            t[c][i] = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int j = 0; j < 3; ++j) cmac(t[c][i], w[3 * i + j], v[c][j]);
-          }
-        } else {
-#pragma unroll
-          for (int i = 0; i < 3; ++i) t[c][i] = v[c][i];
-        }
-      }
-      // rows j * 64 + s_local, j = 2 * colour + (0: re, 1: im); K = half * 8 + g * 4 + 0..3
-#pragma unroll
-      for (int j = 0; j < 6; ++j) {
-        const int i = j >> 1;
-        float x[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) x[c] = (j & 1) ? t[c][i].y : t[c][i].x;
-        split2(x[0], x[1], hw[j][2 * g], lw[j][2 * g]);
-        split2(x[2], x[3], hw[j][2 * g + 1], lw[j][2 * g + 1]);
-      }
-    }
-    // one 16-byte store per row and part: a quarter-warp's eight lanes (eight
-    // consecutive rows of one core matrix) cover 128 contiguous bytes
-#pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      const uint32_t off = (uint32_t)op_offset(j * TILE + s_local, half * 8);
-      st_shared_v4(hi_base + off, hw[j][0], hw[j][1], hw[j][2], hw[j][3]);
-      st_shared_v4(lo_base + off, lw[j][0], lw[j][1], lw[j][2], lw[j][3]);
-    }
-    fence_async_smem();
-    __syncthreads();
-    if (tid == 0 && *s_ok) {
-      tc_fence_after();
-      const uint64_t bdesc = smem_desc(base + L_B, 128, 256);
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        const uint32_t dcol = tmem + 16 * b;
-        mma_bf16(dcol, smem_desc(hi_base + b * 4096, 128, 256), bdesc, IDESC, d > 0 ? 1u : 0u);
-        mma_bf16(dcol, smem_desc(lo_base + b * 4096, 128, 256), bdesc, IDESC, 1u);
-      }
-      mma_commit(bar);
-    }
-#pragma unroll
-    for (int e = 0; e < 9; ++e) w[e] = wn[e];
-    wcur[0] = wnext[0];
-    wcur[1] = wnext[1];
-  }
-  // the commit of direction 8 (the barrier's ninth phase, parity 0) covers every MMA
-  if (tid == 0 && *s_ok && !mbar_wait(bar, 0u, WAIT_CYCLES)) *s_ok = 0;
-  __syncthreads();
-  tc_fence_after();
-  const bool ok = *s_ok != 0;
-  float* E = (float*)(tc_smem + L_S);  // reuses the record buffers: [64 sites][E_STRIDE]
-  if (ok) {
-    // warp w holds rows 32 w .. 32 w + 31 of each 128-row block b:
-    // colour b, component w / 2 (re, im), sites 32 (w % 2) + lane
-    const int sl = 32 * (warp & 1) + lane, comp = warp >> 1;
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      float v[16];
-      tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + 16 * b, v);
-#pragma unroll
-      for (int c = 0; c < 16; ++c) E[sl * E_STRIDE + c * 6 + b * 2 + comp] = v[c];
-    }
-  }
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 0) {
-    tc_fence_after();
-    tmem_dealloc(tmem, TMEM_COLS);
-  }
-  if (!ok) {
-    if (tid == 0) atomicOr(&tc::g_tc_error, 1);
-    return;
-  }
-  for (int q = tid; q < TILE * 16; q += blockDim.x) {
-    const int sl = q >> 4, c = q & 15;
-    const int site = s0 + sl;
-    if (site >= Vh) continue;
-    const float* e = E + sl * E_STRIDE + c * 6;
-    float2 v[3] = {make_float2(e[0], e[1]), make_float2(e[2], e[3]), make_float2(e[4], e[5])};
-    float2* ho = act_ptr(hout, 16, Vh, p, site) + c * 3;
-    if (GATE) {
-      const float n2 = v[0].x * v[0].x + v[0].y * v[0].y + v[1].x * v[1].x + v[1].y * v[1].y + v[2].x * v[2].x +
-                       v[2].y * v[2].y;
-      const float sg = 1.f / (1.f + __expf(-(n2 - bias[c])));
-      float2* po = act_ptr(pre, 16, Vh, p, site) + c * 3;
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        po[i] = v[i];
-        ho[i] = make_float2(v[i].x * sg, v[i].y * sg);
-      }
-    } else {
-#pragma unroll
-      for (int i = 0; i < 3; ++i) ho[i] = v[i];
-    }
-  }
-}
 
 // Check of the tensor-core path on this GPU: one tile (384 x 16 rows of
 // bfloat16 hi/lo operands from a fixed integer pattern, 9 accumulated

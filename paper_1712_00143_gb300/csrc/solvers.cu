@@ -19,6 +19,7 @@
 #include <cmath>
 #include <vector>
 
+#include "flags.h"
 #include "internal.h"
 
 namespace stag {
@@ -216,7 +217,11 @@ static int cg_solve(stag_lattice_s* lat, double2* x_can, const double2* b_can, d
       }
       TRY(cuda_status(cudaMemcpyAsync(hs, dst, sizeof(CgState), cudaMemcpyDeviceToHost, st)));
       TRY(cuda_status(cudaStreamSynchronize(st)));
-      if (loop && hsync[1]) return STAG_ETIMEOUT;
+      if (loop) {
+        auto read = [&](int* v) { return *v = (int)hsync[1], 0; };
+        auto clear = [&] { return hsync[1] = 0, 0; };  // (the device words are cleared before every launch)
+        TRY(take_flag(read, clear, STAG_ETIMEOUT));
+      }
       if ((hs->flags & F_STOP) && !loop) prof_discard_since(mark);  // launches after the flag returned at once
       prof_flush_completed();
       if (hs->flags & F_BREAKDOWN) {
