@@ -14,7 +14,8 @@
 //   whose fragment is then exactly what the lane has; the accumulator's
 //   fragment gives the lane the same two channel pairs of the output, so that
 //   gate and stores need no exchange either.
-// Every warp works by itself: no barrier, no shared memory but the weights.
+// Every warp works by itself: no barrier after the start, its gather running
+// three directions ahead in shared memory of its own.
 // The split of the transports into two bfloat16 parts, the order of the
 // products (direction by direction, high part then low) and the accumulation
 // in FP32 are those of the tcgen05 form, and so are the results, bit for bit
@@ -107,6 +108,98 @@ __device__ __forceinline__ float4 transported(const Pairs& v, const float2 (&w)[
   return make_float4(x[0].x, x[1].x, x[0].y, x[1].y);
 }
 
+// ---- the gather, three directions ahead
+// A lane copies the six words it will read itself (cp.async into its own
+// column of shared memory: no other lane is waited for), and the warp's lanes
+// together the nine words of each site's two hop matrices of a direction mu.
+// (Loads straight into registers left the layer waiting for L2: 206 us at 24^4
+// at four warps per scheduler; there are no registers for a second set.  With
+// the copies ahead it takes 180 us, scheduler 62 % busy with the split and the
+// transports, two blocks per SM at 114 KB of shared memory and 111 registers.)
+constexpr int STAGES = 3;
+struct WarpStage {
+  float4 v[STAGES][6][32];  // [stage][word][lane]
+  uint4 w[2][9][8];         // [slot][chunk][site]
+};
+__device__ __forceinline__ void copy16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tc::smem_u32(dst)), "l"(src) : "memory");
+}
+
+// Walks (group of 8 sites, direction 0..8) and issues one direction's copies
+// per step; consumers follow in the same order.
+struct Gather {
+  const NetGeom& ng;
+  const float2* act;
+  WarpStage* st;
+  int grp, step, total, per;  // current group, groups per step, all groups, groups per parity
+  int lane, d = 0, stage = 0, slot = 0, p = 0, s = 0;
+  Coord c;
+  __device__ __forceinline__ Gather(const NetGeom& ng_, const float2* a, WarpStage* st_, int first, int step_)
+      : ng(ng_), act(a), st(st_), grp(first), step(step_), lane(threadIdx.x & 31) {
+    per = (ng.g.Vh + 7) / 8;
+    total = 2 * per;
+  }
+  __device__ __forceinline__ void issue() {
+    if (grp < total) {
+      const int Vh = ng.g.Vh;
+      if (d == 0) {
+        p = grp >= per;
+        s = (grp - p * per) * 8 + (lane >> 2);
+        s = s < Vh ? s : Vh - 1;
+        c = cb_coords(ng.g, s, p);
+      }
+      const int mu = (d - 1) >> 1;
+      const int ns = d == 0 ? s : cb_neighbour(ng.g, s, c, mu, (d & 1) ? 1 : -1);
+      const float4* f = (const float4*)act_ptr(act, 16, Vh, d ? 1 - p : p, ns) + (lane & 3);
+#pragma unroll
+      for (int k = 0; k < 6; ++k) copy16(&st->v[stage][k][lane], f + 12 * (k / 3) + 4 * (k % 3));
+      if (d & 1) {
+        // chunks t, t + 4, t + 8 of this lane's site
+        const uint4* src = (p ? ng.links[1] : ng.links[0]) + (size_t)(mu * ng.cpm >> 1) * Vh + s;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          const int k = (lane & 3) + 4 * j;
+          if (k < 9) copy16(&st->w[slot][k][lane >> 2], src + (size_t)k * Vh);
+        }
+        slot ^= 1;
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    stage = stage == STAGES - 1 ? 0 : stage + 1;
+    if (++d == NET_NDIR) {
+      d = 0;
+      grp += step;
+    }
+  }
+  __device__ __forceinline__ static void wait() {  // the oldest direction in flight has arrived, for the whole warp
+    asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 1) : "memory");
+    __syncwarp();
+  }
+  __device__ __forceinline__ static void drain() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+};
+__device__ __forceinline__ Pairs staged_pairs(const WarpStage* st, int stage, int lane) {
+  Pairs r;
+#pragma unroll
+  for (int q = 0; q < 2; ++q)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const float4 u = st->v[stage][3 * q + k][lane];
+      r.v[q][(2 * k) / 3][(2 * k) % 3] = make_float2(u.x, u.y);
+      r.v[q][(2 * k + 1) / 3][(2 * k + 1) % 3] = make_float2(u.z, u.w);
+    }
+  return r;
+}
+// hop matrix k (0: +mu, 1: -mu) of the lane's site: entries 9 k .. 9 k + 8 of the slot's eighteen
+template <int K> __device__ __forceinline__ void staged_hop(const WarpStage* st, int slot, int site, float2 (&w)[9]) {
+#pragma unroll
+  for (int j = 4 * K; j < 5 + 4 * K; ++j) {
+    const uint4 c = st->w[slot][j][site];
+    const int e = 2 * j - 9 * K;
+    if (e >= 0) w[e] = make_float2(__uint_as_float(c.x), __uint_as_float(c.y));
+    if (e + 1 < 9) w[e + 1] = make_float2(__uint_as_float(c.z), __uint_as_float(c.w));
+  }
+}
+
 // The weights as B fragments, one uint4 per direction and lane: {b0, b1} of
 // output channels 0..7, then 8..15.  transpose: the adjoint layer's, sign(d)
 // W[partner(d)][c'][c].
@@ -168,6 +261,7 @@ __device__ __forceinline__ void outer(float (&d)[2][4], const uint32_t (&a)[3][4
 
 constexpr int FW = 8;    // warps per block of the forward layer
 constexpr int AW = 4;    // ... of the adjoint layer with its weight gradient
+constexpr int FWD_SMEM = NET_NDIR * 32 * 16 + FW * (int)sizeof(WarpStage);  // two blocks per SM
 constexpr int DWF = NET_NDIR * 256;  // floats of one weight gradient
 // shared memory of the adjoint kernel: weights, and per warp the gradient sums and the site operand
 constexpr int ADJ_SMEM = NET_NDIR * 32 * 16 + AW * (DWF * 4 + 36 * 32 * 4);
@@ -180,16 +274,20 @@ __global__ void __launch_bounds__(32 * nm::FW, 2)
     k_net_layer_mma(NetGeom ng, const float2* __restrict__ hin, float2* __restrict__ pre, float2* __restrict__ hout,
                     const __nv_bfloat16* __restrict__ W, const float* __restrict__ bias) {
   using namespace nm;
-  __shared__ uint4 sB[NET_NDIR * 32];
+  extern __shared__ __align__(16) unsigned char nm_fwd[];
+  uint4* sB = (uint4*)nm_fwd;
+  const int Vh = ng.g.Vh, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  WarpStage* st = (WarpStage*)(nm_fwd + NET_NDIR * 32 * 16) + (threadIdx.x >> 5);
+  const int per = (Vh + 7) / 8, nwarps = gridDim.x * FW, first = blockIdx.x * FW + (threadIdx.x >> 5);
+  Gather ahead(ng, hin, st, first, nwarps);
+#pragma unroll
+  for (int k = 0; k < STAGES; ++k) ahead.issue();
   stage_weights(sB, W, 0);
   __syncthreads();
-  const int Vh = ng.g.Vh, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const int per = (Vh + 7) / 8, nwarps = gridDim.x * FW;
-  for (int grp = blockIdx.x * FW + (threadIdx.x >> 5); grp < 2 * per; grp += nwarps) {
-    const int p = grp >= per, s_raw = (grp - p * per) * 8 + g;
-    const bool in = s_raw < Vh;
-    const int s = in ? s_raw : Vh - 1;
-    const Coord c = cb_coords(ng.g, s, p);
+  int stage = 0, slot = 0;
+  for (int grp = first; grp < 2 * per; grp += nwarps) {
+    const int p = grp >= per, s = (grp - p * per) * 8 + g;
+    const bool in = s < Vh;
     float acc[3][2][4];
 #pragma unroll
     for (int i = 0; i < 3; ++i)
@@ -208,25 +306,44 @@ __global__ void __launch_bounds__(32 * nm::FW, 2)
       mma(acc[i][0], l[0], l[1], l[2], l[3], b.x, b.y);
       mma(acc[i][1], l[0], l[1], l[2], l[3], b.z, b.w);
     };
+    auto done = [&]() {  // the stage has been read by its lane, the slot by the warp: the next direction may come
+      __syncwarp();
+      ahead.issue();
+      stage = stage == STAGES - 1 ? 0 : stage + 1;
+    };
     {
-      const Pairs v = load_pairs(act_ptr(hin, 16, Vh, p, s), t);
+      Gather::wait();
+      const Pairs v = staged_pairs(st, stage, lane);
       const uint4 b = sB[lane];
 #pragma unroll
       for (int i = 0; i < 3; ++i)
         mix(i, make_float4(v.v[0][0][i].x, v.v[0][1][i].x, v.v[0][0][i].y, v.v[0][1][i].y),
             make_float4(v.v[1][0][i].x, v.v[1][1][i].x, v.v[1][0][i].y, v.v[1][1][i].y), b);
+      done();
     }
 #pragma unroll 1
     for (int mu = 0; mu < 4; ++mu) {
-      float2 w[2][9];
-      load_hops(ng, p, s, mu, w);
+      {
+        Gather::wait();
+        float2 w[9];
+        staged_hop<0>(st, slot, g, w);
+        const Pairs v = staged_pairs(st, stage, lane);
+        const uint4 b = sB[(1 + 2 * mu) * 32 + lane];
 #pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const Pairs v = load_pairs(act_ptr(hin, 16, Vh, 1 - p, cb_neighbour(ng.g, s, c, mu, k ? -1 : 1)), t);
-        const uint4 b = sB[(1 + 2 * mu + k) * 32 + lane];
-#pragma unroll
-        for (int i = 0; i < 3; ++i) mix(i, transported(v, w[k], 0, i), transported(v, w[k], 1, i), b);
+        for (int i = 0; i < 3; ++i) mix(i, transported(v, w, 0, i), transported(v, w, 1, i), b);
+        done();
       }
+      {
+        Gather::wait();
+        float2 w[9];
+        staged_hop<1>(st, slot, g, w);
+        const Pairs v = staged_pairs(st, stage, lane);
+        const uint4 b = sB[(2 + 2 * mu) * 32 + lane];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) mix(i, transported(v, w, 0, i), transported(v, w, 1, i), b);
+        done();
+      }
+      slot ^= 1;
     }
     // pair q of the output = accumulator nt = q
     Pairs o, h;
@@ -248,6 +365,7 @@ __global__ void __launch_bounds__(32 * nm::FW, 2)
       store_pairs(act_ptr(hout, 16, Vh, p, s), t, h);
     }
   }
+  Gather::drain();
 }
 
 // Layers with one input and 16 output channels, on the CUDA cores: the first
