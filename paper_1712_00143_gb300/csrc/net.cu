@@ -297,7 +297,7 @@ static int layer_bwd(const NetRun& R, int l, float2* g, float2* gin, bool want_i
     else
       return STAG_EINVAL;
     TRYN(last_launch_status());
-    k_net_sum_parts<<<(co + 31) / 32, 256, 0, st>>>(R.part, G, co, N->grad + N->boff[l]);
+    k_net_sum_parts<<<(co + 31) / 32, 1024, 0, st>>>(R.part, G, co, N->grad + N->boff[l]);
     TRYN(last_launch_status());
   }
   // dW, and the adjoint layer: co -> ci channels with W' (transposed, partner
@@ -313,11 +313,11 @@ static int layer_bwd(const NetRun& R, int l, float2* g, float2* gin, bool want_i
       TRYN(cuda_status(cudaFuncSetAttribute(k_net_adjoint_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, nm::ADJ_SMEM)));
       k_net_adjoint_mma<<<G, 32 * nm::AW, nm::ADJ_SMEM, st>>>(R.ng, g, R.h[l], gin, W, R.part);
     } else if (ci == 1 && co == 16) {
-      G = grid_groups(R.Vh, 4, R.part_blocks);
-      k_net_dw_thin<<<G, 128, 0, st>>>(R.ng, R.h[l], g, 0, R.part);
+      G = grid_groups(R.Vh, nm::TW, 2 * 152);
+      k_net_dw_thin<<<G, 32 * nm::TW, 0, st>>>(R.ng, R.h[l], g, 0, R.part);
     } else if (ci == 16 && co == 1) {
-      G = grid_groups(R.Vh, 4, R.part_blocks);
-      k_net_dw_thin<<<G, 128, 0, st>>>(R.ng, g, R.h[l], 1, R.part);
+      G = grid_groups(R.Vh, nm::TW, 2 * 152);
+      k_net_dw_thin<<<G, 32 * nm::TW, 0, st>>>(R.ng, g, R.h[l], 1, R.part);
     } else if (ci == 1 && co == 1) {
       G = 152;
       k_net_dw_1to1<<<G, 256, 0, st>>>(R.ng, R.h[l], g, R.part);
@@ -326,7 +326,7 @@ static int layer_bwd(const NetRun& R, int l, float2* g, float2* gin, bool want_i
     }
     TRYN(last_launch_status());
     count_launch();
-    k_net_sum_parts<<<(nw + 31) / 32, 256, 0, st>>>(R.part, G, nw, N->grad + N->woff[l]);
+    k_net_sum_parts<<<(nw + 31) / 32, 1024, 0, st>>>(R.part, G, nw, N->grad + N->woff[l]);
     TRYN(last_launch_status());
   }
   if (want_in && co == 1) {

@@ -305,20 +305,21 @@ __global__ void __launch_bounds__(256) k_net_transport_sum(NetGeom ng, const flo
 }
 
 // grad[i] += sum over blocks of part[block][i], in a fixed order: a block takes
-// 32 entries, eight threads each every eighth partial, then the eight in order.
-__global__ void __launch_bounds__(256) k_net_sum_parts(const float* __restrict__ part, int nblocks, int n, float* grad) {
-  __shared__ float sm[8][33];
+// 32 entries, 32 threads each every 32nd partial, then the 32 in order.  (With
+// eight threads the chain of loads took 10 to 12 us.)
+__global__ void __launch_bounds__(1024) k_net_sum_parts(const float* __restrict__ part, int nblocks, int n, float* grad) {
+  __shared__ float sm[32][33];
   const int x = threadIdx.x & 31, y = threadIdx.x >> 5, i = blockIdx.x * 32 + x;
   float s = 0.f;
   if (i < n) {
-#pragma unroll 4
-    for (int b = y; b < nblocks; b += 8) s += part[(size_t)b * n + i];
+#pragma unroll 8
+    for (int b = y; b < nblocks; b += 32) s += part[(size_t)b * n + i];
   }
   sm[y][x] = s;
   __syncthreads();
   if (y == 0 && i < n) {
 #pragma unroll
-    for (int k = 1; k < 8; ++k) s += sm[k][x];
+    for (int k = 1; k < 32; ++k) s += sm[k][x];
     grad[i] += s;
   }
 }

@@ -116,6 +116,7 @@ __device__ __forceinline__ float4 transported(const Pairs& v, const float2 (&w)[
 // at four warps per scheduler; there are no registers for a second set.  With
 // the copies ahead it takes 180 us, scheduler 62 % busy with the split and the
 // transports, two blocks per SM at 114 KB of shared memory and 111 registers.)
+constexpr int TW = 8;  // warps per block of the thin weight gradients
 constexpr int STAGES = 3;
 struct WarpStage {
   float4 v[STAGES][6][32];  // [stage][word][lane]
@@ -578,14 +579,16 @@ __global__ void __launch_bounds__(32 * nm::AW, 3)
 // sum for d belongs to partner(d) with the sign of T_d^dag = -T_partner(d).
 // The nine directions take the place of the channels of the other operand:
 // lane 4 g + t transports u to site g along 2t, 2t + 1 and (t = 0) 8.
-__global__ void __launch_bounds__(128)
+// Bound by the latency of a group's loads: 33 us at 16 x 20 x 12 x 24 with
+// twelve warps per SM (three blocks of four), 28 us with sixteen.
+__global__ void __launch_bounds__(32 * nm::TW, 2)
     k_net_dw_thin(NetGeom ng, const float2* __restrict__ u, const float2* __restrict__ f, int adj,
                   float* __restrict__ part) {
   using namespace nm;
   const int Vh = ng.g.Vh, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const int per = (Vh + 7) / 8, nwarps = gridDim.x * 4;
+  const int per = (Vh + 7) / 8, nwarps = gridDim.x * TW;
   float sum[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-  for (int grp = blockIdx.x * 4 + warp; grp < 2 * per; grp += nwarps) {
+  for (int grp = blockIdx.x * TW + warp; grp < 2 * per; grp += nwarps) {
     const int p = grp >= per, s_raw = (grp - p * per) * 8 + g;
     const bool in = s_raw < Vh;
     const int s = in ? s_raw : Vh - 1;
@@ -651,17 +654,17 @@ __global__ void __launch_bounds__(128)
       for (int e = 0; e < 4; ++e) sum[nt][e] += s4[nt][e];
   }
   // accumulator (nt, lane, e): d = lane / 4 + 8 (e / 2), c = 8 nt + 2 (lane % 4) + e % 2
-  __shared__ float sm[4][2][32][4];
+  __shared__ float sm[TW][2][32][4];
 #pragma unroll
   for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
     for (int e = 0; e < 4; ++e) sm[warp][nt][lane][e] = sum[nt][e];
   __syncthreads();
-  for (int i = threadIdx.x; i < 256; i += 128) {
+  for (int i = threadIdx.x; i < 256; i += 32 * TW) {
     const int e = i & 3, l = (i >> 2) & 31, nt = i >> 7, d = (l >> 2) + 8 * (e >> 1), cc = 8 * nt + 2 * (l & 3) + (e & 1);
     if (d >= NET_NDIR) continue;
     float v = 0.f;
-    for (int k = 0; k < 4; ++k) v += sm[k][nt][l][e];
+    for (int k = 0; k < TW; ++k) v += sm[k][nt][l][e];
     const int dd = !adj || d == 0 ? d : ((d & 1) ? d + 1 : d - 1);
     part[(size_t)blockIdx.x * NET_NDIR * 16 + dd * 16 + cc] = adj && d ? -v : v;
   }
