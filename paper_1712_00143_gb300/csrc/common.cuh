@@ -621,114 +621,6 @@ __device__ inline void finalize(const RedTarget& t, const double* v, int nv) {
       fin_ru_resid((CgState*)t.state, v[0]);
       fin_ru_ortho((CgState*)t.state, v + 1);
       break;
-    case RED_MS_ALPHA: {
-      MsState* ms = (MsState*)t.state;
-      CgState* st = &ms->cg;
-      st->pAp = v[0];
-      if (!(v[0] > 0.0) || !finite_d(v[0])) {
-        st->flags |= F_BREAKDOWN;
-        break;
-      }
-      double a = st->rr / v[0];
-      st->alpha = a;
-      // the previous iteration's shift update has consumed zeta(k+1): rotate,
-      // and retire the shifts that reached their target
-      for (int s = 0; s < ms->nshift; ++s) {
-        ms->zeta_prev[s] = ms->zeta[s];
-        ms->zeta[s] = ms->zeta_next[s];
-      }
-      ms->active_mask &= ~ms->stop_mask;
-      ms->stop_mask = 0;
-      for (int s = 0; s < ms->nshift; ++s) {
-        if (!((ms->active_mask >> s) & 1)) continue;
-        double zp = ms->zeta_prev[s], z = ms->zeta[s];
-        double den = ms->alpha_prev * zp * (1.0 + a * ms->delta[s]) + a * ms->beta_prev * (zp - z);
-        double zn = z * zp * ms->alpha_prev / den;
-        ms->zeta_next[s] = zn;
-        ms->alpha_s[s] = a * zn / z;
-      }
-      break;
-    }
-    case RED_MS_BETA: {
-      MsState* ms = (MsState*)t.state;
-      CgState* st = &ms->cg;
-      double rr_new = v[0];
-      if (!finite_d(rr_new)) {
-        st->flags |= F_BREAKDOWN;
-        break;
-      }
-      double b = rr_new / st->rr;
-      st->beta = b;
-      st->rr_prev = st->rr;
-      st->rr = rr_new;
-      st->iter += 1;
-      double rn = sqrt(rr_new);
-      int mask = ms->active_mask;
-      for (int s = 0; s < ms->nshift; ++s) {
-        if (!((mask >> s) & 1)) continue;
-        double ratio = ms->zeta_next[s] / ms->zeta[s];
-        ms->beta_s[s] = b * ratio * ratio;
-        ms->iters[s] = st->iter;
-      }
-      ms->alpha_prev = st->alpha;
-      ms->beta_prev = b;
-      // shifts whose residual |zeta_s| ||r|| reached the target still take
-      // this iteration's update; they are retired at the next alpha step
-      int stop = 0;
-      for (int s = 0; s < ms->nshift; ++s)
-        if (((mask >> s) & 1) && fabs(ms->zeta_next[s]) * rn <= ms->sqrt_target_bb) stop |= 1 << s;
-      ms->stop_mask = stop;
-      if ((mask & ~stop) == 0) st->flags |= F_CONVERGED;
-      if (st->iter >= st->max_iter) st->flags |= F_ITER_CAP;
-      break;
-    }
-    case RED_MCG_ALPHA: {
-      McgState* g = (McgState*)t.state;
-      for (int i = 0; i < g->n; ++i) {
-        CgState* st = &g->sys[i];
-        if (!((g->active >> i) & 1)) {
-          st->alpha = 0.0;
-          continue;
-        }
-        st->pAp = v[i];
-        if (!(v[i] > 0.0) || !finite_d(v[i])) {
-          st->flags |= F_BREAKDOWN;
-          g->flags |= F_BREAKDOWN;
-        } else {
-          st->alpha = st->rr / v[i];
-        }
-      }
-      break;
-    }
-    case RED_MCG_BETA: {
-      McgState* g = (McgState*)t.state;
-      g->iter += 1;
-      int active = g->active;
-      for (int i = 0; i < g->n; ++i) {
-        CgState* st = &g->sys[i];
-        if (!((active >> i) & 1)) {
-          st->beta = 0.0;
-          continue;
-        }
-        const double rr_new = v[i];
-        if (!finite_d(rr_new)) {
-          st->flags |= F_BREAKDOWN;
-          g->flags |= F_BREAKDOWN;
-          continue;
-        }
-        st->beta = rr_new / st->rr;
-        st->rr_prev = st->rr;
-        st->rr = rr_new;
-        st->iter = g->iter;
-        if (rr_new > st->rr_max) st->rr_max = rr_new;
-        if (rr_new <= st->target) active &= ~(1 << i);
-        if (st->delta2 > 0.0 && rr_new < st->delta2 * st->rr_max) g->flags |= F_NEED_RU;
-      }
-      g->active = active;
-      if (active == 0) g->flags |= F_CONVERGED;
-      if (g->iter >= g->max_iter) g->flags |= F_ITER_CAP;
-      break;
-    }
     case RED_MCG_RU_RESID:
       fin_mcg_ru_resid((McgState*)t.state, v);
       break;
@@ -742,6 +634,148 @@ __device__ inline void finalize(const RedTarget& t, const double* v, int nv) {
       break;
     }
   }
+}
+
+// The same by the first warp of the last block, all its lanes holding the
+// totals, for the operations with a scalar recurrence per shift or per system:
+// lane k does shift or system k.  (One thread doing them in turn, each with two
+// or three FP64 divisions, kept every other block of the grid waiting: with
+// nine shifts at 16^3 x 32 the FP64 operator with MS_ALPHA took 49 us and the
+// residual update with MS_BETA 15 us, 40 and 11 us now.)
+template <int NV> __device__ __forceinline__ void finalize_warp(const RedTarget& t, const double (&v)[NV]) {
+  const unsigned all = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  double mine = v[0];  // system `lane`'s total
+#pragma unroll
+  for (int i = 1; i < NV; ++i) mine = lane == i ? v[i] : mine;
+  switch (t.op) {
+    case RED_MS_ALPHA: {
+      MsState* ms = (MsState*)t.state;
+      const bool ok = v[0] > 0.0 && finite_d(v[0]);
+      if (!ok) {
+        if (lane == 0) {
+          ms->cg.pAp = v[0];
+          ms->cg.flags |= F_BREAKDOWN;
+        }
+        break;
+      }
+      const double a = ms->cg.rr / v[0];
+      const int mask = ms->active_mask & ~ms->stop_mask;
+      __syncwarp();
+      // the previous iteration's shift update has consumed zeta(k+1): rotate,
+      // and retire the shifts that reached their target
+      if (lane < ms->nshift) {
+        const double zp = ms->zeta[lane], z = ms->zeta_next[lane];
+        ms->zeta_prev[lane] = zp;
+        ms->zeta[lane] = z;
+        if ((mask >> lane) & 1) {
+          const double den = ms->alpha_prev * zp * (1.0 + a * ms->delta[lane]) + a * ms->beta_prev * (zp - z);
+          const double zn = z * zp * ms->alpha_prev / den;
+          ms->zeta_next[lane] = zn;
+          ms->alpha_s[lane] = a * zn / z;
+        }
+      }
+      if (lane == 0) {
+        ms->cg.pAp = v[0];
+        ms->cg.alpha = a;
+        ms->active_mask = mask;
+        ms->stop_mask = 0;
+      }
+      break;
+    }
+    case RED_MS_BETA: {
+      MsState* ms = (MsState*)t.state;
+      CgState* st = &ms->cg;
+      const double rr_new = v[0];
+      if (!finite_d(rr_new)) {
+        if (lane == 0) st->flags |= F_BREAKDOWN;
+        break;
+      }
+      const double b = rr_new / st->rr, rn = sqrt(rr_new);
+      const int mask = ms->active_mask, iter = st->iter + 1;
+      bool reached = false;
+      __syncwarp();
+      if (lane < ms->nshift && ((mask >> lane) & 1)) {
+        const double zn = ms->zeta_next[lane], ratio = zn / ms->zeta[lane];
+        ms->beta_s[lane] = b * ratio * ratio;
+        ms->iters[lane] = iter;
+        reached = fabs(zn) * rn <= ms->sqrt_target_bb;
+      }
+      // shifts whose residual |zeta_s| ||r|| reached the target still take
+      // this iteration's update; they are retired at the next alpha step
+      const int stop = (int)__ballot_sync(all, reached);
+      if (lane == 0) {
+        st->beta = b;
+        st->rr_prev = st->rr;
+        st->rr = rr_new;
+        st->iter = iter;
+        ms->alpha_prev = st->alpha;
+        ms->beta_prev = b;
+        ms->stop_mask = stop;
+        if ((mask & ~stop) == 0) st->flags |= F_CONVERGED;
+        if (iter >= st->max_iter) st->flags |= F_ITER_CAP;
+      }
+      break;
+    }
+    case RED_MCG_ALPHA: {
+      McgState* g = (McgState*)t.state;
+      bool bad = false;
+      if (lane < g->n) {
+        CgState* st = &g->sys[lane];
+        if (!((g->active >> lane) & 1)) {
+          st->alpha = 0.0;
+        } else {
+          st->pAp = mine;
+          bad = !(mine > 0.0) || !finite_d(mine);
+          if (bad) st->flags |= F_BREAKDOWN;
+          else st->alpha = st->rr / mine;
+        }
+      }
+      bad = __any_sync(all, bad);
+      if (lane == 0 && bad) g->flags |= F_BREAKDOWN;
+      break;
+    }
+    case RED_MCG_BETA: {
+      McgState* g = (McgState*)t.state;
+      const int active = g->active, iter = g->iter + 1;
+      bool bad = false, reached = false, update = false;
+      __syncwarp();
+      if (lane < g->n) {
+        CgState* st = &g->sys[lane];
+        if (!((active >> lane) & 1)) {
+          st->beta = 0.0;
+        } else if (!finite_d(mine)) {
+          st->flags |= F_BREAKDOWN;
+          bad = true;
+        } else {
+          st->beta = mine / st->rr;
+          st->rr_prev = st->rr;
+          st->rr = mine;
+          st->iter = iter;
+          if (mine > st->rr_max) st->rr_max = mine;
+          reached = mine <= st->target;
+          update = st->delta2 > 0.0 && mine < st->delta2 * st->rr_max;
+        }
+      }
+      const int left = active & ~(int)__ballot_sync(all, reached);
+      bad = __any_sync(all, bad);
+      update = __any_sync(all, update);
+      if (lane == 0) {
+        g->iter = iter;
+        g->active = left;
+        int f = g->flags;
+        if (bad) f |= F_BREAKDOWN;
+        if (update) f |= F_NEED_RU;
+        if (left == 0) f |= F_CONVERGED;
+        if (iter >= g->max_iter) f |= F_ITER_CAP;
+        g->flags = f;
+      }
+      break;
+    }
+    default:
+      if (lane == 0) finalize(t, v, NV);
+  }
+  __syncwarp();
 }
 
 // ------------------------------------------------------------------ accurate sums
@@ -780,7 +814,7 @@ template <> struct Acc1<float> {
   __device__ __forceinline__ double value() const { return df_value(v); }
 };
 
-// Deterministic block sum of NV doubles; the total is valid in thread 0.
+// Deterministic block sum of NV doubles; the total is valid in the first warp's 32 threads.
 template <int NV> __device__ __forceinline__ void block_sum(double (&v)[NV]) {
   __shared__ double sm[NV][32];
 #pragma unroll
@@ -830,10 +864,12 @@ template <int NV> __device__ __forceinline__ void grid_reduce(double (&v)[NV], R
 #pragma unroll
     for (int i = 0; i < NV; ++i) w[i] += __ldcg(rb.partials + i * gridDim.x + b);
   block_sum<NV>(w);
-  if (threadIdx.x == 0) {
-    finalize(tgt, w, NV);
-    *rb.counter = 0u;
-    __threadfence();
+  if (threadIdx.x < 32) {
+    finalize_warp<NV>(tgt, w);
+    if (threadIdx.x == 0) {
+      *rb.counter = 0u;
+      __threadfence();
+    }
   }
 }
 
@@ -865,7 +901,7 @@ template <int NV> __device__ __forceinline__ void warp_sum_df(DF (&v)[NV]) {
     }
 }
 
-// Deterministic block sum of NV double-float values; valid in thread 0.
+// Deterministic block sum of NV double-float values; valid in the first warp's 32 threads.
 template <int NV> __device__ __forceinline__ void block_sum_df(DF (&v)[NV]) {
   __shared__ float2 sm[NV][32];
   warp_sum_df<NV>(v);
@@ -915,13 +951,15 @@ template <int NV> __device__ __forceinline__ void grid_reduce_df(DF (&v)[NV], Re
       df_add_df(w[i], DF{q.x, q.y});
     }
   block_sum_df<NV>(w);
-  if (threadIdx.x == 0) {
+  if (threadIdx.x < 32) {
     double t[NV];
 #pragma unroll
     for (int i = 0; i < NV; ++i) t[i] = df_value(w[i]);
-    finalize(tgt, t, NV);
-    *rb.counter = 0u;
-    __threadfence();
+    finalize_warp<NV>(tgt, t);
+    if (threadIdx.x == 0) {
+      *rb.counter = 0u;
+      __threadfence();
+    }
   }
 }
 
