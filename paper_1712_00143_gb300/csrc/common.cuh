@@ -469,8 +469,8 @@ struct MsState {
   double zeta_prev[MAX_SHIFTS];  // zeta_s(k-1)
   double zeta[MAX_SHIFTS];       // zeta_s(k)
   double zeta_next[MAX_SHIFTS];  // zeta_s(k+1)
-  double alpha_s[MAX_SHIFTS];
-  double beta_s[MAX_SHIFTS];
+  double alpha_s[MAX_SHIFTS];    // steps of x_s along p_s / zeta_s
+  double beta_s[MAX_SHIFTS];     // p_s / zeta_s = r + beta_s (p_s / zeta_s)
   int iters[MAX_SHIFTS];
 };
 
@@ -672,7 +672,7 @@ template <int NV> __device__ __forceinline__ void finalize_warp(const RedTarget&
           const double den = ms->alpha_prev * zp * (1.0 + a * ms->delta[lane]) + a * ms->beta_prev * (zp - z);
           const double zn = z * zp * ms->alpha_prev / den;
           ms->zeta_next[lane] = zn;
-          ms->alpha_s[lane] = a * zn / z;
+          ms->alpha_s[lane] = a * zn;  // (of the direction over zeta)
         }
       }
       if (lane == 0) {
@@ -697,7 +697,7 @@ template <int NV> __device__ __forceinline__ void finalize_warp(const RedTarget&
       __syncwarp();
       if (lane < ms->nshift && ((mask >> lane) & 1)) {
         const double zn = ms->zeta_next[lane], ratio = zn / ms->zeta[lane];
-        ms->beta_s[lane] = b * ratio * ratio;
+        ms->beta_s[lane] = b * ratio;
         ms->iters[lane] = iter;
         reached = fabs(zn) * rn <= ms->sqrt_target_bb;
       }

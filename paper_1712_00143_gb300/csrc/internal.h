@@ -208,7 +208,7 @@ constexpr int kLoopSites = 1 << 15;
 template <int P>
 int launch_ms_r_update(Spinor<Acc<P>::value> r, Spinor<Acc<P>::value> Ap, MsState* state, RedScratch rs,
                        cudaStream_t st);
-// for every active shift s: x_s += alpha_s p_s; p_s = zeta_s r + beta_s p_s
+// for every active shift s: x_s += alpha_s p_s; p_s = r + beta_s p_s (p_s over zeta_s)
 // Runs only when the state's iteration count equals expect_iter (the residual
 // update of this iteration ran); `base` is the smallest shift.
 template <int P>
