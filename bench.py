@@ -769,12 +769,12 @@ def run_config(args):
         lg()
         fam = {f: stag.stag_profile_read(f) for f in ("net", "net_tc", "net_bwd")}
         stag.stag_profile_enable(False)
-        # the 16 -> 16 tensor-core layer against the HBM roofline: per site
-        # 8 fat hops of 72 B, the input record (384 B) and pre + output (768 B)
+        # the 16 -> 16 tensor-core layer (of a training pass) against the HBM roofline:
+        # per site 8 fat hops of 72 B, the input record (384 B) and pre + output (768 B)
         n_tc, ms_tc = fam["net_tc"]
         tc_us = ms_tc / max(n_tc, 1) * 1e3
         tc_bytes = 1728 * 2 * h.Vh
-        tc_roof = {"kernel": "k_net_layer_tc", "avg_launch_us": tc_us, "bytes_per_launch": tc_bytes,
+        tc_roof = {"kernel": "k_net_layer_mma", "avg_launch_us": tc_us, "bytes_per_launch": tc_bytes,
                    "achieved_gbs": tc_bytes / (tc_us * 1e-6) / 1e9 if tc_us > 0 else None}
         if tc_roof["achieved_gbs"]:
             peak, peak_kind = measured_peaks()
@@ -807,11 +807,12 @@ def run_config(args):
             stag.stag_profile_reset()
             stag.stag_profile_select("links", 1)
             stag.stag_profile_enable(True)
-            wall, _ = _timed(lambda: stag.stag_build_links(dims, thin, fat, lng), reps=5)
-            n, ms = stag.stag_profile_read("links")
+            reps = 5
+            wall, _ = _timed(lambda: stag.stag_build_links(dims, thin, fat, lng), reps=reps)
+            _, ms = stag.stag_profile_read("links")
             stag.stag_profile_enable(False)
             stag.stag_profile_select("", 1)
-            per = ms / max(n, 1) * 1e-3
+            per = ms / reps * 1e-3
             tf = 4 * lat.V * flop_per_link / per / 1e12
             rows["x".join(map(str, dims))] = {"device_s": per, "wall_s": wall, "fp64_tflops": tf}
             del thin, fat, lng
@@ -826,8 +827,9 @@ def run_config(args):
         per_site = (time.perf_counter() - t0) / lat.V
         print(json.dumps({"config": "link construction (3-staple fat + Naik) from thin links, FP64",
                           "unit": "s", "results": rows,
-                          "roofline": {"bound": "fp64_alu", "flop_per_link": flop_per_link,
-                                       "note": "FP64 peak about 1.2 TFLOP/s on GB300 (measured DGEMM 1.10)"},
+                          "roofline": {"bound": "integer_multiply", "flop_per_link": flop_per_link,
+                                       "note": "products in fixed point, 81 x 3 wide integer multiply-adds each at 32 per clock and "
+                                               "SM; the FP64 pipe reaches about 1.2 TFLOP/s (measured DGEMM 1.10)"},
                           "cpu_baseline": {"kind": "oracle", "cores": 1, "sample": "16^4, scaled per site",
                                            "s_per_site": per_site,
                                            "value_32_4": per_site * 32 ** 4}}), flush=True)
@@ -859,7 +861,7 @@ def run_config(args):
             stag.stag_profile_enable(True)
             reps = 3
             wall, _ = _timed(lambda: stag.stag_gauge_force(dims, thin, beta, *coef, force=F), reps=reps)
-            n, ms = stag.stag_profile_read("gauge_force")  # two kernels per call
+            n, ms = stag.stag_profile_read("gauge_force")
             stag.stag_profile_enable(False)
             stag.stag_profile_select("", 1)
             per = ms / reps * 1e-3
@@ -879,9 +881,10 @@ def run_config(args):
                           "coefficients": {"beta": beta, "u0": 0.87, "c_pl": coef[0], "c_rt": coef[1], "c_pg": coef[2]},
                           "unit": "s", "results": rows,
                           "algorithm": "three-link staples stored once, reused by every loop",
-                          "roofline": {"bound": "fp64_alu", "flop_per_link": flop_per_link,
+                          "roofline": {"bound": "integer_multiply", "flop_per_link": flop_per_link,
                                        "flop_per_link_walking_each_staple": flop_walk,
-                                       "note": "FP64 peak about 1.2 TFLOP/s on GB300 (measured DGEMM 1.10)"},
+                                       "note": "products in fixed point, 81 x 3 wide integer multiply-adds each at 32 per clock and "
+                                               "SM; the FP64 pipe reaches about 1.2 TFLOP/s (measured DGEMM 1.10)"},
                           "cpu_baseline": {"kind": "oracle", "cores": 1, "sample": "4^4 x 6, scaled per link",
                                            "s_per_link": per_link, "value_24_4": per_link * 4 * 24 ** 4}}),
               flush=True)
@@ -914,7 +917,7 @@ def run_config(args):
             stag.stag_profile_enable(True)
             reps = 3
             wall, _ = _timed(lambda: stag.stag_fermion_force(dims, thin, xs, ys, alphas, force=F), reps=reps)
-            n, ms = stag.stag_profile_read("fermion_force")  # two kernels per call
+            n, ms = stag.stag_profile_read("fermion_force")
             stag.stag_profile_enable(False)
             stag.stag_profile_select("", 1)
             per = ms / reps * 1e-3
@@ -933,8 +936,9 @@ def run_config(args):
         per_link = (time.perf_counter() - t0) / (4 * lat.V)
         print(json.dumps({"config": f"fermion force through the 3-staple fat + Naik links, {nt} terms, FP64",
                           "unit": "s", "results": rows,
-                          "roofline": {"bound": "fp64_alu", "flop_per_link": flop_per_link,
-                                       "note": "FP64 peak about 1.2 TFLOP/s on GB300 (measured DGEMM 1.10)"},
+                          "roofline": {"bound": "integer_multiply", "flop_per_link": flop_per_link,
+                                       "note": "products in fixed point, 81 x 3 wide integer multiply-adds each at 32 per clock and "
+                                               "SM; the FP64 pipe reaches about 1.2 TFLOP/s (measured DGEMM 1.10)"},
                           "cpu_baseline": {"kind": "oracle", "cores": 1, "sample": "6^4, scaled per link",
                                            "s_per_link": per_link, "value_32_4": per_link * 4 * 32 ** 4}}),
               flush=True)

@@ -484,7 +484,10 @@ int stag_dd_cg(stag_dd_t d, void* x, const void* b, double mass, const stag_solv
  * the GPU, periodic boundaries, no staggered phases (stag_load_links folds
  * them in).  thin, fat, lng: device, canonical [V][4][3][3] complex double,
  * caller-owned; fat and lng must not overlap thin or each other
- * (STAG_EINVAL).  dims: even extents >= 4.  Asynchronous on `stream`. */
+ * (STAG_EINVAL).  dims: even extents >= 4.  Products run in fixed point of
+ * FP64-class accuracy where the links allow (unitary to rounding), in FP64
+ * otherwise; scratch 576 B per site, stream-ordered (without it, FP64
+ * arithmetic throughout).  Asynchronous on `stream`. */
 int stag_build_links(const int dims[4], const void* thin, void* fat, void* lng, double c1, double c_staple,
                      double c3, void* stream);
 
@@ -500,6 +503,7 @@ int stag_build_links(const int dims[4], const void* thin, void* fat, void* lng, 
  * so that U_mu(x) -> exp(eps X) U_mu(x) changes S by -eps Re Tr(X force).
  * FP64.  thin, force: device, canonical [V][4][3][3] complex double,
  * caller-owned, not overlapping (STAG_EINVAL).  dims: even extents >= 4.
+ * Scratch: 4608 B per site, stream-ordered (STAG_ENOMEM if unavailable).
  * Asynchronous on `stream`. */
 int stag_gauge_force(const int dims[4], const void* thin, void* force, double beta, double c_pl, double c_rt,
                      double c_pg, void* stream);
@@ -523,15 +527,16 @@ int stag_gauge_force(const int dims[4], const void* thin, void* force, double be
  *   alpha   : host, n_terms weights; 1 <= n_terms <= 32.
  *   force   : device, canonical [V][4][3][3] complex double, caller-owned,
  *             not overlapping thin, x_even or y_odd (STAG_EINVAL).
- * dims: even extents >= 4.  Scratch: 2 V x 4 x 9 complex doubles
- * (1152 B per site), stream-ordered (STAG_ENOMEM if unavailable).
+ * dims: even extents >= 4.  Scratch, stream-ordered: 1760 B per site for the
+ * fixed-point kernels (FP64-class accuracy), else 1152 B for the FP64 ones
+ * (STAG_ENOMEM if neither is available).
  * Asynchronous on `stream`; profiler family "fermion_force". */
 int stag_fermion_force(const int dims[4], const void* thin, int n_terms, const void* x_even, const void* y_odd,
                        const double* alpha, double c1, double c_staple, double c3, void* force, void* stream);
 
-/* Check of this build's tensor-core path on the current GPU (the path the
- * network's 16 -> 16 layers take): one tile of tcgen05 bfloat16 products
- * with FP32 accumulation in tensor memory, 9 accumulated steps, compared
+/* Check of the tcgen05 tensor-core path on the current GPU (the network's
+ * layers feed the tensor cores from registers with mma.sync, whose products
+ * and sums agree with it bit for bit): one tile of bfloat16 products with FP32 accumulation in tensor memory, 9 accumulated steps, compared
  * with the same sums on the CUDA cores.  *max_rel_err: max |difference| /
  * max |reference| (0 expected: the test values are exact in both).
  * STAG_ETIMEOUT if a bounded wait gave up.  Synchronous.  No counterpart in
@@ -550,7 +555,8 @@ const char* stag_strerror(int status);
  * "dslash64_epi" (FP64), "dslash_mrhs", "dslash_mrhs_epi", "dslash_mrhs64",
  * "dslash_mrhs64_epi" (multi-right-hand-side forms), "dslash_df",
  * "dslash_df_epi" (double-float), "blas", "reduce",
- * "convert", "links", "net" (network forward layers), "net_tc" (the
+ * "convert", "cg_loop" (the iterations of a mixed CG on a small lattice, one
+ * launch per reliable-update cycle), "links", "net" (network forward layers), "net_tc" (the
  * 16 -> 16 tensor-core layers of the forward), "net_bwd", "gauge_force",
  * "fermion_force".  stag_launch_count
  * counts all library kernel launches since the last reset, whether or not
