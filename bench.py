@@ -639,7 +639,9 @@ def run_dslash_sweep(args):
                     per = ms / max(n, 1)  # one launch covers min(nrhs, 8) (double-float: 4) right-hand sides
                     k = min(nrhs, 4 if prec == "df64" else 8)
                     nl = 6 if (recon == 12 and prec != "fp64") else 9
-                    byt = ((8 * 9 + 8 * nl) * ELEM_BYTES[prec] + 2 * k * VEC_BYTES[prec]) * h.Vh
+                    # the operator kernel stores the caller's doubles itself (48 B per site and vector)
+                    vec = VEC_BYTES[prec] + (VEC_BYTES[prec] if prec == "df64" else 48)
+                    byt = ((8 * 9 + 8 * nl) * ELEM_BYTES[prec] + k * vec) * h.Vh
                     gbs = byt / (per * 1e-3) / 1e9
                     print(json.dumps({"dslash": "x".join(map(str, dims)), "prec": prec, "recon": recon, "nrhs": k,
                                       "us": per * 1e3, "GB/s": gbs, "frac": gbs / peak, "peak_kind": peak_kind,
