@@ -115,7 +115,7 @@ __device__ __forceinline__ float4 transported(const Pairs& v, const float2 (&w)[
 // (Loads straight into registers left the layer waiting for L2: 206 us at 24^4
 // at four warps per scheduler; there are no registers for a second set.  With
 // the copies ahead it takes 180 us, scheduler 62 % busy with the split and the
-// transports, two blocks per SM at 114 KB of shared memory and 111 registers.)
+// transports, two blocks per SM at 95 KB of shared memory and 111 registers.)
 constexpr int TW = 8;  // warps per block of the thin weight gradients
 constexpr int STAGES = 3;
 struct WarpStage {
