@@ -184,6 +184,29 @@ template <int SLOTS> __device__ __forceinline__ FM ld(const int4* __restrict__ f
   }
   return m;
 }
+// A matrix copied asynchronously into the thread's own column of a [9][128]
+// block of int4 in shared memory, and read from there: no other thread is
+// waited for.
+template <int SLOTS> __device__ __forceinline__ void copy_column(int4* col, const int4* __restrict__ f, int slot, int site) {
+  const int4* p = f + row0(SLOTS, site, slot);
+  const unsigned to = (unsigned)__cvta_generic_to_shared(col);
+#pragma unroll
+  for (int e = 0; e < 9; ++e)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + e * 2048), "l"(p + e * 32) : "memory");
+}
+__device__ __forceinline__ void wait_columns() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ FM from_column(const int4* col) {
+  FM m;
+#pragma unroll
+  for (int e = 0; e < 9; ++e) {
+    const int4 q = col[e * 128];
+    m.h[2 * e] = q.x;
+    m.l[2 * e] = q.y;
+    m.h[2 * e + 1] = q.z;
+    m.l[2 * e + 1] = q.w;
+  }
+  return m;
+}
 template <int SLOTS> __device__ __forceinline__ void st(int4* __restrict__ f, int slot, int site, const FM& m) {
   int4* p = f + row0(SLOTS, site, slot);
 #pragma unroll

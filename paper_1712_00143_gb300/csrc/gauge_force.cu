@@ -251,9 +251,11 @@ __global__ void __launch_bounds__(128, 3) k_gf_staples_fx(Dims d, long long V, i
 // by 2^-k so that |c_pl| 6 + |c_rt| 18 + |c_pg| 24 <= 1, keep S within range.
 // Sums that are touched once per group (S, and a group's rectangle 3) wait in
 // shared memory, a column per thread: in registers they cost the third block
-// of an SM (255 registers, 4.4 ms at 24^4).  Bound by the integer pipe, 67 % busy (ncu),
-// the rest the latency of the table's loads at three warps per scheduler.
-// 24^4: conversion 0.06, table 0.72, force 3.6 ms; the call 4.6 ms against
+// of an SM (255 registers, 4.4 ms at 24^4).  The factors of the next product
+// are copied to shared memory while one runs (loaded into registers where they
+// are used the kernel took 3.57 ms at 24^4, 3.47 so).  Bound by the integer pipe, 67 % busy (ncu),
+// the rest additions, address arithmetic and dependences at three warps per scheduler.
+// 24^4: conversion 0.07, table 0.68, force 3.5 ms; the call 4.2 ms against
 // 21.3 ms with the FP64 kernels.
 struct ForceCoef {
   fx::Coef pl8, rt8, rt, pg4;  // 8 c_pl, 8 c_rt, c_rt, 4 c_pg, each times 2^-k
@@ -266,7 +268,10 @@ __global__ void __launch_bounds__(128, 3) k_gauge_force_fx(Dims d, long long V, 
   extern __shared__ __align__(16) unsigned char gf_sm[];
   long long(*S)[128] = (long long(*)[128])gf_sm;  // [18][128]
   long long(*lone)[128] = S + 18;                  // a group's rectangle 3
-  long long(*hold)[128] = S + 36;                  // a group's sum, then its weighted sum
+  int4(*A)[128] = (int4(*)[128])(S + 36);          // [9][128]: an item's factors on their way, in A
+  int4(*B)[128] = A + 9;                           // and in B; at a group's end the thread's column of B
+  // holds the group's sum, then its weighted sum
+  auto hold = [&](int e) -> long long* { return (long long*)&B[e >> 1][threadIdx.x] + (e & 1); };
   double2* out = (double2*)gf_sm;                  // the block's output, at the end
   const long long x0 = (long long)blockIdx.x * fx::TS;
   const int ns = (int)(V - x0 < fx::TS ? V - x0 : fx::TS);
@@ -294,26 +299,21 @@ __global__ void __launch_bounds__(128, 3) k_gauge_force_fx(Dims d, long long V, 
         lone[e][tid] = 0;
       }
     }
-#pragma unroll 1
-    for (int g = 0; g < 8; ++g) {
-      // group g >= 2: its (nu, s); ps = x + s nu; qs = x (s > 0) or x - nu
+    // copies the factors of item t of group g into the thread's columns of A and B
+    auto fetch = [&](int g, int t) {
       const int gt = g < 2 ? 0 : g - 2, go = gt >> 1, gnu = go < mu ? go : go + 1, gs = (gt & 1) ? -1 : 1;
-      const int ps = fx::next_lex(d, p0, gnu, gs), qs = gs > 0 ? x : ps;
-      long long acc[18];
-      fx::clear(acc);
-      const int items = g < 2 ? 6 : 5;
-#pragma unroll 1
-      for (int t = 0; t < items; ++t) {
-        int sa, sb, xa = ps, xb = qs, adj;
-        if (g < 2) {
-          sa = sb = mu * 6 + t;
-          xa = g == 0 ? pp.lex : x;
-          xb = g == 0 ? x : xm;
-          adj = 0;
-        } else if (t == 0) {
+      int sa, sb, xa, xb;
+      if (g < 2) {
+        sa = sb = mu * 6 + t;
+        xa = g == 0 ? pp.lex : x;
+        xb = g == 0 ? x : xm;
+      } else {
+        // ps = x + s nu; x (s > 0) or x - nu
+        xa = fx::next_lex(d, p0, gnu, gs);
+        xb = gs > 0 ? x : xa;
+        if (t == 0) {
           sa = mu * 6 + gt;
           sb = U0 + gnu;
-          adj = gs > 0 ? -1 : 0;
         } else {
           // (rho, r): the two directions other than mu and nu, both signs
           int rho = (t - 1) >> 1;
@@ -322,11 +322,26 @@ __global__ void __launch_bounds__(128, 3) k_gauge_force_fx(Dims d, long long V, 
           rho += rho >= hi ? 1 : 0;
           sa = fslot(mu, rho, r);
           sb = fslot(gnu, rho, r);
-          adj = gs > 0 ? 0 : -1;
         }
-        const fx::FM a = fx::ld<SLOTS>(T, sa, xa);
-        fx::FM b = fx::ld<SLOTS>(T, sb, xb);
-        fx::adjoint_if(b, adj);
+      }
+      fx::copy_column<SLOTS>(&A[0][tid], T, sa, xa);
+      fx::copy_column<SLOTS>(&B[0][tid], T, sb, xb);
+    };
+    fetch(0, 0);
+#pragma unroll 1
+    for (int g = 0; g < 8; ++g) {
+      // group g >= 2: its (nu, s)
+      const int gt = g < 2 ? 0 : g - 2, go = gt >> 1, gnu = go < mu ? go : go + 1, gs = (gt & 1) ? -1 : 1;
+      long long acc[18];
+      fx::clear(acc);
+      const int items = g < 2 ? 6 : 5;
+#pragma unroll 1
+      for (int t = 0; t < items; ++t) {
+        fx::wait_columns();
+        const fx::FM a = fx::from_column(&A[0][tid]);
+        fx::FM b = fx::from_column(&B[0][tid]);
+        if (t + 1 < items) fetch(g, t + 1);
+        fx::adjoint_if(b, g < 2 ? 0 : (t == 0) == (gs > 0) ? -1 : 0);
         fx::mac(acc, a, b);
         if (g >= 2 && t == 0) {
 #pragma unroll
@@ -337,15 +352,15 @@ __global__ void __launch_bounds__(128, 3) k_gauge_force_fx(Dims d, long long V, 
         }
       }
 #pragma unroll
-      for (int e = 0; e < 18; ++e) hold[e][tid] = acc[e];
+      for (int e = 0; e < 18; ++e) *hold(e) = acc[e];
       {
         const fx::Coef ca = g < 2 ? cf.rt8 : cf.pg4, cb = cf.rt;
         const int sh = g < 2 ? 3 : 2;
 #pragma unroll 2
         for (int e = 0; e < 18; ++e) {
           int h, l;  // lone is 0 for the first two groups
-          fx::split1(fx::scaled(ca, hold[e][tid] >> sh) + fx::scaled(cb, lone[e][tid]), h, l);
-          ((int2*)&hold[e][tid])[0] = make_int2(h, l);
+          fx::split1(fx::scaled(ca, *hold(e) >> sh) + fx::scaled(cb, lone[e][tid]), h, l);
+          *(int2*)hold(e) = make_int2(h, l);
         }
       }
       // the other factor: U_mu(x+mu), U_mu(x-mu), else h(x+mu, nu, s)
@@ -354,12 +369,13 @@ __global__ void __launch_bounds__(128, 3) k_gauge_force_fx(Dims d, long long V, 
       fx::adjoint_if(P, g >= 2 && gs < 0 ? -1 : 0);
 #pragma unroll
       for (int e = 0; e < 18; ++e) {
-        const int2 q = ((const int2*)&hold[e][tid])[0];
+        const int2 q = *(const int2*)hold(e);
         Q.h[e] = g == 1 ? P.h[e] : q.x;
         Q.l[e] = g == 1 ? P.l[e] : q.y;
         P.h[e] = g == 1 ? q.x : P.h[e];
         P.l[e] = g == 1 ? q.y : P.l[e];
       }
+      if (g < 7) fetch(g + 1, 0);
       fx::clear(acc);
       fx::mac(acc, P, Q);
 #pragma unroll
@@ -455,7 +471,7 @@ extern "C" int stag_gauge_force(const int dims[4], const void* thin, void* force
     }
     if (!s) {
       ProfScope ps("gauge_force", st);
-      constexpr int smem = 3 * 18 * 128 * sizeof(long long);  // 54 KB, three blocks per SM
+      constexpr int smem = 4 * 18 * 128 * sizeof(long long);  // 72 KB, three blocks per SM
       s = cuda_status(cudaFuncSetAttribute(gf::k_gauge_force_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
       if (!s) gf::k_gauge_force_fx<<<tiles, 128, smem, st>>>(d, V, Tf, status, (double2*)force, cf);
       if (!s) s = last_launch_status();
