@@ -238,8 +238,9 @@ __global__ void __launch_bounds__(256) k_fx_convert(double2* L, long long n, int
 }
 
 // The FP64 copy to fixed point, if every nonzero matrix lies within 2^-10 of
-// the largest entry (so that all keep FP64's relative accuracy) and the unit
-// is in the middle of the double range; else it stays in doubles.
+// the largest entry (so that all keep FP64's relative accuracy) and the largest
+// entry within 2^+-50 (where the row norms' FP32 squares are normal numbers);
+// else it stays in doubles.
 static int to_fixed(LinkCopy& L, const Geom& g, FxStats* scratch, cudaStream_t st) {
   FxStats h{0, 0x7fffffff, 0u};
   int status = cuda_status(cudaMemcpyAsync(scratch, &h, sizeof(h), cudaMemcpyHostToDevice, st));
@@ -254,10 +255,11 @@ static int to_fixed(LinkCopy& L, const Geom& g, FxStats* scratch, cudaStream_t s
   float row;
   memcpy(&row, &h.row, sizeof(row));
   const int emax = h.max_hi >> 20, emin = h.min_hi >> 20;
-  if (emax < 1023 - 100 || emax > 1023 + 100 || emin < emax - 10) return STAG_OK;
+  if (emax < 1023 - 50 || emax > 1023 + 50 || emin < emax - 10) return STAG_OK;
   int kexp = emax - 1022;  // |entry| < 2^kexp
-  for (double r = std::ldexp((double)row, -kexp); r > 9.0; r *= 0.5) ++kexp;
-  if (kexp > emax - 1022 + 4) return STAG_OK;
+  double r = std::ldexp((double)row, -kexp);
+  for (int k = 0; k < 4 && r > 9.0; ++k, r *= 0.5) ++kexp;
+  if (!(r <= 9.0)) return STAG_OK;
   const long long n = (long long)2 * 144 * g.Vh;
   {
     ProfScope ps("links", st);
