@@ -24,6 +24,7 @@
 // with |ar + ai| and |br + bi| of row norm sqrt 2, below 2 sqrt(2) sqrt(3)
 // 2^60 < 2^62.4.
 #pragma once
+#include "fx_steps.h"
 #include "su3.cuh"
 
 namespace stag {
@@ -35,24 +36,6 @@ using su3::Dims;
 struct FM {
   int h[18], l[18];
 };
-
-// Inline PTX: from C the compiler forms some of these as a 64-bit product and
-// an addition (1.3 times the time of a matrix product).
-__device__ __forceinline__ void wmad(long long& acc, int a, int b) {
-  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
-}
-__device__ __forceinline__ long long wmul(int a, int b) {
-  long long r;
-  asm("mul.wide.s32 %0, %1, %2;" : "=l"(r) : "r"(a), "r"(b));
-  return r;
-}
-
-// int64 in units of 2^-60 -> (h, l): h = round(s / 2^30), l = s - h 2^30
-__device__ __forceinline__ void split1(long long s, int& h, int& l) {
-  h = (int)((s + (1LL << 29)) >> 30);
-  l = ((int)((unsigned)s << 2)) >> 2;
-}
-__device__ __forceinline__ long long join1(int h, int l) { return ((long long)h << 30) + l; }
 
 // One entry of a b, in units of 2^-60.
 __device__ __forceinline__ void entry(const FM& a, const FM& b, int i, int j, long long& re, long long& im) {
@@ -128,16 +111,6 @@ __device__ __forceinline__ long long fixed60(double v) {
   const unsigned long long m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 8;  // 1.f at 2^60
   const long long q = (long long)(m >> (r > 63 ? 63 : r));
   return (long long)b < 0 ? -q : q;
-}
-// s 2^k, rounded to nearest; the result must be a normal number (or s = 0)
-__device__ __forceinline__ double double_of(long long s, int k) {
-  const unsigned long long a0 = (unsigned long long)(s < 0 ? -s : s);
-  const int z = __clzll((long long)a0);
-  const unsigned long long a = a0 << (z & 63);
-  const unsigned long long m = (a >> 11) + ((a >> 10) & 1);  // 53 bits, leading bit at 52
-  unsigned long long b = ((unsigned long long)(unsigned)(1023 + 62 - z + k) << 52) + m;
-  b = a0 == 0 ? 0 : b;
-  return __longlong_as_double((long long)(b | ((unsigned long long)s & 0x8000000000000000ull)));
 }
 // A coefficient |c| <= 1 in the same form, and c s for |s| <= 2^60.
 struct Coef {

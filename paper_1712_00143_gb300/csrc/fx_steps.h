@@ -1,0 +1,210 @@
+// fx_steps.h -- the integer steps of the fixed-point forms, without CUDA types,
+// so that a host program can run them too: the wide multiply-adds, the split
+// of a 64-bit value into two words, and the FP64 operator's running sums over
+// the hops of a site (dslash_fx.cuh).
+#pragma once
+#include <cstring>
+
+#ifdef __CUDACC__
+#define STAG_FX __host__ __device__ __forceinline__
+#else
+#define STAG_FX inline
+#endif
+#ifdef __CUDA_ARCH__
+#define STAG_UNROLL _Pragma("unroll")
+#else
+#define STAG_UNROLL
+#endif
+
+namespace stag {
+namespace fx {
+
+// Inline PTX: from C the compiler forms some of these as a 64-bit product and
+// an addition (1.3 times the time of a matrix product).  Sums are modulo 2^64.
+STAG_FX void wmad(long long& acc, int a, int b) {
+#ifdef __CUDA_ARCH__
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
+#else
+  acc = (long long)((unsigned long long)acc + (unsigned long long)((long long)a * b));
+#endif
+}
+STAG_FX long long wmul(int a, int b) {
+#ifdef __CUDA_ARCH__
+  long long r;
+  asm("mul.wide.s32 %0, %1, %2;" : "=l"(r) : "r"(a), "r"(b));
+  return r;
+#else
+  return (long long)a * b;
+#endif
+}
+// a + b and a - b modulo 2^64
+STAG_FX long long add64(long long a, long long b) {
+  return (long long)((unsigned long long)a + (unsigned long long)b);
+}
+STAG_FX long long sub64(long long a, long long b) {
+  return (long long)((unsigned long long)a - (unsigned long long)b);
+}
+
+// int64 in units of 2^-60 -> (h, l): h = round(s / 2^30), l = s - h 2^30
+STAG_FX void split1(long long s, int& h, int& l) {
+  h = (int)((s + (1LL << 29)) >> 30);
+  l = ((int)((unsigned)s << 2)) >> 2;
+}
+STAG_FX long long join1(int h, int l) { return ((long long)h << 30) + l; }
+
+STAG_FX unsigned long long bits_of(double v) {
+#ifdef __CUDA_ARCH__
+  return (unsigned long long)__double_as_longlong(v);
+#else
+  unsigned long long b;
+  std::memcpy(&b, &v, sizeof(b));
+  return b;
+#endif
+}
+STAG_FX double double_of_bits(unsigned long long b) {
+#ifdef __CUDA_ARCH__
+  return __longlong_as_double((long long)b);
+#else
+  double v;
+  std::memcpy(&v, &b, sizeof(v));
+  return v;
+#endif
+}
+STAG_FX int leading_zeros(unsigned long long a) {
+#ifdef __CUDA_ARCH__
+  return __clzll((long long)a);
+#else
+  return a ? __builtin_clzll(a) : 64;
+#endif
+}
+
+// s 2^k, rounded to nearest; the result must be a normal number (or s = 0)
+STAG_FX double double_of(long long s, int k) {
+  const unsigned long long a0 = s < 0 ? 0ull - (unsigned long long)s : (unsigned long long)s;
+  const int z = leading_zeros(a0);
+  const unsigned long long a = a0 << (z & 63);
+  const unsigned long long m = (a >> 11) + ((a >> 10) & 1);  // 53 bits, leading bit at 52
+  unsigned long long b = ((unsigned long long)(unsigned)(1023 + 62 - z + k) << 52) + m;
+  b = a0 == 0 ? 0 : b;
+  return double_of_bits(b | ((unsigned long long)s & 0x8000000000000000ull));
+}
+
+}  // namespace fx
+
+namespace fxd {
+
+// One link entry in units of 2^kexp, |v| < 2^kexp: v = (h 2^-30 + l 2^-60) 2^kexp, rounded to nearest.
+STAG_FX void fixed_entry(double v, int kexp, int& h, int& l) {
+  const unsigned long long b = fx::bits_of(v);
+  const int r = 1023 + kexp - (int)((b >> 52) & 0x7ff);  // >= 1
+  const unsigned long long m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 8;
+  const long long q = r > 62 ? 0 : (long long)((m + (1ull << (r - 1))) >> r);
+  fx::split1((long long)b < 0 ? -q : q, h, l);
+}
+
+// The running sums of one site.  p[row] = {sum ar br, sum ai bi, sum (ar + ai)
+// (br + bi)}, cross sums folded in, modulo 2^64: only the differences re = p0
+// - p1 and im = p2 - p0 - p1 are bounded (dslash_fx.cuh), and only they are
+// shifted or converted.
+struct Sums {
+  long long p[3][3];
+  int eb;        // biased exponent of the unit (0: nothing met)
+  unsigned any;  // 0 while every component was an exact zero
+};
+
+STAG_FX void init(Sums& S) {
+  for (int i = 0; i < 3; ++i)
+    for (int q = 0; q < 3; ++q) S.p[i][q] = 0;
+  S.eb = 0;
+  S.any = 0;
+}
+STAG_FX long long real_sum(const Sums& S, int i) { return fx::sub64(S.p[i][0], S.p[i][1]); }
+STAG_FX long long imag_sum(const Sums& S, int i) { return fx::sub64(fx::sub64(S.p[i][2], S.p[i][0]), S.p[i][1]); }
+
+// S in units raised to 2^(eb - 1023).  The third sum may have passed 2^63, so
+// the differences are shifted, and the sums replaced by others that have them.
+STAG_FX void raise(Sums& S, int eb) {
+  const int sh = eb - S.eb > 63 ? 63 : eb - S.eb;
+  STAG_UNROLL
+  for (int i = 0; i < 3; ++i) {
+    const long long re = real_sum(S, i) >> sh, im = imag_sum(S, i) >> sh;
+    S.p[i][0] = re;
+    S.p[i][1] = 0;
+    S.p[i][2] = fx::add64(im, re);
+  }
+  S.eb = eb;
+}
+
+// One component (h, l) in units of 2^-30, 2^-60 of 2^(eb - 1023); its exponent is at most eb - 3.
+STAG_FX void component(double v, int eb, int& h, int& l) {
+  const unsigned long long b = fx::bits_of(v);
+  const int hi = (int)(b >> 32);
+  int r = eb - ((hi >> 20) & 0x7ff);
+  r = r > 63 ? 63 : r;
+  const unsigned long long m = (((b & 0xfffffffffffffull) | 0x10000000000000ull) << 8) >> r;
+  const int s = hi >> 31;
+  h = ((int)(m >> 30) ^ s) - s;
+  l = ((int)((unsigned)m & 0x3fffffffu) ^ s) - s;
+}
+
+// One hop: psi[3] with .x and .y, link(e) the matrix entry e = 3 row + column as {re.h, re.l, im.h, im.l}.
+template <class V2, class Link> STAG_FX void hop(Sums& S, const V2 (&psi)[3], Link link) {
+  int mx = 0;
+  unsigned any = 0;
+  STAG_UNROLL
+  for (int c = 0; c < 3; ++c) {
+    const unsigned long long x = fx::bits_of(psi[c].x), y = fx::bits_of(psi[c].y);
+    const int a = (int)(x >> 32) & 0x7fffffff, b = (int)(y >> 32) & 0x7fffffff, ab = a > b ? a : b;
+    mx = mx > ab ? mx : ab;
+    any |= (unsigned)a | (unsigned)b | (unsigned)x | (unsigned)y;
+  }
+  S.any |= any;
+  const int ec = mx >> 20;
+  if (ec + 3 > S.eb) raise(S, ec + 4);
+  int rh[3], rl[3], ih[3], il[3], sh[3], sl[3];
+  STAG_UNROLL
+  for (int c = 0; c < 3; ++c) {
+    component(psi[c].x, S.eb, rh[c], rl[c]);
+    component(psi[c].y, S.eb, ih[c], il[c]);
+    sh[c] = rh[c] + ih[c];
+    sl[c] = rl[c] + il[c];
+  }
+  STAG_UNROLL
+  for (int i = 0; i < 3; ++i) {
+    long long m1 = 0x80000000LL, m2 = m1, m3 = m1;
+    STAG_UNROLL
+    for (int j = 0; j < 3; ++j) {
+      const auto w = link(3 * i + j);
+      const int th = (int)((unsigned)w.x + (unsigned)w.z), tl = w.y + w.w;
+      fx::wmad(S.p[i][0], w.x, rh[j]);
+      fx::wmad(m1, w.x, rl[j]);
+      fx::wmad(m1, w.y, rh[j]);
+      fx::wmad(S.p[i][1], w.z, ih[j]);
+      fx::wmad(m2, w.z, il[j]);
+      fx::wmad(m2, w.w, ih[j]);
+      fx::wmad(S.p[i][2], th, sh[j]);
+      fx::wmad(m3, th, sl[j]);
+      fx::wmad(m3, tl, sh[j]);
+    }
+    S.p[i][0] = fx::add64(S.p[i][0], (long long)(int)(m1 >> 32) * 4);
+    S.p[i][1] = fx::add64(S.p[i][1], (long long)(int)(m2 >> 32) * 4);
+    S.p[i][2] = fx::add64(S.p[i][2], (long long)(int)(m3 >> 32) * 4);
+  }
+}
+
+// Exponents of the unit for which every value on the way is a normal number.
+constexpr int MIN_EB = 256, MAX_EB = 1900;
+
+// The site's sum as doubles, kexp the exponent of the links' unit; false: exponents out of range.
+template <class V2> STAG_FX bool result(const Sums& S, int kexp, V2* out) {
+  const int k = S.eb - 1083 + kexp;
+  STAG_UNROLL
+  for (int i = 0; i < 3; ++i) {
+    out[i].x = fx::double_of(real_sum(S, i), k);
+    out[i].y = fx::double_of(imag_sum(S, i), k);
+  }
+  return S.eb >= MIN_EB && S.eb <= MAX_EB;
+}
+
+}  // namespace fxd
+}  // namespace stag

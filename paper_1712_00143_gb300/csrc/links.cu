@@ -220,19 +220,12 @@ __global__ void __launch_bounds__(128) k_fx_stats(const double2* __restrict__ L,
 }
 
 // in place: two doubles -> {re.h, re.l, im.h, im.l} in units of 2^kexp, rounded to nearest
-__device__ __forceinline__ void fixed_entry(double v, int kexp, int& h, int& l) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-  const int r = 1023 + kexp - (int)((b >> 52) & 0x7ff);  // >= 1: |v| < 2^kexp
-  const unsigned long long m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 8;
-  const long long q = r > 62 ? 0 : (long long)((m + (1ull << (r - 1))) >> r);
-  fx::split1((long long)b < 0 ? -q : q, h, l);
-}
 __global__ void __launch_bounds__(256) k_fx_convert(double2* L, long long n, int kexp) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const double2 v = L[i];
     int4 q;
-    fixed_entry(v.x, kexp, q.x, q.y);
-    fixed_entry(v.y, kexp, q.z, q.w);
+    fxd::fixed_entry(v.x, kexp, q.x, q.y);
+    fxd::fixed_entry(v.y, kexp, q.z, q.w);
     ((int4*)L)[i] = q;
   }
 }

@@ -1,0 +1,92 @@
+"""The integer steps of the FP64 operator on the host (csrc/fx_steps.h through a small C++ program), against
+sums in exact arithmetic, at the largest values their bounds admit."""
+
+import math
+import os
+import shutil
+import subprocess
+from fractions import Fraction
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+pytestmark = pytest.mark.skipif(shutil.which("g++") is None, reason="needs g++")
+
+
+@pytest.fixture(scope="module")
+def steps(tmp_path_factory):
+    exe = tmp_path_factory.mktemp("fx") / "fx_steps_check"
+    src = os.path.join(ROOT, "tests", "native", "fx_steps_check.cpp")
+    inc = os.path.join(ROOT, "paper_1712_00143_gb300", "csrc")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-I" + inc, src, "-o", str(exe)], check=True)
+
+    def run(sites):
+        """sites: [(unit exponent, links [hops, 3, 3], vectors [hops, 3])] -> complex [site, 3] (None: range)"""
+        text = []
+        for kexp, links, psi in sites:
+            text.append(f"site {len(links)} {kexp}")
+            for w, v in zip(links, psi):
+                c = np.concatenate([np.asarray(w).reshape(9), np.asarray(v)])
+                text.append(" ".join(f"{float(z.real).hex()} {float(z.imag).hex()}" for z in c))
+        out = subprocess.run([str(exe)], input="\n".join(text) + "\n", capture_output=True, text=True, check=True)
+        res = []
+        for line in out.stdout.splitlines():
+            f = [float.fromhex(x) for x in line.split()] if line != "range" else None
+            res.append(None if f is None else np.array(f[0::2]) + 1j * np.array(f[1::2]))
+        assert len(res) == len(sites)
+        return res
+
+    return run
+
+
+def exact(links, psi):
+    out = []
+    for i in range(3):
+        re = im = Fraction(0)
+        for w, v in zip(links, psi):
+            for j in range(3):
+                a, b = Fraction(w[i][j].real), Fraction(w[i][j].imag)
+                c, d = Fraction(v[j].real), Fraction(v[j].imag)
+                re += a * c - b * d
+                im += a * d + b * c
+        out.append(complex(float(re), float(im)))
+    return np.array(out)
+
+
+def check(steps, sites):
+    """48 products per sum: FP64 itself rounds to within 96 * 2^-53 = 1.1e-14 of (sum over hops of the row's
+    norm) x (largest vector's norm)."""
+    for (_, links, psi), got in zip(sites, steps(sites)):
+        want = exact(links, psi)
+        row = np.sqrt((np.abs(np.asarray(links)) ** 2).sum(-1)).sum(0).max()
+        size = row * np.sqrt((np.abs(np.asarray(psi)) ** 2).sum(-1)).max()
+        assert got is not None and np.abs(got - want).max() <= 1.1e-14 * size, (got, want)
+
+
+def test_sums_keep_their_value_when_the_unit_is_raised(steps):
+    """Rows of sixteen hops with norms that add up to 8.995 units, entries (1 + i) c and aligned vectors: the
+    third running sum passes 2^63 before a larger last neighbour raises the unit."""
+    sites = []
+    for z in (1e-3, 1e-2):
+        c = (8.995 - 2 * z * math.sqrt(6)) / 14 / math.sqrt(6)
+        for s in (1, -1, 1j, -1j):
+            links = np.full((16, 3, 3), s * (1 + 1j) * c)
+            links[0] = links[15] = (1 + 1j) * z
+            psi = np.full((16, 3), 3.999 + 3.999j)
+            psi[0], psi[15] = 1.99 + 1.99j, 7.99 + 7.99j
+            sites.append((0, links, psi))
+            sites.append((0, links, psi.conj()))
+    check(steps, sites)
+
+
+def test_random_fields(steps):
+    rng = np.random.default_rng(5)
+    sites = []
+    for n in range(40):
+        links = rng.normal(size=(16, 3, 3)) + 1j * rng.normal(size=(16, 3, 3))
+        links *= 0.4 / np.abs(links).max() * rng.choice([1.0, 1 / 16], size=(16, 1, 1))
+        psi = (rng.normal(size=(16, 3)) + 1j * rng.normal(size=(16, 3))) * 2.0 ** rng.integers(-8, 9, size=(16, 1))
+        sites.append((0, links, psi))
+    check(steps, sites)
