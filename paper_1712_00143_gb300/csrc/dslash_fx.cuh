@@ -8,7 +8,7 @@
 // rate; integer pipe 45 % busy) against 522 us in FP64.
 //
 // Links: the handle's FP64 copy holds, in place of two doubles, {re.h, re.l,
-// im.h, im.l} with entry = (h 2^-30 + l 2^-60) 2^kexp, |entry| < 2^kexp
+// im.h, im.l} with entry = (h 2^-30 + l 2^-60) 2^kexp, |entry| <= 1.25 2^kexp
 // (links.cu converts a field when its range allows).
 // Vectors stay doubles in memory.  A site's sum runs in units of 2^-60 2^E
 // with E set by the largest neighbour component met so far (E = eb - 1023,

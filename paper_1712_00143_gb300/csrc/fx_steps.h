@@ -3,6 +3,7 @@
 // of a 64-bit value into two words, and the FP64 operator's running sums over
 // the hops of a site (dslash_fx.cuh).
 #pragma once
+#include <cmath>
 #include <cstring>
 
 #ifdef __CUDACC__
@@ -93,12 +94,25 @@ STAG_FX double double_of(long long s, int k) {
 
 namespace fxd {
 
-// One link entry in units of 2^kexp, |v| < 2^kexp: v = (h 2^-30 + l 2^-60) 2^kexp, rounded to nearest.
+// The exponent of the links' unit, from the largest norm of a matrix row and
+// the largest sum over a site's hops of such norms: rows of at most 1.25 units
+// keep the 32-bit sum of an entry's two parts (1.25 sqrt 2 < 2) and a row's
+// three cross products (see hop: 1.25 sqrt 2 sqrt 3 2^61 + 3 2^59 < 2^63) in
+// range, sums of at most 9 the site's sums.
+inline int unit_exponent(double row, double sum) {
+  int k = 0;
+  const double f = std::frexp(row / 1.25, &k);  // row / 1.25 = f 2^k, f in [1/2, 1)
+  if (f == 0.5) --k;
+  while (std::ldexp(sum, -k) > 9.0) ++k;
+  return k;
+}
+
+// One link entry in units of 2^kexp, |v| <= 1.25 2^kexp: v = (h 2^-30 + l 2^-60) 2^kexp, rounded to nearest.
 STAG_FX void fixed_entry(double v, int kexp, int& h, int& l) {
   const unsigned long long b = fx::bits_of(v);
-  const int r = 1023 + kexp - (int)((b >> 52) & 0x7ff);  // >= 1
+  const int r = 1023 + kexp - (int)((b >> 52) & 0x7ff);  // >= 0
   const unsigned long long m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 8;
-  const long long q = r > 62 ? 0 : (long long)((m + (1ull << (r - 1))) >> r);
+  const long long q = r > 62 ? 0 : r > 0 ? (long long)((m + (1ull << (r - 1))) >> r) : (long long)m;
   fx::split1((long long)b < 0 ? -q : q, h, l);
 }
 
@@ -169,13 +183,14 @@ template <class V2, class Link> STAG_FX void hop(Sums& S, const V2 (&psi)[3], Li
     sh[c] = rh[c] + ih[c];
     sl[c] = rl[c] + il[c];
   }
+  // a row's cross sums: |rl|, |il| < 2^30 and |rh|, |ih| < 2^28, so |sl| < 2^31 and |sh| < 2^29
   STAG_UNROLL
   for (int i = 0; i < 3; ++i) {
     long long m1 = 0x80000000LL, m2 = m1, m3 = m1;
     STAG_UNROLL
     for (int j = 0; j < 3; ++j) {
       const auto w = link(3 * i + j);
-      const int th = (int)((unsigned)w.x + (unsigned)w.z), tl = w.y + w.w;
+      const int th = w.x + w.z, tl = w.y + w.w;
       fx::wmad(S.p[i][0], w.x, rh[j]);
       fx::wmad(m1, w.x, rl[j]);
       fx::wmad(m1, w.y, rh[j]);

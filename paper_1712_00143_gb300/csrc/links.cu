@@ -165,11 +165,11 @@ static double max_abs(const double2* a, long long n_complex, unsigned long long*
 // ------------------------------------------------------------ fixed-point form of the FP64 copy
 // What decides whether (and in which unit) the FP64 copy can be held in fixed
 // point (dslash_fx.cuh): the largest entry, the smallest nonzero matrix (by
-// its largest entry), both as high words of the double, and the largest sum
-// over the sixteen hops of a row's norm.
+// its largest entry), both as high words of the double, the largest norm of a
+// row, and the largest sum over the sixteen hops of a row's norms.
 struct FxStats {
   int max_hi, min_hi;
-  unsigned row;  // a float's bits
+  unsigned row, sum;  // floats' bits
 };
 
 __device__ __forceinline__ float float_of_bits(double v) {  // |v| to float without the FP64 pipe; ends clamped
@@ -184,7 +184,7 @@ __device__ __forceinline__ float float_of_bits(double v) {  // |v| to float with
 __global__ void __launch_bounds__(128) k_fx_stats(const double2* __restrict__ L, int Vh, FxStats* st) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   int mx = 0, mn = 0x7fffffff;
-  float row = 0.f;
+  float row = 0.f, most = 0.f;
   if (idx < 2 * Vh) {
     const int p = idx / Vh, s = idx - p * Vh;
     const double2* src = L + (size_t)p * 144 * Vh + s;
@@ -202,20 +202,24 @@ __global__ void __launch_bounds__(128) k_fx_stats(const double2* __restrict__ L,
           const float a = float_of_bits(w.x), b = float_of_bits(w.y);
           n2 += a * a + b * b;
         }
-        sum[i] += sqrtf(n2);
+        const float n = sqrtf(n2);
+        row = fmaxf(row, n);
+        sum[i] += n;
       }
       mx = max(mx, m);
       if (m > 0) mn = min(mn, m);
     }
-    row = fmaxf(sum[0], fmaxf(sum[1], sum[2]));
+    most = fmaxf(sum[0], fmaxf(sum[1], sum[2]));
   }
   mx = (int)__reduce_max_sync(0xffffffffu, (unsigned)mx);
   mn = (int)__reduce_min_sync(0xffffffffu, (unsigned)mn);
   const unsigned r = __reduce_max_sync(0xffffffffu, __float_as_uint(row));
+  const unsigned q = __reduce_max_sync(0xffffffffu, __float_as_uint(most));
   if ((threadIdx.x & 31) == 0) {
     atomicMax(&st->max_hi, mx);
     atomicMin(&st->min_hi, mn);
     atomicMax(&st->row, r);
+    atomicMax(&st->sum, q);
   }
 }
 
@@ -235,7 +239,7 @@ __global__ void __launch_bounds__(256) k_fx_convert(double2* L, long long n, int
 // entry within 2^+-50 (where the row norms' FP32 squares are normal numbers);
 // else it stays in doubles.
 static int to_fixed(LinkCopy& L, const Geom& g, FxStats* scratch, cudaStream_t st) {
-  FxStats h{0, 0x7fffffff, 0u};
+  FxStats h{0, 0x7fffffff, 0u, 0u};
   int status = cuda_status(cudaMemcpyAsync(scratch, &h, sizeof(h), cudaMemcpyHostToDevice, st));
   if (status) return status;
   {
@@ -245,14 +249,12 @@ static int to_fixed(LinkCopy& L, const Geom& g, FxStats* scratch, cudaStream_t s
   if ((status = last_launch_status())) return status;
   if ((status = cuda_status(cudaMemcpyAsync(&h, scratch, sizeof(h), cudaMemcpyDeviceToHost, st)))) return status;
   if ((status = cuda_status(cudaStreamSynchronize(st)))) return status;
-  float row;
+  float row, sum;
   memcpy(&row, &h.row, sizeof(row));
+  memcpy(&sum, &h.sum, sizeof(sum));
   const int emax = h.max_hi >> 20, emin = h.min_hi >> 20;
   if (emax < 1023 - 50 || emax > 1023 + 50 || emin < emax - 10) return STAG_OK;
-  int kexp = emax - 1022;  // |entry| < 2^kexp
-  double r = std::ldexp((double)row, -kexp);
-  for (int k = 0; k < 4 && r > 9.0; ++k, r *= 0.5) ++kexp;
-  if (!(r <= 9.0)) return STAG_OK;
+  const int kexp = fxd::unit_exponent(row, sum);
   const long long n = (long long)2 * 144 * g.Vh;
   {
     ProfScope ps("links", st);

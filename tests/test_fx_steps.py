@@ -90,3 +90,23 @@ def test_random_fields(steps):
         psi = (rng.normal(size=(16, 3)) + 1j * rng.normal(size=(16, 3))) * 2.0 ** rng.integers(-8, 9, size=(16, 1))
         sites.append((0, links, psi))
     check(steps, sites)
+
+
+# bits of a component that the high word does not hold: nearly all set
+LOW = 1.0 + (2.0**52 - 1) * 2.0**-52
+
+
+@pytest.mark.parametrize("c", [1 - 2.0**-40, 1 - 2.0**-33, 0.95, 0.5, 0.8838834, 0.7216878, 0.51])
+@pytest.mark.parametrize("hops", [1, 2, 3, 16])
+def test_rows_of_the_largest_entries(steps, c, hops):
+    """(1 + i) c in one or all colours, vectors of large low parts: the sum of an entry's parts and a row's
+    cross products at their largest."""
+    sites = []
+    for colours in (1, 3):
+        for s in (1, -1, 1j, -1j):
+            for v in (LOW, 1.5 * LOW, 1.0 + 0.5 * LOW, 1.999999):
+                w = np.zeros((hops, 3, 3), dtype=complex)
+                w[:, :, :colours] = s * (1 + 1j) * c
+                for q in (v + 1j * v, v - 1j * v):
+                    sites.append((9999, w, np.full((hops, 3), q)))
+    check(steps, sites)

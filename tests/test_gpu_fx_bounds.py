@@ -65,3 +65,17 @@ def test_sums_before_a_larger_neighbour(dims, nrhs, phase):
     for t, h in enumerate(_hops(dims, site, 0)):
         psi[h[5]] = (1 + 1j) * (1.99 if t == 0 else 7.99 if t == 15 else 3.999)
     _compare(dims, nrhs, site, fat, lng, psi)
+
+
+@pytest.mark.parametrize("dims,nrhs", FORMS)
+@pytest.mark.parametrize("c", [1 - 2.0**-40, 0.95])
+def test_one_hop_of_large_rows(dims, nrhs, c):
+    """One hop's entries (1 + i) c beside small ones, and vectors whose low words are nearly full."""
+    site = 37
+    low = 1.0 + (2.0**52 - 1) * 2.0**-52
+    matrices = [np.full((3, 3), (1 + 1j) * (c if t == 4 else 0.02)) for t in range(16)]
+    fat, lng = _field(dims, site, 0, matrices, 0.02)
+    psi = synth.random_spinor(dims, 78) * 0.1
+    for h in _hops(dims, site, 0):
+        psi[h[5]] = (1 + 1j) * low
+    _compare(dims, nrhs, site, fat, lng, psi)
