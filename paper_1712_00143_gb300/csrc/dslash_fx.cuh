@@ -4,21 +4,20 @@
 // clock and SM take 2.8 times as long as its 2400 bytes take from HBM.  Here
 // the sixteen link-times-vector products run in the exact fixed-point
 // arithmetic of fx.cuh (81 wide integer multiply-adds per hop) and the
-// operator is bound by HBM again: 32^4, one half 214 us (0.88 of the copy
+// operator is bound by HBM again: 32^4, one half 217 us (0.87 of the copy
 // rate; integer pipe 45 % busy) against 522 us in FP64.
 //
 // Links: the handle's FP64 copy holds, in place of two doubles, {re.h, re.l,
-// im.h, im.l} with entry = (h 2^-30 + l 2^-60) 2^kexp, |entry| <= 1.25 2^kexp
-// (links.cu converts a field when its range allows).
+// im.h, im.l} with entry = (h 2^-30 + l 2^-60) 2^k, and one byte k per matrix
+// (fx_steps.h says how k is chosen; links.cu converts a field).
 // Vectors stay doubles in memory.  A site's sum runs in units of 2^-60 2^E
-// with E set by the largest neighbour component met so far (E = eb - 1023,
-// |component| < 2^(E-2)); a larger one raises E and shifts the sums down,
-// which after the first neighbour is rare.  The neighbours' small components
-// are thus known to 2^-60 of the largest, FP64's rounded sums to 2^-53 of it.
-// The two spare bits and the bound on the link rows that links.cu checks
-// (sum over hops of the row norms <= 9) keep a site's real and imaginary sums
-// below 2^63: 9 sqrt(6) / 4 2^60 < 5.6 2^60.  The three sums they are made of
-// (Gauss) are kept modulo 2^64.
+// with E set by the largest product of a neighbour's largest component and its
+// matrix's unit met so far (E = eb - 1023; a component of matrix unit 2^k is
+// below 2^(E - k - 3)); a larger one raises E and shifts the sums down.  A
+// neighbour seen through a zero matrix sets no unit.
+// A site's real and imaginary sums stay below 2^63: 16 hops x 1.25 x sqrt(6) /
+// 8 2^60 < 6.2 2^60.  The three sums they are made of (Gauss) are kept modulo
+// 2^64.
 // Neighbours with exponents near the ends of the double range (infinities,
 // NaN and subnormals among them) take an FP64 loop over the same links.
 #pragma once
@@ -36,14 +35,15 @@ namespace fxd {
 // FP64 loop over the same links (rare): the sums whose exponents leave the fixed-point range.
 template <class Args> __device__ __noinline__ void site_fp64(const Args& a, int s, double2* out) {
   const Coord c = cb_coords(a.g, s, a.out_parity);
-  const double scale = __longlong_as_double((long long)(1023 + a.kexp) << 52);
   for (int i = 0; i < 3; ++i) out[i] = make_double2(0.0, 0.0);
 #pragma unroll 1
   for (int t = 0; t < 16; ++t) {
     const int k = ((t & 2) ? 3 : 1) * ((t & 1) ? -1 : 1);
     double2 psi[3];
     SpinorLoad<64>::ld(a.in, cb_neighbour(a.g, s, c, t >> 2, k), psi);
-    const int4* L = (const int4*)a.links + (size_t)t * 9 * a.g.Vh + STAG_BOUND(s, a.g.Vh, BOUND_LINK);
+    const int at = STAG_BOUND(s, a.g.Vh, BOUND_LINK);
+    const int4* L = (const int4*)a.links + (size_t)t * 9 * a.g.Vh + at;
+    const double scale = __longlong_as_double((long long)(1023 + __ldg(a.kexp + (size_t)at * 16 + t)) << 52);
 #pragma unroll 1
     for (int i = 0; i < 3; ++i)
 #pragma unroll 1
@@ -56,21 +56,18 @@ template <class Args> __device__ __noinline__ void site_fp64(const Args& a, int 
   }
 }
 
-// hops [t0, t1) of site s
-template <class Args> __device__ __forceinline__ void hops(Sums& S, const Args& a, int s, const Coord& c, int t0, int t1) {
-  const int Vh = a.g.Vh;
-#pragma unroll 1
-  for (int t = t0; t < t1; ++t) {
-    const int k = ((t & 2) ? 3 : 1) * ((t & 1) ? -1 : 1);
-    double2 psi[3];
-    SpinorLoad<64>::ld(a.in, cb_neighbour(a.g, s, c, t >> 2, k), psi);
-    const int4* L = (const int4*)a.links + (size_t)t * 9 * Vh + STAG_BOUND(s, Vh, BOUND_LINK);
-    hop(S, psi, [&](int e) { return __ldg(L + (size_t)e * Vh); });
-  }
+// hop t of site s, kexp the exponent of its matrix
+template <class Args>
+__device__ __forceinline__ void hop_of(Sums& S, const Args& a, int s, const Coord& c, int t, int kexp) {
+  const int Vh = a.g.Vh, k = ((t & 2) ? 3 : 1) * ((t & 1) ? -1 : 1);
+  double2 psi[3];
+  SpinorLoad<64>::ld(a.in, cb_neighbour(a.g, s, c, t >> 2, k), psi);
+  const int4* L = (const int4*)a.links + (size_t)t * 9 * Vh + STAG_BOUND(s, Vh, BOUND_LINK);
+  hop(S, psi, kexp, [&](int e) { return __ldg(L + (size_t)e * Vh); });
 }
 
 template <class Args> __device__ __forceinline__ void finish(const Sums& S, const Args& a, int s, double2 out[3]) {
-  if (!result(S, a.kexp, out)) {
+  if (!result(S, out)) {
     if (S.any == 0) {
 #pragma unroll
       for (int i = 0; i < 3; ++i) out[i] = make_double2(0.0, 0.0);
@@ -83,7 +80,18 @@ template <class Args> __device__ __forceinline__ void finish(const Sums& S, cons
 template <class Args> __device__ __forceinline__ void site(const Args& a, int s, double2 out[3]) {
   Sums S;
   init(S);
-  hops(S, a, s, cb_coords(a.g, s, a.out_parity), 0, 16);
+  const Coord c = cb_coords(a.g, s, a.out_parity);
+  // the sixteen exponents in one load ahead of the hops (a byte per hop, which
+  // each hop's conversion waits for, cost 6 % at 32^4)
+  uint4 k = __ldg((const uint4*)a.kexp + STAG_BOUND(s, a.g.Vh, BOUND_LINK));
+#pragma unroll 1
+  for (int t = 0; t < 16; ++t) {
+    hop_of(S, a, s, c, t, (int)(signed char)(k.x & 0xffu));
+    k.x = __funnelshift_r(k.x, k.y, 8);
+    k.y = __funnelshift_r(k.y, k.z, 8);
+    k.z = __funnelshift_r(k.z, k.w, 8);
+    k.w >>= 8;
+  }
   finish(S, a, s, out);
 }
 
@@ -100,7 +108,8 @@ template <class Args> __device__ __forceinline__ bool component16(const Args& a,
   Sums S;
   init(S);
   int s = s0 + ls;
-  if (s < end) hops(S, a, s, cb_coords(a.g, s, a.out_parity), t, t + 1);
+  if (s < end)
+    hop_of(S, a, s, cb_coords(a.g, s, a.out_parity), t, __ldg(a.kexp + (size_t)STAG_BOUND(s, a.g.Vh, BOUND_LINK) * 16 + t));
   long long v[6];
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
@@ -138,7 +147,7 @@ template <class Args> __device__ __forceinline__ bool component16(const Args& a,
     any |= sa[q][ls];
   }
   if (eb >= MIN_EB && eb <= MAX_EB) {
-    out = fx::double_of(sum, eb - 1083 + a.kexp);
+    out = fx::double_of(sum, eb - 1083);
   } else if (any == 0) {
     out = 0.0;
   } else {

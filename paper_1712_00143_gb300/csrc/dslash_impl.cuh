@@ -27,7 +27,7 @@ template <int P> struct DslashArgs {
   float fat_scale, long_scale;  // long_scale = c3/2 for two-row storage
   Spinor<P> in;
   int s_begin, s_end;  // output sites computed: [s_begin, s_end) (all: 0, Vh)
-  int kexp;            // fixed-point FP64 links: entries in units of 2^kexp
+  const signed char* kexp;  // fixed-point FP64 links: exponents of the matrices' units, [site][hop]
 };
 
 // The complex number k of a group of link chunks held in registers (k is a
@@ -274,7 +274,7 @@ static DslashArgs<P> make_args(const stag_lattice_s* lat, Spinor<P> in, int out_
   a.in = in;
   a.s_begin = 0;
   a.s_end = lat->g.Vh;
-  a.kexp = L.kexp;
+  a.kexp = L.kexp + (size_t)out_parity * 16 * lat->g.Vh;
   return a;
 }
 

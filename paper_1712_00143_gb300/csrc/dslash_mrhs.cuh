@@ -67,7 +67,7 @@ template <int P> struct DslashArgsM {
   const uint4* links;
   float fat_scale, long_scale;
   SpinorM<P> in;
-  int kexp;  // fixed-point FP64 links (dslash_fx.cuh)
+  const signed char* kexp;  // fixed-point FP64 links (dslash_fx.cuh)
 };
 
 // Loads the chunks holding the complex entries [k0, k0 + NE) of one hop and

@@ -94,17 +94,55 @@ STAG_FX double double_of(long long s, int k) {
 
 namespace fxd {
 
-// The exponent of the links' unit, from the largest norm of a matrix row and
-// the largest sum over a site's hops of such norms: rows of at most 1.25 units
-// keep the 32-bit sum of an entry's two parts (1.25 sqrt 2 < 2) and a row's
-// three cross products (see hop: 1.25 sqrt 2 sqrt 3 2^61 + 3 2^59 < 2^63) in
-// range, sums of at most 9 the site's sums.
-inline int unit_exponent(double row, double sum) {
-  int k = 0;
-  const double f = std::frexp(row / 1.25, &k);  // row / 1.25 = f 2^k, f in [1/2, 1)
-  if (f == 0.5) --k;
-  while (std::ldexp(sum, -k) > 9.0) ++k;
-  return k;
+// The unit of a link matrix is 2^k with the smallest k for which no row's norm
+// passes 1.25 units.  That keeps in range the 32-bit sum of an entry's two
+// parts (1.25 sqrt 2 < 2) and a row's three cross products (see hop: 1.25
+// sqrt 2 sqrt 3 2^61 + 3 2^58 < 2^63); every matrix is known to 2^-61 of at
+// most 1.6 times its own largest row norm, FP64's entries to 2^-53.
+// NO_MATRIX: all entries are zero.  BAD_MATRIX: an exponent beyond +-100 (or
+// an infinity, or a NaN); the field then stays in doubles.
+constexpr int NO_MATRIX = -128, BAD_MATRIX = 127;
+
+// |v| 2^-e as a float, without an FP64 instruction; below 2^-126: 0.  |v| < 2^(e + 1).
+STAG_FX float scaled_float(double v, int e) {
+  const unsigned long long b = fx::bits_of(v) & 0x7fffffffffffffffull;
+  const int k = (int)(b >> 52) - e;  // biased exponent of the result (+ 0: that of a double)
+  const unsigned u = k < 897 ? 0u : ((unsigned)(k - 896) << 23) | ((unsigned)(b >> 29) & 0x7fffffu);
+#ifdef __CUDA_ARCH__
+  return __uint_as_float(u);
+#else
+  float f;
+  std::memcpy(&f, &u, sizeof(f));
+  return f;
+#endif
+}
+
+STAG_FX int matrix_exponent(const double (&v)[18]) {
+  int mx = 0;
+  unsigned any = 0;
+  STAG_UNROLL
+  for (int i = 0; i < 18; ++i) {
+    const unsigned long long b = fx::bits_of(v[i]);
+    const int h = (int)(b >> 32) & 0x7fffffff;
+    mx = mx > h ? mx : h;
+    any |= (unsigned)h | (unsigned)b;
+  }
+  if (any == 0) return NO_MATRIX;
+  const int e = (mx >> 20) - 1023;  // the largest entry's exponent
+  if (e < -100 || e > 100) return BAD_MATRIX;
+  float row = 0.f;
+  STAG_UNROLL
+  for (int i = 0; i < 3; ++i) {
+    float n2 = 0.f;
+    STAG_UNROLL
+    for (int j = 0; j < 6; ++j) {
+      const float a = scaled_float(v[6 * i + j], e);
+      n2 += a * a;
+    }
+    row = row > n2 ? row : n2;
+  }
+  // row norms of up to 1.25, 2.5 and 5 (an entry's parts are below 2: at most 2 sqrt 6)
+  return e + (row <= 1.5625f ? 0 : row <= 6.25f ? 1 : 2);
 }
 
 // One link entry in units of 2^kexp, |v| <= 1.25 2^kexp: v = (h 2^-30 + l 2^-60) 2^kexp, rounded to nearest.
@@ -123,7 +161,7 @@ STAG_FX void fixed_entry(double v, int kexp, int& h, int& l) {
 struct Sums {
   long long p[3][3];
   int eb;        // biased exponent of the unit (0: nothing met)
-  unsigned any;  // 0 while every component was an exact zero
+  unsigned any;  // 0 while every component seen through a matrix was an exact zero
 };
 
 STAG_FX void init(Sums& S) {
@@ -149,7 +187,7 @@ STAG_FX void raise(Sums& S, int eb) {
   S.eb = eb;
 }
 
-// One component (h, l) in units of 2^-30, 2^-60 of 2^(eb - 1023); its exponent is at most eb - 3.
+// One component (h, l) in units of 2^-30, 2^-60 of 2^(eb - 1023); its exponent is at most eb - 4.
 STAG_FX void component(double v, int eb, int& h, int& l) {
   const unsigned long long b = fx::bits_of(v);
   const int hi = (int)(b >> 32);
@@ -161,8 +199,11 @@ STAG_FX void component(double v, int eb, int& h, int& l) {
   l = ((int)((unsigned)m & 0x3fffffffu) ^ s) - s;
 }
 
-// One hop: psi[3] with .x and .y, link(e) the matrix entry e = 3 row + column as {re.h, re.l, im.h, im.l}.
-template <class V2, class Link> STAG_FX void hop(Sums& S, const V2 (&psi)[3], Link link) {
+// One hop: psi[3] with .x and .y, kexp the exponent of its matrix (NO_MATRIX:
+// the hop counts for nothing, unless psi is not finite), link(e) the matrix
+// entry e = 3 row + column as {re.h, re.l, im.h, im.l}.  The sums' unit follows
+// the largest vector times its matrix's unit.
+template <class V2, class Link> STAG_FX void hop(Sums& S, const V2 (&psi)[3], int kexp, Link link) {
   int mx = 0;
   unsigned any = 0;
   STAG_UNROLL
@@ -172,18 +213,20 @@ template <class V2, class Link> STAG_FX void hop(Sums& S, const V2 (&psi)[3], Li
     mx = mx > ab ? mx : ab;
     any |= (unsigned)a | (unsigned)b | (unsigned)x | (unsigned)y;
   }
-  S.any |= any;
-  const int ec = mx >> 20;
-  if (ec + 3 > S.eb) raise(S, ec + 4);
+  kexp = kexp == NO_MATRIX ? -4000 : kexp;
+  const int ec = mx >= 0x7ff00000 ? 8000 : (mx >> 20) + kexp;
+  S.any |= ec >= -1000 ? any : 0u;
+  if (ec + 4 > S.eb) raise(S, ec + 4);
+  const int eb = S.eb - kexp;
   int rh[3], rl[3], ih[3], il[3], sh[3], sl[3];
   STAG_UNROLL
   for (int c = 0; c < 3; ++c) {
-    component(psi[c].x, S.eb, rh[c], rl[c]);
-    component(psi[c].y, S.eb, ih[c], il[c]);
+    component(psi[c].x, eb, rh[c], rl[c]);
+    component(psi[c].y, eb, ih[c], il[c]);
     sh[c] = rh[c] + ih[c];
     sl[c] = rl[c] + il[c];
   }
-  // a row's cross sums: |rl|, |il| < 2^30 and |rh|, |ih| < 2^28, so |sl| < 2^31 and |sh| < 2^29
+  // a row's cross sums: |rl|, |il| < 2^30 and |rh|, |ih| < 2^27, so |sl| < 2^31 and |sh| < 2^28
   STAG_UNROLL
   for (int i = 0; i < 3; ++i) {
     long long m1 = 0x80000000LL, m2 = m1, m3 = m1;
@@ -210,9 +253,9 @@ template <class V2, class Link> STAG_FX void hop(Sums& S, const V2 (&psi)[3], Li
 // Exponents of the unit for which every value on the way is a normal number.
 constexpr int MIN_EB = 256, MAX_EB = 1900;
 
-// The site's sum as doubles, kexp the exponent of the links' unit; false: exponents out of range.
-template <class V2> STAG_FX bool result(const Sums& S, int kexp, V2* out) {
-  const int k = S.eb - 1083 + kexp;
+// The site's sum as doubles; false: exponents out of range.
+template <class V2> STAG_FX bool result(const Sums& S, V2* out) {
+  const int k = S.eb - 1083;
   STAG_UNROLL
   for (int i = 0; i < 3; ++i) {
     out[i].x = fx::double_of(real_sum(S, i), k);

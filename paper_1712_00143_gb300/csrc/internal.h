@@ -26,8 +26,8 @@ struct LinkCopy {
   float fat_scale = 1.f;    // 16-bit formats: stored (normalised) value * scale
   float long_scale = 1.f;   //   = matrix entry
   size_t elem_bytes = 0;    // bytes of one stored complex
-  bool fixed = false;       // FP64: entries in fixed point (dslash_fx.cuh), in units
-  int kexp = 0;             //   of 2^kexp, instead of doubles
+  bool fixed = false;       // FP64: entries in fixed point (dslash_fx.cuh) instead of doubles,
+  signed char* kexp = nullptr;  //   [parity][site][hop]: the matrix in units of 2^kexp
   int shape_plain = 1;      // launch shapes chosen by the autotuner
   int shape_epi = 1;        // (default: 256 threads, 4 blocks per SM)
   float tuned_us[2] = {0.f, 0.f};  // their timings (us per launch)

@@ -13,7 +13,6 @@
 // two-row storage of the SU(3) part) form one list of complex numbers,
 // packed PER to a 16-byte chunk; chunk j of all sites is contiguous,
 // [chunk][site], so a warp's 128-bit loads of one chunk are coalesced.
-#include <cmath>
 #include <cstring>
 
 #include "fx.cuh"
@@ -163,106 +162,66 @@ static double max_abs(const double2* a, long long n_complex, unsigned long long*
 }
 
 // ------------------------------------------------------------ fixed-point form of the FP64 copy
-// What decides whether (and in which unit) the FP64 copy can be held in fixed
-// point (dslash_fx.cuh): the largest entry, the smallest nonzero matrix (by
-// its largest entry), both as high words of the double, the largest norm of a
-// row, and the largest sum over the sixteen hops of a row's norms.
-struct FxStats {
-  int max_hi, min_hi;
-  unsigned row, sum;  // floats' bits
-};
-
-__device__ __forceinline__ float float_of_bits(double v) {  // |v| to float without the FP64 pipe; ends clamped
-  const int hi = __double2hiint(v) & 0x7fffffff;
-  const int e = hi >> 20;
-  if (e < 897) return 0.f;
-  if (e > 1150) return __int_as_float(0x7f800000);
-  return __int_as_float(((hi - (896 << 20)) << 3) | (int)((unsigned)__double2loint(v) >> 29));
-}
-
-// one thread per (parity, site); reads the copy once: bound by HBM
-__global__ void __launch_bounds__(128) k_fx_stats(const double2* __restrict__ L, int Vh, FxStats* st) {
+// The exponents of the matrices' units, one thread per (parity, site); *bad is
+// set if some matrix has none.  Reads the copy once: bound by HBM.
+__global__ void __launch_bounds__(128) k_fx_exponents(const double2* __restrict__ L, int Vh,
+                                                      signed char* __restrict__ kexp, int* bad) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  int mx = 0, mn = 0x7fffffff;
-  float row = 0.f, most = 0.f;
-  if (idx < 2 * Vh) {
-    const int p = idx / Vh, s = idx - p * Vh;
-    const double2* src = L + (size_t)p * 144 * Vh + s;
-    float sum[3] = {0.f, 0.f, 0.f};
+  if (idx >= 2 * Vh) return;
+  const int p = idx / Vh, s = idx - p * Vh;
+  const double2* src = L + (size_t)p * 144 * Vh + s;
+  bool out = false;
+  signed char* to = kexp + (size_t)idx * 16;
 #pragma unroll 1
-    for (int t = 0; t < 16; ++t) {
-      int m = 0;
+  for (int t = 0; t < 16; ++t) {
+    double v[18];
 #pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        float n2 = 0.f;
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-          const double2 w = __ldg(src + (size_t)(t * 9 + 3 * i + j) * Vh);
-          m = max(m, max(__double2hiint(w.x) & 0x7fffffff, __double2hiint(w.y) & 0x7fffffff));
-          const float a = float_of_bits(w.x), b = float_of_bits(w.y);
-          n2 += a * a + b * b;
-        }
-        const float n = sqrtf(n2);
-        row = fmaxf(row, n);
-        sum[i] += n;
-      }
-      mx = max(mx, m);
-      if (m > 0) mn = min(mn, m);
+    for (int e = 0; e < 9; ++e) {
+      const double2 w = __ldg(src + (size_t)(t * 9 + e) * Vh);
+      v[2 * e] = w.x;
+      v[2 * e + 1] = w.y;
     }
-    most = fmaxf(sum[0], fmaxf(sum[1], sum[2]));
+    const int k = fxd::matrix_exponent(v);
+    out |= k == fxd::BAD_MATRIX;
+    to[t] = (signed char)k;
   }
-  mx = (int)__reduce_max_sync(0xffffffffu, (unsigned)mx);
-  mn = (int)__reduce_min_sync(0xffffffffu, (unsigned)mn);
-  const unsigned r = __reduce_max_sync(0xffffffffu, __float_as_uint(row));
-  const unsigned q = __reduce_max_sync(0xffffffffu, __float_as_uint(most));
-  if ((threadIdx.x & 31) == 0) {
-    atomicMax(&st->max_hi, mx);
-    atomicMin(&st->min_hi, mn);
-    atomicMax(&st->row, r);
-    atomicMax(&st->sum, q);
-  }
+  if (out) atomicOr(bad, 1);
 }
 
-// in place: two doubles -> {re.h, re.l, im.h, im.l} in units of 2^kexp, rounded to nearest
-__global__ void __launch_bounds__(256) k_fx_convert(double2* L, long long n, int kexp) {
+// in place: two doubles -> {re.h, re.l, im.h, im.l} in the matrix's unit, rounded to nearest
+__global__ void __launch_bounds__(256) k_fx_convert(double2* L, int Vh, const signed char* __restrict__ kexp) {
+  const long long n = (long long)2 * 144 * Vh;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const long long e = i / Vh;  // 144 parity + 9 hop + entry
+    const int p = e >= 144, t = ((int)e - 144 * p) / 9;
+    const int k = __ldg(kexp + ((size_t)p * Vh + (i - e * Vh)) * 16 + t);
     const double2 v = L[i];
     int4 q;
-    fxd::fixed_entry(v.x, kexp, q.x, q.y);
-    fxd::fixed_entry(v.y, kexp, q.z, q.w);
+    fxd::fixed_entry(v.x, k, q.x, q.y);
+    fxd::fixed_entry(v.y, k, q.z, q.w);
     ((int4*)L)[i] = q;
   }
 }
 
-// The FP64 copy to fixed point, if every nonzero matrix lies within 2^-10 of
-// the largest entry (so that all keep FP64's relative accuracy) and the largest
-// entry within 2^+-50 (where the row norms' FP32 squares are normal numbers);
-// else it stays in doubles.
-static int to_fixed(LinkCopy& L, const Geom& g, FxStats* scratch, cudaStream_t st) {
-  FxStats h{0, 0x7fffffff, 0u, 0u};
-  int status = cuda_status(cudaMemcpyAsync(scratch, &h, sizeof(h), cudaMemcpyHostToDevice, st));
+// The FP64 copy to fixed point, unless some matrix's exponent is out of range.
+static int to_fixed(LinkCopy& L, const Geom& g, int* bad, cudaStream_t st) {
+  int status = cuda_status(cudaMemsetAsync(bad, 0, sizeof(int), st));
   if (status) return status;
   {
     ProfScope ps("links", st);
-    k_fx_stats<<<(2 * g.Vh + 127) / 128, 128, 0, st>>>((const double2*)L.data, g.Vh, scratch);
+    k_fx_exponents<<<(2 * g.Vh + 127) / 128, 128, 0, st>>>((const double2*)L.data, g.Vh, L.kexp, bad);
   }
   if ((status = last_launch_status())) return status;
-  if ((status = cuda_status(cudaMemcpyAsync(&h, scratch, sizeof(h), cudaMemcpyDeviceToHost, st)))) return status;
+  int h = 0;
+  if ((status = cuda_status(cudaMemcpyAsync(&h, bad, sizeof(h), cudaMemcpyDeviceToHost, st)))) return status;
   if ((status = cuda_status(cudaStreamSynchronize(st)))) return status;
-  float row, sum;
-  memcpy(&row, &h.row, sizeof(row));
-  memcpy(&sum, &h.sum, sizeof(sum));
-  const int emax = h.max_hi >> 20, emin = h.min_hi >> 20;
-  if (emax < 1023 - 50 || emax > 1023 + 50 || emin < emax - 10) return STAG_OK;
-  const int kexp = fxd::unit_exponent(row, sum);
-  const long long n = (long long)2 * 144 * g.Vh;
+  if (h) return STAG_OK;
   {
     ProfScope ps("links", st);
-    k_fx_convert<<<1216, 256, 0, st>>>((double2*)L.data, n, kexp);
+    k_fx_convert<<<1216, 256, 0, st>>>((double2*)L.data, g.Vh, L.kexp);
   }
   if ((status = last_launch_status())) return status;
   L.fixed = true;
-  L.kexp = kexp;
   return STAG_OK;
 }
 
@@ -275,7 +234,8 @@ int build_link_copy(stag_lattice_s* lat, int prec, int recon, const double2* fat
   size_t bytes = (size_t)2 * 4 * (18 + 2 * nl) * g.Vh * eb;
   if (L.data) cudaFree(L.data);
   L = LinkCopy();
-  if (cudaMalloc(&L.data, bytes) != cudaSuccess) {
+  const size_t kbytes = prec == STAG_FP64 ? (size_t)2 * 16 * g.Vh : 0;
+  if (cudaMalloc(&L.data, bytes + kbytes) != cudaSuccess) {
     cudaGetLastError();
     L.data = nullptr;
     return STAG_ENOMEM;
@@ -283,6 +243,7 @@ int build_link_copy(stag_lattice_s* lat, int prec, int recon, const double2* fat
   L.nl = nl;
   L.elem_bytes = eb;
   L.parity_stride = (size_t)4 * (18 + 2 * nl) * g.Vh * eb;
+  if (kbytes) L.kexp = (signed char*)L.data + bytes;
   int status = 0;
   int* err = (int*)lat->ws.get("links_err", 64, &status);
   if (status) return status;
@@ -322,7 +283,7 @@ int build_link_copy(stag_lattice_s* lat, int prec, int recon, const double2* fat
   if ((status = cuda_status(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st)))) return status;
   if ((status = cuda_status(cudaStreamSynchronize(st)))) return status;
   if (herr) return STAG_ENOTUNITARY;
-  if (prec == STAG_FP64 && (status = to_fixed(L, g, (FxStats*)(err + 8), st))) return status;
+  if (prec == STAG_FP64 && (status = to_fixed(L, g, err + 8, st))) return status;
   L.present = true;
   return STAG_OK;
 }

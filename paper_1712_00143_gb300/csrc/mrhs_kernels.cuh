@@ -177,7 +177,7 @@ template <int P> DslashArgsM<P> make_args_m(const stag_lattice_s* lat, SpinorM<P
   a.fat_scale = (float)(L.fat_scale * fx);
   a.long_scale = (float)((L.nl == 6 ? 0.5 * lat->c3 : (double)L.long_scale) * fx);
   a.in = in;
-  a.kexp = L.kexp;
+  a.kexp = L.kexp + (size_t)out_parity * 16 * lat->g.Vh;
   return a;
 }
 

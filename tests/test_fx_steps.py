@@ -110,3 +110,55 @@ def test_rows_of_the_largest_entries(steps, c, hops):
                 for q in (v + 1j * v, v - 1j * v):
                     sites.append((9999, w, np.full((hops, 3), q)))
     check(steps, sites)
+
+
+def _gaussian(rng, *shape):
+    return rng.normal(size=shape) + 1j * rng.normal(size=shape)
+
+
+def _size(links, psi):
+    """Sum over hops of (row norm) x (vector norm), per row: what the rounding of FP64 sums scales with."""
+    rows = np.sqrt((np.abs(links) ** 2).sum(-1))
+    return (rows * np.sqrt((np.abs(psi) ** 2).sum(-1))[:, None]).sum(0)
+
+
+@pytest.mark.parametrize("small", [0, -3, -7, -10, -20, -40, -90])
+@pytest.mark.parametrize("hop", [0, 5, 15])
+def test_a_small_matrix_keeps_its_accuracy(steps, small, hop):
+    """A vector seen only through a matrix far smaller than the others: six multiply-adds in FP64 are off by at
+    most 6 * 2^-53 of (row norm) x (vector norm)."""
+    rng = np.random.default_rng(100 + hop - small)
+    sites = []
+    for _ in range(40):
+        links, psi = _gaussian(rng, 16, 3, 3), np.zeros((16, 3), dtype=complex)
+        links[hop] *= 2.0**small
+        psi[hop] = _gaussian(rng, 3) * 2.0 ** rng.integers(-3, 4)
+        sites.append((9999, links, psi))
+    for (_, links, psi), got in zip(sites, steps(sites)):
+        assert (np.abs(got - exact(links, psi)) <= 6 * 2.0**-53 * _size(links, psi)).all()
+
+
+@pytest.mark.parametrize("far", [0, 10, 40, 70, 200, 400])
+def test_vectors_behind_zero_matrices_do_not_count(steps, far):
+    """Zero Naik links and far larger vectors three sites away."""
+    rng = np.random.default_rng(far)
+    sites = []
+    for _ in range(20):
+        links, psi = _gaussian(rng, 16, 3, 3), _gaussian(rng, 16, 3)
+        links.reshape(4, 4, 3, 3)[:, 2:] = 0.0
+        psi.reshape(4, 4, 3)[:, 2:] *= 2.0**far
+        sites.append((9999, links, psi))
+    for (_, links, psi), got in zip(sites, steps(sites)):
+        assert (np.abs(got - exact(links, psi)) <= 48 * 2.0**-53 * _size(links, psi)).all()
+
+
+def test_not_finite_vectors_take_the_fp64_loop(steps):
+    rng = np.random.default_rng(9)
+    for bad in (np.nan, np.inf):
+        links, psi = _gaussian(rng, 16, 3, 3), _gaussian(rng, 16, 3)
+        links[3] = 0.0
+        psi[3, 1] = bad
+        assert steps([(9999, links, psi)]) == [None]
+    zero = np.zeros((16, 3, 3), dtype=complex)
+    got = steps([(9999, zero, _gaussian(rng, 16, 3)), (9999, _gaussian(rng, 16, 3, 3), zero[:, 0])])
+    assert all(g is None or (g == 0).all() for g in got)  # ("range" with nothing met: the caller stores zeros)

@@ -79,3 +79,48 @@ def test_one_hop_of_large_rows(dims, nrhs, c):
     for h in _hops(dims, site, 0):
         psi[h[5]] = (1 + 1j) * low
     _compare(dims, nrhs, site, fat, lng, psi)
+
+
+def _sizes(dims, fat, lng, psi, parity):
+    """Per output site and row, the sum over hops of (row norm) x (vector norm)."""
+    Vh = len(psi)
+    lex = oracle.parity_sites(dims, parity)
+    c = oracle.site_coords(dims, lex)
+    norm = np.sqrt((np.abs(psi) ** 2).sum(-1))
+    out = np.zeros((Vh, 3))
+    for mu in range(4):
+        for links, k in ((fat, 1), (lng, 3)):
+            fwd, back = oracle.neighbour_lex(dims, c, mu, k), oracle.neighbour_lex(dims, c, mu, -k)
+            out += 0.5 * np.sqrt((np.abs(links[lex, mu]) ** 2).sum(-1)) * norm[fwd // 2][:, None]
+            out += 0.5 * np.sqrt((np.abs(links[back, mu]) ** 2).sum(-2)) * norm[back // 2][:, None]
+    return out
+
+
+@pytest.mark.parametrize("dims,nrhs", FORMS)
+@pytest.mark.parametrize("kind", ["zero_naik", "zero_matrices", "small_direction", "small_matrices"])
+def test_accuracy_is_that_of_each_matrix(dims, nrhs, kind):
+    """Vectors far larger behind zero matrices, or seen through matrices far smaller than the others: every row
+    is known to within 96 * 2^-53 of the sizes of its own products (twice, with the reference's own rounding)."""
+    fat, lng = synth.gauge_field(dims, 0.3, 1087)
+    rng = np.random.default_rng(4)
+    psi = synth.random_spinor(dims, 79)
+    if kind == "zero_naik":  # a third of the sites far larger: three sites away they must not count
+        lng[:] = 0.0
+        psi *= np.where(rng.uniform(size=(len(psi), 1)) < 0.3, 2.0**40, 1.0)
+    elif kind == "zero_matrices":  # the links that leave every third site
+        lex = np.arange(len(fat))
+        fat[lex % 3 == 0] = 0.0
+        lng[lex % 3 == 0] = 0.0
+        psi *= 2.0 ** rng.integers(-30, 30, size=(len(psi), 1))
+    elif kind == "small_direction":
+        fat[:, 2] *= 2.0**-30
+        lng[:, 2] *= 2.0**-30
+        psi *= np.where(rng.uniform(size=(len(psi), 1)) < 0.01, 1.0, 0.0)
+    else:
+        scale = 2.0 ** rng.integers(-45, 45, size=(len(fat), 4, 1, 1))
+        fat, lng = fat * scale, lng * scale
+    got = _run(dims, fat, lng, np.stack([psi] * nrhs) if nrhs > 1 else psi, 0, nrhs).reshape(nrhs, -1, 3)
+    want = oracle.dslash(fat, lng, psi, dims, 0)
+    size = _sizes(dims, fat, lng, psi, 0)
+    for g in got:
+        assert (np.abs(g - want) <= 2 * BOUND * size).all(), (np.abs(g - want) / np.maximum(size, 1e-300)).max()
