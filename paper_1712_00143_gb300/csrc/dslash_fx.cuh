@@ -4,7 +4,7 @@
 // clock and SM take 2.8 times as long as its 2400 bytes take from HBM.  Here
 // the sixteen link-times-vector products run in the exact fixed-point
 // arithmetic of fx.cuh (81 wide integer multiply-adds per hop) and the
-// operator is bound by HBM again: 32^4, one half 217 us (0.87 of the copy
+// operator is bound by HBM again: 32^4, one half 216 us (0.87 of the copy
 // rate; integer pipe 45 % busy) against 522 us in FP64.
 //
 // Links: the handle's FP64 copy holds, in place of two doubles, {re.h, re.l,

@@ -226,10 +226,12 @@ template <class V2, class Link> STAG_FX void hop(Sums& S, const V2 (&psi)[3], in
     sh[c] = rh[c] + ih[c];
     sl[c] = rl[c] + il[c];
   }
-  // a row's cross sums: |rl|, |il| < 2^30 and |rh|, |ih| < 2^27, so |sl| < 2^31 and |sh| < 2^28
+  // a row's cross sums, in units of 2^-90 (their high words alone, 2^-58, made
+  // a single product less accurate than FP64's): |rl|, |il| < 2^30 and |rh|,
+  // |ih| < 2^27, so |sl| < 2^31 and |sh| < 2^28
   STAG_UNROLL
   for (int i = 0; i < 3; ++i) {
-    long long m1 = 0x80000000LL, m2 = m1, m3 = m1;
+    long long m1 = 1LL << 29, m2 = m1, m3 = m1;  // rounds them to 2^-60
     STAG_UNROLL
     for (int j = 0; j < 3; ++j) {
       const auto w = link(3 * i + j);
@@ -244,9 +246,9 @@ template <class V2, class Link> STAG_FX void hop(Sums& S, const V2 (&psi)[3], in
       fx::wmad(m3, th, sl[j]);
       fx::wmad(m3, tl, sh[j]);
     }
-    S.p[i][0] = fx::add64(S.p[i][0], (long long)(int)(m1 >> 32) * 4);
-    S.p[i][1] = fx::add64(S.p[i][1], (long long)(int)(m2 >> 32) * 4);
-    S.p[i][2] = fx::add64(S.p[i][2], (long long)(int)(m3 >> 32) * 4);
+    S.p[i][0] = fx::add64(S.p[i][0], m1 >> 30);
+    S.p[i][1] = fx::add64(S.p[i][1], m2 >> 30);
+    S.p[i][2] = fx::add64(S.p[i][2], m3 >> 30);
   }
 }
 

@@ -162,3 +162,47 @@ def test_not_finite_vectors_take_the_fp64_loop(steps):
     zero = np.zeros((16, 3, 3), dtype=complex)
     got = steps([(9999, zero, _gaussian(rng, 16, 3)), (9999, _gaussian(rng, 16, 3, 3), zero[:, 0])])
     assert all(g is None or (g == 0).all() for g in got)  # ("range" with nothing met: the caller stores zeros)
+
+
+def _su3(rng, n):
+    return np.linalg.qr(_gaussian(rng, n, 3, 3))[0]
+
+
+@pytest.mark.parametrize("kind", ["field", "equal hops", "point", "one component", "wide", "far large", "scaled"])
+def test_errors_are_no_larger_than_those_of_fp64_sums(steps, kind):
+    """Root mean square over 300 sites of the error against exact sums, this form's and that of one FP64
+    multiply-add after the other; 5 % for the sample (600 numbers or more: 3 % each)."""
+    rng = np.random.default_rng(17)
+    sites = []
+    for _ in range(300):
+        links, psi = 0.5 * _su3(rng, 16), _gaussian(rng, 16, 3)
+        if kind != "equal hops":
+            links.reshape(4, 4, 3, 3)[:, 2:] /= 24
+        if kind in ("point", "one component"):
+            keep = psi[rng.integers(16)].copy()
+            if kind == "one component":
+                keep[1:] = 0.0
+            psi[:] = 0.0
+            psi[rng.integers(16)] = keep
+        elif kind == "wide":
+            psi *= 10.0 ** rng.uniform(-6, 6, size=(16, 1))
+        elif kind == "far large":
+            psi.reshape(4, 4, 3)[:, 2:] *= 100
+        elif kind == "scaled":
+            links *= rng.uniform(0.2, 2, size=(16, 1, 1))
+        sites.append((9999, links, psi))
+    mine, fp64 = steps(sites), steps([(7777, w, v) for _, w, v in sites])
+    total = [0.0, 0.0]
+    for (_, links, psi), got in zip(sites, zip(mine, fp64)):
+        size = Fraction(float(_size(links, psi).max()))
+        for i in range(3):
+            re = im = Fraction(0)
+            for w, v in zip(links[:, i], psi):
+                for j in range(3):
+                    a, b, c, d = (Fraction(float(x)) for x in (w[j].real, w[j].imag, v[j].real, v[j].imag))
+                    re += a * c - b * d
+                    im += a * d + b * c
+            for k in range(2):
+                total[k] += float((Fraction(float(got[k][i].real)) - re) / size) ** 2
+                total[k] += float((Fraction(float(got[k][i].imag)) - im) / size) ** 2
+    assert math.sqrt(total[0]) <= 1.05 * math.sqrt(total[1]), math.sqrt(total[0] / total[1])
