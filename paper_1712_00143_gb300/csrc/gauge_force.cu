@@ -82,40 +82,45 @@ __device__ __forceinline__ M3 ldT(const double2* __restrict__ T, long long y, in
   return m;
 }
 
+// The scratch of a call starts with the status word and the count of marked links.
+struct Header {
+  int status;
+  unsigned long long marked;  // links whose force k_gauge_force_fx leaves to FP64
+};
+// The FP64 table kernels do the whole field when the integer kernels may not,
+// or have marked more links than the list holds.
+__device__ __forceinline__ bool all_fp64(const Header* h, long long cap) {
+  return !fx::usable(&h->status) || (long long)__ldcg(&h->marked) > cap;
+}
+
 // h(p, dir, sgn) without moving p
 __device__ __forceinline__ M3 hop_at(const double2* __restrict__ U, const Dims& d, Pos p, int dir, int sgn) {
   return hop_link(U, d, p, dir, sgn);
 }
 
-// FP64 form; it and k_gauge_force_reuse run only when the integer kernels may
-// not (*status), in grids of a few blocks per SM that return at once otherwise.
-__global__ void __launch_bounds__(128) k_gf_staples(Dims d, long long V, const double2* __restrict__ U,
-                                                    double2* __restrict__ T, const int* status) {
-  if (fx::usable(status)) return;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < 24 * V;
-       idx += (long long)gridDim.x * blockDim.x) {
-  const int k = (int)(idx / V);  // mu * 6 + (other direction index) * 2 + sign
-  const long long x = idx - (long long)k * V;
-  const int mu = k / 6, o = (k % 6) >> 1, s = (k & 1) ? -1 : 1;
-  const int nu = o < mu ? o : o + 1;
-  Pos p0;
-  p0.lex = x;
-  {
-    long long r = x;
-    p0.c.x = (int)(r % d.L0);
-    r /= d.L0;
-    p0.c.y = (int)(r % d.L1);
-    r /= d.L1;
-    p0.c.z = (int)(r % d.L2);
-    p0.c.t = (int)(r / d.L2);
-  }
-  Pos p = step(d, p0, mu, 1);  // walk [nu s, mu -, nu -s] from x + mu
+// T(p0; mu nu s) from the links: the walk [nu s, mu -, nu -s] from p0 + mu
+__device__ __forceinline__ M3 staple(const double2* __restrict__ U, const Dims& d, const Pos& p0, int mu, int nu, int s) {
+  Pos p = step(d, p0, mu, 1);
   M3 m = hop_link(U, d, p, nu, s);
   m = mul(m, hop_link(U, d, p, mu, -1));
-  m = mul(m, hop_link(U, d, p, nu, -s));
-  double2* out = T + tslot(x, mu, nu, s);
+  return mul(m, hop_link(U, d, p, nu, -s));
+}
+
+// FP64 form; it and k_gauge_force_reuse run only when the integer kernels do
+// not serve (all_fp64), in grids of a few blocks per SM that return at once otherwise.
+__global__ void __launch_bounds__(128) k_gf_staples(Dims d, long long V, const double2* __restrict__ U,
+                                                    double2* __restrict__ T, const Header* hd, long long cap) {
+  if (!all_fp64(hd, cap)) return;
+  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < 24 * V;
+       idx += (long long)gridDim.x * blockDim.x) {
+    const int k = (int)(idx / V);  // mu * 6 + (other direction index) * 2 + sign
+    const long long x = idx - (long long)k * V;
+    const int mu = k / 6, o = (k % 6) >> 1, s = (k & 1) ? -1 : 1;
+    const int nu = o < mu ? o : o + 1;
+    const M3 m = staple(U, d, pos_of(d, x), mu, nu, s);
+    double2* out = T + tslot(x, mu, nu, s);
 #pragma unroll
-  for (int i = 0; i < 9; ++i) out[i] = m.e[i];
+    for (int i = 0; i < 9; ++i) out[i] = m.e[i];
   }
 }
 
@@ -128,65 +133,47 @@ __device__ __forceinline__ void axpy3(M3& acc, double c, const M3& m) {
   }
 }
 
-__global__ void __launch_bounds__(128) k_gauge_force_reuse(Dims d, long long V, const double2* __restrict__ U,
-                                                           const double2* __restrict__ T, double2* __restrict__ F,
-                                                           double beta, double cpl, double crt, double cpg,
-                                                           const int* status) {
-  if (fx::usable(status)) return;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < 4 * V;
-       idx += (long long)gridDim.x * blockDim.x) {
-  const int mu = (int)(idx / V);
-  const long long x = idx - (long long)mu * V;
-  Pos p0;
-  p0.lex = x;
-  {
-    long long r = x;
-    p0.c.x = (int)(r % d.L0);
-    r /= d.L0;
-    p0.c.y = (int)(r % d.L1);
-    r /= d.L1;
-    p0.c.z = (int)(r % d.L2);
-    p0.c.t = (int)(r / d.L2);
-  }
+// S += the terms of (nu, s) for the link (p0, mu); staples from the table, or
+// from the links where there is none.
+template <bool TABLE>
+__device__ __forceinline__ void add_pair(M3& S, const double2* __restrict__ U, const double2* __restrict__ T, const Dims& d,
+                                         const Pos& p0, int mu, int nu, int s, double cpl, double crt, double cpg) {
+  auto at = [&](const Pos& p, int a, int b, int sign) {
+    if (TABLE) return ldT(T, p.lex, a, b, sign);
+    return staple(U, d, p, a, b, sign);
+  };
   const Pos pp = step(d, p0, mu, 1), pm = step(d, p0, mu, -1);  // x + mu, x - mu
-  const M3 u_pm = ld(U, pp.lex, mu), u_mm = ld(U, pm.lex, mu);  // U_mu(x+mu), U_mu(x-mu)
-  M3 S;
+  const M3 t0 = at(p0, mu, nu, s);
+  axpy3(S, cpl, t0);                                                    // plaquette
+  axpy3(S, crt, mul(ld(U, pp.lex, mu), mul(at(pp, mu, nu, s), t0)));  // rectangle 1
+  axpy3(S, crt, mul(mul(t0, at(pm, mu, nu, s)), ld(U, pm.lex, mu)));  // rectangle 2
+  // rectangle 3 and the parallelograms share the left factor h(x+mu, nu, s)
+  const Pos ps = step(d, p0, nu, s);  // x + s nu
+  M3 R = mul(at(ps, mu, nu, s), hop_at(U, d, ps, nu, -s));
 #pragma unroll
-  for (int i = 0; i < 9; ++i) S.e[i] = make_double2(0.0, 0.0);
-#pragma unroll 1
-  for (int nu = 0; nu < 4; ++nu) {
-    if (nu == mu) continue;
-#pragma unroll 1
-    for (int s = -1; s <= 1; s += 2) {
-      const M3 t0 = ldT(T, x, mu, nu, s);
-      axpy3(S, cpl, t0);                                          // plaquette
-      axpy3(S, crt, mul(u_pm, mul(ldT(T, pp.lex, mu, nu, s), t0)));  // rectangle 1
-      axpy3(S, crt, mul(mul(t0, ldT(T, pm.lex, mu, nu, s)), u_mm));  // rectangle 2
-      // rectangle 3 and the parallelograms share the left factor h(x+mu, nu, s)
-      const Pos ps = step(d, p0, nu, s);  // x + s nu
-      M3 R = mul(ldT(T, ps.lex, mu, nu, s), hop_at(U, d, ps, nu, -s));
-#pragma unroll
-      for (int i = 0; i < 9; ++i) {
-        R.e[i].x *= crt;
-        R.e[i].y *= crt;
-      }
-      const Pos pmn = step(d, p0, nu, -1);  // x - nu (for s = -1)
-#pragma unroll 1
-      for (int rho = 0; rho < 4; ++rho) {
-        if (rho == mu || rho == nu) continue;
-#pragma unroll 1
-        for (int r = -1; r <= 1; r += 2) {
-          const M3 a = ldT(T, ps.lex, mu, rho, r);
-          M3 q = s > 0 ? ldT(T, x, nu, rho, r) : dagger(ldT(T, pmn.lex, nu, rho, r));
-          const M3 aq = mul(a, q);
-          axpy3(R, cpg, aq);
-        }
-      }
-      const M3 hl = hop_at(U, d, pp, nu, s);
-      const M3 hr = mul(hl, R);
-      axpy3(S, 1.0, hr);
-    }
+  for (int i = 0; i < 9; ++i) {
+    R.e[i].x *= crt;
+    R.e[i].y *= crt;
   }
+  const Pos pq = s > 0 ? p0 : step(d, p0, nu, -1);  // x, or x - nu
+  const int lo = nu < mu ? nu : mu, hi = nu < mu ? mu : nu;
+#pragma unroll 1
+  for (int j = 0; j < 4; ++j) {  // (rho, r): the two directions other than mu and nu, both signs
+    int rho = j >> 1;
+    const int r = (j & 1) ? 1 : -1;
+    rho += rho >= lo ? 1 : 0;
+    rho += rho >= hi ? 1 : 0;
+    const M3 a = at(ps, mu, rho, r);
+    M3 q = at(pq, nu, rho, r);
+    if (s < 0) q = dagger(q);
+    axpy3(R, cpg, mul(a, q));
+  }
+  axpy3(S, 1.0, mul(hop_at(U, d, pp, nu, s), R));
+}
+
+// F_mu(x) = (beta/3) TA[U_mu(x) S]
+__device__ __forceinline__ void store_force(const double2* __restrict__ U, double2* __restrict__ F, long long x, int mu,
+                                            const M3& S, double beta) {
   const M3 us = mul(ld(U, x, mu), S);
   M3 a;
 #pragma unroll
@@ -203,6 +190,54 @@ __global__ void __launch_bounds__(128) k_gauge_force_reuse(Dims d, long long V, 
 #pragma unroll
     for (int j = 0; j < 3; ++j)
       f[3 * i + j] = make_double2(k * a.e[3 * i + j].x, k * (a.e[3 * i + j].y - (i == j ? tr3 : 0.0)));
+}
+
+__global__ void __launch_bounds__(128) k_gauge_force_reuse(Dims d, long long V, const double2* __restrict__ U,
+                                                           const double2* __restrict__ T, double2* __restrict__ F,
+                                                           double beta, double cpl, double crt, double cpg,
+                                                           const Header* hd, long long cap) {
+  if (!all_fp64(hd, cap)) return;
+  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < 4 * V;
+       idx += (long long)gridDim.x * blockDim.x) {
+    const int mu = (int)(idx / V);
+    const long long x = idx - (long long)mu * V;
+    const Pos p0 = pos_of(d, x);
+    M3 S = zero3();
+#pragma unroll 1
+    for (int nu = 0; nu < 4; ++nu) {
+      if (nu == mu) continue;
+#pragma unroll 1
+      for (int s = -1; s <= 1; s += 2) add_pair<true>(S, U, T, d, p0, mu, nu, s, cpl, crt, cpg);
+    }
+    store_force(U, F, x, mu, S, beta);
+  }
+}
+
+// The links that k_gauge_force_fx has marked (its header says which), in FP64
+// without a table: eight lanes per link, six of which take one (nu, s) each --
+// 34 products of a chain of 204, which one thread would take 0.6 ms for.
+__global__ void __launch_bounds__(128) k_gauge_force_marked(Dims d, const double2* __restrict__ U,
+                                                            const long long* __restrict__ list, double2* __restrict__ F,
+                                                            double beta, double cpl, double crt, double cpg,
+                                                            const Header* hd, long long cap) {
+  if (all_fp64(hd, cap)) return;
+  const long long n = (long long)__ldcg(&hd->marked);
+  const int o = threadIdx.x & 7, per = gridDim.x * 16;
+  for (long long i0 = blockIdx.x * 16 + (threadIdx.x >> 5) * 4; i0 < n; i0 += per) {  // (a warp's four links)
+    const long long i = i0 + ((threadIdx.x & 31) >> 3);
+    const bool in = i < n;
+    const long long at = in ? __ldcg(list + i) : 0, x = at >> 2;
+    const int mu = (int)(at & 3), q = o >> 1, nu = q < mu ? q : q + 1;
+    M3 S = zero3();
+    if (in && o < 6) add_pair<false>(S, U, nullptr, d, pos_of(d, x), mu, nu, (o & 1) ? 1 : -1, cpl, crt, cpg);
+#pragma unroll
+    for (int w = 1; w < 8; w <<= 1)
+#pragma unroll
+      for (int e = 0; e < 9; ++e) {
+        S.e[e].x += __shfl_down_sync(0xffffffffu, S.e[e].x, w, 8);
+        S.e[e].y += __shfl_down_sync(0xffffffffu, S.e[e].y, w, 8);
+      }
+    if (in && o == 0) store_force(U, F, x, mu, S, beta);
   }
 }
 
@@ -257,14 +292,23 @@ __global__ void __launch_bounds__(128, 3) k_gf_staples_fx(Dims d, long long V, i
 // the rest additions, address arithmetic and dependences at three warps per scheduler.
 // 24^4: conversion 0.07, table 0.68, force 3.5 ms; the call 4.2 ms against
 // 21.3 ms with the FP64 kernels.
+// Accuracy: about 2^-57 of the coefficients' size, whatever the force.  FP64
+// sums do better where they keep the relative accuracy of a small force: around
+// a link close to a diagonal matrix of 1, -1, i and -i, whose products are
+// exact.  So where a link lies within 3 2^-5 of such a matrix, and the
+// off-diagonal entries and the force in U S below 3 2^-6 of the coefficients'
+// size, the link is marked and done again in FP64.  (Links exp(i eps H), rms
+// error of the force in FP64 and here: eps = 0.08 1.8e-16 and 1.5e-16, eps =
+// 0.04 1.7e-16 and 2.4e-16, eps = 0.005 1.8e-16 and 1.8e-15; the rule marks 3,
+// 70 and 100 % of the links, and none at eps = 0.3.)
 struct ForceCoef {
   fx::Coef pl8, rt8, rt, pg4;  // 8 c_pl, 8 c_rt, c_rt, 4 c_pg, each times 2^-k
   double off, diag;            // beta/3 times 2^(k-60) / 2 and / 3
 };
 __global__ void __launch_bounds__(128, 3) k_gauge_force_fx(Dims d, long long V, const int4* __restrict__ T,
-                                                           const int* __restrict__ status, double2* __restrict__ F,
-                                                           ForceCoef cf) {
-  if (!fx::usable(status)) return;
+                                                           Header* hd, long long* __restrict__ list, long long cap,
+                                                           double2* __restrict__ F, ForceCoef cf) {
+  if (!fx::usable(&hd->status)) return;
   extern __shared__ __align__(16) unsigned char gf_sm[];
   long long(*S)[128] = (long long(*)[128])gf_sm;  // [18][128]
   long long(*lone)[128] = S + 18;                  // a group's rectangle 3
@@ -385,16 +429,28 @@ __global__ void __launch_bounds__(128, 3) k_gauge_force_fx(Dims d, long long V, 
     fx::FM s;
 #pragma unroll
     for (int e = 0; e < 18; ++e) fx::split1(S[e][tid], s.h[e], s.l[e]);
+    const fx::FM u = fx::ld<SLOTS>(T, U0 + mu, x);
     long long w[18];
     fx::clear(w);
-    fx::mac(w, fx::ld<SLOTS>(T, U0 + mu, x), s);
+    fx::mac(w, u, s);
     const long long tr = w[1] + w[9] + w[17];
+    long long size = 0;  // the largest off-diagonal entry, and
+    int away = 0;        // the link's distance from the diagonal matrices of 1, -1, i, -i
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      dg[i] = cf.diag * fx::double_of(3 * w[8 * i + 1] - tr, 0);
+      const long long di = 3 * w[8 * i + 1] - tr;
+      dg[i] = cf.diag * fx::double_of(di, 0);
       const int r = i == 2 ? 1 : 0, c = i == 0 ? 1 : 2;  // entries 01, 02, 12
       const int e = 2 * (3 * r + c), f = 2 * (3 * c + r);
       off[i] = make_double2(cf.off * fx::double_of(w[e] - w[f], 0), cf.off * fx::double_of(w[e + 1] + w[f + 1], 0));
+      size = max(size, max(max(llabs(w[e]), llabs(w[e + 1])), max(llabs(w[f]), llabs(w[f + 1]))));
+      size = max(size, llabs(di) >> 1);  // (a third of it is the force's)
+      away = max(away, max(max(abs(u.h[e]), abs(u.h[e + 1])), max(abs(u.h[f]), abs(u.h[f + 1]))));
+      away = max(away, min(abs(u.h[8 * i]), abs(u.h[8 * i + 1])));
+    }
+    if (away < 3 << 25 && size < 3LL << 54) {
+      const unsigned long long n = atomicAdd(&hd->marked, 1ull);
+      if ((long long)n < cap) list[n] = 4LL * x + mu;
     }
   }
   __syncthreads();  // the sums' memory becomes the output's
@@ -432,24 +488,27 @@ extern "C" int stag_gauge_force(const int dims[4], const void* thin, void* force
   const su3::Dims d{dims[0], dims[1], dims[2], dims[3]};
   cudaStream_t st = (cudaStream_t)stream;
   // stream-ordered scratch: the FP64 staple table (24 of 32 matrix slots per
-  // site, 4608 B) or the fixed-point field (28 matrices, 4032 B), whichever
-  // form runs
+  // site, 4608 B), or the fixed-point field (28 matrices, 4032 B) and the list of
+  // marked links (up to one in 64), whichever form runs
+  const long long cap = V / 16;
   const size_t tbytes = (size_t)V * 32 * 9 * sizeof(double2), fbytes = fx::field_bytes(V, gf::SLOTS);
+  const size_t lbytes = fbytes + (size_t)cap * sizeof(long long);
   char* scratch = nullptr;
-  if (cudaMallocAsync((void**)&scratch, 256 + (tbytes > fbytes ? tbytes : fbytes), st) != cudaSuccess) {
+  if (cudaMallocAsync((void**)&scratch, 256 + (tbytes > lbytes ? tbytes : lbytes), st) != cudaSuccess) {
     cudaGetLastError();
     return STAG_ENOMEM;
   }
-  int* status = (int*)scratch;
+  gf::Header* hd = (gf::Header*)scratch;
   double2* T = (double2*)(scratch + 256);
   int4* Tf = (int4*)(scratch + 256);
+  long long* list = (long long*)(scratch + 256 + fbytes);
   const double2* U = (const double2*)thin;
   // coefficients with a power of two taken out (see k_gauge_force_fx); beyond
   // 2^+-900, or not finite, the FP64 kernels, whose range is wider
   const double big = std::fabs(c_pl) * 6 + std::fabs(c_rt) * 18 + std::fabs(c_pg) * 24;
   const bool fixed = big > 0x1p-900 && big < 0x1p900 && std::fabs(beta) < 0x1p60;
-  int s = STAG_OK;
-  if (fixed) {
+  int s = cuda_status(cudaMemsetAsync(hd, 0, sizeof(*hd), st));
+  if (fixed && !s) {
     int k = 0;
     std::frexp(big, &k);
     gf::ForceCoef cf;
@@ -462,35 +521,40 @@ extern "C" int stag_gauge_force(const int dims[4], const void* thin, void* force
     const unsigned tiles = (unsigned)((V + fx::TS - 1) / fx::TS);
     {
       ProfScope ps("gauge_force", st);
-      s = fx::launch_fx_links(V, U, Tf, gf::SLOTS, gf::U0, status, st);
+      s = fx::launch_fx_links(V, U, Tf, gf::SLOTS, gf::U0, &hd->status, st);
     }
     if (!s) {
       ProfScope ps("gauge_force", st);
-      gf::k_gf_staples_fx<<<tiles, 128, 0, st>>>(d, V, Tf, status);
+      gf::k_gf_staples_fx<<<tiles, 128, 0, st>>>(d, V, Tf, &hd->status);
       s = last_launch_status();
     }
     if (!s) {
       ProfScope ps("gauge_force", st);
       constexpr int smem = 4 * 18 * 128 * sizeof(long long);  // 72 KB, three blocks per SM
       s = cuda_status(cudaFuncSetAttribute(gf::k_gauge_force_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-      if (!s) gf::k_gauge_force_fx<<<tiles, 128, smem, st>>>(d, V, Tf, status, (double2*)force, cf);
+      if (!s) gf::k_gauge_force_fx<<<tiles, 128, smem, st>>>(d, V, Tf, hd, list, cap, (double2*)force, cf);
       if (!s) s = last_launch_status();
     }
-  } else {
-    s = cuda_status(cudaMemsetAsync(status, 0, sizeof(int), st));
+    if (!s) {
+      ProfScope ps("gauge_force", st);
+      const long long want = (cap + 15) / 16;
+      gf::k_gauge_force_marked<<<(unsigned)(want < 152 * 4 ? want : 152 * 4), 128, 0, st>>>(d, U, list, (double2*)force, beta,
+                                                                                         c_pl, c_rt, c_pg, hd, cap);
+      s = last_launch_status();
+    }
   }
   const unsigned few = 152 * 8;
   if (!s) {
     ProfScope ps("gauge_force", st);
     const long long n = (24 * V + 127) / 128;
-    gf::k_gf_staples<<<(unsigned)(fixed && n > few ? few : n), 128, 0, st>>>(d, V, U, T, status);
+    gf::k_gf_staples<<<(unsigned)(fixed && n > few ? few : n), 128, 0, st>>>(d, V, U, T, hd, cap);
     s = last_launch_status();
   }
   if (!s) {
     ProfScope ps("gauge_force", st);
     const long long n = (4 * V + 127) / 128;
     gf::k_gauge_force_reuse<<<(unsigned)(fixed && n > few ? few : n), 128, 0, st>>>(d, V, U, T, (double2*)force, beta, c_pl,
-                                                                                   c_rt, c_pg, status);
+                                                                                   c_rt, c_pg, hd, cap);
     s = last_launch_status();
   }
   const int f = cuda_status(cudaFreeAsync(scratch, st));

@@ -1,0 +1,58 @@
+"""The gauge force on lattices that are ordinary in one part and near the unit matrix (or minus it) in
+another: the small force there keeps FP64's relative accuracy, whether the part is most of the lattice (the
+FP64 kernels then do all of it) or a few links (done one by one)."""
+
+import numpy as np
+import pytest
+import torch
+
+import oracle.gauge_force as ogf
+import synth
+from gpu_common import dev, requires_gpu
+
+pytestmark = [pytest.mark.gpu, requires_gpu]
+
+COEF = (1.0, -0.083, -0.008)
+
+
+def _mixed(dims, eps, inside, seed):
+    """Thin links, near 1 where `inside` (a mask of sites) holds."""
+    thin = synth.gauge_field(dims, 0.3, seed, return_thin=True)[2].copy()
+    thin[inside] = synth.gauge_field(dims, eps, seed + 1, return_thin=True)[2][inside]
+    return thin
+
+
+def _coords(dims):
+    lex = np.arange(np.prod(dims))
+    return np.stack(np.unravel_index(lex, dims[::-1])[::-1], axis=-1)
+
+
+def _interior(dims, inside):
+    """Sites all of whose loops' links lie inside: every site within two steps (and their links' far ends)."""
+    grid = inside.reshape(dims[::-1])
+    for axis in range(4):
+        grid = np.all([np.roll(grid, k, axis) for k in range(-3, 3)], axis=0)
+    return grid.reshape(-1)
+
+
+@pytest.mark.parametrize("eps", [1e-6, 1e-3, 0.02])
+@pytest.mark.parametrize("shape", ["slab", "box"])
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+def test_small_forces_in_part_of_a_lattice(eps, shape, sign):
+    import paper_1712_00143_gb300 as stag
+
+    dims = (4, 4, 4, 12) if shape == "slab" else (8, 8, 10, 10)
+    c = _coords(dims)
+    inside = c[:, 3] >= 3 if shape == "slab" else (c < 6).all(axis=1)
+    thin = _mixed(dims, eps, inside, 1100)
+    if sign < 0:  # antiperiodic in t
+        thin[c[:, 3] == (7 if shape == "slab" else 3), 3] *= -1.0
+    F = stag.stag_gauge_force(dims, dev(thin), 6.0, *COEF)
+    torch.cuda.synchronize()
+    F, want = F.cpu().numpy(), ogf.force(thin, dims, 6.0, *COEF)
+    terms = 2.0 * (6 + 18 * 0.083 + 24 * 0.008)
+    assert np.abs(F - want).max() <= 4e-15 * terms
+    deep = _interior(dims, inside)
+    assert deep.any() and np.abs(want[deep]).max() < 10 * terms * eps
+    # FP64 sums of such links are off by a few 2^-53 of the largest of their own terms, which are of the force's size
+    assert np.linalg.norm((F - want)[deep]) <= 1e-14 * np.linalg.norm(want[deep])
