@@ -24,12 +24,12 @@ __global__ void __launch_bounds__(128) k_fx_links(long long V, const double2* __
 #pragma unroll
     for (int e = 0; e < 9; ++e) {
       const double2 u = sm[s * SITE_W + mu * 9 + e];
-      // exponents of 2 and above (infinity and NaN among them) are out of fixed60's range
+      // exponents of 2 and above (infinity and NaN among them) are out of range
       const int ex = max(__double2hiint(u.x) & 0x7fffffff, __double2hiint(u.y) & 0x7fffffff);
       if (ex >= 0x40000000) flags |= FX_NOT_UNITARY;
       int4 q;
-      split1(fixed60(u.x), q.x, q.y);
-      split1(fixed60(u.y), q.z, q.w);
+      fxd::fixed_entry(u.x, 0, q.x, q.y);
+      fxd::fixed_entry(u.y, 0, q.z, q.w);
       o[e * 32] = q;
       f[e] = make_float2((float)q.x * 0x1p-30f, (float)q.z * 0x1p-30f);
     }

@@ -103,15 +103,7 @@ __device__ __forceinline__ void clear(long long (&s)[18]) {
   for (int i = 0; i < 18; ++i) s[i] = 0;
 }
 
-// ------------------------------------------------------------ conversions (no FP64 instruction)
-// v 2^60 (|v| < 2, truncated towards zero)
-__device__ __forceinline__ long long fixed60(double v) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-  const int r = 1023 - (int)((b >> 52) & 0x7ff);
-  const unsigned long long m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 8;  // 1.f at 2^60
-  const long long q = (long long)(m >> (r > 63 ? 63 : r));
-  return (long long)b < 0 ? -q : q;
-}
+// ------------------------------------------------------------ coefficients
 // A coefficient |c| <= 1 in the same form, and c s for |s| <= 2^60.
 struct Coef {
   int h, l;
@@ -259,6 +251,22 @@ enum : int { FX_NOT_UNITARY = 1, FX_AWAY = 2, FX_RANGE = 4 };
 // matrix stay on the FP64 kernels: their small entries, and a force made of
 // them, would be known to 2^-58 absolute where FP64 keeps 2^-53 relative.
 __device__ __forceinline__ bool usable(const int* status) { return __ldcg(status) == FX_AWAY; }
+
+// What a call's scratch starts with where the integer kernels may leave single
+// results to the FP64 ones: the status word, and the count of those marked.
+struct Header {
+  int status;
+  unsigned long long marked;
+};
+__device__ __forceinline__ void mark(Header* hd, long long* __restrict__ list, long long cap, long long item) {
+  const unsigned long long n = atomicAdd(&hd->marked, 1ull);
+  if ((long long)n < cap) list[n] = item;
+}
+// The FP64 kernels do the whole field when the integer kernels may not, or have
+// marked more results than the list holds.
+__device__ __forceinline__ bool all_fp64(const Header* hd, long long cap) {
+  return !usable(&hd->status) || (long long)__ldcg(&hd->marked) > cap;
+}
 
 // Fixed-point copy of the thin links [V][4][3][3] into slots slot0 + mu of a
 // field with `slots` slots, and *status (fx.cu).

@@ -82,17 +82,6 @@ __device__ __forceinline__ M3 ldT(const double2* __restrict__ T, long long y, in
   return m;
 }
 
-// The scratch of a call starts with the status word and the count of marked links.
-struct Header {
-  int status;
-  unsigned long long marked;  // links whose force k_gauge_force_fx leaves to FP64
-};
-// The FP64 table kernels do the whole field when the integer kernels may not,
-// or have marked more links than the list holds.
-__device__ __forceinline__ bool all_fp64(const Header* h, long long cap) {
-  return !fx::usable(&h->status) || (long long)__ldcg(&h->marked) > cap;
-}
-
 // h(p, dir, sgn) without moving p
 __device__ __forceinline__ M3 hop_at(const double2* __restrict__ U, const Dims& d, Pos p, int dir, int sgn) {
   return hop_link(U, d, p, dir, sgn);
@@ -107,10 +96,10 @@ __device__ __forceinline__ M3 staple(const double2* __restrict__ U, const Dims& 
 }
 
 // FP64 form; it and k_gauge_force_reuse run only when the integer kernels do
-// not serve (all_fp64), in grids of a few blocks per SM that return at once otherwise.
+// not serve (fx::all_fp64), in grids of a few blocks per SM that return at once otherwise.
 __global__ void __launch_bounds__(128) k_gf_staples(Dims d, long long V, const double2* __restrict__ U,
-                                                    double2* __restrict__ T, const Header* hd, long long cap) {
-  if (!all_fp64(hd, cap)) return;
+                                                    double2* __restrict__ T, const fx::Header* hd, long long cap) {
+  if (!fx::all_fp64(hd, cap)) return;
   for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < 24 * V;
        idx += (long long)gridDim.x * blockDim.x) {
     const int k = (int)(idx / V);  // mu * 6 + (other direction index) * 2 + sign
@@ -195,8 +184,8 @@ __device__ __forceinline__ void store_force(const double2* __restrict__ U, doubl
 __global__ void __launch_bounds__(128) k_gauge_force_reuse(Dims d, long long V, const double2* __restrict__ U,
                                                            const double2* __restrict__ T, double2* __restrict__ F,
                                                            double beta, double cpl, double crt, double cpg,
-                                                           const Header* hd, long long cap) {
-  if (!all_fp64(hd, cap)) return;
+                                                           const fx::Header* hd, long long cap) {
+  if (!fx::all_fp64(hd, cap)) return;
   for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < 4 * V;
        idx += (long long)gridDim.x * blockDim.x) {
     const int mu = (int)(idx / V);
@@ -219,8 +208,8 @@ __global__ void __launch_bounds__(128) k_gauge_force_reuse(Dims d, long long V, 
 __global__ void __launch_bounds__(128) k_gauge_force_marked(Dims d, const double2* __restrict__ U,
                                                             const long long* __restrict__ list, double2* __restrict__ F,
                                                             double beta, double cpl, double crt, double cpg,
-                                                            const Header* hd, long long cap) {
-  if (all_fp64(hd, cap)) return;
+                                                            const fx::Header* hd, long long cap) {
+  if (fx::all_fp64(hd, cap)) return;
   const long long n = (long long)__ldcg(&hd->marked);
   const int o = threadIdx.x & 7, per = gridDim.x * 16;
   for (long long i0 = blockIdx.x * 16 + (threadIdx.x >> 5) * 4; i0 < n; i0 += per) {  // (a warp's four links)
@@ -306,7 +295,7 @@ struct ForceCoef {
   double off, diag;            // beta/3 times 2^(k-60) / 2 and / 3
 };
 __global__ void __launch_bounds__(128, 3) k_gauge_force_fx(Dims d, long long V, const int4* __restrict__ T,
-                                                           Header* hd, long long* __restrict__ list, long long cap,
+                                                           fx::Header* hd, long long* __restrict__ list, long long cap,
                                                            double2* __restrict__ F, ForceCoef cf) {
   if (!fx::usable(&hd->status)) return;
   extern __shared__ __align__(16) unsigned char gf_sm[];
@@ -448,10 +437,7 @@ __global__ void __launch_bounds__(128, 3) k_gauge_force_fx(Dims d, long long V, 
       away = max(away, max(max(abs(u.h[e]), abs(u.h[e + 1])), max(abs(u.h[f]), abs(u.h[f + 1]))));
       away = max(away, min(abs(u.h[8 * i]), abs(u.h[8 * i + 1])));
     }
-    if (away < 3 << 25 && size < 3LL << 54) {
-      const unsigned long long n = atomicAdd(&hd->marked, 1ull);
-      if ((long long)n < cap) list[n] = 4LL * x + mu;
-    }
+    if (away < 3 << 25 && size < 3LL << 54) fx::mark(hd, list, cap, 4LL * x + mu);
   }
   __syncthreads();  // the sums' memory becomes the output's
   if (lane < ns) {
@@ -498,7 +484,7 @@ extern "C" int stag_gauge_force(const int dims[4], const void* thin, void* force
     cudaGetLastError();
     return STAG_ENOMEM;
   }
-  gf::Header* hd = (gf::Header*)scratch;
+  fx::Header* hd = (fx::Header*)scratch;
   double2* T = (double2*)(scratch + 256);
   int4* Tf = (int4*)(scratch + 256);
   long long* list = (long long*)(scratch + 256 + fbytes);

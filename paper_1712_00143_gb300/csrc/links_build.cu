@@ -21,63 +21,74 @@ namespace stag {
 namespace lb {
 using namespace su3;
 
-// FP64 form: bound by the FP64 pipe (10.8 ms at 32^4, 1.2 TFLOP/s).  With a
-// status word it runs only when the integer kernel may not, in a grid of a
-// few blocks per SM whose blocks return at once otherwise.
-__global__ void __launch_bounds__(128) k_build_links(Dims d, long long V, const double2* __restrict__ U,
-                                                     double2* __restrict__ F, double2* __restrict__ Lk, double c1,
-                                                     double cst, double c3, const int* status) {
-  if (status && fx::usable(status)) return;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < 4 * V;
-       idx += (long long)gridDim.x * blockDim.x) {
-  const int mu = (int)(idx / V);
-  const long long x = idx - (long long)mu * V;
-  C4 c;
-  {
-    long long r = x;
-    c.x = (int)(r % d.L0);
-    r /= d.L0;
-    c.y = (int)(r % d.L1);
-    r /= d.L1;
-    c.z = (int)(r % d.L2);
-    c.t = (int)(r / d.L2);
-  }
-  const long long x_pmu = shifted(d, x, c, mu, 1);
-  M3 S;
-#pragma unroll
-  for (int i = 0; i < 9; ++i) S.e[i] = make_double2(0.0, 0.0);
+// F_mu(x) in FP64
+__device__ __forceinline__ M3 fat_link(const Dims& d, const double2* __restrict__ U, const Pos& p, int mu, double c1,
+                                       double cst) {
+  const Pos pm = step(d, p, mu, 1);
+  M3 S = zero3();
 #pragma unroll 1
   for (int nu = 0; nu < 4; ++nu) {
     if (nu == mu) continue;
     // upper staple U_nu(x) U_mu(x+nu) U_nu(x+mu)^dag
     {
-      const M3 ab = mul(ld(U, x, nu), ld(U, shifted(d, x, c, nu, 1), mu));
-      mac_mul_dag(S, ab, ld(U, x_pmu, nu));
+      const M3 ab = mul(ld(U, p.lex, nu), ld(U, shifted(d, p.lex, p.c, nu, 1), mu));
+      mac_mul_dag(S, ab, ld(U, pm.lex, nu));
     }
-    // lower staple U_nu(x-nu)^dag U_mu(x-nu) U_nu(x-nu+mu): x - nu + mu is
-    // x + mu moved by -nu (mu != nu)
+    // lower staple U_nu(x-nu)^dag U_mu(x-nu) U_nu(x-nu+mu)
     {
-      const long long x_mnu = shifted(d, x, c, nu, -1);
-      C4 cp = c;  // coordinates of x + mu
-      const int Lm = extent(d, mu), vm = c.get(mu) + 1 == Lm ? 0 : c.get(mu) + 1;
-      cp.x = mu == 0 ? vm : cp.x;
-      cp.y = mu == 1 ? vm : cp.y;
-      cp.z = mu == 2 ? vm : cp.z;
-      cp.t = mu == 3 ? vm : cp.t;
+      const long long x_mnu = shifted(d, p.lex, p.c, nu, -1);
       const M3 ab = dag_mul(ld(U, x_mnu, nu), ld(U, x_mnu, mu));
-      mac_mul(S, ab, ld(U, shifted(d, x_pmu, cp, nu, -1), nu));
+      mac_mul(S, ab, ld(U, shifted(d, pm.lex, pm.c, nu, -1), nu));
     }
   }
-  const M3 u = ld(U, x, mu);
-  double2* f = F + (x * 4 + mu) * 9;
+  const M3 u = ld(U, p.lex, mu);
 #pragma unroll
-  for (int i = 0; i < 9; ++i) f[i] = make_double2(c1 * u.e[i].x + cst * S.e[i].x, c1 * u.e[i].y + cst * S.e[i].y);
-  // Naik: c3 U_mu(x) U_mu(x+mu) U_mu(x+2mu)
-  const M3 uu = mul(u, ld(U, x_pmu, mu));
-  const M3 l3 = mul(uu, ld(U, shifted(d, x, c, mu, 2), mu));
-  double2* l = Lk + (x * 4 + mu) * 9;
+  for (int i = 0; i < 9; ++i) S.e[i] = make_double2(c1 * u.e[i].x + cst * S.e[i].x, c1 * u.e[i].y + cst * S.e[i].y);
+  return S;
+}
+// L_mu(x) = c3 U_mu(x) U_mu(x+mu) U_mu(x+2mu) in FP64
+__device__ __forceinline__ M3 naik_link(const Dims& d, const double2* __restrict__ U, const Pos& p, int mu, double c3) {
+  const M3 uu = mul(ld(U, p.lex, mu), ld(U, shifted(d, p.lex, p.c, mu, 1), mu));
+  M3 l = mul(uu, ld(U, shifted(d, p.lex, p.c, mu, 2), mu));
 #pragma unroll
-  for (int i = 0; i < 9; ++i) l[i] = make_double2(c3 * l3.e[i].x, c3 * l3.e[i].y);
+  for (int i = 0; i < 9; ++i) l.e[i] = make_double2(c3 * l.e[i].x, c3 * l.e[i].y);
+  return l;
+}
+__device__ __forceinline__ void st(double2* __restrict__ out, long long link, const M3& m) {
+#pragma unroll
+  for (int i = 0; i < 9; ++i) out[link * 9 + i] = m.e[i];
+}
+
+// FP64 form: bound by the FP64 pipe (10.8 ms at 32^4, 1.2 TFLOP/s).  With a
+// header it runs only when the integer kernels do not serve, in a grid of a few
+// blocks per SM whose blocks return at once otherwise.
+__global__ void __launch_bounds__(128) k_build_links(Dims d, long long V, const double2* __restrict__ U,
+                                                     double2* __restrict__ F, double2* __restrict__ Lk, double c1,
+                                                     double cst, double c3, const fx::Header* hd, long long cap) {
+  if (hd && !fx::all_fp64(hd, cap)) return;
+  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < 4 * V;
+       idx += (long long)gridDim.x * blockDim.x) {
+    const int mu = (int)(idx / V);
+    const Pos p = pos_of(d, idx - (long long)mu * V);
+    st(F, p.lex * 4 + mu, fat_link(d, U, p, mu, c1, cst));
+    st(Lk, p.lex * 4 + mu, naik_link(d, U, p, mu, c3));
+  }
+}
+// The fat and Naik links that k_build_links_fx has marked, one thread each.
+__global__ void __launch_bounds__(128) k_build_marked(Dims d, const double2* __restrict__ U,
+                                                      const long long* __restrict__ list, double2* __restrict__ F,
+                                                      double2* __restrict__ Lk, double c1, double cst, double c3,
+                                                      const fx::Header* hd, long long cap) {
+  if (fx::all_fp64(hd, cap)) return;
+  const long long n = (long long)__ldcg(&hd->marked);
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const long long at = __ldcg(list + i), link = at >> 1;
+    const int mu = (int)(link & 3);
+    const Pos p = pos_of(d, link >> 2);
+    if (at & 1)
+      st(Lk, link, naik_link(d, U, p, mu, c3));
+    else
+      st(F, link, fat_link(d, U, p, mu, c1, cst));
   }
 }
 
@@ -90,12 +101,20 @@ __global__ void __launch_bounds__(128) k_build_links(Dims d, long long V, const 
 // FP64 instructions at the end would cost a tenth of the whole kernel.  Bound
 // by the integer pipe (65 % busy with two blocks per SM; three or four blocks
 // measured the same).  24^4: conversion 0.06, fat 0.84, Naik 0.17 ms; the call
-// at 32^4 3.42 ms against 10.84 ms with the FP64 kernel.
+// at 32^4 3.46 ms against 10.84 ms with the FP64 kernel.
+// Accuracy: half of FP64's error in every matrix's norm.  FP64 does better on
+// small off-diagonal entries, which it knows to their own size where the links
+// are close to a diagonal matrix; so where the link lies within 3 2^-6 of a
+// diagonal matrix of 1, -1, i, -i and the result's off-diagonal entries are
+// below 3 2^-7 (of the larger coefficient), the result is marked and done again
+// in FP64.  (Off-diagonal entries of fat links from exp(i eps H), rms error in
+// FP64 and here: eps = 0.04 1.2e-16 and 1.0e-16, eps = 0.02 1.1e-16 and 2.0e-16,
+// eps = 0.005 1.1e-16 and 7.7e-16.)
 template <bool FAT>
 __global__ void __launch_bounds__(128, FAT ? 2 : 3) k_build_links_fx(Dims d, long long V, const int4* __restrict__ U,
-                                                        const int* __restrict__ status, double2* __restrict__ out,
-                                                        fx::Coef c1, fx::Coef cst, int k) {
-  if (!fx::usable(status)) return;
+                                                        fx::Header* hd, long long* __restrict__ list, long long cap,
+                                                        double2* __restrict__ out, fx::Coef c1, fx::Coef cst, int k) {
+  if (!fx::usable(&hd->status)) return;
   __shared__ double2 sm[fx::TS * fx::SITE_W];
   const long long x0 = (long long)blockIdx.x * fx::TS;
   const int ns = (int)(V - x0 < fx::TS ? V - x0 : fx::TS);
@@ -105,6 +124,12 @@ __global__ void __launch_bounds__(128, FAT ? 2 : 3) k_build_links_fx(Dims d, lon
     double2* o = sm + s * fx::SITE_W + mu * 9;
     long long acc[18];
     fx::clear(acc);
+    int away = 0;  // the link's distance from the diagonal matrices of 1, -1, i, -i
+    auto look = [&](const fx::FM& u) {
+#pragma unroll
+      for (int e = 0; e < 9; ++e)
+        away = max(away, e % 4 == 0 ? min(abs(u.h[2 * e]), abs(u.h[2 * e + 1])) : max(abs(u.h[2 * e]), abs(u.h[2 * e + 1])));
+    };
     if constexpr (FAT) {
       // t = 0..5: direction nu, upper (U_nu(x) U_mu(x+nu) U_nu(x+mu)^dag) and
       // lower (U_nu(x-nu)^dag U_mu(x-nu) U_nu(x-nu+mu)) staple
@@ -120,18 +145,26 @@ __global__ void __launch_bounds__(128, FAT ? 2 : 3) k_build_links_fx(Dims d, lon
         fx::mac(acc, a, c);
       }
       const fx::FM u = fx::ld<4>(U, mu, p.lex);
+      look(u);
 #pragma unroll
       for (int e = 0; e < 18; ++e)  // the staple sum, of norm up to 6, enters as an eighth
         acc[e] = fx::scaled(c1, fx::join1(u.h[e], u.l[e])) + fx::scaled(cst, (acc[e] + 4) >> 3);
     } else {
       // U_mu(x) U_mu(x+mu) U_mu(x+2mu)
-      fx::FM a = fx::mul(fx::ld<4>(U, mu, p.lex), fx::ld<4>(U, mu, pm.lex));
+      fx::FM a = fx::ld<4>(U, mu, p.lex);
+      look(a);
+      a = fx::mul(a, fx::ld<4>(U, mu, pm.lex));
       fx::mac(acc, a, fx::ld<4>(U, mu, fx::next_lex(d, pm, mu, 1)));
 #pragma unroll
       for (int e = 0; e < 18; ++e) acc[e] = fx::scaled(c1, acc[e]);
     }
+    long long size = 0;  // the largest off-diagonal entry
 #pragma unroll
-    for (int e = 0; e < 9; ++e) o[e] = make_double2(fx::double_of(acc[2 * e], k), fx::double_of(acc[2 * e + 1], k));
+    for (int e = 0; e < 9; ++e) {
+      o[e] = make_double2(fx::double_of(acc[2 * e], k), fx::double_of(acc[2 * e + 1], k));
+      if (e % 4) size = max(size, max(llabs(acc[2 * e]), llabs(acc[2 * e + 1])));
+    }
+    if (away < 3 << 24 && size < 3LL << 53) fx::mark(hd, list, cap, (4LL * p.lex + mu) * 2 + (FAT ? 0 : 1));
   }
   __syncthreads();
   for (int i = threadIdx.x; i < ns * 36; i += 128) out[x0 * 36 + i] = sm[(i / 36) * fx::SITE_W + i % 36];
@@ -161,11 +194,12 @@ extern "C" int stag_build_links(const int dims[4], const void* thin, void* fat, 
   if (overlap(thin, fat) || overlap(thin, lng) || overlap(fat, lng)) return STAG_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
   const double2* U = (const double2*)thin;
-  auto fp64 = [&](const int* status) {
+  const long long cap = V / 16;  // marked results that the list holds
+  auto fp64 = [&](const fx::Header* hd) {
     ProfScope ps("links", st);
     const long long want = (4 * V + 127) / 128;
-    const unsigned grid = (unsigned)(status && want > 152 * 8 ? 152 * 8 : want);
-    lb::k_build_links<<<grid, 128, 0, st>>>(d, V, U, (double2*)fat, (double2*)lng, c1, c_staple, c3, status);
+    const unsigned grid = (unsigned)(hd && want > 152 * 8 ? 152 * 8 : want);
+    lb::k_build_links<<<grid, 128, 0, st>>>(d, V, U, (double2*)fat, (double2*)lng, c1, c_staple, c3, hd, cap);
     return last_launch_status();
   };
   // Coefficients as fixed point with a power of two taken out; beyond 2^+-900
@@ -178,33 +212,42 @@ extern "C" int stag_build_links(const int dims[4], const void* thin, void* fat, 
   std::frexp(big3, &k3);
   // the fixed-point copy of the links (576 B per site) in stream-ordered
   // scratch; without room for it the FP64 kernel does the work
+  const size_t fbytes = fx::field_bytes(V, 4);
   char* scratch = nullptr;
-  if (cudaMallocAsync((void**)&scratch, 256 + fx::field_bytes(V, 4), st) != cudaSuccess) {
+  if (cudaMallocAsync((void**)&scratch, 256 + fbytes + (size_t)cap * sizeof(long long), st) != cudaSuccess) {
     cudaGetLastError();
     return fp64(nullptr);
   }
-  int* status = (int*)scratch;
+  fx::Header* hd = (fx::Header*)scratch;
   int4* Uf = (int4*)(scratch + 256);
+  long long* list = (long long*)(scratch + 256 + fbytes);
   const unsigned tiles = (unsigned)((V + fx::TS - 1) / fx::TS);
   const fx::Coef none{0, 0};
-  int s;
-  {
+  int s = cuda_status(cudaMemsetAsync(hd, 0, sizeof(*hd), st));
+  if (!s) {
     ProfScope ps("links", st);
-    s = fx::launch_fx_links(V, U, Uf, 4, 0, status, st);
+    s = fx::launch_fx_links(V, U, Uf, 4, 0, &hd->status, st);
   }
   if (!s) {
     ProfScope ps("links", st);
-    lb::k_build_links_fx<true><<<tiles, 128, 0, st>>>(d, V, Uf, status, (double2*)fat, fx::make_coef(std::ldexp(c1, -k)),
+    lb::k_build_links_fx<true><<<tiles, 128, 0, st>>>(d, V, Uf, hd, list, cap, (double2*)fat, fx::make_coef(std::ldexp(c1, -k)),
                                                       fx::make_coef(std::ldexp(c_staple, 3 - k)), k - 60);
     s = last_launch_status();
   }
   if (!s) {
     ProfScope ps("links", st);
-    lb::k_build_links_fx<false><<<tiles, 128, 0, st>>>(d, V, Uf, status, (double2*)lng,
+    lb::k_build_links_fx<false><<<tiles, 128, 0, st>>>(d, V, Uf, hd, list, cap, (double2*)lng,
                                                        fx::make_coef(std::ldexp(c3, -k3)), none, k3 - 60);
     s = last_launch_status();
   }
-  if (!s) s = fp64(status);
+  if (!s) {
+    ProfScope ps("links", st);
+    const long long want = (cap + 127) / 128;
+    lb::k_build_marked<<<(unsigned)(want < 152 * 8 ? want : 152 * 8), 128, 0, st>>>(d, U, list, (double2*)fat, (double2*)lng,
+                                                                                 c1, c_staple, c3, hd, cap);
+    s = last_launch_status();
+  }
+  if (!s) s = fp64(hd);
   const int f = cuda_status(cudaFreeAsync(scratch, st));
   return s ? s : f;
 }

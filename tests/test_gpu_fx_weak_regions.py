@@ -1,12 +1,13 @@
-"""The gauge force on lattices that are ordinary in one part and near the unit matrix (or minus it) in
-another: the small force there keeps FP64's relative accuracy, whether the part is most of the lattice (the
-FP64 kernels then do all of it) or a few links (done one by one)."""
+"""Lattices that are ordinary in one part and near the unit matrix (or minus it) in another: the small gauge
+force there, and the small off-diagonal entries of the fat and Naik links, keep FP64's relative accuracy,
+whether the part is most of the lattice (the FP64 kernels then do all of it) or a few links (done one by one)."""
 
 import numpy as np
 import pytest
 import torch
 
 import oracle.gauge_force as ogf
+import oracle.links as olk
 import synth
 from gpu_common import dev, requires_gpu
 
@@ -56,3 +57,24 @@ def test_small_forces_in_part_of_a_lattice(eps, shape, sign):
     assert deep.any() and np.abs(want[deep]).max() < 10 * terms * eps
     # FP64 sums of such links are off by a few 2^-53 of the largest of their own terms, which are of the force's size
     assert np.linalg.norm((F - want)[deep]) <= 1e-14 * np.linalg.norm(want[deep])
+
+
+@pytest.mark.parametrize("eps", [1e-6, 1e-3, 0.01])
+@pytest.mark.parametrize("shape", ["slab", "box"])
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+def test_small_entries_of_built_links(eps, shape, sign):
+    import paper_1712_00143_gb300 as stag
+
+    dims = (4, 4, 4, 12) if shape == "slab" else (8, 8, 10, 10)
+    c = _coords(dims)
+    inside = c[:, 3] >= 3 if shape == "slab" else (c < 6).all(axis=1)
+    thin = _mixed(dims, eps, inside, 1102)
+    if sign < 0:
+        thin[c[:, 3] == (7 if shape == "slab" else 3), 3] *= -1.0
+    fat, lng = stag.stag_build_links(dims, dev(thin))
+    torch.cuda.synchronize()
+    deep, off = _interior(dims, inside), ~np.eye(3, dtype=bool)
+    for got, want in ((fat.cpu().numpy(), olk.fat_links(thin, dims)), (lng.cpu().numpy(), olk.naik_links(thin, dims))):
+        assert np.linalg.norm(got - want) <= 1e-15 * np.linalg.norm(want)
+        got, want = got[deep][..., off], want[deep][..., off]
+        assert np.linalg.norm(got - want) <= 1e-14 * np.linalg.norm(want)
