@@ -490,9 +490,11 @@ extern "C" int stag_gauge_force(const int dims[4], const void* thin, void* force
   long long* list = (long long*)(scratch + 256 + fbytes);
   const double2* U = (const double2*)thin;
   // coefficients with a power of two taken out (see k_gauge_force_fx); beyond
-  // 2^+-900, or not finite, the FP64 kernels, whose range is wider
+  // 2^+-900, with a beta that would make the last factor (ForceCoef) subnormal, or
+  // not finite, the FP64 kernels, whose range is wider
   const double big = std::fabs(c_pl) * 6 + std::fabs(c_rt) * 18 + std::fabs(c_pg) * 24;
-  const bool fixed = big > 0x1p-900 && big < 0x1p900 && std::fabs(beta) < 0x1p60;
+  const double b = std::fabs(beta);
+  const bool fixed = big > 0x1p-900 && big < 0x1p900 && (b == 0.0 || (b > 0x1p-50 && b < 0x1p60));
   int s = cuda_status(cudaMemsetAsync(hd, 0, sizeof(*hd), st));
   if (fixed && !s) {
     int k = 0;
