@@ -316,7 +316,10 @@ __global__ void __launch_bounds__(128) k_ff_outer_fx(Dims d, long long V, long l
 // B = U_n(y), C = U_r(y+n), lower ones B = U_n(y-n), C = U_r(y-n):
 //   t = G^F_r B' + C^dag G',  w = C^dag B',  Z += A' t + G'' w
 // in the notation at the top of the file (B' = B^dag or B, and so on).
-// Every G is shifted to the largest exponent E among the 22 the link reads.
+// Every G is shifted to the largest exponent E among those of its part: the
+// staples' eighteen, the Naik products' three, G^F_r(y) (with one exponent for
+// all, a part whose coefficient is small or 0 took the others' bits where its G
+// is larger).
 // The staples' sum (up to 9.6 with G's norm, held halved), c1 G and the Naik
 // sum are each brought to full width before their coefficient is applied and
 // they are added (add_part), and Z again before the last product: scaling the
@@ -351,8 +354,9 @@ __global__ void __launch_bounds__(128, 3) k_ff_chain_fx(Dims d, long long V, con
   if (lane < ns) {
     const fx::Site py = fx::site_of(d, (int)x0 + lane), pr = fx::next(d, py, r, 1), pmr = fx::next(d, py, r, -1);
     const int y = py.lex, p2 = fx::next_lex(d, pr, r, 1), pm2 = fx::next_lex(d, pmr, r, -1);
-    int E = max(max(exps[eat(GF0 + r, y)], exps[eat(GL0 + r, y)]),
-                max(exps[eat(GL0 + r, pmr.lex)], exps[eat(GL0 + r, pm2)]));
+    const int EF = exps[eat(GF0 + r, y)];
+    const int EL = max(exps[eat(GL0 + r, y)], max(exps[eat(GL0 + r, pmr.lex)], exps[eat(GL0 + r, pm2)]));
+    int E = ZERO_E;  // the common exponent of the part at hand: the staples' first
 #pragma unroll 1
     for (int g = 0; g < 6; ++g) {
       const int o = g >> 1, n = o < r ? o : o + 1, low = g & 1;
@@ -373,8 +377,8 @@ __global__ void __launch_bounds__(128, 3) k_ff_chain_fx(Dims d, long long V, con
       fx::adjoint_if(m, adj);
       return m;
     };
-    int eZ = ZERO_E;  // Z in units of 2^-60 2^(E + eZ)
-    // Z += coefficient i times the sum in `hold` (units of 2^-60 2^(E + e0))
+    int eZ = ZERO_E;  // Z in units of 2^-60 2^eZ
+    // Z += coefficient i times the sum in `hold` (units of 2^-60 2^e0)
     auto add_part = [&](int i, int e0) {
       long long(*src)[128] = (long long(*)[128])hold;
       unsigned long long mx = 0;
@@ -461,12 +465,14 @@ __global__ void __launch_bounds__(128, 3) k_ff_chain_fx(Dims d, long long V, con
         part[e][tid] = naik ? acc[e] : Z[e][tid];
         if (!naik) Z[e][tid] = 0;
       }
-      add_part(naik ? 2 : 1, naik ? 0 : 1);
+      add_part(naik ? 2 : 1, naik ? E : E + 1);
       if (!naik) {
+        E = EF;
         const fx::FM gy = fetch(GF0 + r, y, 0);
 #pragma unroll
         for (int e = 0; e < 18; ++e) part[e][tid] = fx::join1(gy.h[e], gy.l[e]);
-        add_part(0, 0);
+        add_part(0, E);
+        E = EL;
       }
     }
     // force = -TA[U Z]; the differences are exact
@@ -484,7 +490,7 @@ __global__ void __launch_bounds__(128, 3) k_ff_chain_fx(Dims d, long long V, con
     fx::clear(w);
     fx::mac(w, fx::ld<SLOTS>(T, r, y), z);
     const long long tr = w[1] + w[9] + w[17];
-    const int k = E + eZ - up - 60;  // (no use where every sum is zero)
+    const int k = eZ - up - 60;  // (no use where every sum is zero)
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       dg[i] = (-1.0 / 3.0) * fx::double_of(3 * w[8 * i + 1] - tr, k);
