@@ -16,10 +16,13 @@
 //   gate and stores need no exchange either.
 // Every warp works by itself: no barrier after the start, its gather running
 // three directions ahead in shared memory of its own.
-// The split of the transports into two bfloat16 parts, the order of the
-// products (direction by direction, high part then low) and the accumulation
-// in FP32 are those of the tcgen05 form, and so are the results, bit for bit
-// (both units were compared on random operands).
+// The transports enter as two bfloat16 parts (16 bits), products and sums are
+// FP32.  The unit truncates its sums, and over a chain of them that shrinks
+// every result by the same few 2^-22, which a gradient, a sum over all sites,
+// keeps while the sites' own errors average out.  So a product starts from zero
+// for each direction, the low parts first, and is added with rounding outside:
+// gradient at 16 x 20 x 12 x 24 3.0e-7 from the 64-bit one against 3.4e-6, for
+// 542 in place of 524 us per forward pass at 24^4.
 #pragma once
 #include "net_tc.cuh"
 
@@ -248,16 +251,28 @@ __device__ __forceinline__ void site_operand(const Pairs& h, uint32_t (&o)[36]) 
 
 // d[nt] += sum over the 8 sites and (re, im) of colour i: a (channels or
 // directions m: transposed parts [part]{re t, re t+4, im t, im t+4}) times the
-// site operand (parts b[part][nt]{re, im}).  Six products of parts, the small
-// ones first, carry 24 bits of each factor.  The unit truncates its sums, so d
-// starts from zero for every 8 sites and is added to the running sum outside.
+// site operand (parts b[part][nt]{re, im}).  Six products of parts carry 24 bits
+// of each factor; the five small ones, the smallest first, have a sum of their
+// own, and both are added with rounding.
 __device__ __forceinline__ void outer(float (&d)[2][4], const uint32_t (&a)[3][4], const uint2 (&b)[3][2]) {
 #pragma unroll
-  for (int n = 2; n >= 0; --n)
+  for (int nt = 0; nt < 2; ++nt) {
+    float s[4] = {0.f, 0.f, 0.f, 0.f}, m[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int k = 0; k <= n; ++k)
+    for (int n = 2; n > 0; --n)
 #pragma unroll
-      for (int nt = 0; nt < 2; ++nt) mma(d[nt], a[k][0], a[k][1], a[k][2], a[k][3], b[n - k][nt].x, b[n - k][nt].y);
+      for (int k = 0; k <= n; ++k) mma(s, a[k][0], a[k][1], a[k][2], a[k][3], b[n - k][nt].x, b[n - k][nt].y);
+    mma(m, a[0][0], a[0][1], a[0][2], a[0][3], b[0][nt].x, b[0][nt].y);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) d[nt][e] += m[e] + s[e];
+  }
+}
+// acc += s, rounded to nearest
+__device__ __forceinline__ void add(float (&acc)[2][4], const float (&s)[2][4]) {
+#pragma unroll
+  for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) acc[nt][e] += s[nt][e];
 }
 
 constexpr int FW = 8;    // warps per block of the forward layer
@@ -302,10 +317,12 @@ __global__ void __launch_bounds__(32 * nm::FW, 2)
       tc::split2(x0.z, x0.w, h[1], l[1]);
       tc::split2(x1.x, x1.y, h[2], l[2]);
       tc::split2(x1.z, x1.w, h[3], l[3]);
-      mma(acc[i][0], h[0], h[1], h[2], h[3], b.x, b.y);
-      mma(acc[i][1], h[0], h[1], h[2], h[3], b.z, b.w);
-      mma(acc[i][0], l[0], l[1], l[2], l[3], b.x, b.y);
-      mma(acc[i][1], l[0], l[1], l[2], l[3], b.z, b.w);
+      float s[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+      mma(s[0], l[0], l[1], l[2], l[3], b.x, b.y);
+      mma(s[1], l[0], l[1], l[2], l[3], b.z, b.w);
+      mma(s[0], h[0], h[1], h[2], h[3], b.x, b.y);
+      mma(s[1], h[0], h[1], h[2], h[3], b.z, b.w);
+      add(acc[i], s);
     };
     auto done = [&]() {  // the stage has been read by its lane, the slot by the warp: the next direction may come
       __syncwarp();
@@ -507,10 +524,14 @@ __global__ void __launch_bounds__(32 * nm::AW, 3)
         split3(x0.z, x0.w, i0);
         split3(x1.x, x1.y, r1);
         split3(x1.z, x1.w, i1);
+        {
+          float s[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          mma(acc[i][0], r0[k], i0[k], r1[k], i1[k], b.x, b.y);
-          mma(acc[i][1], r0[k], i0[k], r1[k], i1[k], b.z, b.w);
+          for (int k = 1; k >= 0; --k) {
+            mma(s[0], r0[k], i0[k], r1[k], i1[k], b.x, b.y);
+            mma(s[1], r0[k], i0[k], r1[k], i1[k], b.z, b.w);
+          }
+          add(acc[i], s);
         }
         uint32_t a[3][4];
         uint2 q[3][2];
