@@ -68,6 +68,7 @@ EXPORTS = (
     "stag_net_loss_grad",
     "stag_net_train",
     "stag_tc_selftest",
+    "stag_cg_loop_test",
     "stag_build_links",
     "stag_gauge_force",
     "stag_fermion_force",
@@ -204,6 +205,7 @@ def load_library(path=LIB_PATH):
         ),
         "stag_net_train": (ci, [vp, ctypes.POINTER(TrainPair), ci, ctypes.POINTER(TrainParams), ctypes.POINTER(cd), vp]),
         "stag_tc_selftest": (ci, [ctypes.POINTER(cd)]),
+        "stag_cg_loop_test": (ci, [vp, ctypes.c_uint, ci]),
         "stag_build_links": (ci, [ctypes.POINTER(ci), vp, vp, vp, cd, cd, cd, vp]),
         "stag_gauge_force": (ci, [ctypes.POINTER(ci), vp, vp, cd, cd, cd, cd, vp]),
         "stag_fermion_force": (ci, [ctypes.POINTER(ci), vp, ci, vp, vp, ctypes.POINTER(cd), cd, cd, cd, vp, vp]),
@@ -578,6 +580,11 @@ def stag_tc_selftest():
     err = ctypes.c_double()
     _check(_lib.stag_tc_selftest(ctypes.byref(err)), "stag_tc_selftest")
     return err.value
+
+
+def stag_cg_loop_test(lattice, polls=0, what=0):
+    """Testing aid: bound the waits of this handle's small-lattice CG kernel (see include/stag.h)."""
+    _check(_lib.stag_cg_loop_test(lattice.ptr, int(polls), int(what)), "stag_cg_loop_test")
 
 
 def stag_strerror(status):

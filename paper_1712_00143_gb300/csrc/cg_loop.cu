@@ -35,6 +35,7 @@ constexpr unsigned SPIN_LIMIT = 1u << 22;  // polls of a barrier, about a second
 struct LoopSync {
   unsigned* arrived;  // zero at the start
   unsigned* gave_up;  // set when a wait ran out
+  unsigned limit;     // polls of one wait
 };
 
 // The two halves of a grid barrier, called by all threads.  arrive: what the
@@ -51,7 +52,7 @@ __device__ __forceinline__ bool grid_wait(const LoopSync& sy, unsigned target) {
     unsigned n = 0, seen;
     do {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(sy.arrived) : "memory");
-    } while ((int)(seen - target) < 0 && ++n < SPIN_LIMIT);
+    } while ((int)(seen - target) < 0 && ++n < sy.limit);
     ok = (int)(seen - target) >= 0;
     if (!ok) atomicExch(sy.gave_up, 1u);
   }
@@ -357,7 +358,8 @@ __global__ void __launch_bounds__(LB)
 
 // Iterations until a stop flag is raised or `most` have run.  `gave_up`
 // (device, beside the barrier's counter) is set if a wait ran out: the fields
-// are then not usable.  STAG_EINVAL where the form does not apply or the grid
+// are then not usable, and the state is as it was or the loop's (the caller
+// solves again with queued launches).  STAG_EINVAL where the form does not apply or the grid
 // cannot be resident at once (the caller queues the iterations instead).
 template <int P>
 int launch_cg_loop(stag_lattice_s* lat, Spinor<P> p, Spinor<P> p2, Spinor<P> t, Spinor<32> Ap, Spinor<32> xh,
@@ -384,8 +386,9 @@ int launch_cg_loop(stag_lattice_s* lat, Spinor<P> p, Spinor<P> p2, Spinor<P> t, 
   const void* k = kernel(want <= sms);
   if (2 * G > rs.max_grid * 3) return STAG_EINVAL;  // (the caller's partials hold three per block of max_grid)
   float2* partials = (float2*)rs.partials;
-  LoopSync sy{sync, sync + 1};
+  LoopSync sy{sync, sync + 1, lat->loop_polls ? lat->loop_polls : SPIN_LIMIT};
   int s = cuda_status(cudaMemsetAsync(sync, 0, 2 * sizeof(unsigned), st));
+  if (!s && lat->loop_test == 1) s = cuda_status(cudaMemsetAsync(sync, 0xc0, sizeof(unsigned), st));
   if (s) return s;
   void* args[] = {&odd, &even, &p, &p2, &t, &Ap, &xh, &rh, &state, &partials, &sy, &pending, &most};
   ProfScope ps("cg_loop", st);

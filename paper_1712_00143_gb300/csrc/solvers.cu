@@ -61,10 +61,11 @@ static int true_residual(stag_lattice_s* lat, Spinor<64> r, Spinor<64> b, Spinor
 }
 
 // Solve (m^2 + sigma - D_eo D_oe) x = b with sloppy precision P (P = 64: plain
-// FP64 CG).  x_can/b_can: canonical device fields.
+// FP64 CG).  x_can/b_can: canonical device fields.  may_loop: a small lattice's
+// iterations may run as one kernel.
 template <int P>
 static int cg_solve(stag_lattice_s* lat, double2* x_can, const double2* b_can, double shift,
-                    const stag_solve_params& prm, stag_solve_info* info, cudaStream_t st) {
+                    const stag_solve_params& prm, stag_solve_info* info, cudaStream_t st, bool may_loop = true) {
   constexpr int PV = Acc<P>::value;
   const double t0 = now_s();
   const int Vh = lat->g.Vh;
@@ -102,7 +103,7 @@ static int cg_solve(stag_lattice_s* lat, double2* x_can, const double2* b_can, d
     return launch_dslash_df_epi(lat, rdf, tdf, 1, 0, ydf, -shift, radf, 1.0, 1.0, nullptr, st);
   };
   // small lattices: the iterations between two updates as one kernel
-  bool loop = P != 64 && Vh <= kLoopSites;
+  bool loop = P != 64 && Vh <= kLoopSites && may_loop;
   Spinor<P> p2{nullptr, Vh};
   unsigned* sync = nullptr;
   if (loop) {
@@ -220,7 +221,13 @@ static int cg_solve(stag_lattice_s* lat, double2* x_can, const double2* b_can, d
       if (loop) {
         auto read = [&](int* v) { return *v = (int)hsync[1], 0; };
         auto clear = [&] { return hsync[1] = 0, 0; };  // (the device words are cleared before every launch)
-        TRY(take_flag(read, clear, STAG_ETIMEOUT));
+        const int f = take_flag(read, clear, STAG_ETIMEOUT);
+        if (f == STAG_ETIMEOUT) {  // a barrier's wait ran out: from the start, with launches that wait for nothing
+          const int again = cg_solve<P>(lat, x_can, b_can, shift, prm, info, st, false);
+          if (info) info->seconds = now_s() - t0;
+          return again;
+        }
+        if (f) return f;
       }
       if ((hs->flags & F_STOP) && !loop) prof_discard_since(mark);  // launches after the flag returned at once
       prof_flush_completed();
