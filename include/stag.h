@@ -546,9 +546,9 @@ int stag_tc_selftest(double* max_rel_err);
 /* Testing aid for this handle's mixed-precision solves on small lattices, whose
  * iterations run as one kernel with bounded waits: a wait gives up after
  * `polls` polls (0: the default, about a second).  what: 0 nothing else; 1 a
- * wait is never satisfied.  A solve whose wait gave up starts again with one
- * launch per step, so it returns what it would have returned without that
- * kernel. */
+ * wait is never satisfied; 2 the kernel's scratch cannot be had.  A solve whose
+ * wait gave up starts again with one launch per step, and one without scratch
+ * runs so, so it returns what it would have returned without that kernel. */
 int stag_cg_loop_test(stag_lattice_t lat, unsigned polls, int what);
 
 /* Human-readable text of a status code (static storage). */

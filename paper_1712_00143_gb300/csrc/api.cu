@@ -426,7 +426,7 @@ int stag_tuned_shape(stag_lattice_t lat, int prec, int kernel, int* block, int* 
 }
 
 int stag_cg_loop_test(stag_lattice_t lat, unsigned polls, int what) {
-  if (!lat || what < 0 || what > 1) return STAG_EINVAL;
+  if (!lat || what < 0 || what > 2) return STAG_EINVAL;
   lat->loop_polls = polls;
   lat->loop_test = what;
   return STAG_OK;

@@ -60,7 +60,8 @@ struct stag_lattice_s {
     float us_epi = 0.f;
   } mrhs[6][5];  // by the ABI precision (stag_prec), tuned per format
   // bounded waits of the small-lattice CG loop (stag_cg_loop_test): polls of a
-  // barrier (0: the default), and 1 if its counter starts out of reach
+  // barrier (0: the default), and 1 if its counter starts out of
+  // reach, 2 if its scratch cannot be had
   unsigned loop_polls = 0;
   int loop_test = 0;
   stag::LinkCopy links[5];  // by stag_prec (STAG_DF64 = 4: FP64 split into hi + lo floats)

@@ -107,9 +107,10 @@ static int cg_solve(stag_lattice_s* lat, double2* x_can, const double2* b_can, d
   Spinor<P> p2{nullptr, Vh};
   unsigned* sync = nullptr;
   if (loop) {
-    if (P == 32 || P == 31) p2 = ws_spinor<P>(lat, "cg.p2", &s);
-    sync = (unsigned*)lat->ws.get("cg.sync", 64, &s);
-    if (s) return s;
+    int none = STAG_OK;  // without this scratch: queued launches
+    if (P == 32 || P == 31) p2 = ws_spinor<P>(lat, "cg.p2", &none);
+    sync = (unsigned*)lat->ws.get("cg.sync", lat->loop_test == 2 ? (size_t)1 << 60 : 64, &none);
+    loop = none == STAG_OK;
   }
   PinnedState pin(sizeof(CgState) + 64);
   if (!pin.h) return STAG_ENOMEM;

@@ -45,3 +45,22 @@ def test_an_initial_guess_survives():
     info = stag.stag_cg(h, x, dev(b), 0.1, mode="mixed32", tol=1e-11, use_initial_guess=1)
     assert info["converged"] and oracle.true_residual(fat, lng, x.cpu().numpy(), b, 0.1, dims) <= 1.01e-11
     h.free()
+
+
+@pytest.mark.parametrize("mode", ["mixed32", "mixedfx16"])
+def test_without_scratch_the_launches_are_queued(mode):
+    import paper_1712_00143_gb300 as stag
+
+    dims = (6, 6, 8, 4)
+    fat, lng = synth.gauge_field(dims, 0.3, 1113)
+    h = stag.stag_load_links(dims, dev(fat), dev(lng))
+    b = synth.gaussian_source(dims, 5202)
+    runs = []
+    for polls, what in ((300, 1), (0, 2), (0, 0), (0, 2)):
+        stag.stag_cg_loop_test(h, polls, what)
+        x = torch.zeros((h.Vh, 3), dtype=torch.complex128, device="cuda")
+        info = stag.stag_cg(h, x, dev(b), 0.2, mode=mode, tol=1e-10)
+        assert info["converged"] and oracle.true_residual(fat, lng, x.cpu().numpy(), b, 0.2, dims) <= 1.001e-10
+        runs.append(x)
+    assert torch.equal(runs[0], runs[1]) and torch.equal(runs[1], runs[3])
+    h.free()
