@@ -63,6 +63,21 @@ int get_red_scratch(stag_lattice_s* lat, const char* name, RedScratch* out, int 
   return STAG_OK;
 }
 
+int sm_count() {
+  static std::atomic<int> n{0};
+  int v = n.load();
+  if (v == 0) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) {
+      cudaGetLastError();
+      v = 152;
+    }
+    n.store(v);
+  }
+  return v;
+}
+
 int last_launch_status() {
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? STAG_OK : STAG_ECUDA;

@@ -30,27 +30,13 @@ namespace {
     if (_s) return _s;         \
   } while (0)
 
-int sm_count_b() {
-  static int n = 0;
-  if (n == 0) {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
-      n = v;
-    else {
-      cudaGetLastError();
-      n = 152;
-    }
-  }
-  return n;
-}
 int grid_red(int Vh, int cap) {
-  int g = (Vh + 255) / 256, m = 4 * sm_count_b();
+  int g = (Vh + 255) / 256, m = 4 * sm_count();
   g = g < m ? g : m;
   return g < cap ? g : cap;
 }
 int grid_bw(int Vh) {
-  int g = (Vh + 255) / 256, m = 8 * sm_count_b();
+  int g = (Vh + 255) / 256, m = 8 * sm_count();
   return g < m ? g : m;
 }
 

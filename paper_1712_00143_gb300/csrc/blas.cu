@@ -14,21 +14,6 @@ namespace stag {
 
 static constexpr int BB = 256;  // threads per block of the level-1 kernels
 
-static int sm_count() {
-  static int n = 0;
-  if (n == 0) {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0) {
-      n = v;
-    } else {
-      cudaGetLastError();
-      n = 152;
-    }
-  }
-  return n;
-}
-
 // Grids: reductions use up to 4 blocks per SM (each block reduces once, at
 // the end), streaming kernels up to 8.
 static inline int red_grid(int Vh, int cap) {

@@ -165,26 +165,12 @@ int hop_launches(const stag_lattice_s* lat, DfField out, DfField in, int n, int 
 // ------------------------------------------------------------ level 1
 #define DGRID(s, Vh) for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < (Vh); s += gridDim.x * blockDim.x)
 
-int sm_count_df() {
-  static int n = 0;
-  if (n == 0) {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
-      n = v;
-    else {
-      cudaGetLastError();
-      n = 152;
-    }
-  }
-  return n;
-}
 int grid_bw_df(int Vh) {
-  const int g = (Vh + 255) / 256, m = 8 * sm_count_df();
+  const int g = (Vh + 255) / 256, m = 8 * sm_count();
   return g < m ? g : m;
 }
 int grid_red_df(int Vh, int cap) {
-  int g = (Vh + 255) / 256, m = 4 * sm_count_df();
+  int g = (Vh + 255) / 256, m = 4 * sm_count();
   g = g < m ? g : m;
   return g < cap ? g : cap;
 }

@@ -65,7 +65,7 @@ __device__ __forceinline__ void st3x3(double2* __restrict__ p, const M3& m) {
 }
 
 // FP64 forms.  With a status word they run only when the integer kernels may
-// not, in grids of a few blocks per SM that return at once otherwise.
+// not, in grids that return at once otherwise.
 // One thread per (site x, direction mu), idx = x * 4 + mu: consecutive threads
 // write consecutive matrices.  X, Y: [n][V/2][3], checkerboard index lex / 2.
 __global__ void __launch_bounds__(128) k_ff_outer(Dims d, long long V, long long Vh, int n, Alphas al,
@@ -600,7 +600,7 @@ extern "C" int stag_fermion_force(const int dims[4], const void* thin, int n_ter
     }
   }
   const long long n = (4 * V + 127) / 128;
-  const unsigned grid = (unsigned)(fixed && n > 152 * 8 ? 152 * 8 : n);
+  const unsigned grid = fixed ? beside_grid(n) : (unsigned)n;
   const int* when = fixed ? status : nullptr;
   if (!s) {
     ProfScope ps("fermion_force", st);

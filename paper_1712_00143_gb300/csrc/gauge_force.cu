@@ -96,7 +96,7 @@ __device__ __forceinline__ M3 staple(const double2* __restrict__ U, const Dims& 
 }
 
 // FP64 form; it and k_gauge_force_reuse run only when the integer kernels do
-// not serve (fx::all_fp64), in grids of a few blocks per SM that return at once otherwise.
+// not serve (fx::all_fp64), in grids that return at once otherwise.
 __global__ void __launch_bounds__(128) k_gf_staples(Dims d, long long V, const double2* __restrict__ U,
                                                     double2* __restrict__ T, const fx::Header* hd, long long cap) {
   if (!fx::all_fp64(hd, cap)) return;
@@ -122,20 +122,21 @@ __device__ __forceinline__ void axpy3(M3& acc, double c, const M3& m) {
   }
 }
 
-// S += the terms of (nu, s) for the link (p0, mu); staples from the table, or
-// from the links where there is none.
+// S += the terms of (nu, s) for the link (p0, mu), with pp = x + mu, pm = x - mu
+// and their links U_mu; staples from the table, or from the links where there
+// is none.
 template <bool TABLE>
 __device__ __forceinline__ void add_pair(M3& S, const double2* __restrict__ U, const double2* __restrict__ T, const Dims& d,
-                                         const Pos& p0, int mu, int nu, int s, double cpl, double crt, double cpg) {
+                                         const Pos& p0, const Pos& pp, const Pos& pm, const M3& u_pm, const M3& u_mm,
+                                         int mu, int nu, int s, double cpl, double crt, double cpg) {
   auto at = [&](const Pos& p, int a, int b, int sign) {
     if (TABLE) return ldT(T, p.lex, a, b, sign);
     return staple(U, d, p, a, b, sign);
   };
-  const Pos pp = step(d, p0, mu, 1), pm = step(d, p0, mu, -1);  // x + mu, x - mu
   const M3 t0 = at(p0, mu, nu, s);
-  axpy3(S, cpl, t0);                                                    // plaquette
-  axpy3(S, crt, mul(ld(U, pp.lex, mu), mul(at(pp, mu, nu, s), t0)));  // rectangle 1
-  axpy3(S, crt, mul(mul(t0, at(pm, mu, nu, s)), ld(U, pm.lex, mu)));  // rectangle 2
+  axpy3(S, cpl, t0);                                       // plaquette
+  axpy3(S, crt, mul(u_pm, mul(at(pp, mu, nu, s), t0)));  // rectangle 1
+  axpy3(S, crt, mul(mul(t0, at(pm, mu, nu, s)), u_mm));  // rectangle 2
   // rectangle 3 and the parallelograms share the left factor h(x+mu, nu, s)
   const Pos ps = step(d, p0, nu, s);  // x + s nu
   M3 R = mul(at(ps, mu, nu, s), hop_at(U, d, ps, nu, -s));
@@ -144,18 +145,34 @@ __device__ __forceinline__ void add_pair(M3& S, const double2* __restrict__ U, c
     R.e[i].x *= crt;
     R.e[i].y *= crt;
   }
-  const Pos pq = s > 0 ? p0 : step(d, p0, nu, -1);  // x, or x - nu
-  const int lo = nu < mu ? nu : mu, hi = nu < mu ? mu : nu;
+  const Pos pmn = step(d, p0, nu, -1);  // x - nu (for s = -1)
+  if constexpr (TABLE) {
 #pragma unroll 1
-  for (int j = 0; j < 4; ++j) {  // (rho, r): the two directions other than mu and nu, both signs
-    int rho = j >> 1;
-    const int r = (j & 1) ? 1 : -1;
-    rho += rho >= lo ? 1 : 0;
-    rho += rho >= hi ? 1 : 0;
-    const M3 a = at(ps, mu, rho, r);
-    M3 q = at(pq, nu, rho, r);
-    if (s < 0) q = dagger(q);
-    axpy3(R, cpg, mul(a, q));
+    for (int rho = 0; rho < 4; ++rho) {
+      if (rho == mu || rho == nu) continue;
+#pragma unroll 1
+      for (int r = -1; r <= 1; r += 2) {
+        const M3 a = at(ps, mu, rho, r);
+        const M3 q = s > 0 ? at(p0, nu, rho, r) : dagger(at(pmn, nu, rho, r));
+        axpy3(R, cpg, mul(a, q));
+      }
+    }
+  } else {
+    // the same in a form that lanes of other (mu, nu, s) run together (for the
+    // table kernel, whose warps share them, it is 1.5 % slower)
+    const Pos pq = s > 0 ? p0 : pmn;
+    const int lo = nu < mu ? nu : mu, hi = nu < mu ? mu : nu;
+#pragma unroll 1
+    for (int j = 0; j < 4; ++j) {
+      int rho = j >> 1;
+      const int r = (j & 1) ? 1 : -1;
+      rho += rho >= lo ? 1 : 0;
+      rho += rho >= hi ? 1 : 0;
+      const M3 a = at(ps, mu, rho, r);
+      M3 q = at(pq, nu, rho, r);
+      if (s < 0) q = dagger(q);
+      axpy3(R, cpg, mul(a, q));
+    }
   }
   axpy3(S, 1.0, mul(hop_at(U, d, pp, nu, s), R));
 }
@@ -190,13 +207,14 @@ __global__ void __launch_bounds__(128) k_gauge_force_reuse(Dims d, long long V, 
        idx += (long long)gridDim.x * blockDim.x) {
     const int mu = (int)(idx / V);
     const long long x = idx - (long long)mu * V;
-    const Pos p0 = pos_of(d, x);
+    const Pos p0 = pos_of(d, x), pp = step(d, p0, mu, 1), pm = step(d, p0, mu, -1);
+    const M3 u_pm = ld(U, pp.lex, mu), u_mm = ld(U, pm.lex, mu);
     M3 S = zero3();
 #pragma unroll 1
     for (int nu = 0; nu < 4; ++nu) {
       if (nu == mu) continue;
 #pragma unroll 1
-      for (int s = -1; s <= 1; s += 2) add_pair<true>(S, U, T, d, p0, mu, nu, s, cpl, crt, cpg);
+      for (int s = -1; s <= 1; s += 2) add_pair<true>(S, U, T, d, p0, pp, pm, u_pm, u_mm, mu, nu, s, cpl, crt, cpg);
     }
     store_force(U, F, x, mu, S, beta);
   }
@@ -218,7 +236,11 @@ __global__ void __launch_bounds__(128) k_gauge_force_marked(Dims d, const double
     const long long at = in ? __ldcg(list + i) : 0, x = at >> 2;
     const int mu = (int)(at & 3), q = o >> 1, nu = q < mu ? q : q + 1;
     M3 S = zero3();
-    if (in && o < 6) add_pair<false>(S, U, nullptr, d, pos_of(d, x), mu, nu, (o & 1) ? 1 : -1, cpl, crt, cpg);
+    if (in && o < 6) {
+      const Pos p0 = pos_of(d, x), pp = step(d, p0, mu, 1), pm = step(d, p0, mu, -1);
+      add_pair<false>(S, U, nullptr, d, p0, pp, pm, ld(U, pp.lex, mu), ld(U, pm.lex, mu), mu, nu, (o & 1) ? 1 : -1, cpl, crt,
+                      cpg);
+    }
 #pragma unroll
     for (int w = 1; w < 8; w <<= 1)
 #pragma unroll
@@ -526,22 +548,20 @@ extern "C" int stag_gauge_force(const int dims[4], const void* thin, void* force
     if (!s) {
       ProfScope ps("gauge_force", st);
       const long long want = (cap + 15) / 16;
-      gf::k_gauge_force_marked<<<(unsigned)(want < 152 * 4 ? want : 152 * 4), 128, 0, st>>>(d, U, list, (double2*)force, beta,
-                                                                                         c_pl, c_rt, c_pg, hd, cap);
+      gf::k_gauge_force_marked<<<beside_grid(want), 128, 0, st>>>(d, U, list, (double2*)force, beta, c_pl, c_rt, c_pg, hd, cap);
       s = last_launch_status();
     }
   }
-  const unsigned few = 152 * 8;
   if (!s) {
     ProfScope ps("gauge_force", st);
     const long long n = (24 * V + 127) / 128;
-    gf::k_gf_staples<<<(unsigned)(fixed && n > few ? few : n), 128, 0, st>>>(d, V, U, T, hd, cap);
+    gf::k_gf_staples<<<fixed ? beside_grid(n) : (unsigned)n, 128, 0, st>>>(d, V, U, T, hd, cap);
     s = last_launch_status();
   }
   if (!s) {
     ProfScope ps("gauge_force", st);
     const long long n = (4 * V + 127) / 128;
-    gf::k_gauge_force_reuse<<<(unsigned)(fixed && n > few ? few : n), 128, 0, st>>>(d, V, U, T, (double2*)force, beta, c_pl,
+    gf::k_gauge_force_reuse<<<fixed ? beside_grid(n) : (unsigned)n, 128, 0, st>>>(d, V, U, T, (double2*)force, beta, c_pl,
                                                                                    c_rt, c_pg, hd, cap);
     s = last_launch_status();
   }

@@ -201,6 +201,17 @@ template <int P> int launch_ru_p(Spinor<P> p, Spinor<Acc<P>::value> rh, CgState*
 template <int P>
 int launch_cg_loop(stag_lattice_s* lat, Spinor<P> p, Spinor<P> p2, Spinor<P> t, Spinor<32> Ap, Spinor<32> xh,
                    Spinor<32> rh, CgState* state, int pending, int most, RedScratch rs, unsigned* sync, cudaStream_t st);
+// SMs of the current device (152 where it cannot be asked).
+int sm_count();
+// Grid of an FP64 kernel that is launched beside the integer kernels and returns
+// at once unless they do not serve: n blocks of work, grid-stride.  32 blocks
+// per SM cost 3 us when they return at once, and leave the last wave short when
+// they do not (with 8 per SM some blocks had nine parts and some eight: links at
+// 24^4 5 %, gauge force 3 % slower than one block per part).
+inline unsigned beside_grid(long long n) {
+  const long long most = 32LL * sm_count();
+  return (unsigned)(n < most ? n : most);
+}
 // Sites per parity up to which the fixed-point FP64 operator runs one hop per
 // thread (dslash_impl.cuh says why the line lies there).
 constexpr int kFewSites = 1 << 15;

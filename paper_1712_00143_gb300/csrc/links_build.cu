@@ -60,8 +60,8 @@ __device__ __forceinline__ void st(double2* __restrict__ out, long long link, co
 }
 
 // FP64 form: bound by the FP64 pipe (10.8 ms at 32^4, 1.2 TFLOP/s).  With a
-// header it runs only when the integer kernels do not serve, in a grid of a few
-// blocks per SM whose blocks return at once otherwise.
+// header it runs only when the integer kernels do not serve, in a grid
+// whose blocks return at once otherwise.
 __global__ void __launch_bounds__(128) k_build_links(Dims d, long long V, const double2* __restrict__ U,
                                                      double2* __restrict__ F, double2* __restrict__ Lk, double c1,
                                                      double cst, double c3, const fx::Header* hd, long long cap) {
@@ -198,7 +198,7 @@ extern "C" int stag_build_links(const int dims[4], const void* thin, void* fat, 
   auto fp64 = [&](const fx::Header* hd) {
     ProfScope ps("links", st);
     const long long want = (4 * V + 127) / 128;
-    const unsigned grid = (unsigned)(hd && want > 152 * 8 ? 152 * 8 : want);
+    const unsigned grid = hd ? beside_grid(want) : (unsigned)want;
     lb::k_build_links<<<grid, 128, 0, st>>>(d, V, U, (double2*)fat, (double2*)lng, c1, c_staple, c3, hd, cap);
     return last_launch_status();
   };
@@ -243,8 +243,7 @@ extern "C" int stag_build_links(const int dims[4], const void* thin, void* fat, 
   if (!s) {
     ProfScope ps("links", st);
     const long long want = (cap + 127) / 128;
-    lb::k_build_marked<<<(unsigned)(want < 152 * 8 ? want : 152 * 8), 128, 0, st>>>(d, U, list, (double2*)fat, (double2*)lng,
-                                                                                 c1, c_staple, c3, hd, cap);
+    lb::k_build_marked<<<beside_grid(want), 128, 0, st>>>(d, U, list, (double2*)fat, (double2*)lng, c1, c_staple, c3, hd, cap);
     s = last_launch_status();
   }
   if (!s) s = fp64(hd);

@@ -234,7 +234,7 @@ static int net_run_init(stag_net_s* net, stag_lattice_s* lat, NetRun& R, bool tr
   if (training) {
     R.g0 = (float2*)net->ws.get(pre + "g0", sites * cmax * 3 * sizeof(float2), &s);
     R.g1 = (float2*)net->ws.get(pre + "g1", sites * cmax * 3 * sizeof(float2), &s);
-    R.part_blocks = 3 * 152;
+    R.part_blocks = 3 * sm_count();
     R.part = (float*)net->ws.get(pre + "part", (size_t)R.part_blocks * NET_NDIR * cmax * cmax * sizeof(float), &s);
   }
   R.scal = (double*)net->ws.get(pre + "scal", 64, &s);
@@ -265,7 +265,7 @@ static int layer_fwd(const NetRun& R, int l, cudaStream_t st) {
   } else if (ci == 16 && co == 16 && gate) {
     if (((uintptr_t)in & 15u) != 0) return STAG_EINVAL;  // records are read as 16-byte words
     TRYN(cuda_status(cudaFuncSetAttribute(k_net_layer_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, nm::FWD_SMEM)));
-    k_net_layer_mma<<<grid_groups(R.Vh, nm::FW, 2 * 152), 32 * nm::FW, nm::FWD_SMEM, st>>>(R.ng, in, pre, out, W, b);
+    k_net_layer_mma<<<grid_groups(R.Vh, nm::FW, 2 * sm_count()), 32 * nm::FW, nm::FWD_SMEM, st>>>(R.ng, in, pre, out, W, b);
   } else if (ci == 16 && co == 1 && !gate) {
     // one output channel: site-local mix into the directions, then one
     // transport per direction, for the even sites the prediction is read on
@@ -313,13 +313,13 @@ static int layer_bwd(const NetRun& R, int l, float2* g, float2* gin, bool want_i
       TRYN(cuda_status(cudaFuncSetAttribute(k_net_adjoint_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, nm::ADJ_SMEM)));
       k_net_adjoint_mma<<<G, 32 * nm::AW, nm::ADJ_SMEM, st>>>(R.ng, g, R.h[l], gin, W, R.part);
     } else if (ci == 1 && co == 16) {
-      G = grid_groups(R.Vh, nm::TW, 2 * 152);
+      G = grid_groups(R.Vh, nm::TW, 2 * sm_count());
       k_net_dw_thin<<<G, 32 * nm::TW, 0, st>>>(R.ng, R.h[l], g, 0, R.part);
     } else if (ci == 16 && co == 1) {
-      G = grid_groups(R.Vh, nm::TW, 2 * 152);
+      G = grid_groups(R.Vh, nm::TW, 2 * sm_count());
       k_net_dw_thin<<<G, 32 * nm::TW, 0, st>>>(R.ng, g, R.h[l], 1, R.part);
     } else if (ci == 1 && co == 1) {
-      G = 152;
+      G = sm_count();
       k_net_dw_1to1<<<G, 256, 0, st>>>(R.ng, R.h[l], g, R.part);
     } else {
       return STAG_EINVAL;
