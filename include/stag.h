@@ -486,7 +486,7 @@ int stag_dd_cg(stag_dd_t d, void* x, const void* b, double mass, const stag_solv
  * caller-owned; fat and lng must not overlap thin or each other
  * (STAG_EINVAL).  dims: even extents >= 4.  Products run in fixed point of
  * FP64-class accuracy where the links allow (unitary to rounding), in FP64
- * otherwise; scratch 576 B per site, stream-ordered (without it, FP64
+ * otherwise; scratch 608 B per site, stream-ordered (without it, FP64
  * arithmetic throughout).  Asynchronous on `stream`. */
 int stag_build_links(const int dims[4], const void* thin, void* fat, void* lng, double c1, double c_staple,
                      double c3, void* stream);

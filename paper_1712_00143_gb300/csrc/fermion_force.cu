@@ -573,7 +573,8 @@ extern "C" int stag_fermion_force(const int dims[4], const void* thin, int n_ter
     cudaGetLastError();
     return STAG_ENOMEM;
   }
-  int* status = (int*)scratch;
+  fx::Header* hd = (fx::Header*)scratch;
+  int* status = &hd->status;
   int4* T = (int4*)(scratch + 256);
   int* exps = (int*)(scratch + 256 + gbytes);
   double2* GF = (double2*)(scratch + 256);
@@ -584,7 +585,7 @@ extern "C" int stag_fermion_force(const int dims[4], const void* thin, int n_ter
     const unsigned tiles = (unsigned)((V + fx::TS - 1) / fx::TS);
     {
       ProfScope ps("fermion_force", st);
-      s = fx::launch_fx_links(V, U, T, ffc::SLOTS, 0, status, st);
+      s = fx::launch_fx_links(V, U, T, ffc::SLOTS, 0, hd, st);
     }
     if (!s) {
       ProfScope ps("fermion_force", st);

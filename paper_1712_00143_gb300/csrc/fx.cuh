@@ -252,25 +252,34 @@ enum : int { FX_NOT_UNITARY = 1, FX_AWAY = 2, FX_RANGE = 4 };
 // them, would be known to 2^-58 absolute where FP64 keeps 2^-53 relative.
 __device__ __forceinline__ bool usable(const int* status) { return __ldcg(status) == FX_AWAY; }
 
-// What a call's scratch starts with where the integer kernels may leave single
-// results to the FP64 ones: the status word, and the count of those marked.
+// What a call's scratch starts with: the status word, the count of single
+// results that the integer kernels leave to the FP64 ones, and the counts of
+// links within 3 2^-6 and 3 2^-5 of a diagonal matrix of 1, -1, i, -i.
 struct Header {
   int status;
   unsigned long long marked;
+  unsigned long long near[2];
 };
+enum : int { ANY_LINKS = -1, NEAR_6 = 0, NEAR_5 = 1 };
+// Whether the integer kernels run.  Where more than half of the links are near
+// (at the distance at which a routine marks its results) they would leave most
+// of the work to the FP64 kernels anyway.
+__device__ __forceinline__ bool serve(const Header* hd, int which, long long V) {
+  return usable(&hd->status) && (which == ANY_LINKS || (long long)__ldcg(&hd->near[which < 0 ? 0 : which]) <= 2 * V);
+}
 __device__ __forceinline__ void mark(Header* hd, long long* __restrict__ list, long long cap, long long item) {
   const unsigned long long n = atomicAdd(&hd->marked, 1ull);
   if ((long long)n < cap) list[n] = item;
 }
 // The FP64 kernels do the whole field when the integer kernels may not, or have
 // marked more results than the list holds.
-__device__ __forceinline__ bool all_fp64(const Header* hd, long long cap) {
-  return !usable(&hd->status) || (long long)__ldcg(&hd->marked) > cap;
+__device__ __forceinline__ bool all_fp64(const Header* hd, int which, long long V, long long cap) {
+  return !serve(hd, which, V) || (long long)__ldcg(&hd->marked) > cap;
 }
 
 // Fixed-point copy of the thin links [V][4][3][3] into slots slot0 + mu of a
-// field with `slots` slots, and *status (fx.cu).
-int launch_fx_links(long long V, const double2* U, int4* out, int slots, int slot0, int* status, cudaStream_t st);
+// field with `slots` slots, and *hd (fx.cu).
+int launch_fx_links(long long V, const double2* U, int4* out, int slots, int slot0, Header* hd, cudaStream_t st);
 
 }  // namespace fx
 }  // namespace stag

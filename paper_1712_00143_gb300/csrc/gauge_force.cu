@@ -99,7 +99,7 @@ __device__ __forceinline__ M3 staple(const double2* __restrict__ U, const Dims& 
 // not serve (fx::all_fp64), in grids that return at once otherwise.
 __global__ void __launch_bounds__(128) k_gf_staples(Dims d, long long V, const double2* __restrict__ U,
                                                     double2* __restrict__ T, const fx::Header* hd, long long cap) {
-  if (!fx::all_fp64(hd, cap)) return;
+  if (!fx::all_fp64(hd, fx::NEAR_5, V, cap)) return;
   for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < 24 * V;
        idx += (long long)gridDim.x * blockDim.x) {
     const int k = (int)(idx / V);  // mu * 6 + (other direction index) * 2 + sign
@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(128) k_gauge_force_reuse(Dims d, long long V, 
                                                            const double2* __restrict__ T, double2* __restrict__ F,
                                                            double beta, double cpl, double crt, double cpg,
                                                            const fx::Header* hd, long long cap) {
-  if (!fx::all_fp64(hd, cap)) return;
+  if (!fx::all_fp64(hd, fx::NEAR_5, V, cap)) return;
   for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < 4 * V;
        idx += (long long)gridDim.x * blockDim.x) {
     const int mu = (int)(idx / V);
@@ -223,11 +223,11 @@ __global__ void __launch_bounds__(128) k_gauge_force_reuse(Dims d, long long V, 
 // The links that k_gauge_force_fx has marked (its header says which), in FP64
 // without a table: eight lanes per link, six of which take one (nu, s) each --
 // 34 products of a chain of 204, which one thread would take 0.6 ms for.
-__global__ void __launch_bounds__(128) k_gauge_force_marked(Dims d, const double2* __restrict__ U,
+__global__ void __launch_bounds__(128) k_gauge_force_marked(Dims d, long long V, const double2* __restrict__ U,
                                                             const long long* __restrict__ list, double2* __restrict__ F,
                                                             double beta, double cpl, double crt, double cpg,
                                                             const fx::Header* hd, long long cap) {
-  if (fx::all_fp64(hd, cap)) return;
+  if (fx::all_fp64(hd, fx::NEAR_5, V, cap)) return;
   const long long n = (long long)__ldcg(&hd->marked);
   const int o = threadIdx.x & 7, per = gridDim.x * 16;
   for (long long i0 = blockIdx.x * 16 + (threadIdx.x >> 5) * 4; i0 < n; i0 += per) {  // (a warp's four links)
@@ -263,8 +263,8 @@ __device__ __forceinline__ int fslot(int mu, int nu, int s) {
 // takes 32 sites, its warp w the six staples of mu = w.  T is stored as the
 // adjoint of the path walked the other way, A B C with A or C daggered.
 __global__ void __launch_bounds__(128, 3) k_gf_staples_fx(Dims d, long long V, int4* __restrict__ T,
-                                                          const int* __restrict__ status) {
-  if (!fx::usable(status)) return;
+                                                          const fx::Header* hd) {
+  if (!fx::serve(hd, fx::NEAR_5, V)) return;
   const int x = blockIdx.x * fx::TS + (threadIdx.x & 31);
   const int mu = threadIdx.x >> 5;
   if (x >= V) return;
@@ -319,7 +319,7 @@ struct ForceCoef {
 __global__ void __launch_bounds__(128, 3) k_gauge_force_fx(Dims d, long long V, const int4* __restrict__ T,
                                                            fx::Header* hd, long long* __restrict__ list, long long cap,
                                                            double2* __restrict__ F, ForceCoef cf) {
-  if (!fx::usable(&hd->status)) return;
+  if (!fx::serve(hd, fx::NEAR_5, V)) return;
   extern __shared__ __align__(16) unsigned char gf_sm[];
   long long(*S)[128] = (long long(*)[128])gf_sm;  // [18][128]
   long long(*lone)[128] = S + 18;                  // a group's rectangle 3
@@ -497,8 +497,9 @@ extern "C" int stag_gauge_force(const int dims[4], const void* thin, void* force
   cudaStream_t st = (cudaStream_t)stream;
   // stream-ordered scratch: the FP64 staple table (24 of 32 matrix slots per
   // site, 4608 B), or the fixed-point field (28 matrices, 4032 B) and the list of
-  // marked links (up to one in 64), whichever form runs
-  const long long cap = V / 16;
+  // marked links (up to one in four: one by one they take 2.2 times as long as
+  // with the table), whichever form runs
+  const long long cap = V;
   const size_t tbytes = (size_t)V * 32 * 9 * sizeof(double2), fbytes = fx::field_bytes(V, gf::SLOTS);
   const size_t lbytes = fbytes + (size_t)cap * sizeof(long long);
   char* scratch = nullptr;
@@ -531,11 +532,11 @@ extern "C" int stag_gauge_force(const int dims[4], const void* thin, void* force
     const unsigned tiles = (unsigned)((V + fx::TS - 1) / fx::TS);
     {
       ProfScope ps("gauge_force", st);
-      s = fx::launch_fx_links(V, U, Tf, gf::SLOTS, gf::U0, &hd->status, st);
+      s = fx::launch_fx_links(V, U, Tf, gf::SLOTS, gf::U0, hd, st);
     }
     if (!s) {
       ProfScope ps("gauge_force", st);
-      gf::k_gf_staples_fx<<<tiles, 128, 0, st>>>(d, V, Tf, &hd->status);
+      gf::k_gf_staples_fx<<<tiles, 128, 0, st>>>(d, V, Tf, hd);
       s = last_launch_status();
     }
     if (!s) {
@@ -548,7 +549,7 @@ extern "C" int stag_gauge_force(const int dims[4], const void* thin, void* force
     if (!s) {
       ProfScope ps("gauge_force", st);
       const long long want = (cap + 15) / 16;
-      gf::k_gauge_force_marked<<<beside_grid(want), 128, 0, st>>>(d, U, list, (double2*)force, beta, c_pl, c_rt, c_pg, hd, cap);
+      gf::k_gauge_force_marked<<<beside_grid(want), 128, 0, st>>>(d, V, U, list, (double2*)force, beta, c_pl, c_rt, c_pg, hd, cap);
       s = last_launch_status();
     }
   }

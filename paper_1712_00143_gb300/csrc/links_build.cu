@@ -65,7 +65,7 @@ __device__ __forceinline__ void st(double2* __restrict__ out, long long link, co
 __global__ void __launch_bounds__(128) k_build_links(Dims d, long long V, const double2* __restrict__ U,
                                                      double2* __restrict__ F, double2* __restrict__ Lk, double c1,
                                                      double cst, double c3, const fx::Header* hd, long long cap) {
-  if (hd && !fx::all_fp64(hd, cap)) return;
+  if (hd && !fx::all_fp64(hd, fx::NEAR_6, V, cap)) return;
   for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < 4 * V;
        idx += (long long)gridDim.x * blockDim.x) {
     const int mu = (int)(idx / V);
@@ -75,11 +75,11 @@ __global__ void __launch_bounds__(128) k_build_links(Dims d, long long V, const 
   }
 }
 // The fat and Naik links that k_build_links_fx has marked, one thread each.
-__global__ void __launch_bounds__(128) k_build_marked(Dims d, const double2* __restrict__ U,
+__global__ void __launch_bounds__(128) k_build_marked(Dims d, long long V, const double2* __restrict__ U,
                                                       const long long* __restrict__ list, double2* __restrict__ F,
                                                       double2* __restrict__ Lk, double c1, double cst, double c3,
                                                       const fx::Header* hd, long long cap) {
-  if (fx::all_fp64(hd, cap)) return;
+  if (fx::all_fp64(hd, fx::NEAR_6, V, cap)) return;
   const long long n = (long long)__ldcg(&hd->marked);
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const long long at = __ldcg(list + i), link = at >> 1;
@@ -114,7 +114,7 @@ template <bool FAT>
 __global__ void __launch_bounds__(128, FAT ? 2 : 3) k_build_links_fx(Dims d, long long V, const int4* __restrict__ U,
                                                         fx::Header* hd, long long* __restrict__ list, long long cap,
                                                         double2* __restrict__ out, fx::Coef c1, fx::Coef cst, int k) {
-  if (!fx::usable(&hd->status)) return;
+  if (!fx::serve(hd, fx::NEAR_6, V)) return;
   __shared__ double2 sm[fx::TS * fx::SITE_W];
   const long long x0 = (long long)blockIdx.x * fx::TS;
   const int ns = (int)(V - x0 < fx::TS ? V - x0 : fx::TS);
@@ -194,7 +194,7 @@ extern "C" int stag_build_links(const int dims[4], const void* thin, void* fat, 
   if (overlap(thin, fat) || overlap(thin, lng) || overlap(fat, lng)) return STAG_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
   const double2* U = (const double2*)thin;
-  const long long cap = V / 16;  // marked results that the list holds
+  const long long cap = 4 * V;  // marked results that the list holds (of 8 V)
   auto fp64 = [&](const fx::Header* hd) {
     ProfScope ps("links", st);
     const long long want = (4 * V + 127) / 128;
@@ -210,7 +210,7 @@ extern "C" int stag_build_links(const int dims[4], const void* thin, void* fat, 
     return fp64(nullptr);
   std::frexp(big, &k);
   std::frexp(big3, &k3);
-  // the fixed-point copy of the links (576 B per site) in stream-ordered
+  // the fixed-point copy of the links and the list (608 B per site) in stream-ordered
   // scratch; without room for it the FP64 kernel does the work
   const size_t fbytes = fx::field_bytes(V, 4);
   char* scratch = nullptr;
@@ -223,10 +223,10 @@ extern "C" int stag_build_links(const int dims[4], const void* thin, void* fat, 
   long long* list = (long long*)(scratch + 256 + fbytes);
   const unsigned tiles = (unsigned)((V + fx::TS - 1) / fx::TS);
   const fx::Coef none{0, 0};
-  int s = cuda_status(cudaMemsetAsync(hd, 0, sizeof(*hd), st));
-  if (!s) {
+  int s;
+  {
     ProfScope ps("links", st);
-    s = fx::launch_fx_links(V, U, Uf, 4, 0, &hd->status, st);
+    s = fx::launch_fx_links(V, U, Uf, 4, 0, hd, st);
   }
   if (!s) {
     ProfScope ps("links", st);
@@ -243,7 +243,7 @@ extern "C" int stag_build_links(const int dims[4], const void* thin, void* fat, 
   if (!s) {
     ProfScope ps("links", st);
     const long long want = (cap + 127) / 128;
-    lb::k_build_marked<<<beside_grid(want), 128, 0, st>>>(d, U, list, (double2*)fat, (double2*)lng, c1, c_staple, c3, hd, cap);
+    lb::k_build_marked<<<beside_grid(want), 128, 0, st>>>(d, V, U, list, (double2*)fat, (double2*)lng, c1, c_staple, c3, hd, cap);
     s = last_launch_status();
   }
   if (!s) s = fp64(hd);

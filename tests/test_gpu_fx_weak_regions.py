@@ -78,3 +78,22 @@ def test_small_entries_of_built_links(eps, shape, sign):
         assert np.linalg.norm(got - want) <= 1e-15 * np.linalg.norm(want)
         got, want = got[deep][..., off], want[deep][..., off]
         assert np.linalg.norm(got - want) <= 1e-14 * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("eps", [0.02, 0.05, 0.08, 0.1, 0.15])
+def test_weak_fields_on_every_route(eps):
+    """Whole lattices from all links near 1 (FP64 at once) through a share of them (marked, done one by one) to
+    none; a force's error against the reference's own, 4e-15 of the sum of its terms, and its own size."""
+    import paper_1712_00143_gb300 as stag
+
+    dims = (4, 6, 10, 6)
+    thin = synth.gauge_field(dims, eps, 1104, return_thin=True)[2]
+    F = stag.stag_gauge_force(dims, dev(thin), 6.0, *COEF)
+    fat, lng = stag.stag_build_links(dims, dev(thin))
+    torch.cuda.synchronize()
+    want = ogf.force(thin, dims, 6.0, *COEF)
+    assert np.linalg.norm(F.cpu().numpy() - want) <= 5e-16 * np.linalg.norm(want)
+    off = ~np.eye(3, dtype=bool)
+    for got, ref in ((fat.cpu().numpy(), olk.fat_links(thin, dims)), (lng.cpu().numpy(), olk.naik_links(thin, dims))):
+        assert np.linalg.norm(got - ref) <= 4e-16 * np.linalg.norm(ref)
+        assert np.linalg.norm((got - ref)[..., off]) <= 6e-16 * np.linalg.norm(ref[..., off])
