@@ -252,6 +252,17 @@ enum : int { FX_NOT_UNITARY = 1, FX_AWAY = 2, FX_RANGE = 4 };
 // them, would be known to 2^-58 absolute where FP64 keeps 2^-53 relative.
 __device__ __forceinline__ bool usable(const int* status) { return __ldcg(status) == FX_AWAY; }
 
+// The distance of m from the diagonal matrices of 1, -1, i, -i, in units of 2^-30.
+__device__ __forceinline__ int away(const FM& m) {
+  int d = 0;
+#pragma unroll
+  for (int e = 0; e < 9; ++e) {
+    const int re = abs(m.h[2 * e]), im = abs(m.h[2 * e + 1]);
+    d = max(d, e % 4 == 0 ? min(re, im) : max(re, im));
+  }
+  return d;
+}
+
 // What a call's scratch starts with: the status word, the count of single
 // results that the integer kernels leave to the FP64 ones, and the counts of
 // links within 3 2^-6 and 3 2^-5 of a diagonal matrix of 1, -1, i, -i.

@@ -440,13 +440,12 @@ __global__ void __launch_bounds__(128, 3) k_gauge_force_fx(Dims d, long long V, 
     fx::FM s;
 #pragma unroll
     for (int e = 0; e < 18; ++e) fx::split1(S[e][tid], s.h[e], s.l[e]);
-    const fx::FM u = fx::ld<SLOTS>(T, U0 + mu, x);
     long long w[18];
     fx::clear(w);
-    fx::mac(w, u, s);
+    fx::mac(w, fx::ld<SLOTS>(T, U0 + mu, x), s);
     const long long tr = w[1] + w[9] + w[17];
-    long long size = 0;  // the largest off-diagonal entry, and
-    int away = 0;        // the link's distance from the diagonal matrices of 1, -1, i, -i
+    int size = 0;  // the largest off-diagonal entry, in units of 2^-28
+    auto top = [](long long v) { return abs((int)(v >> 32)); };
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       const long long di = 3 * w[8 * i + 1] - tr;
@@ -454,12 +453,10 @@ __global__ void __launch_bounds__(128, 3) k_gauge_force_fx(Dims d, long long V, 
       const int r = i == 2 ? 1 : 0, c = i == 0 ? 1 : 2;  // entries 01, 02, 12
       const int e = 2 * (3 * r + c), f = 2 * (3 * c + r);
       off[i] = make_double2(cf.off * fx::double_of(w[e] - w[f], 0), cf.off * fx::double_of(w[e + 1] + w[f + 1], 0));
-      size = max(size, max(max(llabs(w[e]), llabs(w[e + 1])), max(llabs(w[f]), llabs(w[f + 1]))));
-      size = max(size, llabs(di) >> 1);  // (a third of it is the force's)
-      away = max(away, max(max(abs(u.h[e]), abs(u.h[e + 1])), max(abs(u.h[f]), abs(u.h[f + 1]))));
-      away = max(away, min(abs(u.h[8 * i]), abs(u.h[8 * i + 1])));
+      size = max(size, max(max(top(w[e]), top(w[e + 1])), max(top(w[f]), top(w[f + 1]))));
+      size = max(size, top(di) >> 1);  // (a third of it is the force's)
     }
-    if (away < 3 << 25 && size < 3LL << 54) fx::mark(hd, list, cap, 4LL * x + mu);
+    if (size < 3 << 22 && fx::away(fx::ld<SLOTS>(T, U0 + mu, x)) < 3 << 25) fx::mark(hd, list, cap, 4LL * x + mu);
   }
   __syncthreads();  // the sums' memory becomes the output's
   if (lane < ns) {
@@ -549,7 +546,7 @@ extern "C" int stag_gauge_force(const int dims[4], const void* thin, void* force
     if (!s) {
       ProfScope ps("gauge_force", st);
       const long long want = (cap + 15) / 16;
-      gf::k_gauge_force_marked<<<beside_grid(want), 128, 0, st>>>(d, V, U, list, (double2*)force, beta, c_pl, c_rt, c_pg, hd, cap);
+      gf::k_gauge_force_marked<<<beside_grid(want, 4), 128, 0, st>>>(d, V, U, list, (double2*)force, beta, c_pl, c_rt, c_pg, hd, cap);
       s = last_launch_status();
     }
   }

@@ -204,12 +204,12 @@ int launch_cg_loop(stag_lattice_s* lat, Spinor<P> p, Spinor<P> p2, Spinor<P> t, 
 // SMs of the current device (152 where it cannot be asked).
 int sm_count();
 // Grid of an FP64 kernel that is launched beside the integer kernels and returns
-// at once unless they do not serve: n blocks of work, grid-stride.  32 blocks
-// per SM cost 3 us when they return at once, and leave the last wave short when
-// they do not (with 8 per SM some blocks had nine parts and some eight: links at
-// 24^4 5 %, gauge force 3 % slower than one block per part).
-inline unsigned beside_grid(long long n) {
-  const long long most = 32LL * sm_count();
+// at once unless they do not serve: n blocks of work, grid-stride.  Blocks that
+// return cost a launch 4 us at 8 per SM, 8 at 16 and 14 at 32 (few fit at a time:
+// their registers); fewer blocks cost the FP64 kernels a last wave that is
+// longer (1 % at 8, half of it at 16).
+inline unsigned beside_grid(long long n, int per_sm = 16) {
+  const long long most = (long long)per_sm * sm_count();
   return (unsigned)(n < most ? n : most);
 }
 // Sites per parity up to which the fixed-point FP64 operator runs one hop per

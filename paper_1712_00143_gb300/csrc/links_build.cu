@@ -124,12 +124,6 @@ __global__ void __launch_bounds__(128, FAT ? 2 : 3) k_build_links_fx(Dims d, lon
     double2* o = sm + s * fx::SITE_W + mu * 9;
     long long acc[18];
     fx::clear(acc);
-    int away = 0;  // the link's distance from the diagonal matrices of 1, -1, i, -i
-    auto look = [&](const fx::FM& u) {
-#pragma unroll
-      for (int e = 0; e < 9; ++e)
-        away = max(away, e % 4 == 0 ? min(abs(u.h[2 * e]), abs(u.h[2 * e + 1])) : max(abs(u.h[2 * e]), abs(u.h[2 * e + 1])));
-    };
     if constexpr (FAT) {
       // t = 0..5: direction nu, upper (U_nu(x) U_mu(x+nu) U_nu(x+mu)^dag) and
       // lower (U_nu(x-nu)^dag U_mu(x-nu) U_nu(x-nu+mu)) staple
@@ -145,26 +139,24 @@ __global__ void __launch_bounds__(128, FAT ? 2 : 3) k_build_links_fx(Dims d, lon
         fx::mac(acc, a, c);
       }
       const fx::FM u = fx::ld<4>(U, mu, p.lex);
-      look(u);
 #pragma unroll
       for (int e = 0; e < 18; ++e)  // the staple sum, of norm up to 6, enters as an eighth
         acc[e] = fx::scaled(c1, fx::join1(u.h[e], u.l[e])) + fx::scaled(cst, (acc[e] + 4) >> 3);
     } else {
       // U_mu(x) U_mu(x+mu) U_mu(x+2mu)
-      fx::FM a = fx::ld<4>(U, mu, p.lex);
-      look(a);
-      a = fx::mul(a, fx::ld<4>(U, mu, pm.lex));
+      fx::FM a = fx::mul(fx::ld<4>(U, mu, p.lex), fx::ld<4>(U, mu, pm.lex));
       fx::mac(acc, a, fx::ld<4>(U, mu, fx::next_lex(d, pm, mu, 1)));
 #pragma unroll
       for (int e = 0; e < 18; ++e) acc[e] = fx::scaled(c1, acc[e]);
     }
-    long long size = 0;  // the largest off-diagonal entry
+    int size = 0;  // the largest off-diagonal entry, in units of 2^-28
 #pragma unroll
     for (int e = 0; e < 9; ++e) {
       o[e] = make_double2(fx::double_of(acc[2 * e], k), fx::double_of(acc[2 * e + 1], k));
-      if (e % 4) size = max(size, max(llabs(acc[2 * e]), llabs(acc[2 * e + 1])));
+      if (e % 4) size = max(size, max(abs((int)(acc[2 * e] >> 32)), abs((int)(acc[2 * e + 1] >> 32))));
     }
-    if (away < 3 << 24 && size < 3LL << 53) fx::mark(hd, list, cap, (4LL * p.lex + mu) * 2 + (FAT ? 0 : 1));
+    if (size < 3 << 21 && fx::away(fx::ld<4>(U, mu, p.lex)) < 3 << 24)
+      fx::mark(hd, list, cap, (4LL * p.lex + mu) * 2 + (FAT ? 0 : 1));
   }
   __syncthreads();
   for (int i = threadIdx.x; i < ns * 36; i += 128) out[x0 * 36 + i] = sm[(i / 36) * fx::SITE_W + i % 36];
@@ -243,7 +235,7 @@ extern "C" int stag_build_links(const int dims[4], const void* thin, void* fat, 
   if (!s) {
     ProfScope ps("links", st);
     const long long want = (cap + 127) / 128;
-    lb::k_build_marked<<<beside_grid(want), 128, 0, st>>>(d, V, U, list, (double2*)fat, (double2*)lng, c1, c_staple, c3, hd, cap);
+    lb::k_build_marked<<<beside_grid(want, 4), 128, 0, st>>>(d, V, U, list, (double2*)fat, (double2*)lng, c1, c_staple, c3, hd, cap);
     s = last_launch_status();
   }
   if (!s) s = fp64(hd);
