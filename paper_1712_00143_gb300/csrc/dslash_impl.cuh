@@ -507,10 +507,12 @@ int tune_dslash(stag_lattice_s* lat, cudaStream_t st) {
     return STAG_ECUDA;
   }
   const int reps = 5;
+  // (few sites with fixed-point links run in one shape of their own)
+  const int shapes = P == 64 && L.fixed && lat->g.Vh <= kFewSites ? 1 : kNumShapes;
   float best[2] = {1e30f, 1e30f};
   int pick[2] = {0, 0};
   for (int kind = 0; kind < 2 && !s; ++kind) {
-    for (int v = 0; v < kNumShapes && !s; ++v) {
+    for (int v = 0; v < shapes && !s; ++v) {
       for (int it = -2; it < reps && !s; ++it) {
         if (it == 0) s = cuda_status(cudaEventRecord(e0, st));
         if (s) break;
