@@ -534,13 +534,13 @@ int stag_gauge_force(const int dims[4], const void* thin, void* force, double be
 int stag_fermion_force(const int dims[4], const void* thin, int n_terms, const void* x_even, const void* y_odd,
                        const double* alpha, double c1, double c_staple, double c3, void* force, void* stream);
 
-/* Check of the tcgen05 tensor-core path on the current GPU (the network's
- * layers feed the tensor cores from registers with mma.sync, whose products
- * and sums agree with it bit for bit): one tile of bfloat16 products with FP32 accumulation in tensor memory, 9 accumulated steps, compared
- * with the same sums on the CUDA cores.  *max_rel_err: max |difference| /
- * max |reference| (0 expected: the test values are exact in both).
- * STAG_ETIMEOUT if a bounded wait gave up.  Synchronous.  No counterpart in
- * the paper, which predates these tensor cores. */
+/* Check of the tensor cores on the current GPU against the CUDA cores: the
+ * register fragments of the network's layers and weight gradients (mma.sync,
+ * both weight forms, the splits into bfloat16 parts, the products over sites),
+ * and one tile of tcgen05 products accumulated in tensor memory.  *max_rel_err:
+ * max |difference| / max |reference| (0 expected: the test values' sums are
+ * exact).  STAG_ETIMEOUT if a bounded wait gave up.  Synchronous.  No
+ * counterpart in the paper, which predates these tensor cores. */
 int stag_tc_selftest(double* max_rel_err);
 
 /* Testing aid for this handle's mixed-precision solves on small lattices, whose

@@ -565,20 +565,35 @@ int stag_net_loss_grad(stag_net_t n, stag_lattice_t lat, const void* r, const vo
 
 int stag_tc_selftest(double* max_rel_err) {
   if (!max_rel_err) return STAG_EINVAL;
+  // {difference (relative), finished} of tcgen05; {difference, largest} of the layers' fragments; weights
+  constexpr int NW = NET_NDIR * 256;
   float* d = nullptr;
-  if (cudaMalloc(&d, 2 * sizeof(float)) != cudaSuccess) {
+  if (cudaMalloc(&d, 4 * sizeof(float) + NW * sizeof(__nv_bfloat16)) != cudaSuccess) {
     cudaGetLastError();
     return STAG_ENOMEM;
   }
+  __nv_bfloat16* W = (__nv_bfloat16*)(d + 4);
+  std::vector<__nv_bfloat16> w(NW);
+  for (int i = 0; i < NW; ++i)
+    w[i] = __float2bfloat16((float)(((i >> 8) * 3 + ((i >> 4) & 15) * 11 + (i & 15) * 7) % 13 - 6) * 0.0625f);
+  int s = cuda_status(cudaMemcpy(W, w.data(), NW * sizeof(__nv_bfloat16), cudaMemcpyHostToDevice));
   cudaFuncSetAttribute(k_tc_selftest, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_BYTES);
-  count_launch();
-  k_tc_selftest<<<1, 128, tc::SMEM_BYTES>>>(d);
-  int s = last_launch_status();
-  float h[2] = {0.f, 0.f};
+  if (!s) {
+    count_launch();
+    k_tc_selftest<<<1, 128, tc::SMEM_BYTES>>>(d);
+    s = last_launch_status();
+  }
+  if (!s) {
+    count_launch();
+    k_mma_selftest<<<1, 32>>>(W, d + 2);
+    s = last_launch_status();
+  }
+  float h[4] = {0.f, 0.f, 0.f, 0.f};
   if (!s) s = cuda_status(cudaMemcpy(h, d, sizeof(h), cudaMemcpyDeviceToHost));
   cudaFree(d);
   if (s) return s;
-  *max_rel_err = h[0];
+  const float mma = h[3] > 0.f ? h[2] / h[3] : 1.f;
+  *max_rel_err = h[0] > mma ? h[0] : mma;
   return h[1] == 1.f ? STAG_OK : STAG_ETIMEOUT;
 }
 

@@ -691,4 +691,114 @@ __global__ void __launch_bounds__(32 * nm::TW, 2)
   }
 }
 
+// The fragments above (weights, splits, products, transposes, outer products),
+// one warp, on values whose sums are exact in FP32, against the CUDA cores:
+// out = {max |difference|, max |reference|}.
+__global__ void __launch_bounds__(32) k_mma_selftest(const __nv_bfloat16* __restrict__ W, float* out) {
+  using namespace nm;
+  __shared__ uint4 sB[2][NET_NDIR * 32];
+  stage_weights(sB[0], W, 0);
+  stage_weights(sB[1], W, 1);
+  __syncthreads();
+  const int lane = threadIdx.x, g = lane >> 2, t = lane & 3;
+  // multiples of 2^-12 below 1 (fine) or of 1/8
+  auto val = [](int d, int site, int c, int i, int im, bool fine) {
+    const int h = (d * 7 + site * 13 + c * 5 + i * 3 + im) % 15 - 7;
+    return (float)h * 0.125f + (fine ? (float)((site + c + d + im) % 5 - 2) * (1.f / 4096.f) : 0.f);
+  };
+  auto pairs = [&](int d, bool fine) {
+    Pairs v;
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+      for (int e = 0; e < 2; ++e)
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+          v.v[q][e][i] = make_float2(val(d, g, 2 * t + 8 * q + e, i, 0, fine), val(d, g, 2 * t + 8 * q + e, i, 1, fine));
+    return v;
+  };
+  float err = 0.f, most = 0.f;
+  auto meet = [&](float got, float want) {
+    err = fmaxf(err, fabsf(got - want));
+    most = fmaxf(most, fabsf(want));
+  };
+  for (int tr = 0; tr < 2; ++tr) {
+    float acc[3][2][4] = {};
+    for (int d = 0; d < NET_NDIR; ++d) {
+      const Pairs v = pairs(d, true);
+      const uint4 b = sB[tr][d * 32 + lane];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        uint32_t h[4], l[4];
+        tc::split2(v.v[0][0][i].x, v.v[0][1][i].x, h[0], l[0]);
+        tc::split2(v.v[0][0][i].y, v.v[0][1][i].y, h[1], l[1]);
+        tc::split2(v.v[1][0][i].x, v.v[1][1][i].x, h[2], l[2]);
+        tc::split2(v.v[1][0][i].y, v.v[1][1][i].y, h[3], l[3]);
+        float s[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+        mma(s[0], l[0], l[1], l[2], l[3], b.x, b.y);
+        mma(s[1], l[0], l[1], l[2], l[3], b.z, b.w);
+        mma(s[0], h[0], h[1], h[2], h[3], b.x, b.y);
+        mma(s[1], h[0], h[1], h[2], h[3], b.z, b.w);
+        add(acc[i], s);
+      }
+    }
+    for (int i = 0; i < 3; ++i)
+      for (int q = 0; q < 2; ++q)
+        for (int k = 0; k < 4; ++k) {
+          const int c = 2 * t + 8 * q + (k & 1), im = k >> 1;
+          float ref = 0.f;
+          for (int d = 0; d < NET_NDIR; ++d) {
+            const int dd = d == 0 ? 0 : ((d & 1) ? d + 1 : d - 1);
+            for (int cp = 0; cp < 16; ++cp) {
+              const float w = !tr ? __bfloat162float(W[(d * 16 + c) * 16 + cp])
+                                  : (d ? -1.f : 1.f) * __bfloat162float(W[(dd * 16 + cp) * 16 + c]);
+              ref += w * val(d, g, cp, i, im, true);
+            }
+          }
+          meet(acc[i][q][k], ref);
+        }
+  }
+  // sum over the eight sites, colours and (re, im) of a_c h_c'
+  const Pairs a = pairs(2, true);
+  uint32_t o[36];
+  site_operand(pairs(5, false), o);
+  float sum[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    uint32_t r0[3], i0[3], r1[3], i1[3], f[3][4];
+    uint2 q[3][2];
+    split3(a.v[0][0][i].x, a.v[0][1][i].x, r0);
+    split3(a.v[0][0][i].y, a.v[0][1][i].y, i0);
+    split3(a.v[1][0][i].x, a.v[1][1][i].x, r1);
+    split3(a.v[1][0][i].y, a.v[1][1][i].y, i1);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      f[k][0] = trans(r0[k]);
+      f[k][1] = trans(r1[k]);
+      f[k][2] = trans(i0[k]);
+      f[k][3] = trans(i1[k]);
+#pragma unroll
+      for (int nt = 0; nt < 2; ++nt) q[k][nt] = make_uint2(o[((k * 3 + i) * 2 + nt) * 2], o[((k * 3 + i) * 2 + nt) * 2 + 1]);
+    }
+    outer(sum, f, q);
+  }
+  for (int nt = 0; nt < 2; ++nt)
+    for (int k = 0; k < 4; ++k) {
+      const int c = (lane >> 2) + 8 * (k >> 1), cp = 8 * nt + 2 * (lane & 3) + (k & 1);
+      float ref = 0.f;
+      for (int site = 0; site < 8; ++site)
+        for (int i = 0; i < 3; ++i)
+          for (int im = 0; im < 2; ++im) ref += val(2, site, c, i, im, true) * val(5, site, cp, i, im, false);
+      meet(sum[nt][k], ref);
+    }
+  for (int w = 16; w > 0; w >>= 1) {
+    err = fmaxf(err, __shfl_xor_sync(0xffffffffu, err, w));
+    most = fmaxf(most, __shfl_xor_sync(0xffffffffu, most, w));
+  }
+  if (lane == 0) {
+    out[0] = err;
+    out[1] = most;
+  }
+}
+
 }  // namespace stag

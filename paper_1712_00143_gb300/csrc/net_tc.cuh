@@ -2,7 +2,7 @@
 // cores on this GPU (stag_tc_selftest): 384 x 16 rows of bfloat16 operands,
 // nine accumulated K = 16 steps into tensor memory, against the CUDA cores.
 // The network's layers once ran in this form; they now take mma.sync straight
-// from registers (net_mma.cuh says why) with the same results.
+// from registers (net_mma.cuh says why).
 //
 // Shared-memory operand layout (no swizzle, K-major): 8-row x 16-byte core
 // matrices stored as 128 contiguous bytes; the two 16-byte K halves of a row
