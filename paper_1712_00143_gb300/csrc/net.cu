@@ -264,8 +264,9 @@ static int layer_fwd(const NetRun& R, int l, cudaStream_t st) {
     k_net_layer_1to16<true><<<grid_groups(R.Vh, 8, 1 << 20), 256, 0, st>>>(R.ng, in, pre, out, W, b);
   } else if (ci == 16 && co == 16 && gate) {
     if (((uintptr_t)in & 15u) != 0) return STAG_EINVAL;  // records are read as 16-byte words
-    TRYN(cuda_status(cudaFuncSetAttribute(k_net_layer_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, nm::FWD_SMEM)));
-    k_net_layer_mma<<<grid_groups(R.Vh, nm::FW, 2 * sm_count()), 32 * nm::FW, nm::FWD_SMEM, st>>>(R.ng, in, pre, out, W, b);
+    auto layer = R.training ? k_net_layer_mma<true> : k_net_layer_mma<false>;
+    TRYN(cuda_status(cudaFuncSetAttribute(layer, cudaFuncAttributeMaxDynamicSharedMemorySize, nm::FWD_SMEM)));
+    layer<<<grid_groups(R.Vh, nm::FW, 2 * sm_count()), 32 * nm::FW, nm::FWD_SMEM, st>>>(R.ng, in, pre, out, W, b);
   } else if (ci == 16 && co == 1 && !gate) {
     // one output channel: site-local mix into the directions, then one
     // transport per direction, for the even sites the prediction is read on

@@ -19,10 +19,12 @@
 // The transports enter as two bfloat16 parts (16 bits), products and sums are
 // FP32.  The unit truncates its sums, and over a chain of them that shrinks
 // every result by the same few 2^-22, which a gradient, a sum over all sites,
-// keeps while the sites' own errors average out.  So a product starts from zero
-// for each direction, the low parts first, and is added with rounding outside:
-// gradient at 16 x 20 x 12 x 24 3.0e-7 from the 64-bit one against 3.4e-6, for
-// 542 in place of 524 us per forward pass at 24^4.
+// keeps while the sites' own errors average out.  So in training a product
+// starts from zero for each direction, the low parts first, and is added with
+// rounding outside: gradient at 16 x 20 x 12 x 24 3.0e-7 from the 64-bit one
+// against 3.4e-6, for 3.5 % more time per layer.  Applied as a preconditioner
+// the network's values are as good either way (4.2e-6 and 4.5e-6), and the
+// products are summed in one chain.
 #pragma once
 #include "net_tc.cuh"
 
@@ -284,8 +286,9 @@ constexpr int ADJ_SMEM = NET_NDIR * 32 * 16 + AW * (DWF * 4 + 36 * 32 * 4);
 
 }  // namespace nm
 
-// The forward layer.  GATE: hout = pre * sigmoid(|pre|^2 - b_c), pre stored if
-// wanted (training); a warp takes every nwarps-th group of 8 sites.
+// The forward layer: hout = pre * sigmoid(|pre|^2 - b_c).  TRAIN: pre is stored
+// and the sums are rounded.  A warp takes every nwarps-th group of 8 sites.
+template <bool TRAIN>
 __global__ void __launch_bounds__(32 * nm::FW, 2)
     k_net_layer_mma(NetGeom ng, const float2* __restrict__ hin, float2* __restrict__ pre, float2* __restrict__ hout,
                     const __nv_bfloat16* __restrict__ W, const float* __restrict__ bias) {
@@ -317,12 +320,19 @@ __global__ void __launch_bounds__(32 * nm::FW, 2)
       tc::split2(x0.z, x0.w, h[1], l[1]);
       tc::split2(x1.x, x1.y, h[2], l[2]);
       tc::split2(x1.z, x1.w, h[3], l[3]);
-      float s[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-      mma(s[0], l[0], l[1], l[2], l[3], b.x, b.y);
-      mma(s[1], l[0], l[1], l[2], l[3], b.z, b.w);
-      mma(s[0], h[0], h[1], h[2], h[3], b.x, b.y);
-      mma(s[1], h[0], h[1], h[2], h[3], b.z, b.w);
-      add(acc[i], s);
+      if constexpr (TRAIN) {
+        float s[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+        mma(s[0], l[0], l[1], l[2], l[3], b.x, b.y);
+        mma(s[1], l[0], l[1], l[2], l[3], b.z, b.w);
+        mma(s[0], h[0], h[1], h[2], h[3], b.x, b.y);
+        mma(s[1], h[0], h[1], h[2], h[3], b.z, b.w);
+        add(acc[i], s);
+      } else {
+        mma(acc[i][0], h[0], h[1], h[2], h[3], b.x, b.y);
+        mma(acc[i][1], h[0], h[1], h[2], h[3], b.z, b.w);
+        mma(acc[i][0], l[0], l[1], l[2], l[3], b.x, b.y);
+        mma(acc[i][1], l[0], l[1], l[2], l[3], b.z, b.w);
+      }
     };
     auto done = [&]() {  // the stage has been read by its lane, the slot by the warp: the next direction may come
       __syncwarp();
@@ -379,7 +389,7 @@ __global__ void __launch_bounds__(32 * nm::FW, 2)
         for (int i = 0; i < 3; ++i) h.v[q][e][i] = make_float2(v[i].x * sg, v[i].y * sg);
       }
     if (in) {
-      if (pre) store_pairs(act_ptr(pre, 16, Vh, p, s), t, o);
+      if (TRAIN) store_pairs(act_ptr(pre, 16, Vh, p, s), t, o);
       store_pairs(act_ptr(hout, 16, Vh, p, s), t, h);
     }
   }
