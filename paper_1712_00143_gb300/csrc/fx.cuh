@@ -271,12 +271,15 @@ struct Header {
   unsigned long long marked;
   unsigned long long near[2];
 };
-enum : int { ANY_LINKS = -1, NEAR_6 = 0, NEAR_5 = 1 };
+enum : int { NEAR_6 = 0, NEAR_5 = 1 };
 // Whether the integer kernels run.  Where more than half of the links are near
 // (at the distance at which a routine marks its results) they would leave most
 // of the work to the FP64 kernels anyway.
-__device__ __forceinline__ bool serve(const Header* hd, int which, long long V) {
-  return usable(&hd->status) && (which == ANY_LINKS || (long long)__ldcg(&hd->near[which < 0 ? 0 : which]) <= 2 * V);
+__device__ __forceinline__ bool serve(const Header* hd, int which, long long V, unsigned long long* count = nullptr) {
+  const unsigned long long n = __ldcg(&hd->near[which]);  // (both words are asked for before either is waited for)
+  const bool ok = usable(&hd->status);
+  if (count) *count = n;
+  return ok & ((long long)n <= 2 * V);
 }
 __device__ __forceinline__ void mark(Header* hd, long long* __restrict__ list, long long cap, long long item) {
   const unsigned long long n = atomicAdd(&hd->marked, 1ull);

@@ -198,37 +198,12 @@ __device__ __forceinline__ void store_force(const double2* __restrict__ U, doubl
       f[3 * i + j] = make_double2(k * a.e[3 * i + j].x, k * (a.e[3 * i + j].y - (i == j ? tr3 : 0.0)));
 }
 
-__global__ void __launch_bounds__(128) k_gauge_force_reuse(Dims d, long long V, const double2* __restrict__ U,
-                                                           const double2* __restrict__ T, double2* __restrict__ F,
-                                                           double beta, double cpl, double crt, double cpg,
-                                                           const fx::Header* hd, long long cap) {
-  if (!fx::all_fp64(hd, fx::NEAR_5, V, cap)) return;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < 4 * V;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const int mu = (int)(idx / V);
-    const long long x = idx - (long long)mu * V;
-    const Pos p0 = pos_of(d, x), pp = step(d, p0, mu, 1), pm = step(d, p0, mu, -1);
-    const M3 u_pm = ld(U, pp.lex, mu), u_mm = ld(U, pm.lex, mu);
-    M3 S = zero3();
-#pragma unroll 1
-    for (int nu = 0; nu < 4; ++nu) {
-      if (nu == mu) continue;
-#pragma unroll 1
-      for (int s = -1; s <= 1; s += 2) add_pair<true>(S, U, T, d, p0, pp, pm, u_pm, u_mm, mu, nu, s, cpl, crt, cpg);
-    }
-    store_force(U, F, x, mu, S, beta);
-  }
-}
-
-// The links that k_gauge_force_fx has marked (its header says which), in FP64
-// without a table: eight lanes per link, six of which take one (nu, s) each --
-// 34 products of a chain of 204, which one thread would take 0.6 ms for.
-__global__ void __launch_bounds__(128) k_gauge_force_marked(Dims d, long long V, const double2* __restrict__ U,
-                                                            const long long* __restrict__ list, double2* __restrict__ F,
-                                                            double beta, double cpl, double crt, double cpg,
-                                                            const fx::Header* hd, long long cap) {
-  if (fx::all_fp64(hd, fx::NEAR_5, V, cap)) return;
-  const long long n = (long long)__ldcg(&hd->marked);
+// The links that k_gauge_force_fx has marked (its header says which), without a
+// table: eight lanes per link, six of which take one (nu, s) each -- 34 products
+// of a chain of 204, which one thread would take 0.6 ms for.
+__device__ __forceinline__ void marked_links(const Dims& d, const double2* __restrict__ U, const long long* __restrict__ list,
+                                             long long n, double2* __restrict__ F, double beta, double cpl, double crt,
+                                             double cpg) {
   const int o = threadIdx.x & 7, per = gridDim.x * 16;
   for (long long i0 = blockIdx.x * 16 + (threadIdx.x >> 5) * 4; i0 < n; i0 += per) {  // (a warp's four links)
     const long long i = i0 + ((threadIdx.x & 31) >> 3);
@@ -249,6 +224,34 @@ __global__ void __launch_bounds__(128) k_gauge_force_marked(Dims d, long long V,
         S.e[e].y += __shfl_down_sync(0xffffffffu, S.e[e].y, w, 8);
       }
     if (in && o == 0) store_force(U, F, x, mu, S, beta);
+  }
+}
+
+// The force from the table, or the marked links alone (in a launch of its own
+// that cost small lattices 4 us).
+__global__ void __launch_bounds__(128) k_gauge_force_reuse(Dims d, long long V, const double2* __restrict__ U,
+                                                           const double2* __restrict__ T, double2* __restrict__ F,
+                                                           double beta, double cpl, double crt, double cpg,
+                                                           const fx::Header* hd, const long long* __restrict__ list,
+                                                           long long cap) {
+  if (!fx::all_fp64(hd, fx::NEAR_5, V, cap)) {
+    marked_links(d, U, list, (long long)__ldcg(&hd->marked), F, beta, cpl, crt, cpg);
+    return;
+  }
+  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < 4 * V;
+       idx += (long long)gridDim.x * blockDim.x) {
+    const int mu = (int)(idx / V);
+    const long long x = idx - (long long)mu * V;
+    const Pos p0 = pos_of(d, x), pp = step(d, p0, mu, 1), pm = step(d, p0, mu, -1);
+    const M3 u_pm = ld(U, pp.lex, mu), u_mm = ld(U, pm.lex, mu);
+    M3 S = zero3();
+#pragma unroll 1
+    for (int nu = 0; nu < 4; ++nu) {
+      if (nu == mu) continue;
+#pragma unroll 1
+      for (int s = -1; s <= 1; s += 2) add_pair<true>(S, U, T, d, p0, pp, pm, u_pm, u_mm, mu, nu, s, cpl, crt, cpg);
+    }
+    store_force(U, F, x, mu, S, beta);
   }
 }
 
@@ -515,8 +518,8 @@ extern "C" int stag_gauge_force(const int dims[4], const void* thin, void* force
   const double big = std::fabs(c_pl) * 6 + std::fabs(c_rt) * 18 + std::fabs(c_pg) * 24;
   const double b = std::fabs(beta);
   const bool fixed = big > 0x1p-900 && big < 0x1p900 && (b == 0.0 || (b > 0x1p-50 && b < 0x1p60));
-  int s = cuda_status(cudaMemsetAsync(hd, 0, sizeof(*hd), st));
-  if (fixed && !s) {
+  int s = fixed ? STAG_OK : cuda_status(cudaMemsetAsync(hd, 0, sizeof(*hd), st));
+  if (fixed) {
     int k = 0;
     std::frexp(big, &k);
     gf::ForceCoef cf;
@@ -543,12 +546,6 @@ extern "C" int stag_gauge_force(const int dims[4], const void* thin, void* force
       if (!s) gf::k_gauge_force_fx<<<tiles, 128, smem, st>>>(d, V, Tf, hd, list, cap, (double2*)force, cf);
       if (!s) s = last_launch_status();
     }
-    if (!s) {
-      ProfScope ps("gauge_force", st);
-      const long long want = (cap + 15) / 16;
-      gf::k_gauge_force_marked<<<beside_grid(want, 4), 128, 0, st>>>(d, V, U, list, (double2*)force, beta, c_pl, c_rt, c_pg, hd, cap);
-      s = last_launch_status();
-    }
   }
   if (!s) {
     ProfScope ps("gauge_force", st);
@@ -560,7 +557,7 @@ extern "C" int stag_gauge_force(const int dims[4], const void* thin, void* force
     ProfScope ps("gauge_force", st);
     const long long n = (4 * V + 127) / 128;
     gf::k_gauge_force_reuse<<<fixed ? beside_grid(n) : (unsigned)n, 128, 0, st>>>(d, V, U, T, (double2*)force, beta, c_pl,
-                                                                                   c_rt, c_pg, hd, cap);
+                                                                               c_rt, c_pg, hd, list, cap);
     s = last_launch_status();
   }
   const int f = cuda_status(cudaFreeAsync(scratch, st));

@@ -208,8 +208,8 @@ int sm_count();
 // return cost a launch 4 us at 8 per SM, 8 at 16 and 14 at 32 (few fit at a time:
 // their registers); fewer blocks cost the FP64 kernels a last wave that is
 // longer (1 % at 8, half of it at 16).
-inline unsigned beside_grid(long long n, int per_sm = 16) {
-  const long long most = (long long)per_sm * sm_count();
+inline unsigned beside_grid(long long n) {
+  const long long most = 16LL * sm_count();
   return (unsigned)(n < most ? n : most);
 }
 // Sites per parity up to which the fixed-point FP64 operator runs one hop per

@@ -60,32 +60,30 @@ __device__ __forceinline__ void st(double2* __restrict__ out, long long link, co
 }
 
 // FP64 form: bound by the FP64 pipe (10.8 ms at 32^4, 1.2 TFLOP/s).  With a
-// header it runs only when the integer kernels do not serve, in a grid
-// whose blocks return at once otherwise.
+// header it does the whole field only when the integer kernels do not serve,
+// otherwise the fat and Naik links that k_build_links_fx has marked, one per
+// thread (in a launch of its own that cost small lattices 3 us).
 __global__ void __launch_bounds__(128) k_build_links(Dims d, long long V, const double2* __restrict__ U,
                                                      double2* __restrict__ F, double2* __restrict__ Lk, double c1,
-                                                     double cst, double c3, const fx::Header* hd, long long cap) {
-  if (hd && !fx::all_fp64(hd, fx::NEAR_6, V, cap)) return;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < 4 * V;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const int mu = (int)(idx / V);
-    const Pos p = pos_of(d, idx - (long long)mu * V);
-    st(F, p.lex * 4 + mu, fat_link(d, U, p, mu, c1, cst));
-    st(Lk, p.lex * 4 + mu, naik_link(d, U, p, mu, c3));
-  }
-}
-// The fat and Naik links that k_build_links_fx has marked, one thread each.
-__global__ void __launch_bounds__(128) k_build_marked(Dims d, long long V, const double2* __restrict__ U,
-                                                      const long long* __restrict__ list, double2* __restrict__ F,
-                                                      double2* __restrict__ Lk, double c1, double cst, double c3,
-                                                      const fx::Header* hd, long long cap) {
-  if (fx::all_fp64(hd, fx::NEAR_6, V, cap)) return;
-  const long long n = (long long)__ldcg(&hd->marked);
+                                                     double cst, double c3, const fx::Header* hd,
+                                                     const long long* __restrict__ list, long long cap) {
+  const bool all = !hd || fx::all_fp64(hd, fx::NEAR_6, V, cap);
+  const long long n = all ? 8 * V : (long long)__ldcg(&hd->marked);
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const long long at = __ldcg(list + i), link = at >> 1;
+    long long link;  // 4 site + mu; a warp of the whole field shares mu and the kind
+    int kind;
+    if (all) {
+      const long long q = i / V;
+      kind = q >= 4;
+      link = 4 * (i - q * V) + (q & 3);
+    } else {
+      const long long at = __ldcg(list + i);
+      kind = (int)(at & 1);
+      link = at >> 1;
+    }
     const int mu = (int)(link & 3);
     const Pos p = pos_of(d, link >> 2);
-    if (at & 1)
+    if (kind)
       st(Lk, link, naik_link(d, U, p, mu, c3));
     else
       st(F, link, fat_link(d, U, p, mu, c1, cst));
@@ -114,7 +112,8 @@ template <bool FAT>
 __global__ void __launch_bounds__(128, FAT ? 2 : 3) k_build_links_fx(Dims d, long long V, const int4* __restrict__ U,
                                                         fx::Header* hd, long long* __restrict__ list, long long cap,
                                                         double2* __restrict__ out, fx::Coef c1, fx::Coef cst, int k) {
-  if (!fx::serve(hd, fx::NEAR_6, V)) return;
+  unsigned long long near = 0;
+  if (!fx::serve(hd, fx::NEAR_6, V, &near)) return;
   __shared__ double2 sm[fx::TS * fx::SITE_W];
   const long long x0 = (long long)blockIdx.x * fx::TS;
   const int ns = (int)(V - x0 < fx::TS ? V - x0 : fx::TS);
@@ -149,14 +148,16 @@ __global__ void __launch_bounds__(128, FAT ? 2 : 3) k_build_links_fx(Dims d, lon
 #pragma unroll
       for (int e = 0; e < 18; ++e) acc[e] = fx::scaled(c1, acc[e]);
     }
-    int size = 0;  // the largest off-diagonal entry, in units of 2^-28
 #pragma unroll
-    for (int e = 0; e < 9; ++e) {
-      o[e] = make_double2(fx::double_of(acc[2 * e], k), fx::double_of(acc[2 * e + 1], k));
-      if (e % 4) size = max(size, max(abs((int)(acc[2 * e] >> 32)), abs((int)(acc[2 * e + 1] >> 32))));
+    for (int e = 0; e < 9; ++e) o[e] = make_double2(fx::double_of(acc[2 * e], k), fx::double_of(acc[2 * e + 1], k));
+    if (near != 0) {
+      int size = 0;  // the largest off-diagonal entry, in units of 2^-28
+#pragma unroll
+      for (int e = 0; e < 9; ++e)
+        if (e % 4) size = max(size, max(abs((int)(acc[2 * e] >> 32)), abs((int)(acc[2 * e + 1] >> 32))));
+      if (size < 3 << 21 && fx::away(fx::ld<4>(U, mu, p.lex)) < 3 << 24)
+        fx::mark(hd, list, cap, (4LL * p.lex + mu) * 2 + (FAT ? 0 : 1));
     }
-    if (size < 3 << 21 && fx::away(fx::ld<4>(U, mu, p.lex)) < 3 << 24)
-      fx::mark(hd, list, cap, (4LL * p.lex + mu) * 2 + (FAT ? 0 : 1));
   }
   __syncthreads();
   for (int i = threadIdx.x; i < ns * 36; i += 128) out[x0 * 36 + i] = sm[(i / 36) * fx::SITE_W + i % 36];
@@ -187,11 +188,11 @@ extern "C" int stag_build_links(const int dims[4], const void* thin, void* fat, 
   cudaStream_t st = (cudaStream_t)stream;
   const double2* U = (const double2*)thin;
   const long long cap = 4 * V;  // marked results that the list holds (of 8 V)
-  auto fp64 = [&](const fx::Header* hd) {
+  auto fp64 = [&](const fx::Header* hd, const long long* list) {
     ProfScope ps("links", st);
-    const long long want = (4 * V + 127) / 128;
+    const long long want = (8 * V + 127) / 128;
     const unsigned grid = hd ? beside_grid(want) : (unsigned)want;
-    lb::k_build_links<<<grid, 128, 0, st>>>(d, V, U, (double2*)fat, (double2*)lng, c1, c_staple, c3, hd, cap);
+    lb::k_build_links<<<grid, 128, 0, st>>>(d, V, U, (double2*)fat, (double2*)lng, c1, c_staple, c3, hd, list, cap);
     return last_launch_status();
   };
   // Coefficients as fixed point with a power of two taken out; beyond 2^+-900
@@ -199,7 +200,7 @@ extern "C" int stag_build_links(const int dims[4], const void* thin, void* fat, 
   const double big = std::fmax(std::fabs(c1), 8.0 * std::fabs(c_staple)), big3 = std::fabs(c3);
   int k = 0, k3 = 0;
   if (!(big > 0x1p-900 && big < 0x1p900 && big3 > 0x1p-900 && big3 < 0x1p900) || c1 != c1 || c_staple != c_staple)
-    return fp64(nullptr);
+    return fp64(nullptr, nullptr);
   std::frexp(big, &k);
   std::frexp(big3, &k3);
   // the fixed-point copy of the links and the list (608 B per site) in stream-ordered
@@ -208,7 +209,7 @@ extern "C" int stag_build_links(const int dims[4], const void* thin, void* fat, 
   char* scratch = nullptr;
   if (cudaMallocAsync((void**)&scratch, 256 + fbytes + (size_t)cap * sizeof(long long), st) != cudaSuccess) {
     cudaGetLastError();
-    return fp64(nullptr);
+    return fp64(nullptr, nullptr);
   }
   fx::Header* hd = (fx::Header*)scratch;
   int4* Uf = (int4*)(scratch + 256);
@@ -232,13 +233,7 @@ extern "C" int stag_build_links(const int dims[4], const void* thin, void* fat, 
                                                        fx::make_coef(std::ldexp(c3, -k3)), none, k3 - 60);
     s = last_launch_status();
   }
-  if (!s) {
-    ProfScope ps("links", st);
-    const long long want = (cap + 127) / 128;
-    lb::k_build_marked<<<beside_grid(want, 4), 128, 0, st>>>(d, V, U, list, (double2*)fat, (double2*)lng, c1, c_staple, c3, hd, cap);
-    s = last_launch_status();
-  }
-  if (!s) s = fp64(hd);
+  if (!s) s = fp64(hd, list);
   const int f = cuda_status(cudaFreeAsync(scratch, st));
   return s ? s : f;
 }
